@@ -23,6 +23,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // range of the work unit, keeps the running maximum M, S = sum exp(z-M), A = sum exp(z-M) z and
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
 struct EpiStats {
+  static constexpr bool kTileFlags = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;   // [rows] compact sampled-token ids
@@ -103,6 +104,116 @@ struct EpiStats {
 };
 
 // ---------------------------------------------------------------------------------------------
+// 16-bit logarithmic code of exp(z - m): what the one-sweep path keeps of a logit between the pass that forms it and the
+// point where the row's log-sum-exp and loss coefficients are known.  With t = (z - m) log2(e) and m an estimate of
+// the log-sum-exp of the row, code = round(max(1024 t + 57344, 512 t + 38912)) clamped at 0: steps of 2^-10 of an
+// octave down to t = -36 (relative error of p at most 2^-11.5, an eighth of the bf16 rounding that follows; rms of
+// the two together 0.7 % above bf16 alone), 2^-9 of an octave down to t = -76.  t reaches up to 8 before the code
+// leaves 16 bits: rows whose estimate is that far off are recomputed (kCodeTop, kCodeLow below).
+constexpr float kCodeSlope1 = 1024.f, kCodeBase1 = 57344.f, kCodeSlope2 = 512.f, kCodeBase2 = 38912.f;
+constexpr float kCodeTop = 7.9f;    // largest t of a row that its codes can hold
+constexpr float kCodeLow = -14.f;   // least log2 of the row's sum of exp(z - m): below, too little of the fine range is left
+
+// p's exponent t of the code in the low 16 bits of the float 2^23 + code.
+__device__ __forceinline__ float code_exponent(float f) {
+  return fminf(fmaf(f, 1.f / kCodeSlope1, -(8388608.f + kCodeBase1) / kCodeSlope1),
+               fmaf(f, 1.f / kCodeSlope2, -(8388608.f + kCodeBase2) / kCodeSlope2));
+}
+
+// 32 rows x 32 columns of 16-bit values (two per word, one row per lane) into one half of a 128-byte-swizzled 32 x 64
+// box; c = index of the 32-column chunk.  The second half hands the box to the TMA unit.
+__device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, uint32_t staging, uint32_t& n_issued,
+                                               const CUtensorMap* map, int col, int row0) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t buf = staging + (n_issued & 1u) * 4096u;
+  if ((c & 1) == 0) {
+    // first half of a new box: the store issued from this buffer two boxes ago must have read it
+    if (lane == 0) bulk_wait_group_read<1>();
+    __syncwarp();
+  }
+  // row `lane` of the box is 128 bytes = 8 chunks of 8 values; chunk j sits at position j ^ (row & 7)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t jj = uint32_t(4 * (c & 1) + j);
+    const uint32_t addr = buf + lane * 128u + ((jj ^ uint32_t(lane & 7)) << 4);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[4 * j]), "r"(w[4 * j + 1]),
+                 "r"(w[4 * j + 2]), "r"(w[4 * j + 3])
+                 : "memory");
+  }
+  if (c & 1) {
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_2d(map, buf, col - 32, row0);
+      bulk_commit_group();
+    }
+    n_issued++;
+  }
+}
+
+// Forward statistics of EpiStats for one slab of rows, plus the code of every logit written to the slab scratch (the
+// place the gradient with respect to the logits then takes).  Forming the logits once instead of twice (statistics,
+// then recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  At d = 2048 the extra
+// arithmetic (about 3 instructions per logit on top of the statistics' 3) still hides behind the next tile's MMAs.
+struct EpiSweep {
+  static constexpr bool kTileFlags = false;
+  static constexpr int kStagingBytes = 4 * kStagingPerWarp;
+  struct Params {
+    EpiStats::Params stats;
+    const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
+  };
+  struct State {
+    EpiStats::State s;
+    float k1, k2;
+    uint32_t n_issued;
+    int grow;   // compact row
+  };
+  __device__ static __forceinline__ void init(State& st) { st.n_issued = 0; }
+  __device__ static __forceinline__ void finish(State& st) {
+    if ((threadIdx.x & 31) == 0 && st.n_issued) bulk_wait_group_all();
+    __syncwarp();
+  }
+  __device__ static __forceinline__ void begin_unit(const Params& p, State& st, int m_tile, int, int row_in_tile,
+                                                    int m_rows, int slab_off, int) {
+    const int rl = m_tile * BM + row_in_tile;
+    const bool valid = rl < m_rows;
+    st.grow = valid ? slab_off + rl : -1;
+    st.s.m = -CUDART_INF_F;
+    st.s.s = 0.f;
+    st.s.a = 0.f;
+    st.s.zy = 0.f;
+    st.s.y = valid ? p.stats.tokens_c[st.grow] : -1;
+    const float sh = valid ? p.shift2[st.grow] : 0.f;
+    st.k1 = fmaf(-kCodeSlope1, sh, kCodeBase1);
+    st.k2 = fmaf(-kCodeSlope2, sh, kCodeBase2);
+  }
+  __device__ static __forceinline__ void chunk(const Params& p, State& st, int m_tile, int n_tile, int c,
+                                               int row_in_tile, int m_rows, const float (&v)[32],
+                                               const CUtensorMap* map, uint32_t staging) {
+    // a CTA pair may own a 128-row tile that lies wholly past the slab's rows: nothing to write
+    if (m_tile * BM >= ((m_rows + BM - 1) / BM) * BM) return;
+    EpiStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
+    const float2 a1 = make_float2(kLog2e * kCodeSlope1, kLog2e * kCodeSlope1), b1 = make_float2(st.k1, st.k1);
+    const float2 a2 = make_float2(kLog2e * kCodeSlope2, kLog2e * kCodeSlope2), b2 = make_float2(st.k2, st.k2);
+    const float2 magic = make_float2(8388608.f, 8388608.f);   // low 16 bits of 2^23 + x are round(x)
+    uint32_t w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float2 z2 = make_float2(v[2 * i], v[2 * i + 1]);
+      const float2 x = __ffma2_rn(z2, a1, b1), y = __ffma2_rn(z2, a2, b2);
+      const float2 q = __fadd2_rn(make_float2(fmaxf(fmaxf(x.x, y.x), 0.f), fmaxf(fmaxf(x.y, y.y), 0.f)), magic);
+      w[i] = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x5410);
+    }
+    const int lane = threadIdx.x & 31;
+    stage_half_box(w, c, staging, st.n_issued, map, n_tile * BN + c * 32, m_tile * BM + (row_in_tile - lane));
+  }
+  __device__ static __forceinline__ void end_unit(const Params& p, State& st, int, int nr, int, int) {
+    if (st.grow >= 0)
+      p.stats.partials[(size_t)nr * p.stats.part_stride + st.grow] = make_float4(st.s.m, st.s.s, st.s.a, st.s.zy);
+  }
+};
+
+// ---------------------------------------------------------------------------------------------
 // Gradient with respect to the logits for one slab of rows x vocabulary columns, rounded to
 // bf16 and written to the slab scratch (row-major) by bulk tensor stores: each epilogue warp packs
 // two consecutive 32-column chunks of its 32 rows into a 128-byte-swizzled 32x64 bf16 box in
@@ -111,6 +222,7 @@ struct EpiStats {
 // cp_t = -w_t dloss_t/dlogp_t and ce_t = w_t ent_coef come from the per-token loss kernel.
 // Rows past the valid rows of the slab and columns past V are written as zero.
 struct EpiGrad {
+  static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     const int* tokens_c;
@@ -195,36 +307,14 @@ struct EpiGrad {
         for (int i = 0; i < 32; ++i) g[i] = i < nvalid ? g[i] : 0.f;
       }
     }
-    const int lane = threadIdx.x & 31;
-    const uint32_t buf = staging + (st.n_issued & 1u) * 4096u;
-    if ((c & 1) == 0) {
-      // first half of a new box: the store issued from this buffer two boxes ago must have read it
-      if (lane == 0) bulk_wait_group_read<1>();
-      __syncwarp();
-    }
-    // row `lane` of the box is 128 bytes = 8 chunks of 8 bf16; chunk j sits at position j ^ (row & 7)
+    uint32_t w[16];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      __nv_bfloat162 b0 = __floats2bfloat162_rn(g[8 * j + 0], g[8 * j + 1]);
-      __nv_bfloat162 b1 = __floats2bfloat162_rn(g[8 * j + 2], g[8 * j + 3]);
-      __nv_bfloat162 b2 = __floats2bfloat162_rn(g[8 * j + 4], g[8 * j + 5]);
-      __nv_bfloat162 b3 = __floats2bfloat162_rn(g[8 * j + 6], g[8 * j + 7]);
-      const uint32_t jj = uint32_t(4 * (c & 1) + j);
-      const uint32_t addr = buf + lane * 128u + ((jj ^ uint32_t(lane & 7)) << 4);
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(*reinterpret_cast<uint32_t*>(&b0)),
-                   "r"(*reinterpret_cast<uint32_t*>(&b1)), "r"(*reinterpret_cast<uint32_t*>(&b2)),
-                   "r"(*reinterpret_cast<uint32_t*>(&b3))
-                   : "memory");
+    for (int i = 0; i < 16; ++i) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(g[2 * i], g[2 * i + 1]);
+      w[i] = *reinterpret_cast<const uint32_t*>(&b);
     }
-    if (c & 1) {
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) {
-        tma_store_2d(tmG, buf, col_l - 32, m_tile * BM + (row_in_tile - lane));
-        bulk_commit_group();
-      }
-      st.n_issued++;
-    }
+    const int lane = threadIdx.x & 31;
+    stage_half_box(w, c, staging, st.n_issued, tmG, col_l, m_tile * BM + (row_in_tile - lane));
   }
   __device__ static __forceinline__ void end_unit(const Params&, State&, int, int, int, int) {}
 };
@@ -237,6 +327,7 @@ struct EpiGrad {
 // also clips rows past the tensor.  Every element is written by exactly one tile per launch, so
 // the result does not depend on timing.
 struct EpiAcc {
+  static constexpr bool kTileFlags = false;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     int n_cols;

@@ -60,6 +60,7 @@ constexpr int kGemmSmemBytes = kTileSmemBytes + 1024;  // + slack for 1024-byte 
 constexpr int kStagingPerWarp = 8192;                  // two 32x32 fp32 boxes per epilogue warp
 constexpr int kTmemCols = 512;
 constexpr int kMaxSplit = 16;   // most column ranges per row tile when the split is chosen to fill the machine
+constexpr int kFlagRows = 256;  // rows one entry of GemmShape::tile_flags stands for
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
 
 enum TileMode { kTileSquare = 0, kTileWide = 1, kTileDual = 2 };
@@ -133,6 +134,10 @@ struct GemmShape {
   // walked for one group before the next group starts, so that the A panels the CTAs running at any
   // moment keep re-reading stay in L2; B is then fetched once per group instead of once per launch.
   int m_group;
+  // Row-tile selection: when tile_flags is set, only row tiles whose flag (indexed from the slab's first row, one per
+  // kFlagRows rows) is non-zero are walked, and the launch returns at once when *flag_count is 0.
+  const int* tile_flags;
+  const int* flag_count;
   // coordinate offsets into the operands' global tensors
   int a_mn_off, a_k_off, b_mn_off, b_k_off;
 };
@@ -170,6 +175,7 @@ __host__ __device__ inline int choose_range(int m_units, int n_tiles, int n_work
 }
 
 struct GemmExtents {
+  int tile_rows;   // rows of one row tile (BM x CTAs per tile)
   int m_rows, m_units, k_blocks, n_range, n_ranges, n_units, slab_off, k_split, kb_per, stream_k, m_group;
 };
 
@@ -213,6 +219,7 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
   e.m_rows = sh.m_dyn ? m : sh.m_rows_cap;
   k = k < 0 ? 0 : (k > sh.k_cap ? sh.k_cap : k);
   const int k_len = sh.k_dyn ? k : sh.k_cap;
+  e.tile_rows = BM * cg;
   e.m_units = (e.m_rows + BM * cg - 1) / (BM * cg);
   e.k_blocks = (k_len + BK - 1) / BK;
   const bool plenty = (long)e.m_units * ((sh.n_tiles + kFwdRange - 1) / kFwdRange) >= 4L * n_workers;
@@ -272,6 +279,8 @@ __host__ __device__ inline void unit_coords(const GemmShape& sh, const GemmExten
 // remaining tiles (between one and two per worker) are balanced: their (tile, k-block) iterations,
 // tile-major, are cut into one contiguous share per worker, one unit per tile a share touches; ks
 // is then the output slice of the part: 0 when it starts at k-block 0, else 1.
+// FLAGS: row tiles whose GemmShape::tile_flags entry is zero are passed over.
+template <bool FLAGS = false>
 struct UnitWalk {
   const GemmShape& sh;
   const GemmExtents& ex;
@@ -287,9 +296,10 @@ struct UnitWalk {
     }
   }
   __host__ __device__ inline bool next(int& mu, int& nr, int& ks, int& kb0, int& kb1) {
-    if (u < plain_units) {
+    while (u < plain_units) {
       unit_coords(sh, ex, u, mu, nr, ks, kb0, kb1);
       u += n_workers;
+      if (FLAGS && sh.tile_flags && !sh.tile_flags[(ex.slab_off + mu * ex.tile_rows) / kFlagRows]) continue;
       return true;
     }
     if (it >= it_end) return false;
@@ -313,7 +323,8 @@ struct UnitWalk {
 //                       const CUtensorMap* out_map, uint32_t staging);
 //     static void end_unit(const Params&, State&, int m_tile, int n_range_idx, int row_in_tile, int m_rows);
 //     static void init(State&); static void finish(State&);     // once per kernel, per thread
-//     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB) };
+//     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
+//     static constexpr bool kTileFlags; };                     // launches may be restricted by GemmShape::tile_flags
 //   kTileDual: chunk receives the chunk of the second product as well (..., v, v2, out_map, staging).
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
 // sh.n_tiles then counts 512-wide tiles).  tmA2 / tmB2 / k2_len are read by kTileDual only.
@@ -323,6 +334,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
             const typename Epi::Params ep, DevStatus* status) {
+  if (Epi::kTileFlags && sh.flag_count && *sh.flag_count == 0) return;   // no flagged row tile
   static_assert(MODE != kTileWide || CG == 2, "wide tiles run on CTA pairs");
   static_assert(MODE != kTileDual || (A_MN == 0 && B_MN == 0), "the two-product mode takes K-major operands");
   using Cfg = StageCfg<CG, MODE, Epi::kStagingBytes>;
@@ -376,7 +388,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      UnitWalk walk(sh, ex, worker, n_workers);
+      UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
       int mu, nr, ks, kb0, kb1;
       while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
         const int m = mu * CG + (int)rank;
@@ -463,7 +475,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       uint32_t t = 0;   // tiles issued so far
       bool ok = true;
       if (run && ex.k_blocks > 0) {
-        UnitWalk walk(sh, ex, worker, n_workers);
+        UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
         int mu, nr, ks, kb0, kb1;
         while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
           if (kb1 <= kb0) continue;   // empty K slice: the epilogue handles it without an accumulator
@@ -539,7 +551,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     Epi::init(st);
     uint32_t t = 0;
     bool ok = true;
-    UnitWalk walk(sh, ex, worker, n_workers);
+    UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
     int mu, nr, ks, kb0, kb1;
     while (ok && run && walk.next(mu, nr, ks, kb0, kb1)) {
       const bool has_k = kb1 > kb0;   // an empty K slice contributes zeros

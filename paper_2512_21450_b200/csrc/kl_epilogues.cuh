@@ -11,6 +11,7 @@ namespace rlh {
 //   Mr, Sr = running max and sum exp(zr - Mr) of the reference logits (for lse_ref).
 // Two float4 per (range, row): {M, S, A, z_y} and {D, Mr, Sr, 0}.
 struct EpiStatsKL {
+  static constexpr bool kTileFlags = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;
@@ -86,6 +87,7 @@ struct EpiStatsKL {
 //                  + ce_t p_tj (log p_tj + Ent_t),   cb_t = w_t beta,
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
+  static constexpr bool kTileFlags = false;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     const int* tokens_c;

@@ -33,6 +33,7 @@ struct rl_ctx {
   EncodeTiledFn encode;
   int slab_rows;  // rows of one gradient slab (multiple of 128)
   int slab_cols;  // vocabulary columns of one gradient slab (multiple of 256)
+  int slab_auto;  // 1: rl_set_slab_limits() left the slab's shape to the library (whole rows where they fit)
   int cta_group;  // 1: one CTA per 128x256 tile; 2: CTA pairs on 256x256 tiles
   int dh_k_slices;  // upper bound on the K slices of the dH pass (1 = tiles are not cut)
   long long row_group_bytes;  // forward / dlogits: bytes of A panels walked together (0 = all row tiles at once)
@@ -59,6 +60,12 @@ namespace {
 
 constexpr long long kRowGroupBytes = 36ll << 20;   // A panels walked together by the rows-first passes (L2 is 126 MB)
 constexpr int kSlabRowsMax = 32768;        // rows of one gradient slab
+// Slab shape when the caller sets none: rows over the WHOLE vocabulary, as many as kSlabElements allows (14080 rows at
+// 152 K words, 4.3 GB).  A row that is complete in the slab needs its logits formed only once.  Fewer rows per slab mean
+// more passes over dW (8 bytes per entry and slab, beside 10 bytes per entry of the slab itself); below
+// kSlabRowsMin rows a slab is cut by columns instead.
+constexpr long long kSlabElements = 1ll << 31;
+constexpr int kSlabRowsMin = 2048;
 // Device words a context owns besides the workspace: the status record, a few scalars of the small kernels
 // (byte 64: batch statistics, 96: longest response, 128: valid-row count of rl_token_loss) and, from byte 256 on,
 // the block partials of rl_token_loss.
@@ -77,6 +84,8 @@ inline int dh_buffers(const rl_ctx* c) { return dh_uses_stream_k(c) ? 2 : c->dh_
 struct WsLayout {
   int Tpad, Ts, Vs;
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
+  size_t shift2, flags;                              // one-sweep path: log-sum-exp estimates, row-tile flags
+  int n_row_slabs, n_flags;                          // n_flags: row tiles, then one count per row slab
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
 };
 
@@ -121,9 +130,18 @@ inline size_t carve_stage(char* base, int64_t T, int64_t d, HostStage* hs) {
 WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_slots, int64_t d_ref = 0) {
   WsLayout L;
   L.Tpad = (int)align_up((size_t)(T > 0 ? T : 1), 128);
-  L.Ts = L.Tpad < c->slab_rows ? L.Tpad : c->slab_rows;
   const int Vpad = (int)align_up((size_t)V, 256);
+  long long rows = c->slab_rows;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
+  if (c->slab_auto) {
+    const long long whole = kSlabElements / Vpad / 256 * 256;
+    if (whole >= kSlabRowsMin || whole >= L.Tpad) {
+      rows = whole < kSlabRowsMax ? whole : kSlabRowsMax;
+      L.Vs = Vpad;
+    }
+  }
+  L.Ts = L.Tpad < rows ? L.Tpad : (int)rows;
+  L.n_row_slabs = (L.Tpad + L.Ts - 1) / L.Ts;
   size_t o = 0;
   size_t n_part_ranges = kMaxSplit;
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 1024); return at; };
@@ -145,6 +163,9 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.Hc = take((size_t)L.Tpad * d * 2);
   L.G = take((size_t)L.Ts * L.Vs * 2);
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
+  L.shift2 = take((size_t)L.Tpad * 4);
+  L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
+  L.flags = take((size_t)L.n_flags * 4);
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
@@ -338,6 +359,7 @@ struct FwdPlan {
   bool stats = true;         // tensor-core pass that leaves per-range statistics in the workspace
   int64_t vocab_off = 0;     // first vocabulary id of W's rows (vocabulary-parallel head)
   int64_t V_total = 0;       // size of the whole vocabulary for the token-range check (0: V)
+  const float* old_logp = nullptr;   // one-sweep path: estimate every row's log-sum-exp while its row is copied
 };
 
 // Mask scan + row compaction + forward statistics.  Leaves per-range partials in the workspace.
@@ -358,10 +380,20 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     prof_end(c, pr, 4);
     c->launches += 3;
   }
+  SweepPrep sp;
+  memset(&sp, 0, sizeof(sp));
+  if (plan.old_logp) {
+    sp.W = static_cast<const __nv_bfloat16*>(W);
+    sp.ldW = ldW;
+    sp.old_logp = plan.old_logp;
+    sp.shift2 = reinterpret_cast<float*>(ws + L.shift2);
+    sp.flags = reinterpret_cast<int*>(ws + L.flags);
+    sp.n_flags = L.n_flags;
+  }
   const int pr_gather = prof_begin(c, 5);
   gather_rows_kernel<<<c->n_sm * 4, 256, 0, c->stream>>>(static_cast<const __nv_bfloat16*>(H), ldH, (int)d, row_map,
                                                          tokens, (int)(plan.V_total > 0 ? plan.V_total : V),
-                                                         (int)plan.vocab_off, Hc, tokens_c, c->dstatus);
+                                                         (int)plan.vocab_off, Hc, tokens_c, sp, c->dstatus);
   prof_end(c, pr_gather, 5);
   c->launches += 1;
   if (!plan.stats) {
@@ -445,6 +477,7 @@ rl_status rl_create(rl_ctx** out, int device) {
   c->ws_bytes = 0;
   c->slab_rows = kSlabRowsMax;
   c->slab_cols = kSlabColsMax;
+  c->slab_auto = 1;
   c->cta_group = 1;
   c->dh_k_slices = 1;
   c->dh_stream_k = 0;
@@ -472,6 +505,7 @@ rl_status rl_create(rl_ctx** out, int device) {
   if (cudaMalloc(&c->dstatus, kStatusBytes) != cudaSuccess) { delete c; return RL_ERR_CUDA; }
   cudaMemset(c->dstatus, 0, kStatusBytes);
   bool ok = set_smem_attr<EpiStats, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiSweep, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
@@ -653,12 +687,14 @@ rl_status rl_profile_read(rl_ctx* c, double* ms, int64_t* launches) {
 
 rl_status rl_set_slab_limits(rl_ctx* c, int max_rows, int max_cols) {
   if (!c) return RL_ERR_INVALID_ARG;
+  const int automatic = max_rows == 0 && max_cols == 0;
   if (max_rows == 0) max_rows = kSlabRowsMax;
   if (max_cols == 0) max_cols = kSlabColsMax;
   if (max_rows < 128 || max_rows % 128 != 0 || max_cols < 256 || max_cols % 256 != 0) return RL_ERR_SHAPE;
   if ((int64_t)max_rows * max_cols > (int64_t(1) << 31)) return RL_ERR_SHAPE;
   c->slab_rows = max_rows;
   c->slab_cols = max_cols;
+  c->slab_auto = automatic;
   return RL_OK;
 }
 
@@ -961,9 +997,19 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   if (o.logp_out) cudaMemsetAsync(o.logp_out, 0, (size_t)T * 4, st);
   if (o.entropy_out) cudaMemsetAsync(o.entropy_out, 0, (size_t)T * 4, st);
 
-  // ---- forward: statistics per (row, vocabulary range)
+  // ---- forward: statistics per (row, vocabulary range).  One sweep: a slab that holds whole rows lets the pass that
+  // forms their logits leave them there as 16-bit codes, which an elementwise pass turns into the gradient once the
+  // rows' coefficients are known.  Not where the coefficients of a row need rows of another slab, nor where the
+  // statistics come from elsewhere: those paths form the logits a second time.
+  const int Vpad = (int)align_up((size_t)V, 256);
+  const bool sweep = L.Vs == Vpad && !shard && !o.kl_full &&
+                     (L.n_row_slabs == 1 || (L.Ts % kFlagRows == 0 && !seq_path));
   GemmShape fwd_shape;
   FwdPlan plan;
+  if (sweep) {
+    plan.stats = false;
+    plan.old_logp = old_logp;
+  }
   if (shard) {
     // the statistics of the whole vocabulary are given: only the row compaction is needed
     plan.stats = false;
@@ -997,6 +1043,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
   p.cp_c = reinterpret_cast<float*>(ws + L.cp_c);
   p.ce_c = reinterpret_cast<float*>(ws + L.ce_c);
+  if (sweep || seq_path) p.logp_c = reinterpret_cast<float*>(ws + L.logp_c);
   p.logp_out = o.logp_out;
   p.ent_out = o.entropy_out;
   p.block_sums = reinterpret_cast<double*>(ws + L.block_sums);
@@ -1014,47 +1061,61 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     p.kl_out = o.kl_out;
     if (o.kl_out) cudaMemsetAsync(o.kl_out, 0, (size_t)T * 4, st);
   }
-  int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
-  if (blocks > 1024) blocks = 1024;
-  const int pr_loss = prof_begin(c, 6);
-  if (!seq_path) {
-    combine_loss_kernel<<<blocks, kLossThreads, 0, st>>>(p, c->dstatus);
+  int blocks = 0;   // blocks whose partial sums make up the loss
+  // merge of slab r (one sweep) or of all rows, then the loss and the coefficients of the backward pass
+  auto merge_and_loss = [&](int r) {
+    const int rows_cap = sweep ? L.Ts : (int)T;
+    int nb = (rows_cap + kLossThreads - 1) / kLossThreads;
+    const int nb_max = 1024 / (sweep ? L.n_row_slabs : 1);
+    if (nb > nb_max) nb = nb_max;
+    const int pr_loss = prof_begin(c, 6);
+    if (!seq_path) {
+      LossParams ps = p;
+      ps.block_sums = p.block_sums + (size_t)r * nb * kLossSums;
+      blocks = (r + 1) * nb;
+      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(ps, c->dstatus);
+      c->launches++;
+    } else {
+      // merge the statistics first, then one warp per response forms weights, ratios and the loss
+      p.with_loss = 0;
+      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(p, c->dstatus);
+      SeqParams q;
+      memset(&q, 0, sizeof(q));
+      q.seq_offsets = o.seq_offsets;
+      q.n_seq = (int)o.n_seq;
+      q.agg_mode = o.token_weight ? 0 : o.agg_mode;
+      q.sequence_level = o.sequence_level ? 1 : 0;
+      q.row_map = p.row_map;
+      q.logp_c = p.logp_c;
+      q.ent_c = p.ent_c;
+      q.old_logp = old_logp;
+      q.ref_logp = ref_logp;
+      q.adv = adv;
+      q.token_weight = o.token_weight;
+      q.eps_low = eps_low; q.eps_high = eps_high; q.beta = beta; q.ent_coef = o.ent_coef;
+      q.l_max = reinterpret_cast<int*>(reinterpret_cast<char*>(c->dstatus) + 96);
+      q.cp_c = p.cp_c;
+      q.ce_c = p.ce_c;
+      q.block_sums = p.block_sums;
+      // valid rows that lie outside every response range take no part: their coefficients stay 0
+      cudaMemsetAsync(q.cp_c, 0, (size_t)L.Tpad * 4, st);
+      cudaMemsetAsync(q.ce_c, 0, (size_t)L.Tpad * 4, st);
+      seq_lmax_kernel<<<1, 1024, 0, st>>>(o.seq_offsets, (int)o.n_seq, q.l_max);
+      blocks = (int)((o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32));
+      if (blocks > 1024) blocks = 1024;
+      seq_loss_kernel<<<blocks, kLossThreads, 0, st>>>(q, c->dstatus);
+      c->launches += 3;
+    }
+    prof_end(c, pr_loss, 6);
+  };
+  auto finalize = [&]() {
+    finalize_loss_kernel<<<1, 32 * kLossSums, 0, st>>>(p.block_sums, blocks, loss, o.metrics_out, c->dstatus);
     c->launches++;
-  } else {
-    // merge the statistics first, then one warp per response forms weights, ratios and the loss
-    p.with_loss = 0;
-    p.logp_c = reinterpret_cast<float*>(ws + L.logp_c);
-    combine_loss_kernel<<<blocks, kLossThreads, 0, st>>>(p, c->dstatus);
-    SeqParams q;
-    memset(&q, 0, sizeof(q));
-    q.seq_offsets = o.seq_offsets;
-    q.n_seq = (int)o.n_seq;
-    q.agg_mode = o.token_weight ? 0 : o.agg_mode;
-    q.sequence_level = o.sequence_level ? 1 : 0;
-    q.row_map = p.row_map;
-    q.logp_c = p.logp_c;
-    q.ent_c = p.ent_c;
-    q.old_logp = old_logp;
-    q.ref_logp = ref_logp;
-    q.adv = adv;
-    q.token_weight = o.token_weight;
-    q.eps_low = eps_low; q.eps_high = eps_high; q.beta = beta; q.ent_coef = o.ent_coef;
-    q.l_max = reinterpret_cast<int*>(reinterpret_cast<char*>(c->dstatus) + 96);
-    q.cp_c = p.cp_c;
-    q.ce_c = p.ce_c;
-    q.block_sums = p.block_sums;
-    // valid rows that lie outside every response range take no part: their coefficients stay 0
-    cudaMemsetAsync(q.cp_c, 0, (size_t)L.Tpad * 4, st);
-    cudaMemsetAsync(q.ce_c, 0, (size_t)L.Tpad * 4, st);
-    seq_lmax_kernel<<<1, 1024, 0, st>>>(o.seq_offsets, (int)o.n_seq, q.l_max);
-    blocks = (int)((o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32));
-    if (blocks > 1024) blocks = 1024;
-    seq_loss_kernel<<<blocks, kLossThreads, 0, st>>>(q, c->dstatus);
-    c->launches += 3;
+  };
+  if (!sweep) {
+    merge_and_loss(0);
+    finalize();
   }
-  finalize_loss_kernel<<<1, 32 * kLossSums, 0, st>>>(p.block_sums, blocks, loss, o.metrics_out, c->dstatus);
-  prof_end(c, pr_loss, 6);
-  c->launches++;
 
   // ---- backward, one (row slab x vocabulary slab) at a time
   __nv_bfloat16* Hc = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc);
@@ -1080,9 +1141,10 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             map_out_f32(c, &tm_dW, dW, (uint64_t)V, (uint64_t)d, (uint64_t)d, 1, (uint64_t)V);
   if (!ok) return RL_ERR_CUDA;
 
-  const int n_row_slabs = (L.Tpad + L.Ts - 1) / L.Ts;
+  const int n_row_slabs = L.n_row_slabs;
   const int n_col_slabs = (int)((V + L.Vs - 1) / L.Vs);
   const int d_tiles = (int)((d + BN - 1) / BN);
+  int hook_slab = 0;
   for (int r = 0; r < n_row_slabs; ++r) {
     GemmShape dh_shape;
     memset(&dh_shape, 0, sizeof(dh_shape));
@@ -1092,8 +1154,46 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     for (int cs = 0; cs < n_col_slabs; ++cs) {
       const int vocab_base = cs * L.Vs;
       const int cols = (int)((V - vocab_base) < L.Vs ? (V - vocab_base) : L.Vs);
-      // (1) recompute the logits of the slab, write G = dloss/dlogits as bf16
+      // (1) the slab's G = dloss/dlogits as bf16: from the codes of a first pass, or by forming the logits again
       {
+        int* flags = reinterpret_cast<int*>(ws + L.flags);
+        int* flag_count = flags + (L.n_flags - n_row_slabs) + r;
+        if (sweep) {
+          GemmShape sw;
+          memset(&sw, 0, sizeof(sw));
+          sw.n_valid = n_valid;
+          sw.m_rows_cap = rows_cap; sw.m_dyn = 1; sw.slab_cap = L.Ts; sw.slab_index = r;
+          sw.k_cap = (int)d;
+          sw.n_tiles = (cols + BN - 1) / BN;
+          sw.a_mn_slab = 1;
+          sw.m_group = row_group_tiles(c, d);
+          EpiSweep::Params ep;
+          ep.stats.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
+          ep.stats.partials = reinterpret_cast<float4*>(ws + L.partials);
+          ep.stats.part_stride = L.Tpad;
+          ep.stats.V = (int)V;
+          ep.shift2 = reinterpret_cast<const float*>(ws + L.shift2);
+          launch_gemm<EpiSweep, 0, 0>(c, 0, tmHc_k, tmW_k, tm_G_out, sw, ep);
+          p.fwd_shape = sw;
+          p.slab_cap = L.Ts;
+          p.slab_index = r;
+          p.shift2 = ep.shift2;
+          p.tile_flags = flags;
+          p.flag_count = flag_count;
+          merge_and_loss(r);
+          LogitGradParams lg;
+          lg.slab = reinterpret_cast<uint16_t*>(G);
+          lg.ld = L.Vs;
+          lg.V = (int)V;
+          lg.slab_cap = L.Ts; lg.slab_index = r;
+          lg.tokens_c = ep.stats.tokens_c;
+          lg.shift2 = ep.shift2;
+          lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
+          const int pr_lg = prof_begin(c, 1);
+          logit_grad_kernel<<<c->n_sm * 8, 256, 0, st>>>(lg, c->dstatus);
+          prof_end(c, pr_lg, 1);
+          c->launches++;
+        }
         GemmShape sh;
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
@@ -1104,12 +1204,16 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.a_mn_slab = 1;
         sh.b_mn_off = vocab_base;
         sh.m_group = row_group_tiles(c, d + (o.kl_full ? o.d_ref : 0));
+        if (sweep) {   // only row tiles whose codes could not hold their logits (none as a rule)
+          sh.tile_flags = flags;
+          sh.flag_count = flag_count;
+        }
         if (!o.kl_full) {
           EpiGrad::Params ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.lse = p.lse_c; ep.ent = p.ent_c; ep.cp = p.cp_c; ep.ce = p.ce_c;
           ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_gemm<EpiGrad, 0, 0>(c, 1, tmHc_k, tmW_k, tm_G_out, sh, ep);
+          launch_gemm<EpiGrad, 0, 0>(c, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, sh, ep);
         } else {
           EpiGradKL::Params ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
@@ -1143,29 +1247,36 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           launch_gemm<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, sh, ep);
         }
       }
-      // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab
-      {
+      // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab.  A caller that wants to
+      // be told as rows of dW are completed gets them in pieces.
+      const bool report = c->dw_hook && r == n_row_slabs - 1;
+      const int step = report && cols > kSlabColsMax ? kSlabColsMax : cols;
+      for (int c0 = 0; c0 < cols; c0 += step) {
         GemmShape sh;
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
-        sh.m_rows_cap = cols;
+        sh.m_rows_cap = cols - c0 < step ? cols - c0 : step;
         sh.k_cap = rows_cap; sh.k_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
         sh.n_tiles = d_tiles;
         sh.n_range = 1;
         sh.skip_if_k0 = (r > 0 || o.accumulate_dW) ? 1 : 0;
+        sh.a_mn_off = c0;
         sh.b_k_slab = 1;
         sh.n_fastest = 1;
         EpiAcc::Params ep;
         ep.n_cols = (int)d; ep.accumulate = (r > 0 || o.accumulate_dW) ? 1 : 0;
-        ep.row_base = vocab_base; ep.slice_add = 0;
+        ep.row_base = vocab_base + c0; ep.slice_add = 0;
         if (use_wide(c)) {
           sh.n_tiles = (int)((d + 2 * BN - 1) / (2 * BN));
           launch_wide<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, sh, ep);
         } else {
           launch_gemm<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, sh, ep);
         }
-        // rows [vocab_base, vocab_base + cols) of dW are complete once the last row slab has added to them
-        if (c->dw_hook && r == n_row_slabs - 1) c->dw_hook(c->dw_hook_user, cs, vocab_base, (int64_t)vocab_base + cols);
+        // these rows of dW are complete once the last row slab has added to them
+        if (report) {
+          const int64_t row0 = (int64_t)vocab_base + c0;
+          c->dw_hook(c->dw_hook_user, hook_slab++, row0, row0 + sh.m_rows_cap);
+        }
       }
     }
     const int pr_sc = prof_begin(c, 7);
@@ -1180,6 +1291,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     prof_end(c, pr_sc, 7);
     c->launches++;
   }
+  if (sweep) finalize();
   return cuda_ok();
 }
 
@@ -1506,7 +1618,7 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
   const GemmExtents ex = gemm_extents(sh, nv, cta_group, n_workers);
   int64_t n = 0;
   for (int worker = 0; worker < n_workers; ++worker) {
-    UnitWalk walk(sh, ex, worker, n_workers);
+    UnitWalk<> walk(sh, ex, worker, n_workers);
     int mu, nr, ks, kb0, kb1;
     while (walk.next(mu, nr, ks, kb0, kb1)) {
       if (n < max_units) {

@@ -120,12 +120,26 @@ __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t*
 // vocabulary [0, V) and stored relative to vocab_off, the first id of the rows of W this call
 // holds (0 unless the head is split by vocabulary): an id outside the held slice becomes a
 // negative or too large column that no tile ever matches.
+// SweepPrep (shift2 != NULL): the one-sweep path also needs an estimate of every row's log-sum-exp before its logits are
+// formed.  The behaviour policy supplies it: lse ~ z_y - old_logp, with z_y the sampled token's logit, taken here from
+// the row that is being copied anyway (exact up to the drift between the two policies, which the codes have room for).
+struct SweepPrep {
+  const __nv_bfloat16* W;
+  long long ldW;
+  const float* old_logp;   // [T] original rows
+  float* shift2;           // [rows] compact: the estimate in units of log 2, or NULL
+  int* flags;              // words cleared for the launches that follow
+  int n_flags;
+};
+
 __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* __restrict__ H, long long ldH, int d,
                                                           const int* __restrict__ row_map,
                                                           const int* __restrict__ tokens, int V, int vocab_off,
                                                           __nv_bfloat16* __restrict__ Hc,
-                                                          int* __restrict__ tokens_c, DevStatus* st) {
+                                                          int* __restrict__ tokens_c, const SweepPrep sp,
+                                                          DevStatus* st) {
   const int n = st->n_valid;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sp.n_flags; i += gridDim.x * blockDim.x) sp.flags[i] = 0;
   const int n_pad = (n + 127) / 128 * 128;
   const int lane = threadIdx.x & 31;
   const int warps_per_block = blockDim.x >> 5;
@@ -135,10 +149,31 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* _
     if (i < n) {
       const int r = row_map[i];
       const uint4* src = reinterpret_cast<const uint4*>(H + (size_t)r * ldH);
-      for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
+      const int y = tokens[r];
+      const bool in_range = y >= 0 && y < V;
+      if (sp.shift2) {
+        const uint4* wrow = reinterpret_cast<const uint4*>(sp.W + (size_t)(in_range ? y : 0) * sp.ldW);
+        float2 acc = make_float2(0.f, 0.f);
+        for (int v = lane; v < vec_per_row; v += 32) {
+          const uint4 h = __ldg(src + v), w = __ldg(wrow + v);
+          dst[v] = h;
+          const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
+                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
+        }
+        float z = acc.x + acc.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (lane == 0) {
+          const float est = z - sp.old_logp[r];
+          sp.shift2[i] = (isfinite(est) ? est : 0.f) * kLog2e;
+        }
+      } else {
+        for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
+      }
       if (lane == 0) {
-        const int y = tokens[r];
-        const bool in_range = y >= 0 && y < V;
         tokens_c[i] = in_range ? y - vocab_off : -1;
         if (!in_range) latch_status(st, kStatusTokenRange, r);
       }
@@ -541,6 +576,12 @@ struct LossParams {
   const float* ext_logp;
   const float* ext_ent;
   const float* ext_lse;
+  // one row slab of the one-sweep path (slab_cap > 0): only its rows are merged, and the row tiles whose estimated
+  // log-sum-exp lies too far from the true one for the 16-bit codes are flagged
+  int slab_cap, slab_index;
+  const float* shift2;
+  int* tile_flags;   // [rows / kFlagRows], over all rows
+  int* flag_count;   // non-zero: this slab has a flagged tile
 };
 constexpr int kLossSums = 8;  // loss, pg, kl, ent, clip, ratio, ratio_max, unused
 constexpr int kLossThreads = 256;
@@ -571,7 +612,12 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
   const long long n_mean = p.token_count ? *p.token_count : (long long)n;
   const float w_mean = n_mean > 0 ? (float)(1.0 / (double)n_mean) : 0.f;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  int i_begin = 0, i_end = n;
+  if (p.slab_cap > 0) {
+    slab_extent(n, p.slab_cap, p.slab_index, i_begin, i_end);
+    i_end += i_begin;
+  }
+  for (int i = i_begin + blockIdx.x * blockDim.x + threadIdx.x; i < i_end; i += gridDim.x * blockDim.x) {
     float lse, logp, ent;
     float M = -CUDART_INF_F, S = 0.f, A = 0.f;
     if (p.ext_lse) {
@@ -611,6 +657,14 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       kl = (A - D) / S - lse + lse_ref;      // sum_j p_j (z_j - zr_j) - lse + lse_ref
       p.lse_ref_c[i] = lse_ref;
       p.kl_c[i] = kl;
+    }
+    if (p.shift2) {
+      const float shift2 = p.shift2[i];
+      // (the comparison is written so that a NaN counts as too far)
+      if (!(fmaf(M, kLog2e, -shift2) <= kCodeTop && fmaf(lse, kLog2e, -shift2) >= kCodeLow)) {
+        p.tile_flags[i / kFlagRows] = 1;
+        *p.flag_count = 1;
+      }
     }
     const int row = p.row_map[i];
     if (p.kl_out) p.kl_out[row] = kl;
@@ -669,6 +723,91 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     double v = red[0][k];
     for (int w = 1; w < kLossThreads / 32; ++w) v = (k == 6) ? fmax(v, red[w][k]) : v + red[w][k];
     p.block_sums[(size_t)blockIdx.x * kLossSums + k] = v;
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// One-sweep path: the 16-bit codes of a slab's logits become, in place, the bf16 gradient with respect to the logits
+//   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),  log p_tj = code exponent + (estimate - lse_t),
+// rows past the slab's valid rows (up to a multiple of 128) and columns past V become zero.  The sampled token's own
+// entry uses its exact log-probability.  Bound by memory: 2 bytes in and 2 out per entry and nothing read twice.  A
+// warp takes kGradUnit consecutive columns of one row, all its 16-byte loads in flight before the first is used.
+constexpr int kGradVecs = 4;                       // 16-byte words per lane and unit
+constexpr int kGradUnit = 32 * 8 * kGradVecs;      // columns per warp and unit
+struct LogitGradParams {
+  uint16_t* slab;          // [slab rows][ld]
+  int ld;                  // multiple of 256
+  int V;
+  int slab_cap, slab_index;
+  const int* tokens_c;     // per compact row, as the arrays below
+  const float* shift2;
+  const float* lse;
+  const float* logp;
+  const float* ent;
+  const float* cp;
+  const float* ce;
+};
+
+__global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
+  int off, rows;
+  slab_extent(st->n_valid, p.slab_cap, p.slab_index, off, rows);
+  const int rows_pad = (rows + 127) / 128 * 128;
+  const int units_per_row = (p.ld + kGradUnit - 1) / kGradUnit;
+  const long long n_units = (long long)rows_pad * units_per_row;
+  const int lane = threadIdx.x & 31;
+  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
+    const int r = (int)(u / units_per_row);
+    const int c0 = (int)(u - (long long)r * units_per_row) * kGradUnit;
+    uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
+    if (r >= rows) {
+#pragma unroll
+      for (int k = 0; k < kGradVecs; ++k)
+        if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
+      continue;
+    }
+    uint4 q[kGradVecs];
+#pragma unroll
+    for (int k = 0; k < kGradVecs; ++k)
+      if (c0 + k * 256 < p.ld) q[k] = base[k * 32];
+    const int i = off + r;
+    const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i];
+    const int y = p.tokens_c[i];
+    const float shift = fmaf(-lse, kLog2e, p.shift2[i]);   // log2 p = exponent of the code + shift
+    const float kc = fmaf(ce, ent, cp), kl = ce * kLn2;     // g = p (kc + kl log2 p)
+    // the sampled token's entry from its exact log-probability
+    const float gy = fmaf(ex2_approx(logp * kLog2e), fmaf(ce, logp, kc), -cp);
+#pragma unroll
+    for (int k = 0; k < kGradVecs; ++k) {
+      const int c = c0 + k * 256 + lane * 8;
+      if (c0 + k * 256 >= p.ld) break;
+      const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+      float g[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // 0x4B00 above a 16-bit code is the float 2^23 + code
+        const float t0 = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5410))) + shift;
+        const float t1 = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5432))) + shift;
+        g[2 * j] = ex2_approx(t0) * fmaf(kl, t0, kc);
+        g[2 * j + 1] = ex2_approx(t1) * fmaf(kl, t1, kc);
+      }
+      const unsigned rel = (unsigned)(y - c);
+      if (rel < 8u) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) g[j] = rel == (unsigned)j ? gy : g[j];
+      }
+      if (c + 8 > p.V) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) g[j] = c + j < p.V ? g[j] : 0.f;
+      }
+      uint32_t o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
+        o[j] = *reinterpret_cast<const uint32_t*>(&b);
+      }
+      base[k * 32] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
   }
 }
 

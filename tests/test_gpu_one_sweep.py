@@ -1,0 +1,88 @@
+"""The one-sweep backward (logits formed once per slab of whole rows, kept as 16-bit codes until the loss coefficients are
+known) where it can go wrong: slab edges, ragged vocabulary tails, and rows whose log-sum-exp is badly estimated by
+their behaviour log-probability, which have to be recomputed.  Oracle and tolerances of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import grpo_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _np64(t):
+    return t.detach().double().cpu().numpy()
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+# the codes hold estimates that are 5.4 nats too low to 9.7 nats too high; beyond that the row tile is recomputed
+@pytest.mark.parametrize("cta_group", [2, 1])
+@pytest.mark.parametrize("rows,V,d,ent,off", [
+    (256, 300, 64, 0.0, 0.0),        # slabs of one row tile, one ragged column tile
+    (256, 1024, 128, 0.01, 0.0),     # entropy term, vocabulary a whole number of warp units
+    (512, 2085, 192, 0.0, 5.0),      # estimates off by up to 5 nats: still within the codes
+    (512, 1025, 64, 0.01, 20.0),     # single rows far off in both directions: those tiles are recomputed
+    (0, 70001, 64, 0.0, 12.0),       # default limits: one slab, several row tiles of it recomputed
+])
+def test_one_sweep_matches_oracle(cta_group, rows, V, d, ent, off):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    w = make_workload(1, prompts=1, L_max=150, d=d, V=V, seed=1000 + V)
+    assert w.n_valid > 512
+    adv = torch.randn(w.T, device="cuda")
+    valid = torch.nonzero(w.mask)[:, 0]
+    hit = valid[::max(1, valid.numel() // 3)]            # a few rows of different tiles
+    w.old_logp[hit[0::2]] += off
+    w.old_logp[hit[1::2]] -= off
+    adv[hit] = adv[hit].abs() * 0.1                      # a ratio of e^20 is then clipped and does not drown the rest
+    c = Context(0)
+    try:
+        c.set_cta_group(cta_group)
+        c.set_slab_limits(rows, -(-V // 256) * 256 if rows else 0)
+        dH = torch.full((w.T, d), float("nan"), device="cuda")
+        dW = torch.full((V, d), float("nan"), device="cuda")
+        c.ensure_workspace(w.T, d, V)
+        c._ws.fill_(0xFF)
+        out = c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, w.ref_logp, adv, w.mask, w.eps_low, w.eps_high,
+                                       w.beta, ent_coef=ent, dH=dH, dW=dW, dH_fp32=True)
+        status, detail = c.last_device_status()
+        assert status == 0, (status, hex(detail & 0xffffffff))
+    finally:
+        c.close()
+    oo = O.policy_loss_fwd_bwd(_np64(w.H), _np64(w.W), w.tokens.cpu().numpy(), _np64(w.old_logp), _np64(w.ref_logp),
+                               _np64(adv), w.mask.cpu().numpy(), w.eps_low, w.eps_high, w.beta, ent_coef=ent)
+    assert np.abs(_np64(out["logp"]) - oo["logp"]).max() <= 2e-3
+    assert abs(out["loss"].item() - oo["loss"]) <= 1e-3 * abs(oo["loss"]) + 1e-7
+    m = w.mask.cpu().numpy().astype(bool)
+    got, want = _np64(out["dH"]), oo["dH"]
+    assert not got[~m].any()
+    # every row by itself: one bf16 rounding per factor, a row that kept wrong codes would be off by its own size
+    err, size = np.linalg.norm(got[m] - want[m], axis=1), np.linalg.norm(want[m], axis=1)
+    assert (err <= 1e-2 * size + 1e-2 * np.median(size)).all()
+    assert _rel(got, want) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
+
+
+def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
+    # the coefficients of a response's rows need all its rows: with more than one row slab the logits are recomputed, and
+    # the result is that of one slab up to fp32 summation order and the rounding of the codes
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    w = make_workload(1, prompts=1, L_max=150, d=128, V=2000, seed=77)
+    adv = torch.randn(w.T, device="cuda")
+    outs = []
+    for rows in (256, 32768):
+        c = Context(0)
+        try:
+            c.set_slab_limits(rows, 2048)
+            outs.append(c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, w.ref_logp, adv, w.mask, 0.2, 0.2, 0.04,
+                                                 sequence_level=True, seq_offsets=w.seq_offsets, dH_fp32=True))
+            assert c.last_device_status()[0] == 0
+        finally:
+            c.close()
+    a, b = outs
+    assert torch.allclose(a["loss"], b["loss"], rtol=1e-5)
+    # two roundings to bf16 (2^-9 each) of the same gradient
+    assert _rel(_np64(a["dH"]), _np64(b["dH"])) <= 4e-3 and _rel(_np64(a["dW"]), _np64(b["dW"])) <= 4e-3
