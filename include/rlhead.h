@@ -90,8 +90,8 @@ rl_status rl_set_cta_group(rl_ctx* ctx, int cta_group);
  * rl_workspace_bytes().  On the measured workloads the gain was within 1 %. */
 rl_status rl_set_dh_k_slices(rl_ctx* ctx, int max_slices);
 /* Tile shape of the two long-K gradient products, dH = G W and dW = G^T H (default on, used when the
- * tensor-core passes run as CTA pairs and neither rl_set_dh_k_slices nor rl_set_dh_stream_k is in
- * effect): 256 x 512 output tiles that fill both accumulators of tensor memory, so a CTA pulls a
+ * tensor-core passes run as CTA pairs, the last tile of a row would not be half empty for nothing, and, for dW, K
+ * is long): 256 x 512 output tiles that fill both accumulators of tensor memory, so a CTA pulls a
  * quarter fewer operand bytes from L2 per flop, at the price of not overlapping a tile's epilogue
  * with the next tile's main loop (about 1 % of a tile at K of 17-19 thousand).  Off: 256 x 256 tiles
  * with a double-buffered accumulator, as the forward and gradient-of-logits passes always use.
@@ -475,8 +475,9 @@ rl_status rl_selftest_cluster_exchange(rl_ctx* ctx, int mode, int cluster_size, 
  * no counterpart).  For a pass over n_valid rows (at most rows_cap), K extent k_len, n_tiles column
  * tiles walked n_range at a time (0: split that fills the SMs, or 8 with plenty of work; -h with 1 <= h < 100:
  * chosen in [1, h] as the gradient-of-the-logits pass does; -100 - h: chosen in [8, h] when there is plenty of
- * work, else as 0), with the ordering options
- * of the library (n_fastest, row groups of m_group row tiles, stream-K, K slices) on n_workers
+ * work, else as 0; -1000 - r: as the passes that form logits, at most r ranges per row tile), with the ordering options
+ * of the library (n_fastest, row groups of m_group row tiles, stream-K, K slices; stream_k = 2: only the ragged last
+ * wave is cut, and a part's output slice is 1 + the slot it goes to) on n_workers
  * workers of cta_group CTAs each, writes one record of eight int32 per work unit, worker by worker
  * in the order the worker walks them: {worker, row tile, first column tile, end column tile,
  * output slice, first k-block, end k-block, k-blocks per tile}.  units (host, may be NULL when

@@ -24,6 +24,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
 struct EpiStats {
   static constexpr bool kTileFlags = false;
+  static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;   // [rows] compact sampled-token ids
@@ -157,6 +158,7 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // arithmetic (about 3 instructions per logit on top of the statistics' 3) still hides behind the next tile's MMAs.
 struct EpiSweep {
   static constexpr bool kTileFlags = false;
+  static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     EpiStats::Params stats;
@@ -223,6 +225,7 @@ struct EpiSweep {
 // Rows past the valid rows of the slab and columns past V are written as zero.
 struct EpiGrad {
   static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
+  static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     const int* tokens_c;
@@ -328,12 +331,15 @@ struct EpiGrad {
 // the result does not depend on timing.
 struct EpiAcc {
   static constexpr bool kTileFlags = false;
+  static constexpr bool kParts = true;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     int n_cols;
     int accumulate;
     int row_base;
     int slice_add;   // stream-K launches: output slices past the first are always added to
+    int tile_cols;   // > 0: k_slice > 0 names slot k_slice - 1, a box of tile_cols columns x tile_rows rows of its own
+    int tile_rows;
   };
   struct State {
     int k_slice;
@@ -354,6 +360,7 @@ struct EpiAcc {
     const int row0 = m_tile * BM + (row_in_tile - lane);   // first row of this warp's 32
     const int col0 = n_tile * BN + c * 32;
     if (row0 >= m_rows || col0 >= p.n_cols) return;        // warp-uniform
+    const bool part = p.tile_cols > 0 && st.k_slice > 0;
     const uint32_t buf = staging + (st.n_issued & 1u) * 4096u;
     // the store issued from this buffer two chunks ago must have finished reading it
     if (lane == 0) bulk_wait_group_read<1>();
@@ -369,7 +376,8 @@ struct EpiAcc {
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
-      if (p.accumulate || (p.slice_add && st.k_slice > 0)) tma_reduce_add_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
+      if (part) tma_store_3d(tmC, buf, col0 % p.tile_cols, row0 % p.tile_rows, st.k_slice - 1);
+      else if (p.accumulate || (p.slice_add && st.k_slice > 0)) tma_reduce_add_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
       else              tma_store_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
       bulk_commit_group();
     }

@@ -59,7 +59,10 @@ constexpr int kTileSmemBytes = 224 * 1024;             // operand ring + epilogu
 constexpr int kGemmSmemBytes = kTileSmemBytes + 1024;  // + slack for 1024-byte alignment
 constexpr int kStagingPerWarp = 8192;                  // two 32x32 fp32 boxes per epilogue warp
 constexpr int kTmemCols = 512;
-constexpr int kMaxSplit = 16;   // most column ranges per row tile when the split is chosen to fill the machine
+constexpr int kMaxSplit = 16;   // most column ranges per row tile unless GemmShape::n_split_max says otherwise
+constexpr int kFewRowTiles = 16;   // row tiles up to which the column split is chosen by waves (choose_split)
+constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
+constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
 constexpr int kFlagRows = 256;  // rows one entry of GemmShape::tile_flags stands for
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
 
@@ -108,6 +111,7 @@ struct GemmShape {
   // With n_range == 0 and n_range_hi > 0 the range length is chosen in [n_range_lo, n_range_hi] by choose_range():
   // always (n_range_always != 0) or only when there is plenty of work (otherwise the split that fills the SMs).
   int n_range_lo, n_range_hi, n_range_always;
+  int n_split_max;  // most column ranges per row tile (what the partials have room for); 0: kMaxSplit
   int skip_if_k0;   // nothing to do at all when K is empty (otherwise the epilogue sees zeros)
   int n_fastest;    // 1: consecutive units walk the column ranges of one row tile first
   // Row slabs of the backward pass: when slab_cap > 0 the valid rows are cut into
@@ -128,6 +132,9 @@ struct GemmShape {
   // caller zeroes beforehand), so each output element still has exactly one writer per slice and
   // launch.  Every share holds at least one whole tile's worth of iterations, so a tile has at
   // most two parts.
+  // 2: only the tiles of the ragged last wave (all tiles, when there are fewer than workers) are cut, see cut_tiles().
+  // Every part goes to a slot of its own and whoever reads the output adds the slots of a tile in a fixed order:
+  // nothing is zeroed beforehand and every element has one writer.
   int stream_k;
   // Row groups (only when the units are walked rows-first, n_fastest == 0): when m_group > 0 the row
   // tiles are taken at most m_group at a time (in groups of equal size) and all column ranges are
@@ -143,16 +150,23 @@ struct GemmShape {
 };
 
 // Number of vocabulary ranges each row tile is split into so that (row tiles x ranges) fills the
-// machine: minimises waves * tiles-per-range, preferring fewer ranges on ties.  m_units = row
-// tiles of 128*CG rows, n_workers = CTAs (CG = 1) or CTA pairs (CG = 2).
-__host__ __device__ inline int choose_split(int m_units, int n_tiles, int n_workers) {
+// machine: minimises waves * (tiles-per-range, and 5 % of a tile for what the roles do between units).  m_units = row
+// tiles of 128*CG rows, n_workers = CTAs (CG = 1) or CTA pairs (CG = 2).  For a given number of waves the best split is
+// the largest that needs no more, so only one candidate per wave count is looked at.  77 rows against 152 K words at
+// d = 2560: 478 us when no more than 16 ranges (16 of 74 pairs) were allowed, 172 us with 148 on single CTAs.
+__host__ __device__ inline int choose_split(int m_units, int n_tiles, int n_workers, int smax) {
   int best = 1;
   long best_cost = -1;
-  for (int s = 1; s <= kMaxSplit && s <= n_tiles; ++s) {
-    long units = (long)m_units * s;
-    long waves = (units + n_workers - 1) / n_workers;
-    long cost = waves * ((n_tiles + s - 1) / s);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
+  const int w0 = (m_units + n_workers - 1) / n_workers;
+  for (int waves = w0; waves < w0 + 5; ++waves) {
+    long sp = m_units > 0 ? (long)waves * n_workers / m_units : 1;
+    if (sp > smax) sp = smax;
+    if (sp > n_tiles) sp = n_tiles;
+    if (sp < 1) sp = 1;
+    const int per = (int)((n_tiles + sp - 1) / sp);
+    const int ranges = (n_tiles + per - 1) / per;
+    const long cost = ((long)m_units * ranges + n_workers - 1) / n_workers * (100L * per + 5);
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = (int)sp; }
   }
   return best;
 }
@@ -177,6 +191,7 @@ __host__ __device__ inline int choose_range(int m_units, int n_tiles, int n_work
 struct GemmExtents {
   int tile_rows;   // rows of one row tile (BM x CTAs per tile)
   int m_rows, m_units, k_blocks, n_range, n_ranges, n_units, slab_off, k_split, kb_per, stream_k, m_group;
+  int cut, cut_parts, cut_len;   // stream_k == 2: tiles that are cut, parts each, k-blocks of a part (0: all of its range)
 };
 
 // Number of K slices per tile (1..smax) that minimises the number of waves the tiles take on
@@ -203,6 +218,40 @@ __host__ __device__ inline void slab_extent(int n_valid, int cap, int index, int
   rows = rows < 0 ? 0 : (rows > per ? per : rows);
 }
 
+// How the tiles of a ragged last wave are cut.  With R of them on n workers every tile's K range is cut into
+// S = n / R equal ranges.  Worker r + R s takes range s of tile r, so that the workers of one s start on the same k and share
+// operand panels through L2 (one contiguous run of (tile, k) per worker, the usual stream-K, lost that: 640 rows against
+// 152 K words at d = 2048 took 405 us, bound by 2.8 GB of DRAM reads).  When n - R S workers would be left idle and S is
+// small enough for that to matter, each part stops after cut_len k-blocks and the ends of the parts, in order of
+// (tile, range), are shared equally among the remaining workers.  A wave that is nearly full is left alone.
+__host__ __device__ inline void cut_tiles(GemmExtents& e, int n_workers) {
+  const int R = e.n_units % n_workers, waves = e.n_units / n_workers + 1;
+  if (R == 0 || e.k_blocks == 0 || (n_workers - R) * 20 < n_workers * waves) return;
+  int S = n_workers / R;
+  if (S > e.k_blocks / kMinShare) S = e.k_blocks / kMinShare;
+  if (S < 1) return;
+  const int len = e.k_blocks / S;   // shortest range
+  const int fair = (int)(((long long)R * e.k_blocks + n_workers - 1) / n_workers);
+  e.cut_len = S == n_workers / R && R * S < n_workers && S <= kHelpSplit && len - fair >= kMinShare ? fair : 0;
+  if (S == 1 && e.cut_len == 0) return;
+  e.cut = R;
+  e.cut_parts = S;
+}
+// First k-block of range s of a cut tile, and the position of the end of part s in the list of its tile's ends.
+__host__ __device__ inline int cut_begin(const GemmExtents& e, int s) {
+  return (int)((long long)e.k_blocks * s / e.cut_parts);
+}
+__host__ __device__ inline int cut_end_pos(const GemmExtents& e, int s) { return cut_begin(e, s) - s * e.cut_len; }
+// k-blocks in all ends of one tile, and in those of all tiles.
+__host__ __device__ inline int cut_tile_ends(const GemmExtents& e) { return e.k_blocks - e.cut_parts * e.cut_len; }
+// Slots: part s of tile r has slot r S + s; the piece of the end of that part that helper h does has slot
+// R S + (r S + s) + h (from one piece to the next r S + s or h grows, so no two share a slot; fewer than 2 n in all).
+// Helper that does block `pos` of the list of all ends.
+__host__ __device__ inline int cut_helper(const GemmExtents& e, int n_workers, long long pos) {
+  const long long total = (long long)e.cut * cut_tile_ends(e);
+  return (int)(((pos + 1) * (n_workers - e.cut * e.cut_parts) - 1) / total);
+}
+
 // cg = CTAs per output row tile, n_workers = gridDim.x / cg.
 __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_valid, int cg, int n_workers) {
   GemmExtents e;
@@ -222,7 +271,9 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
   e.tile_rows = BM * cg;
   e.m_units = (e.m_rows + BM * cg - 1) / (BM * cg);
   e.k_blocks = (k_len + BK - 1) / BK;
-  const bool plenty = (long)e.m_units * ((sh.n_tiles + kFwdRange - 1) / kFwdRange) >= 4L * n_workers;
+  const int smax = sh.n_split_max > 0 ? sh.n_split_max : kMaxSplit;
+  const bool few_rows = sh.n_split_max > 0 && e.m_units <= kFewRowTiles;
+  const bool plenty = !few_rows && (long)e.m_units * ((sh.n_tiles + kFwdRange - 1) / kFwdRange) >= 4L * n_workers;
   if (sh.n_range > 0) {
     e.n_range = sh.n_range;
   } else if (sh.n_range_hi > 0 && (sh.n_range_always || plenty)) {
@@ -232,7 +283,7 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
     // column tiles of the others, so the B operand is fetched from DRAM about once
     e.n_range = kFwdRange;
   } else {
-    const int split = choose_split(e.m_units, sh.n_tiles, n_workers);
+    const int split = choose_split(e.m_units, sh.n_tiles, n_workers, smax);
     e.n_range = (sh.n_tiles + split - 1) / split;
   }
   if (e.n_range < 1) e.n_range = 1;
@@ -250,6 +301,11 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
   }
   e.stream_k = (sh.stream_k && e.k_split == 1 && e.n_range == 1 && e.k_blocks > 0 && e.n_units >= n_workers &&
                 e.n_units % n_workers != 0) ? 1 : 0;
+  e.cut = e.cut_parts = e.cut_len = 0;
+  if (sh.stream_k == 2) {
+    if (e.k_split == 1 && e.n_range == 1) cut_tiles(e, n_workers);
+    e.stream_k = e.cut > 0 ? 2 : 0;
+  }
   return e;
 }
 
@@ -278,17 +334,29 @@ __host__ __device__ inline void unit_coords(const GemmShape& sh, const GemmExten
 // but the last are walked the same way (CTAs that run together then share operand panels); the
 // remaining tiles (between one and two per worker) are balanced: their (tile, k-block) iterations,
 // tile-major, are cut into one contiguous share per worker, one unit per tile a share touches; ks
-// is then the output slice of the part: 0 when it starts at k-block 0, else 1.
+// is then the output slice of the part: 0 when it starts at k-block 0, else 1.  stream_k == 2: full waves, then this
+// worker's parts of cut tiles (cut_tiles); ks is 0 for a whole tile, else 1 + the slot of the part.
 // FLAGS: row tiles whose GemmShape::tile_flags entry is zero are passed over.
 template <bool FLAGS = false>
 struct UnitWalk {
   const GemmShape& sh;
   const GemmExtents& ex;
-  int n_workers, u, plain_units;
+  int n_workers, u, me, plain_units;
   long long it, it_end;
   __host__ __device__ inline UnitWalk(const GemmShape& sh_, const GemmExtents& ex_, int worker, int n_workers_)
-      : sh(sh_), ex(ex_), n_workers(n_workers_), u(worker), plain_units(ex_.n_units), it(0), it_end(0) {
-    if (ex.stream_k) {
+      : sh(sh_), ex(ex_), n_workers(n_workers_), u(worker), me(worker), plain_units(ex_.n_units), it(0), it_end(0) {
+    if (ex.stream_k == 2) {
+      plain_units = ex.n_units - ex.cut;
+      const int mains = ex.cut * ex.cut_parts, helpers = n_workers - mains;
+      if (worker < mains) {
+        it = 0;
+        it_end = 1;
+      } else if (ex.cut_len > 0) {
+        const long long total = (long long)ex.cut * cut_tile_ends(ex);
+        it = total * (worker - mains) / helpers;
+        it_end = total * (worker - mains + 1) / helpers;
+      }
+    } else if (ex.stream_k) {
       plain_units = (ex.n_units / n_workers - 1) * n_workers;
       const long long total = (long long)(ex.n_units - plain_units) * ex.k_blocks;
       it = total * worker / n_workers;
@@ -303,6 +371,7 @@ struct UnitWalk {
       return true;
     }
     if (it >= it_end) return false;
+    if (ex.stream_k == 2) return next_part(mu, nr, ks, kb0, kb1);
     const int t_rel = (int)(it / ex.k_blocks);
     kb0 = (int)(it - (long long)t_rel * ex.k_blocks);
     const long long left = it_end - it;
@@ -310,6 +379,32 @@ struct UnitWalk {
     ks = kb0 > 0 ? 1 : 0;
     it += kb1 - kb0;
     const int tile = plain_units + t_rel;
+    if (sh.n_fastest) { nr = tile % ex.n_ranges; mu = tile / ex.n_ranges; }
+    else              { mu = tile % ex.m_units;  nr = tile / ex.m_units; }
+    return true;
+  }
+  __host__ __device__ inline bool next_part(int& mu, int& nr, int& ks, int& kb0, int& kb1) {
+    const int S = ex.cut_parts, mains = ex.cut * S;
+    int r, s;
+    if (me < mains) {
+      r = me % ex.cut;
+      s = me / ex.cut;
+      kb0 = cut_begin(ex, s);
+      kb1 = ex.cut_len > 0 ? kb0 + ex.cut_len : cut_begin(ex, s + 1);
+      ks = 1 + r * S + s;
+      it = it_end;
+    } else {
+      const int ends = cut_tile_ends(ex);
+      r = (int)(it / ends);
+      const int pos = (int)(it - (long long)r * ends);
+      for (s = 0; s + 1 < S && cut_end_pos(ex, s + 1) <= pos; ++s) {}
+      kb0 = cut_begin(ex, s) + ex.cut_len + pos - cut_end_pos(ex, s);
+      kb1 = cut_begin(ex, s + 1);
+      if (kb1 - kb0 > it_end - it) kb1 = kb0 + (int)(it_end - it);
+      ks = 1 + mains + r * S + s + (me - mains);
+      it += kb1 - kb0;
+    }
+    const int tile = plain_units + r;
     if (sh.n_fastest) { nr = tile % ex.n_ranges; mu = tile / ex.n_ranges; }
     else              { mu = tile % ex.m_units;  nr = tile / ex.m_units; }
     return true;
@@ -324,7 +419,8 @@ struct UnitWalk {
 //     static void end_unit(const Params&, State&, int m_tile, int n_range_idx, int row_in_tile, int m_rows);
 //     static void init(State&); static void finish(State&);     // once per kernel, per thread
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
-//     static constexpr bool kTileFlags; };                     // launches may be restricted by GemmShape::tile_flags
+//     static constexpr bool kTileFlags;                        // launches may be restricted by GemmShape::tile_flags
+//     static constexpr bool kParts; };                         // knows what to do with parts of tiles (stream_k == 2)
 //   kTileDual: chunk receives the chunk of the second product as well (..., v, v2, out_map, staging).
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
 // sh.n_tiles then counts 512-wide tiles).  tmA2 / tmB2 / k2_len are read by kTileDual only.
@@ -377,6 +473,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   const uint32_t tmem_base = tmem_base_smem;
   volatile int* abort_p = &abort_flag;
 
+  // parts of cut tiles go to slots, seen through the second map of operand A (one-product passes only)
+  const CUtensorMap* part_map = MODE == kTileDual ? &tmC : &tmA2;
   const GemmExtents ex = gemm_extents(sh, sh.n_valid ? *sh.n_valid : 0, CG, n_workers);
   const int k2_blocks = MODE == kTileDual ? (k2_len + BK - 1) / BK : 0;
   // the two-product mode has nothing to do unless both products have a K range
@@ -597,7 +695,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = 0.f;
               }
-              Epi::chunk(ep, st, m, n * Cfg::kBBoxes + s, c, row_in_tile, ex.m_rows, v, &tmC, staging);
+              Epi::chunk(ep, st, m, n * Cfg::kBBoxes + s, c, row_in_tile, ex.m_rows, v,
+                         Epi::kParts && ex.stream_k == 2 && ks > 0 ? part_map : &tmC, staging);
             }
           }
           if (has_k) {

@@ -12,6 +12,7 @@ namespace rlh {
 // Two float4 per (range, row): {M, S, A, z_y} and {D, Mr, Sr, 0}.
 struct EpiStatsKL {
   static constexpr bool kTileFlags = false;
+  static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;
@@ -88,6 +89,7 @@ struct EpiStatsKL {
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
   static constexpr bool kTileFlags = false;
+  static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 4 * kStagingPerWarp;
   struct Params {
     const int* tokens_c;

@@ -40,6 +40,7 @@ struct rl_ctx {
   int wide_tiles;   // 1: dH and dW run on 256 x 512 tiles (both accumulators hold one tile)
   int dh_stream_k;  // 1: the dH pass balances its tiles over the SMs by stream-K (needs a second accumulator buffer)
   int grid[3];    // persistent grid for cta_group 1 and 2 (index = cta_group)
+  int fixed_scratch;  // 1: the context of rl_token_logprobs_static, whose scratch has a documented size
   int grid_full[3];   // the same before rl_set_max_ctas() capped it
   rl_dw_slab_hook dw_hook;   // called after the launch that completes a slab of dW rows was enqueued
   void* dw_hook_user;
@@ -72,6 +73,8 @@ constexpr int kSlabRowsMin = 2048;
 constexpr int kTokenLossBlocks = 1024;
 constexpr size_t kStatusBytes = 256 + (size_t)kTokenLossBlocks * kLossSums * sizeof(double);
 constexpr int kAdvRowsMinGroups = 2048;     // from this many groups on, GRPO advantages run one thread per group
+constexpr int kWideGain = 96;              // time of a 256 x 512 tile, in % of two 256 x 256 tiles of the same K
+constexpr int kWideMinRows = 8192;         // rows of a slab (K of the dW pass) from which its tiles are 512 wide
 constexpr int kDhSplitMax = 4;             // most K slices (separate fp32 accumulators) of the dH pass
 constexpr int kSlabColsMax = 148 * 256;    // vocabulary columns of one gradient slab (148 tiles of 256: two per SM pair)
 
@@ -80,11 +83,27 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // fp32 accumulator buffers of the dH pass: one per K slice, or two when stream-K balancing is on
 inline bool dh_uses_stream_k(const rl_ctx* c) { return c->dh_stream_k && c->dh_k_slices == 1; }
 inline int dh_buffers(const rl_ctx* c) { return dh_uses_stream_k(c) ? 2 : c->dh_k_slices; }
+// Neither option set: the tiles of the dH pass's ragged last wave are cut into parts that lie in slots.
+inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_slices == 1; }
+// 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
+// tile that is half empty costs as much as a full one.
+inline bool use_wide(const rl_ctx* c, int64_t d) {
+  const int64_t wide = (d + 2 * BN - 1) / (2 * BN) * 2, square = (d + BN - 1) / BN;
+  return c->wide_tiles && c->cta_group == 2 && wide * kWideGain <= square * 100;
+}
+// Width of a dH tile, and bytes of the slots its parts may need (two per worker).
+inline int dh_tile_cols(const rl_ctx* c, int64_t d) { return use_wide(c, d) ? 2 * BN : BN; }
+inline size_t dh_slot_bytes(const rl_ctx* c, int64_t d) {
+  const int workers = c->grid_full[c->cta_group] / c->cta_group;
+  return (size_t)2 * workers * BM * c->cta_group * dh_tile_cols(c, d) * 4;
+}
 
 struct WsLayout {
   int Tpad, Ts, Vs;
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
   size_t shift2, flags;                              // one-sweep path: log-sum-exp estimates, row-tile flags
+  int part_ranges;                                   // column ranges per row that the partials have room for
+  size_t dH_slots;                                   // parts of cut dH tiles (0: none)
   int n_row_slabs, n_flags;                          // n_flags: row tiles, then one count per row slab
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
 };
@@ -154,15 +173,25 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.cp_c = take((size_t)L.Tpad * 4);
   L.ce_c = take((size_t)L.Tpad * 4);
   {
-    // one float4 per (column range, row): at most kMaxSplit ranges, or one per kFwdRange column tiles
-    const size_t by_range = (size_t)(((V + BN - 1) / BN + kFwdRange - 1) / kFwdRange);
+    // one float4 per (column range, row): at most kMaxSplit ranges, or one per kFwdRange column tiles; with few rows
+    // enough ranges to give every SM a unit
+    const size_t tiles = (size_t)((V + BN - 1) / BN);
+    const size_t by_range = (tiles + kFwdRange - 1) / kFwdRange;
     n_part_ranges = by_range > (size_t)kMaxSplit ? by_range : (size_t)kMaxSplit;
+    if (!c->fixed_scratch) {
+      size_t fill = (size_t)c->n_sm * 512 / L.Tpad;
+      if (fill > (size_t)c->n_sm) fill = c->n_sm;
+      if (fill > tiles) fill = tiles;
+      if (n_part_ranges < fill) n_part_ranges = fill;
+    }
+    L.part_ranges = (int)n_part_ranges;
     L.partials = take(n_part_ranges * L.Tpad * sizeof(float4));
   }
   L.block_sums = take((size_t)1024 * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
   L.G = take((size_t)L.Ts * L.Vs * 2);
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
+  L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
   L.shift2 = take((size_t)L.Tpad * 4);
   L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
   L.flags = take((size_t)L.n_flags * 4);
@@ -247,8 +276,14 @@ cudaError_t set_smem_attr_dual() {
 
 // Rows of B that one CTA stages per k-slice (box height of a K-major B map) and the number of
 // 64-wide panels of an MN-major B map, for the context's CTA grouping.
-inline uint32_t b_box_rows(const rl_ctx* c) { return BN / c->cta_group; }
+inline uint32_t b_box_rows(int cg) { return BN / cg; }
+inline uint32_t b_box_rows(const rl_ctx* c) { return b_box_rows(c->cta_group); }
 inline uint32_t b_box_panels(const rl_ctx* c) { return BN / 64 / c->cta_group; }
+
+// CTAs per row tile of the passes that form logits: a pair would spend half its tensor work on padding when at most 128
+// rows exist, and with so few rows the pass is a stream of W.
+inline int fwd_cta_group(const rl_ctx* c, const WsLayout& L) { return L.Tpad <= BM ? 1 : c->cta_group; }
+inline int fwd_workers(const rl_ctx* c, const WsLayout& L) { const int cg = fwd_cta_group(c, L); return c->grid[cg] / cg; }
 
 // Optional timing of a group of launches: event pair on the context's stream, tagged with a kind.
 int prof_begin(rl_ctx* c, int kind) {
@@ -269,11 +304,11 @@ void prof_end(rl_ctx* c, int i, int kind) {
 // One launch of the tensor-core engine in tile mode MODE on the context's persistent grid (CTA pairs
 // when cta_group is 2; wide tiles exist for pairs only).  a2 / b2 / k2_len: second product (kTileDual).
 template <class Epi, int A_MN, int B_MN, int MODE>
-void launch_tiles(rl_ctx* c, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2,
+void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2,
                   const CUtensorMap& b2, const CUtensorMap& out, const GemmShape& sh, int k2_len,
                   const typename Epi::Params& ep) {
   const int prof = prof_begin(c, kind);
-  if (c->cta_group == 2) {
+  if (cg == 2) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(c->grid[2]);
@@ -296,26 +331,25 @@ void launch_tiles(rl_ctx* c, int kind, const CUtensorMap& a, const CUtensorMap& 
   prof_end(c, prof, kind);
 }
 
+// 256-column tiles, cg CTAs each; parts: the slots of cut tiles (any map where no tile is cut).
 template <class Epi, int A_MN, int B_MN>
-void launch_gemm(rl_ctx* c, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out,
-                 const GemmShape& sh, const typename Epi::Params& ep) {
-  launch_tiles<Epi, A_MN, B_MN, kTileSquare>(c, kind, a, b, a, b, out, sh, 0, ep);
+void launch_gemm(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out,
+                 const CUtensorMap& parts, const GemmShape& sh, const typename Epi::Params& ep) {
+  launch_tiles<Epi, A_MN, B_MN, kTileSquare>(c, cg, kind, a, b, parts, b, out, sh, 0, ep);
 }
 
 // 256 x 512 tiles on CTA pairs; sh.n_tiles counts 512-wide column tiles.
-inline bool use_wide(const rl_ctx* c) { return c->wide_tiles && c->cta_group == 2; }
-
 template <class Epi, int A_MN, int B_MN>
 void launch_wide(rl_ctx* c, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out,
-                 const GemmShape& sh, const typename Epi::Params& ep) {
-  launch_tiles<Epi, A_MN, B_MN, kTileWide>(c, kind, a, b, a, b, out, sh, 0, ep);
+                 const CUtensorMap& parts, const GemmShape& sh, const typename Epi::Params& ep) {
+  launch_tiles<Epi, A_MN, B_MN, kTileWide>(c, 2, kind, a, b, parts, b, out, sh, 0, ep);
 }
 
 template <class Epi>
 void launch_dual(rl_ctx* c, int kind, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2,
                  const CUtensorMap& b2, const CUtensorMap& out, const GemmShape& sh, int k2_len,
                  const typename Epi::Params& ep) {
-  launch_tiles<Epi, 0, 0, kTileDual>(c, kind, a, b, a2, b2, out, sh, k2_len, ep);
+  launch_tiles<Epi, 0, 0, kTileDual>(c, c->cta_group, kind, a, b, a2, b2, out, sh, k2_len, ep);
 }
 
 rl_status check_hw(const void* H, int64_t ldH, const void* W, int64_t ldW, int64_t T, int64_t d, int64_t V) {
@@ -400,9 +434,10 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     memset(shape_out, 0, sizeof(*shape_out));
     return cuda_ok();
   }
+  const int cg = kl ? c->cta_group : fwd_cta_group(c, L);
   CUtensorMap tmA, tmB;
   if (!map_kmajor(c, &tmA, Hc, (uint64_t)L.Tpad, (uint64_t)d, (uint64_t)d, BM)) return RL_ERR_CUDA;
-  if (!map_kmajor(c, &tmB, W, (uint64_t)V, (uint64_t)d, (uint64_t)ldW, b_box_rows(c))) return RL_ERR_CUDA;
+  if (!map_kmajor(c, &tmB, W, (uint64_t)V, (uint64_t)d, (uint64_t)ldW, b_box_rows(cg))) return RL_ERR_CUDA;
   GemmShape sh;
   memset(&sh, 0, sizeof(sh));
   sh.n_valid = &c->dstatus->n_valid;
@@ -411,6 +446,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   sh.k_cap = (int)d;
   sh.n_tiles = (int)((V + BN - 1) / BN);
   sh.n_range = 0;  // split chosen on the device from the number of valid rows
+  sh.n_split_max = L.part_ranges;
   sh.m_group = row_group_tiles(c, d + (kl ? kl->d_ref : 0));
   EpiStats::Params ep;
   ep.tokens_c = tokens_c;
@@ -418,7 +454,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   ep.part_stride = L.Tpad;
   ep.V = (int)V;
   if (!kl) {
-    launch_gemm<EpiStats, 0, 0>(c, 0, tmA, tmB, tmA, sh, ep);   // no output map
+    launch_gemm<EpiStats, 0, 0>(c, cg, 0, tmA, tmB, tmA, tmA, sh, ep);   // no output map
   } else {
     // full KL: compact the reference hidden states with the same row map and form both logit
     // tiles per output tile
@@ -483,6 +519,7 @@ rl_status rl_create(rl_ctx** out, int device) {
   c->dh_stream_k = 0;
   c->wide_tiles = 1;
   c->row_group_bytes = kRowGroupBytes;
+  c->fixed_scratch = 0;
   c->grid[0] = 0;
   c->grid[1] = c->n_sm;
   c->grid[2] = c->n_sm / 2 * 2;
@@ -920,8 +957,8 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
   p.fwd_shape = fwd_shape;
-  p.fwd_cg = c->cta_group;
-  p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+  p.fwd_cg = fwd_cta_group(c, L);
+  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.with_loss = 0;
   p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);
@@ -1026,8 +1063,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
   p.fwd_shape = fwd_shape;
-  p.fwd_cg = c->cta_group;
-  p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+  p.fwd_cg = fwd_cta_group(c, L);
+  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.old_logp = old_logp;
   p.ref_logp = ref_logp;
@@ -1054,6 +1091,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   }
   if (o.kl_full) {
     p.kl_full = 1;
+    p.fwd_cg = c->cta_group;   // two-product tiles
+    p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
     p.partials2 = reinterpret_cast<const float4*>(ws + L.partials2);
     p.lse_ref_c = reinterpret_cast<float*>(ws + L.lse_ref_c);
     p.kl_c = reinterpret_cast<float*>(ws + L.kl_c);
@@ -1124,7 +1163,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int* row_map = reinterpret_cast<const int*>(ws + L.row_map);
   const int* n_valid = &c->dstatus->n_valid;
 
-  CUtensorMap tmHc_k, tmW_k, tmG_k, tmW_mn, tmG_mn, tmHc_mn, tm_dH, tm_dW, tm_G_out, tmHr_k, tmWr_k;
+  CUtensorMap tmHc_k, tmW_k, tmG_k, tmW_mn, tmG_mn, tmHc_mn, tm_dH, tm_dW, tm_G_out, tmHr_k, tmWr_k, tm_slots, tmW_fwd;
   if (o.kl_full) {
     if (!map_kmajor(c, &tmHr_k, ws + L.Hc_ref, (uint64_t)L.Tpad, (uint64_t)o.d_ref, (uint64_t)o.d_ref, BM) ||
         !map_kmajor(c, &tmWr_k, o.W_ref, (uint64_t)V, (uint64_t)o.d_ref, (uint64_t)o.ldW_ref, b_box_rows(c)))
@@ -1139,6 +1178,17 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             map_out_bf16(c, &tm_G_out, G, (uint64_t)L.Ts, (uint64_t)L.Vs, (uint64_t)L.Vs) &&
             map_out_f32(c, &tm_dH, dH_acc, (uint64_t)L.Ts, (uint64_t)d, (uint64_t)d, (uint64_t)dh_buffers(c), (uint64_t)L.Ts) &&
             map_out_f32(c, &tm_dW, dW, (uint64_t)V, (uint64_t)d, (uint64_t)d, 1, (uint64_t)V);
+  const int dh_tile_rows = BM * c->cta_group, dh_cols = dh_tile_cols(c, d);
+  const int dh_workers = c->grid[c->cta_group] / c->cta_group;
+  float* dH_slots = reinterpret_cast<float*>(ws + L.dH_slots);
+  tm_slots = tm_dH;
+  if (L.dH_slots)
+    ok = ok && map_out_f32(c, &tm_slots, dH_slots, (uint64_t)dh_tile_rows, (uint64_t)dh_cols, (uint64_t)dh_cols,
+                           (uint64_t)2 * dh_workers, (uint64_t)dh_tile_rows);
+  const int cg_fwd = fwd_cta_group(c, L);
+  tmW_fwd = tmW_k;
+  if (cg_fwd != c->cta_group)
+    ok = ok && map_kmajor(c, &tmW_fwd, W, (uint64_t)V, (uint64_t)d, (uint64_t)ldW, b_box_rows(cg_fwd));
   if (!ok) return RL_ERR_CUDA;
 
   const int n_row_slabs = L.n_row_slabs;
@@ -1165,6 +1215,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sw.m_rows_cap = rows_cap; sw.m_dyn = 1; sw.slab_cap = L.Ts; sw.slab_index = r;
           sw.k_cap = (int)d;
           sw.n_tiles = (cols + BN - 1) / BN;
+          sw.n_split_max = L.part_ranges;
           sw.a_mn_slab = 1;
           sw.m_group = row_group_tiles(c, d);
           EpiSweep::Params ep;
@@ -1173,7 +1224,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           ep.stats.part_stride = L.Tpad;
           ep.stats.V = (int)V;
           ep.shift2 = reinterpret_cast<const float*>(ws + L.shift2);
-          launch_gemm<EpiSweep, 0, 0>(c, 0, tmHc_k, tmW_k, tm_G_out, sw, ep);
+          launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
           p.fwd_shape = sw;
           p.slab_cap = L.Ts;
           p.slab_index = r;
@@ -1213,7 +1264,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.lse = p.lse_c; ep.ent = p.ent_c; ep.cp = p.cp_c; ep.ce = p.ce_c;
           ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_gemm<EpiGrad, 0, 0>(c, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, sh, ep);
+          launch_gemm<EpiGrad, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
         } else {
           EpiGradKL::Params ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
@@ -1230,22 +1281,19 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.n_valid = n_valid;
         sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
         sh.k_cap = cols;
-        sh.n_tiles = d_tiles;
+        sh.n_tiles = (int)((d + dh_cols - 1) / dh_cols);
         sh.n_range = 1;
         sh.b_k_off = vocab_base;
         sh.n_fastest = 1;   // the CTAs that share a panel of G rows run together
         sh.k_split_max = c->dh_k_slices;
-        sh.stream_k = dh_uses_stream_k(c) ? 1 : 0;
-        dh_shape = sh;      // the slice count depends only on rows, d tiles and grid: same for every slab
+        sh.stream_k = dh_uses_stream_k(c) ? 1 : (L.dH_slots ? 2 : 0);
+        dh_shape = sh;      // how tiles are cut depends only on rows, d tiles and grid: same for every slab
         EpiAcc::Params ep;
-        ep.n_cols = (int)d; ep.accumulate = cs > 0; ep.row_base = 0; ep.slice_add = sh.stream_k;
-        if (use_wide(c)) {
-          sh.n_tiles = (int)((d + 2 * BN - 1) / (2 * BN));
-          dh_shape = sh;
-          launch_wide<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, sh, ep);
-        } else {
-          launch_gemm<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, sh, ep);
-        }
+        ep.n_cols = (int)d; ep.accumulate = cs > 0; ep.row_base = 0; ep.slice_add = sh.stream_k == 1;
+        ep.tile_cols = sh.stream_k == 2 ? dh_cols : 0;
+        ep.tile_rows = dh_tile_rows;
+        if (use_wide(c, d)) launch_wide<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
+        else launch_gemm<EpiAcc, 0, 1>(c, c->cta_group, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
       }
       // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab.  A caller that wants to
       // be told as rows of dW are completed gets them in pieces.
@@ -1257,7 +1305,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.n_valid = n_valid;
         sh.m_rows_cap = cols - c0 < step ? cols - c0 : step;
         sh.k_cap = rows_cap; sh.k_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
-        sh.n_tiles = d_tiles;
+        const bool wide = use_wide(c, d) && L.Ts >= kWideMinRows;
+        sh.n_tiles = wide ? (int)((d + 2 * BN - 1) / (2 * BN)) : d_tiles;
         sh.n_range = 1;
         sh.skip_if_k0 = (r > 0 || o.accumulate_dW) ? 1 : 0;
         sh.a_mn_off = c0;
@@ -1265,13 +1314,9 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.n_fastest = 1;
         EpiAcc::Params ep;
         ep.n_cols = (int)d; ep.accumulate = (r > 0 || o.accumulate_dW) ? 1 : 0;
-        ep.row_base = vocab_base + c0; ep.slice_add = 0;
-        if (use_wide(c)) {
-          sh.n_tiles = (int)((d + 2 * BN - 1) / (2 * BN));
-          launch_wide<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, sh, ep);
-        } else {
-          launch_gemm<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, sh, ep);
-        }
+        ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
+        if (wide) launch_wide<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
+        else launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
         // these rows of dW are complete once the last row slab has added to them
         if (report) {
           const int64_t row0 = (int64_t)vocab_base + c0;
@@ -1280,14 +1325,18 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       }
     }
     const int pr_sc = prof_begin(c, 7);
-    if (o.dH_dtype)
-      scatter_dH_f32_kernel<<<c->n_sm * 4, 256, 0, st>>>(dH_acc, (int)d, dh_shape, c->cta_group,
-                                                         c->grid[c->cta_group] / c->cta_group, (long long)L.Ts * d, row_map,
-                                                         static_cast<float*>(dH), c->dstatus);
-    else
-      scatter_dH_kernel<<<c->n_sm * 4, 256, 0, st>>>(dH_acc, (int)d, dh_shape, c->cta_group,
-                                                     c->grid[c->cta_group] / c->cta_group, (long long)L.Ts * d, row_map,
-                                                     static_cast<__nv_bfloat16*>(dH), c->dstatus);
+    DhSource src;
+    src.acc = dH_acc;
+    src.d = (int)d;
+    src.shape = dh_shape;
+    src.cg = c->cta_group;
+    src.workers = dh_workers;
+    src.split_stride = (long long)L.Ts * d;
+    src.slots = dH_slots;
+    src.tile_rows = dh_tile_rows;
+    src.tile_cols = dh_cols;
+    if (o.dH_dtype) scatter_dH_kernel<true><<<c->n_sm * 8, 256, 0, st>>>(src, row_map, dH, c->dstatus);
+    else            scatter_dH_kernel<false><<<c->n_sm * 8, 256, 0, st>>>(src, row_map, dH, c->dstatus);
     prof_end(c, pr_sc, 7);
     c->launches++;
   }
@@ -1345,8 +1394,8 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
   p.fwd_shape = fwd_shape;
-  p.fwd_cg = c->cta_group;
-  p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+  p.fwd_cg = fwd_cta_group(c, L);
+  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.stats_out = reinterpret_cast<float4*>(stats);
   int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
@@ -1406,8 +1455,8 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
     p.partials = reinterpret_cast<const float4*>(ws + L.partials);
     p.part_stride = L.Tpad;
     p.fwd_shape = fwd_shape;
-    p.fwd_cg = c->cta_group;
-    p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+    p.fwd_cg = fwd_cta_group(c, L);
+    p.fwd_workers = fwd_workers(c, L);
     p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
     p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);
     p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
@@ -1606,6 +1655,8 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
   sh.n_tiles = (int)n_tiles;
   if (n_range >= 0) {
     sh.n_range = n_range;
+  } else if (n_range <= -1000) {   // as the passes that form logits: at most -n_range - 1000 ranges per row tile
+    sh.n_split_max = -n_range - 1000;
   } else if (n_range > -100) {   // as the gradient-of-the-logits pass: always chosen in [1, -n_range]
     sh.n_range_lo = 1; sh.n_range_hi = -n_range; sh.n_range_always = 1;
   } else {                       // as the forward pass: chosen in [8, -n_range - 100] when there is plenty of work
@@ -1716,17 +1767,17 @@ rl_status rl_selftest_gemm(rl_ctx* c, const void* A, const void* B, float* C, in
   CUtensorMap tc;
   if (!map_out_f32(c, &tc, C, (uint64_t)M, (uint64_t)N, (uint64_t)N, 1, (uint64_t)M)) return RL_ERR_CUDA;
   EpiAcc::Params ep;
-  ep.n_cols = (int)N; ep.accumulate = accumulate; ep.row_base = 0; ep.slice_add = 0;
-  if (use_wide(c)) {
+  ep.n_cols = (int)N; ep.accumulate = accumulate; ep.row_base = 0; ep.slice_add = 0; ep.tile_cols = 0;
+  if (c->wide_tiles && c->cta_group == 2) {
     sh.n_tiles = (int)((N + 2 * BN - 1) / (2 * BN));
-    if (!a_mn && !b_mn) launch_wide<EpiAcc, 0, 0>(c, -1, ta, tb, tc, sh, ep);
-    else if (!a_mn && b_mn) launch_wide<EpiAcc, 0, 1>(c, -1, ta, tb, tc, sh, ep);
-    else if (a_mn && !b_mn) launch_wide<EpiAcc, 1, 0>(c, -1, ta, tb, tc, sh, ep);
-    else launch_wide<EpiAcc, 1, 1>(c, -1, ta, tb, tc, sh, ep);
-  } else if (!a_mn && !b_mn) launch_gemm<EpiAcc, 0, 0>(c, -1, ta, tb, tc, sh, ep);
-  else if (!a_mn && b_mn) launch_gemm<EpiAcc, 0, 1>(c, -1, ta, tb, tc, sh, ep);
-  else if (a_mn && !b_mn) launch_gemm<EpiAcc, 1, 0>(c, -1, ta, tb, tc, sh, ep);
-  else launch_gemm<EpiAcc, 1, 1>(c, -1, ta, tb, tc, sh, ep);
+    if (!a_mn && !b_mn) launch_wide<EpiAcc, 0, 0>(c, -1, ta, tb, tc, tc, sh, ep);
+    else if (!a_mn && b_mn) launch_wide<EpiAcc, 0, 1>(c, -1, ta, tb, tc, tc, sh, ep);
+    else if (a_mn && !b_mn) launch_wide<EpiAcc, 1, 0>(c, -1, ta, tb, tc, tc, sh, ep);
+    else launch_wide<EpiAcc, 1, 1>(c, -1, ta, tb, tc, tc, sh, ep);
+  } else if (!a_mn && !b_mn) launch_gemm<EpiAcc, 0, 0>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
+  else if (!a_mn && b_mn) launch_gemm<EpiAcc, 0, 1>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
+  else if (a_mn && !b_mn) launch_gemm<EpiAcc, 1, 0>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
+  else launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
   return cuda_ok();
 }
 
@@ -1788,6 +1839,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
     c.dh_stream_k = 0;
     c.wide_tiles = 0;
     c.row_group_bytes = kRowGroupBytes;
+    c.fixed_scratch = 1;
     c.grid[1] = c.n_sm;
     slot.ready = true;
   }
@@ -1814,8 +1866,8 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
   p.fwd_shape = fwd_shape;
-  p.fwd_cg = c->cta_group;
-  p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+  p.fwd_cg = fwd_cta_group(c, L);
+  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.with_loss = 0;
   p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);

@@ -1168,63 +1168,93 @@ __global__ void __launch_bounds__(256) merge_shard_stats_kernel(const float4* __
 }
 
 // ------------------------------------------------------------------------------------------
-// dH of one row slab: fp32 accumulator rows -> bf16 rows of the caller's dH at their original
-// positions.  One warp per row.
-// The dH pass may have cut K into slices that accumulate in separate buffers, split_stride
-// elements apart (same slice count as gemm_extents chose for the pass): summed here in slice order.
-__device__ __forceinline__ float4 sum_k_slices(const float4* p, int n_slices, long long split_stride) {
-  float4 x = __ldcs(p);
-  if (n_slices == 1) return x;
-  for (int s = 1; s < n_slices; ++s) {
-    const float4 y = __ldcs(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + s * split_stride));
-    x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
-  }
-  return x;
-}
+// dH of one row slab: fp32 accumulator rows -> rows of the caller's dH at their original positions, fp32 or bf16.
+// The dH pass may have cut K into slices that accumulate in separate buffers, split_stride elements apart, or cut the
+// tiles of its last wave into parts that lie in slots: summed here in a fixed order.
+struct DhSource {
+  const float* acc;        // [slab rows][d]
+  int d;
+  GemmShape shape;         // the dH pass: together with its grid it fixes how tiles were cut
+  int cg, workers;
+  long long split_stride;
+  const float* slots;      // [slots][tile_rows][tile_cols], tiles cut by stream_k == 2
+  int tile_rows, tile_cols;
+};
 
-// Same with an fp32 destination.
-__global__ void __launch_bounds__(256) scatter_dH_f32_kernel(const float* __restrict__ acc, int d, const GemmShape dh_shape,
-                                                             int dh_cg, int dh_workers, long long split_stride,
-                                                             const int* __restrict__ row_map,
-                                                             float* __restrict__ dH, const DevStatus* st) {
-  int slab_base, rows;
-  slab_extent(st->n_valid, dh_shape.slab_cap, dh_shape.slab_index, slab_base, rows);
-  // stream-K launches always keep two buffers (the second holds the parts that finished a tile)
-  const int n_slices = dh_shape.stream_k ? 2 : gemm_extents(dh_shape, st->n_valid, dh_cg, dh_workers).k_split;
-  const int lane = threadIdx.x & 31;
-  const int warps_per_block = blockDim.x >> 5;
-  for (int i = blockIdx.x * warps_per_block + (threadIdx.x >> 5); i < rows; i += gridDim.x * warps_per_block) {
-    const float4* src = reinterpret_cast<const float4*>(acc + (size_t)i * d);
-    float4* dst = reinterpret_cast<float4*>(dH + (size_t)row_map[slab_base + i] * d);
-    for (int v = lane; v < d / 4; v += 32) dst[v] = sum_k_slices(src + v, n_slices, split_stride);
+__device__ __forceinline__ void add_piece(float4 (&x)[4], const float* q, int cols, int lane) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int v = lane + 32 * k;
+    if (v * 8 < cols) {
+      const float4 a = __ldcs(reinterpret_cast<const float4*>(q) + 2 * v);
+      const float4 b = __ldcs(reinterpret_cast<const float4*>(q) + 2 * v + 1);
+      x[2 * k].x += a.x; x[2 * k].y += a.y; x[2 * k].z += a.z; x[2 * k].w += a.w;
+      x[2 * k + 1].x += b.x; x[2 * k + 1].y += b.y; x[2 * k + 1].z += b.z; x[2 * k + 1].w += b.w;
+    }
   }
 }
 
-__global__ void __launch_bounds__(256) scatter_dH_kernel(const float* __restrict__ acc, int d, const GemmShape dh_shape,
-                                                         int dh_cg, int dh_workers, long long split_stride,
-                                                         const int* __restrict__ row_map,
-                                                         __nv_bfloat16* __restrict__ dH, const DevStatus* st) {
+// One warp per row and column tile (at most 512 columns: two groups of eight per lane).
+template <bool F32>
+__global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const int* __restrict__ row_map,
+                                                         void* __restrict__ dH, const DevStatus* st) {
   int slab_base, rows;
-  slab_extent(st->n_valid, dh_shape.slab_cap, dh_shape.slab_index, slab_base, rows);
-  // stream-K launches always keep two buffers (the second holds the parts that finished a tile)
-  const int n_slices = dh_shape.stream_k ? 2 : gemm_extents(dh_shape, st->n_valid, dh_cg, dh_workers).k_split;
+  slab_extent(st->n_valid, s.shape.slab_cap, s.shape.slab_index, slab_base, rows);
+  const GemmExtents ex = gemm_extents(s.shape, st->n_valid, s.cg, s.workers);
+  const int slices = s.shape.stream_k == 1 ? 2 : ex.k_split;   // stream-K launches always keep two buffers
   const int lane = threadIdx.x & 31;
   const int warps_per_block = blockDim.x >> 5;
-  for (int i = blockIdx.x * warps_per_block + (threadIdx.x >> 5); i < rows; i += gridDim.x * warps_per_block) {
-    // eight elements per lane: two 16-byte loads, one 16-byte store (d is a multiple of 64)
-    const float4* src = reinterpret_cast<const float4*>(acc + (size_t)i * d);
-    uint4* dst = reinterpret_cast<uint4*>(dH + (size_t)row_map[slab_base + i] * d);
-    for (int v = lane; v < d / 8; v += 32) {
-      const float4 x = sum_k_slices(src + 2 * v, n_slices, split_stride);
-      const float4 y = sum_k_slices(src + 2 * v + 1, n_slices, split_stride);
-      __nv_bfloat162 b0 = __floats2bfloat162_rn(x.x, x.y), b1 = __floats2bfloat162_rn(x.z, x.w);
-      __nv_bfloat162 b2 = __floats2bfloat162_rn(y.x, y.y), b3 = __floats2bfloat162_rn(y.z, y.w);
-      uint4 o;
-      o.x = *reinterpret_cast<uint32_t*>(&b0);
-      o.y = *reinterpret_cast<uint32_t*>(&b1);
-      o.z = *reinterpret_cast<uint32_t*>(&b2);
-      o.w = *reinterpret_cast<uint32_t*>(&b3);
-      __stcs(dst + v, o);
+  const unsigned col_tiles = (s.d + s.tile_cols - 1) / s.tile_cols;
+  const unsigned units = (unsigned)rows * col_tiles;
+  for (unsigned u = blockIdx.x * warps_per_block + (threadIdx.x >> 5); u < units; u += gridDim.x * warps_per_block) {
+    const int i = (int)(u / col_tiles), nt = (int)(u - i * col_tiles);
+    const int cols = min(s.tile_cols, s.d - nt * s.tile_cols);
+    const size_t col0 = (size_t)nt * s.tile_cols;
+    float4 x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int r = i / s.tile_rows * ex.n_ranges + nt - (ex.n_units - ex.cut);
+    if (ex.stream_k == 2 && r >= 0) {
+      const int S = ex.cut_parts, mains = ex.cut * S;
+      const size_t slot = (size_t)s.tile_rows * s.tile_cols;
+      const float* base = s.slots + (size_t)(i % s.tile_rows) * s.tile_cols;
+      int h0 = 1, h1 = 0;   // lane s: helpers that did the end of part s
+      if (ex.cut_len > 0 && lane < S) {
+        const long long pos = (long long)r * cut_tile_ends(ex);
+        h0 = cut_helper(ex, s.workers, pos + cut_end_pos(ex, lane));
+        h1 = cut_helper(ex, s.workers, pos + cut_end_pos(ex, lane + 1) - 1);
+      }
+      for (int p = 0; p < S; ++p) {
+        add_piece(x, base + slot * (r * S + p), cols, lane);
+        if (ex.cut_len > 0) {
+          const int a = __shfl_sync(0xffffffffu, h0, p), b = __shfl_sync(0xffffffffu, h1, p);
+          for (int h = a; h <= b; ++h) add_piece(x, base + slot * (mains + r * S + p + h), cols, lane);
+        }
+      }
+    } else {
+      const float* q = s.acc + (size_t)i * s.d + col0;
+      for (int k = 0; k < slices; ++k, q += s.split_stride) add_piece(x, q, cols, lane);
+    }
+    const size_t out = (size_t)row_map[slab_base + i] * s.d + col0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int v = lane + 32 * k;
+      if (v * 8 >= cols) break;
+      const float4 a = x[2 * k], b = x[2 * k + 1];
+      if (F32) {
+        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(dH) + out) + 2 * v;
+        __stcs(dst, a);
+        __stcs(dst + 1, b);
+      } else {
+        __nv_bfloat162 b0 = __floats2bfloat162_rn(a.x, a.y), b1 = __floats2bfloat162_rn(a.z, a.w);
+        __nv_bfloat162 b2 = __floats2bfloat162_rn(b.x, b.y), b3 = __floats2bfloat162_rn(b.z, b.w);
+        uint4 o;
+        o.x = *reinterpret_cast<uint32_t*>(&b0);
+        o.y = *reinterpret_cast<uint32_t*>(&b1);
+        o.z = *reinterpret_cast<uint32_t*>(&b2);
+        o.w = *reinterpret_cast<uint32_t*>(&b3);
+        __stcs(reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(dH) + out) + v, o);
+      }
     }
   }
 }

@@ -1,0 +1,70 @@
+"""Schedules for calls with few rows: column ranges chosen by waves, tiles of the ragged last wave cut into parts.  The
+distribution itself on the CPU, the passes that use it against the oracle on the GPU."""
+import numpy as np
+import pytest
+
+
+@pytest.mark.parametrize("cta_group,workers", [(2, 74), (1, 148), (2, 3), (2, 1)])
+def test_cut_tiles_cover_every_block_once(cta_group, workers):
+    from paper_2512_21450_b200.binding import debug_schedule
+    rng = np.random.default_rng(workers)
+    sizes = [(1, 64, 1), (1, 64 * 9, 1), (300, 152064, 4), (2757, 152064, 7), (5000, 152064, 4), (18947, 4160, 5)]
+    sizes += [(int(rng.integers(1, 20000)), 64 * int(rng.integers(1, 600)), int(rng.integers(1, 12))) for _ in range(60)]
+    for rows, k_len, n_tiles in sizes:
+        u = debug_schedule(rows, 32768, k_len, n_tiles, n_range=1, n_fastest=1, stream_k=2, cta_group=cta_group,
+                           n_workers=workers)
+        m_units, kb = -(-rows // (128 * cta_group)), -(-k_len // 64)
+        cover = np.zeros((m_units, n_tiles, kb), dtype=np.int32)
+        slots, work = set(), np.zeros(workers, dtype=np.int64)
+        for w, mu, c0, c1, ks, kb0, kb1, _ in u:
+            assert c1 == c0 + 1 and kb1 > kb0
+            cover[mu, c0, kb0:kb1] += 1
+            work[w] += kb1 - kb0
+            if ks == 0:
+                assert kb1 - kb0 == kb                           # a whole tile
+            else:
+                assert ks not in slots and ks <= 2 * workers     # a slot of its own
+                slots.add(ks)
+        assert (cover == 1).all()
+        # within 8 % of an even split of all blocks plus what one part may be too long by, unless parts would get too short
+        even = m_units * n_tiles * kb / workers
+        if kb >= 8 * workers:
+            assert work.max() <= 1.08 * even + 8, (rows, k_len, n_tiles, work.max(), even)
+
+
+@pytest.mark.parametrize("rows,n_tiles,most,expect", [(77, 594, 148, 0.88), (276, 594, 118, 0.9), (2757, 594, 75, 0.9),
+                                                      (60, 16, 16, 0.0), (1, 1, 16, 0.0), (4096, 594, 75, 0.9)])
+def test_column_ranges_fill_the_machine(rows, n_tiles, most, expect):
+    from paper_2512_21450_b200.binding import debug_schedule
+    u = debug_schedule(rows, 32768, 2048, n_tiles, n_range=-1000 - most, cta_group=2, n_workers=74)
+    m_units = -(-rows // 256)
+    cover, work = np.zeros((m_units, n_tiles), dtype=np.int32), np.zeros(74, dtype=np.int64)
+    for w, mu, c0, c1, *_ in u:
+        cover[mu, c0:c1] += 1
+        work[w] += c1 - c0
+    assert (cover == 1).all() and len({(r[2], r[3]) for r in u}) <= most
+    assert work.mean() >= expect * work.max()          # 594 tiles on 74 workers: 9 each at best, 8.03 on average
+
+
+# T: one 128-row tile (single CTAs form the logits), one and several pairs; V and d: ranges of a few and of many k-blocks,
+# tiles of 256 and of 512 columns, ends of parts shared among helpers (11, 13, 21 tiles on 74 pairs); masked rows make the
+# valid ones fewer than T says
+@pytest.mark.gpu
+@pytest.mark.parametrize("L_max,d,V,kw", [
+    (1, 64, 300, {}), (16, 64, 70001, {}), (16, 512, 9000, {}), (40, 320, 5000, {}), (150, 768, 40000, {}),
+    (150, 1024, 3000, {}), (400, 512, 90000, {}), (40, 512, 9000, dict(cta_group=1)), (150, 512, 40000, dict(max_ctas=10)),
+])
+@pytest.mark.parametrize("f32", [False, True])
+def test_few_rows_match_oracle(L_max, d, V, kw, f32):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    from tests.test_gpu_parity import _check_against_oracle
+    c = Context(0)
+    try:
+        if "cta_group" in kw:
+            c.set_cta_group(kw["cta_group"])
+        if "max_ctas" in kw:
+            c.set_max_ctas(kw["max_ctas"])
+        _check_against_oracle(c, make_workload(1, prompts=1, L_max=L_max, d=d, V=V, seed=4000 + V + L_max), dH_fp32=f32)
+    finally:
+        c.close()
