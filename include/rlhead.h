@@ -222,8 +222,8 @@ rl_status rl_token_loss(rl_ctx* ctx, const float* logp, const float* entropy, co
 /* Padding-free row map on its own (section 4.4, training without padding tokens): row_map[i] = index of
  * the i-th row with mask != 0, ascending, for i < *n_valid; entries past that are left untouched.
  * mask NULL = all rows valid.  row_map[T] (int32) and n_valid[1] (int32) are device pointers; the
- * workspace needs (T / 4096 + 3) * 4 bytes.  Every other call of this library runs the same
- * three kernels internally; this entry exists so that the map can be checked and timed by itself.
+ * workspace needs (T / 4096 + 3) * 4 bytes.  Calls of more than 32768 rows run the same
+ * kernels internally; this entry exists so that the map can be checked and timed by itself.
  * Errors: T < 0 or T >= 2^31, NULL outputs -> RL_ERR_INVALID_ARG; RL_ERR_WORKSPACE. */
 rl_status rl_mask_scan(rl_ctx* ctx, const uint8_t* mask, int64_t T, int32_t* row_map, int32_t* n_valid);
 

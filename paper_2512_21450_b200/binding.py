@@ -154,7 +154,8 @@ def load_library():
 
 
 def _ptr(t):
-    return c_void_p(t.data_ptr()) if t is not None else c_void_p(0)
+    """Device address as a plain int (0 = NULL): ctypes turns it into the declared c_void_p itself."""
+    return 0 if t is None else t.data_ptr()
 
 
 def _check(status, where):
@@ -188,7 +189,8 @@ class Context:
             pass
 
     def _bind_stream(self):
-        _check(self.lib.rl_set_stream(self.handle, c_void_p(torch.cuda.current_stream(self.device).cuda_stream)),
+        # the raw handle of torch's current stream, without building a Stream object for every call
+        _check(self.lib.rl_set_stream(self.handle, torch._C._cuda_getCurrentRawStream(self.device.index)),
                "rl_set_stream")
 
     def workspace_bytes(self, T, d, V, host=False, d_ref=0):

@@ -68,13 +68,17 @@ constexpr int kSlabRowsMax = 32768;        // rows of one gradient slab
 constexpr long long kSlabElements = 1ll << 31;
 constexpr int kSlabRowsMin = 2048;
 // Device words a context owns besides the workspace: the status record, a few scalars of the small kernels
-// (byte 64: batch statistics, 96: longest response, 128: valid-row count of rl_token_loss) and, from byte 256 on,
-// the block partials of rl_token_loss.
+// (byte 64: batch statistics, 96: longest response, kTicketOffset: ticket counter of the loss kernels), the valid-row
+// counts of rl_token_loss and, behind them, its block partials.
 constexpr int kTokenLossBlocks = 1024;
-constexpr size_t kStatusBytes = 256 + (size_t)kTokenLossBlocks * kLossSums * sizeof(double);
+constexpr size_t kCountOffset = 256;
+constexpr size_t kSumsOffset = kCountOffset + kCountBlocks * sizeof(unsigned);
+constexpr size_t kStatusBytes = kSumsOffset + (size_t)kTokenLossBlocks * kLossSums * sizeof(double);
 constexpr int kAdvRowsMinGroups = 2048;     // from this many groups on, GRPO advantages run one thread per group
 constexpr int kWideGain = 96;              // time of a 256 x 512 tile, in % of two 256 x 256 tiles of the same K
 constexpr int kWideMinRows = 8192;         // rows of a slab (K of the dW pass) from which its tiles are 512 wide
+constexpr int kMergeBlocks = 512;          // blocks per merge launch when a call makes several (kLossThreads threads each)
+constexpr size_t kTicketOffset = 192;      // in the device block: blocks of a loss kernel that are done (0 between calls)
 constexpr int kDhSplitMax = 4;             // most K slices (separate fp32 accumulators) of the dH pass
 constexpr int kSlabColsMax = 148 * 256;    // vocabulary columns of one gradient slab (148 tiles of 256: two per SM pair)
 
@@ -83,6 +87,11 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // fp32 accumulator buffers of the dH pass: one per K slice, or two when stream-K balancing is on
 inline bool dh_uses_stream_k(const rl_ctx* c) { return c->dh_stream_k && c->dh_k_slices == 1; }
 inline int dh_buffers(const rl_ctx* c) { return dh_uses_stream_k(c) ? 2 : c->dh_k_slices; }
+// Blocks of the merge of `rows` rows, 32 at a time; all launches of a call together have at most kMergeBlocks * (1 + slabs).
+inline int merge_blocks(int64_t rows, int slabs) {
+  const int64_t n = (rows + 31) / 32, most = slabs > 1 ? kMergeBlocks : 2 * kMergeBlocks;
+  return (int)(n < most ? n : most);
+}
 // Neither option set: the tiles of the dH pass's ragged last wave are cut into parts that lie in slots.
 inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_slices == 1; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
@@ -101,6 +110,7 @@ inline size_t dh_slot_bytes(const rl_ctx* c, int64_t d) {
 struct WsLayout {
   int Tpad, Ts, Vs;
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
+  size_t row_pos;                                    // position of every row in the row map (large T)
   size_t shift2, flags;                              // one-sweep path: log-sum-exp estimates, row-tile flags
   int part_ranges;                                   // column ranges per row that the partials have room for
   size_t dH_slots;                                   // parts of cut dH tiles (0: none)
@@ -187,12 +197,13 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
     L.part_ranges = (int)n_part_ranges;
     L.partials = take(n_part_ranges * L.Tpad * sizeof(float4));
   }
-  L.block_sums = take((size_t)1024 * kLossSums * sizeof(double));
+  L.block_sums = take((size_t)kMergeBlocks * (1 + L.n_row_slabs) * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
   L.G = take((size_t)L.Ts * L.Vs * 2);
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
   L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
   L.shift2 = take((size_t)L.Tpad * 4);
+  L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
   L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
   L.flags = take((size_t)L.n_flags * 4);
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = 0;
@@ -387,6 +398,18 @@ inline int row_group_tiles(const rl_ctx* c, int64_t k) {
 
 inline rl_status cuda_ok() { return cudaGetLastError() == cudaSuccess ? RL_OK : RL_ERR_CUDA; }
 
+// Mask scan of T rows in two launches (three for very many), row_pos may be NULL.
+void launch_mask_scan(rl_ctx* c, const uint8_t* mask, int64_t T, int* block_counts, int* row_map, int* row_pos) {
+  const int pr = prof_begin(c, 4);
+  const int n_blocks = (int)((T + kScanRowsPerBlock - 1) / kScanRowsPerBlock);
+  const int sums = n_blocks <= kScanSumBlocks ? 1 : 0;
+  mask_count_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts);
+  if (!sums) mask_offsets_kernel<<<1, 1024, 0, c->stream>>>(block_counts, n_blocks, c->dstatus);
+  mask_write_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts, sums, row_map, row_pos, c->dstatus);
+  prof_end(c, pr, 4);
+  c->launches += sums ? 2 : 3;
+}
+
 // Which part of the forward stage a call needs, and where its rows of W sit in the vocabulary.
 struct FwdPlan {
   bool scan = true;          // mask scan (false: the row map of an earlier call on this workspace is reused)
@@ -394,6 +417,7 @@ struct FwdPlan {
   int64_t vocab_off = 0;     // first vocabulary id of W's rows (vocabulary-parallel head)
   int64_t V_total = 0;       // size of the whole vocabulary for the token-range check (0: V)
   const float* old_logp = nullptr;   // one-sweep path: estimate every row's log-sum-exp while its row is copied
+  RowOutputs out = {};       // per-row outputs of the call, zeroed where the mask is 0
 };
 
 // Mask scan + row compaction + forward statistics.  Leaves per-range partials in the workspace.
@@ -404,18 +428,9 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   int* row_map = reinterpret_cast<int*>(ws + L.row_map);
   int* tokens_c = reinterpret_cast<int*>(ws + L.tokens_c);
   __nv_bfloat16* Hc = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc);
-  if (plan.scan) {
-    const int pr = prof_begin(c, 4);
-    int* block_counts = reinterpret_cast<int*>(ws + L.scan_counts);
-    const int n_blocks = (int)((T + kScanRowsPerBlock - 1) / kScanRowsPerBlock);
-    mask_count_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts);
-    mask_offsets_kernel<<<1, 1024, 0, c->stream>>>(block_counts, n_blocks, c->dstatus);
-    mask_write_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts, row_map);
-    prof_end(c, pr, 4);
-    c->launches += 3;
-  }
-  SweepPrep sp;
-  memset(&sp, 0, sizeof(sp));
+  PrepParams pp;
+  memset(&pp, 0, sizeof(pp));
+  SweepPrep& sp = pp.sp;
   if (plan.old_logp) {
     sp.W = static_cast<const __nv_bfloat16*>(W);
     sp.ldW = ldW;
@@ -424,11 +439,33 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     sp.flags = reinterpret_cast<int*>(ws + L.flags);
     sp.n_flags = L.n_flags;
   }
-  const int pr_gather = prof_begin(c, 5);
-  gather_rows_kernel<<<c->n_sm * 4, 256, 0, c->stream>>>(static_cast<const __nv_bfloat16*>(H), ldH, (int)d, row_map,
-                                                         tokens, (int)(plan.V_total > 0 ? plan.V_total : V),
-                                                         (int)plan.vocab_off, Hc, tokens_c, sp, c->dstatus);
-  prof_end(c, pr_gather, 5);
+  pp.H = static_cast<const __nv_bfloat16*>(H);
+  pp.ldH = ldH;
+  pp.d = (int)d;
+  pp.mask = mask;
+  pp.T = (int)T;
+  pp.tokens = tokens;
+  pp.V = (int)(plan.V_total > 0 ? plan.V_total : V);
+  pp.vocab_off = (int)plan.vocab_off;
+  pp.Hc = Hc;
+  pp.tokens_c = tokens_c;
+  pp.row_map = row_map;
+  pp.out = plan.out;
+  if (T <= kPrepRows) {
+    const int pr = prof_begin(c, 5);
+    int rows = (int)align_up((size_t)(T + c->n_sm * 4 - 1) / (c->n_sm * 4), 16);   // at most 256: kPrepRows / (4 n_sm)
+    if (rows > 256) rows = 256;
+    pp.rows_per_block = rows;
+    prep_rows_kernel<true><<<(int)((T + rows - 1) / rows), 256, 0, c->stream>>>(pp, c->dstatus);
+    prof_end(c, pr, 5);
+  } else {
+    int* row_pos = reinterpret_cast<int*>(ws + L.row_pos);
+    if (plan.scan) launch_mask_scan(c, mask, T, reinterpret_cast<int*>(ws + L.scan_counts), row_map, row_pos);
+    pp.row_pos = row_pos;
+    const int pr = prof_begin(c, 5);
+    prep_rows_kernel<false><<<c->n_sm * 8, 256, 0, c->stream>>>(pp, c->dstatus);
+    prof_end(c, pr, 5);
+  }
   c->launches += 1;
   if (!plan.stats) {
     memset(shape_out, 0, sizeof(*shape_out));
@@ -773,7 +810,10 @@ rl_status rl_grpo_advantages_ex(rl_ctx* c, const float* rewards, int64_t n_seq, 
   // many groups of 4, 8, ... 32 responses in 16-byte aligned arrays: one thread per group; else shuffle segments
   const bool rows_path = n_groups >= kAdvRowsMinGroups && group_size % 4 == 0 && group_size <= 32 &&
                          ((reinterpret_cast<uintptr_t>(rewards) | reinterpret_cast<uintptr_t>(adv_seq)) & 15) == 0;
-  if (rows_path) {
+  // few groups of few responses: the broadcast works the advantages out itself
+  const bool fused = adv_tok && T > 0 && n_groups < kAdvRowsMinGroups && group_size <= 32 && rewards != adv_seq;
+  if (fused) {
+  } else if (rows_path) {
     const int blocks = (n_groups + 255) / 256;
     const float4* r4 = reinterpret_cast<const float4*>(rewards);
     float4* a4 = reinterpret_cast<float4*>(adv_seq);
@@ -791,15 +831,19 @@ rl_status rl_grpo_advantages_ex(rl_ctx* c, const float* rewards, int64_t n_seq, 
     grpo_adv_kernel<<<(n_groups + groups_per_block - 1) / groups_per_block, warps * 32, 0, c->stream>>>(
         rewards, n_groups, group_size, ddof, eps_std, adv_seq);
   }
-  c->launches++;
-  if (adv_tok) {
-    if (T > 0) {
-      const long long rows_per_block = (long long)kBroadcastSweeps * 1024;
-      long long blocks = (T + rows_per_block - 1) / rows_per_block;
-      if (blocks > (long long)c->n_sm * 32) blocks = (long long)c->n_sm * 32;
-      broadcast_adv_kernel<<<(int)blocks, 256, 0, c->stream>>>(adv_seq, seq_offsets, (int)n_seq, (long long)T, adv_tok);
-      c->launches++;
-    }
+  c->launches += fused ? 0 : 1;
+  if (adv_tok && T > 0) {
+    long long sweeps = T / (1024ll * 2 * c->n_sm);   // two blocks per SM before a block takes more than one sweep
+    sweeps = sweeps < 1 ? 1 : (sweeps > kBroadcastSweeps ? kBroadcastSweeps : sweeps);
+    long long blocks = (T + sweeps * 1024 - 1) / (sweeps * 1024);
+    if (blocks > (long long)c->n_sm * 32) blocks = (long long)c->n_sm * 32;
+    if (fused)
+      broadcast_adv_kernel<true><<<(int)blocks, 256, 0, c->stream>>>(rewards, group_size, ddof, eps_std, adv_seq, seq_offsets,
+                                                                     (int)n_seq, (long long)T, (int)sweeps, adv_tok);
+    else
+      broadcast_adv_kernel<false><<<(int)blocks, 256, 0, c->stream>>>(rewards, group_size, ddof, eps_std, adv_seq, seq_offsets,
+                                                                      (int)n_seq, (long long)T, (int)sweeps, adv_tok);
+    c->launches++;
   }
   prof_end(c, pr_adv, 8);
   return cuda_ok();
@@ -850,25 +894,26 @@ rl_status rl_token_loss(rl_ctx* c, const float* logp, const float* entropy, cons
     return cuda_ok();
   }
   char* base = reinterpret_cast<char*>(c->dstatus);
-  unsigned long long* count = reinterpret_cast<unsigned long long*>(base + 128);
-  double* block_sums = reinterpret_cast<double*>(base + 256);
+  unsigned* counts = reinterpret_cast<unsigned*>(base + kCountOffset);
+  double* block_sums = reinterpret_cast<double*>(base + kSumsOffset);
   const int pr = prof_begin(c, 6);
+  long long cb = 0;
   if (mask) {
-    cudaMemsetAsync(count, 0, 8, st);
-    long long cb = (T / 16 + 255) / 256 + 1;
-    if (cb > (long long)c->n_sm * 8) cb = (long long)c->n_sm * 8;
-    count_valid_kernel<<<(int)cb, 256, 0, st>>>(mask, (long long)T, count);
+    cb = (T / 16 + 255) / 256 + 1;
+    if (cb > kCountBlocks) cb = kCountBlocks;
+    count_valid_kernel<<<(int)cb, 256, 0, st>>>(mask, (long long)T, counts);
     c->launches++;
   }
   TokenLossParams p;
   memset(&p, 0, sizeof(p));
   p.logp = logp; p.entropy = entropy; p.old_logp = old_logp; p.ref_logp = beta != 0.f ? ref_logp : nullptr;
   p.adv = adv; p.mask = mask; p.token_weight = token_weight;
-  p.count = token_count ? reinterpret_cast<const unsigned long long*>(token_count) : (mask ? count : nullptr);
-  p.n_known = (unsigned long long)T;
+  p.counts = mask ? counts : nullptr;
+  p.n_counts = (int)cb;
+  p.token_count = reinterpret_cast<const unsigned long long*>(token_count);
   p.T = (long long)T;
   p.eps_low = eps_low; p.eps_high = eps_high; p.beta = beta; p.ent_coef = ent_coef;
-  p.dlogp = dlogp; p.dentropy = dentropy; p.block_sums = block_sums;
+  p.dlogp = dlogp; p.dentropy = dentropy;
   long long blocks = ((T + 3) / 4 + kLossThreads - 1) / kLossThreads;
   if (blocks > kTokenLossBlocks) blocks = kTokenLossBlocks;
   if (blocks > (long long)c->n_sm * 4) blocks = (long long)c->n_sm * 4;   // one wave: four blocks are resident per SM
@@ -877,11 +922,15 @@ rl_status rl_token_loss(rl_ctx* c, const float* logp, const float* entropy, cons
                   reinterpret_cast<uintptr_t>(token_weight) | reinterpret_cast<uintptr_t>(dlogp) |
                   reinterpret_cast<uintptr_t>(dentropy);
   const bool vec = (all & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0;
+  p.fin.block_sums = block_sums;
+  p.fin.ticket = reinterpret_cast<unsigned*>(base + kTicketOffset);
+  p.fin.base = 0;
+  p.fin.total = (int)blocks;
+  p.fin.loss = loss;
+  p.fin.metrics = metrics_out;
   if (vec) token_loss_kernel<true><<<(int)blocks, kLossThreads, 0, st>>>(p);
   else     token_loss_kernel<false><<<(int)blocks, kLossThreads, 0, st>>>(p);
-  finalize_token_loss_kernel<<<1, 32 * kLossSums, 0, st>>>(block_sums, (int)blocks, loss, metrics_out, mask ? count : nullptr,
-                                               (unsigned long long)T);
-  c->launches += 2;
+  c->launches += 1;
   prof_end(c, pr, 6);
   return cuda_ok();
 }
@@ -905,17 +954,18 @@ rl_status rl_kl_shaped_returns(rl_ctx* c, const float* seq_value, const float* l
   }
   if (!seq_value || !seq_offsets) return RL_ERR_INVALID_ARG;
   if (kl_estimate == RL_KL_GIVEN ? !kl_tok : (!logp || !ref_logp)) return RL_ERR_INVALID_ARG;
-  const int warps = 8;
-  long long blocks = (n_seq + warps - 1) / warps;
-  if (blocks > (long long)c->n_sm * 64) blocks = (long long)c->n_sm * 64;
+  const bool by_block = T >= 32 * kShapeChunks * n_seq;   // a block per response, else a warp
+  int64_t blocks = by_block ? n_seq : (n_seq + kShapeWarps - 1) / kShapeWarps;
+  if (blocks > (int64_t)c->n_sm * 64) blocks = (int64_t)c->n_sm * 64;
   const int pr = prof_begin(c, 8);
-  zero_outside_ranges_kernel<<<c->n_sm, 256, 0, c->stream>>>(seq_offsets, (int)n_seq, (long long)T, returns,
-                                                             shaped_reward);
-  kl_shaped_returns_kernel<<<(int)blocks, warps * 32, 0, c->stream>>>(seq_value, logp, ref_logp, kl_tok, mask,
-                                                                      seq_offsets, (int)n_seq, beta, gamma, kl_estimate,
-                                                                      shaped_reward, returns);
+  auto launch = [&](auto kernel) {
+    kernel<<<(int)blocks, 32 * kShapeWarps, 0, c->stream>>>(seq_value, logp, ref_logp, kl_tok, mask, seq_offsets, (int)n_seq,
+                                                            (long long)T, beta, gamma, kl_estimate, shaped_reward, returns);
+  };
+  if (by_block) launch(kl_shaped_returns_kernel<kShapeWarps>);
+  else          launch(kl_shaped_returns_kernel<1>);
   prof_end(c, pr, 8);
-  c->launches += 2;
+  c->launches += 1;
   return cuda_ok();
 }
 
@@ -925,12 +975,7 @@ rl_status rl_mask_scan(rl_ctx* c, const uint8_t* mask, int64_t T, int32_t* row_m
   const int n_blocks = (int)((T + kScanRowsPerBlock - 1) / kScanRowsPerBlock);
   if (!c->ws || c->ws_bytes < ((size_t)n_blocks + 2) * 4) return RL_ERR_WORKSPACE;
   int* block_counts = static_cast<int*>(c->ws);
-  const int pr = prof_begin(c, 4);
-  mask_count_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts);
-  mask_offsets_kernel<<<1, 1024, 0, c->stream>>>(block_counts, n_blocks, c->dstatus);
-  mask_write_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts, row_map);
-  prof_end(c, pr, 4);
-  c->launches += 3;
+  launch_mask_scan(c, mask, T, block_counts, row_map, nullptr);
   if (cudaMemcpyAsync(n_valid, &c->dstatus->n_valid, 4, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
     return RL_ERR_CUDA;
   return cuda_ok();
@@ -947,11 +992,10 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   const WsLayout L = ws_layout(c, T, d, V, false);
   if ((s = check_ws(c, L)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
-  cudaMemsetAsync(logp, 0, (size_t)T * 4, c->stream);
-  if (entropy) cudaMemsetAsync(entropy, 0, (size_t)T * 4, c->stream);
-  if (lse) cudaMemsetAsync(lse, 0, (size_t)T * 4, c->stream);
   GemmShape fwd_shape;
-  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape)) != RL_OK) return s;
+  FwdPlan plan;
+  plan.out.value[0] = logp; plan.out.value[1] = entropy; plan.out.value[2] = lse;
+  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape, nullptr, plan)) != RL_OK) return s;
   LossParams p;
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
@@ -966,8 +1010,7 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   p.logp_out = logp;
   p.ent_out = entropy;
   p.lse_out = lse;
-  int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
-  if (blocks > 1024) blocks = 1024;
+  const int blocks = merge_blocks(T, 1);
   combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
   c->launches++;
   return cuda_ok();
@@ -1030,9 +1073,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     if (o.metrics_out) cudaMemsetAsync(o.metrics_out, 0, 32, st);
     return cuda_ok();
   }
-  cudaMemsetAsync(dH, 0, (size_t)T * d * (o.dH_dtype ? 4 : 2), st);
-  if (o.logp_out) cudaMemsetAsync(o.logp_out, 0, (size_t)T * 4, st);
-  if (o.entropy_out) cudaMemsetAsync(o.entropy_out, 0, (size_t)T * 4, st);
 
   // ---- forward: statistics per (row, vocabulary range).  One sweep: a slab that holds whole rows lets the pass that
   // forms their logits leave them there as 16-bit codes, which an elementwise pass turns into the gradient once the
@@ -1043,6 +1083,10 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
                      (L.n_row_slabs == 1 || (L.Ts % kFlagRows == 0 && !seq_path));
   GemmShape fwd_shape;
   FwdPlan plan;
+  plan.out.dH = dH;
+  plan.out.dH_row_bytes = (long long)d * (o.dH_dtype ? 4 : 2);
+  plan.out.value[0] = o.logp_out; plan.out.value[1] = o.entropy_out;
+  plan.out.value[2] = o.kl_full ? o.kl_out : nullptr;
   if (sweep) {
     plan.stats = false;
     plan.old_logp = old_logp;
@@ -1083,7 +1127,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   if (sweep || seq_path) p.logp_c = reinterpret_cast<float*>(ws + L.logp_c);
   p.logp_out = o.logp_out;
   p.ent_out = o.entropy_out;
-  p.block_sums = reinterpret_cast<double*>(ws + L.block_sums);
   if (shard) {
     p.ext_logp = shard->logp;
     p.ext_ent = shard->entropy;
@@ -1098,25 +1141,28 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     p.kl_c = reinterpret_cast<float*>(ws + L.kl_c);
     p.cb_c = reinterpret_cast<float*>(ws + L.cb_c);
     p.kl_out = o.kl_out;
-    if (o.kl_out) cudaMemsetAsync(o.kl_out, 0, (size_t)T * 4, st);
   }
-  int blocks = 0;   // blocks whose partial sums make up the loss
   // merge of slab r (one sweep) or of all rows, then the loss and the coefficients of the backward pass
+  LossFinish fin;
+  fin.block_sums = reinterpret_cast<double*>(ws + L.block_sums);
+  fin.ticket = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(c->dstatus) + kTicketOffset);
+  fin.loss = loss;
+  fin.metrics = o.metrics_out;
   auto merge_and_loss = [&](int r) {
-    const int rows_cap = sweep ? L.Ts : (int)T;
-    int nb = (rows_cap + kLossThreads - 1) / kLossThreads;
-    const int nb_max = 1024 / (sweep ? L.n_row_slabs : 1);
-    if (nb > nb_max) nb = nb_max;
+    const int slabs = sweep ? L.n_row_slabs : 1;
+    const int nb = merge_blocks(sweep ? L.Ts : T, slabs);
     const int pr_loss = prof_begin(c, 6);
     if (!seq_path) {
-      LossParams ps = p;
-      ps.block_sums = p.block_sums + (size_t)r * nb * kLossSums;
-      blocks = (r + 1) * nb;
-      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(ps, c->dstatus);
+      p.fin = fin;
+      p.fin.base = r * nb;
+      p.fin.total = slabs * nb;
+      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(p, c->dstatus);
       c->launches++;
     } else {
-      // merge the statistics first, then one warp per response forms weights, ratios and the loss
+      // merge the statistics first, then one team per response forms weights, ratios and the loss; valid rows that lie
+      // outside every response range take no part: their coefficients stay 0
       p.with_loss = 0;
+      p.zero_coef = 1;
       combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(p, c->dstatus);
       SeqParams q;
       memset(&q, 0, sizeof(q));
@@ -1135,27 +1181,23 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       q.l_max = reinterpret_cast<int*>(reinterpret_cast<char*>(c->dstatus) + 96);
       q.cp_c = p.cp_c;
       q.ce_c = p.ce_c;
-      q.block_sums = p.block_sums;
-      // valid rows that lie outside every response range take no part: their coefficients stay 0
-      cudaMemsetAsync(q.cp_c, 0, (size_t)L.Tpad * 4, st);
-      cudaMemsetAsync(q.ce_c, 0, (size_t)L.Tpad * 4, st);
-      seq_lmax_kernel<<<1, 1024, 0, st>>>(o.seq_offsets, (int)o.n_seq, q.l_max);
-      blocks = (int)((o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32));
-      if (blocks > 1024) blocks = 1024;
-      seq_loss_kernel<<<blocks, kLossThreads, 0, st>>>(q, c->dstatus);
-      c->launches += 3;
+      q.fin = fin;
+      q.fin.base = 0;
+      if (q.agg_mode == 2) {
+        seq_lmax_kernel<<<1, 1024, 0, st>>>(o.seq_offsets, (int)o.n_seq, q.l_max);
+        c->launches++;
+      }
+      // a block per response unless that would be mostly idle threads
+      const bool by_block = T >= 64 * o.n_seq;
+      const int64_t teams = by_block ? o.n_seq : (o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32);
+      q.fin.total = (int)(teams < 1024 ? teams : 1024);
+      if (by_block) seq_loss_kernel<kLossThreads><<<q.fin.total, kLossThreads, 0, st>>>(q, c->dstatus);
+      else          seq_loss_kernel<32><<<q.fin.total, kLossThreads, 0, st>>>(q, c->dstatus);
+      c->launches += 2;
     }
     prof_end(c, pr_loss, 6);
   };
-  auto finalize = [&]() {
-    finalize_loss_kernel<<<1, 32 * kLossSums, 0, st>>>(p.block_sums, blocks, loss, o.metrics_out, c->dstatus);
-    c->launches++;
-  };
-  if (!sweep) {
-    merge_and_loss(0);
-    finalize();
-  }
-
+  if (!sweep) merge_and_loss(0);
   // ---- backward, one (row slab x vocabulary slab) at a time
   __nv_bfloat16* Hc = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc);
   __nv_bfloat16* G = reinterpret_cast<__nv_bfloat16*>(ws + L.G);
@@ -1340,7 +1382,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     prof_end(c, pr_sc, 7);
     c->launches++;
   }
-  if (sweep) finalize();
   return cuda_ok();
 }
 
@@ -1382,11 +1423,11 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   const WsLayout L = ws_layout(c, T, d, V_shard, false);
   if ((s = check_ws(c, L)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
-  cudaMemsetAsync(stats, 0, (size_t)T * 16, c->stream);
   GemmShape fwd_shape;
   FwdPlan plan;
   plan.vocab_off = vocab_offset;
   plan.V_total = V_total;
+  plan.out.stats = reinterpret_cast<float4*>(stats);
   if ((s = run_forward(c, L, H, ldH, W_shard, ldW, tokens, mask, T, d, V_shard, &fwd_shape, nullptr, plan)) != RL_OK)
     return s;
   LossParams p;
@@ -1398,8 +1439,7 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.stats_out = reinterpret_cast<float4*>(stats);
-  int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
-  if (blocks > 1024) blocks = 1024;
+  const int blocks = merge_blocks(T, 1);
   const int pr = prof_begin(c, 6);
   combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
   prof_end(c, pr, 6);
@@ -1443,10 +1483,9 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
   if (s != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
   for (int i = 0; i < n_models; ++i) {
-    cudaMemsetAsync(logp[i], 0, (size_t)T * 4, c->stream);
-    if (entropy && entropy[i]) cudaMemsetAsync(entropy[i], 0, (size_t)T * 4, c->stream);
     GemmShape fwd_shape;
     FwdPlan plan;
+    plan.out.value[0] = logp[i]; plan.out.value[1] = entropy ? entropy[i] : nullptr;
     plan.scan = i == 0;   // the mask is scanned once; every model reuses the row map
     if ((s = run_forward(c, L, H[i], ldH[i], W[i], ldW[i], tokens, mask, T, d[i], V, &fwd_shape, nullptr, plan)) != RL_OK)
       return s;
@@ -1462,8 +1501,7 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
     p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
     p.logp_out = logp[i];
     p.ent_out = entropy ? entropy[i] : nullptr;
-    int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
-    if (blocks > 1024) blocks = 1024;
+    const int blocks = merge_blocks(T, 1);
     combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
     c->launches++;
   }
@@ -1856,11 +1894,10 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   char* ws = static_cast<char*>(c->ws);
   // the array keeps the previous call's contents: the status word and the valid-row count start at zero
   if (cudaMemsetAsync(c->dstatus, 0, sizeof(DevStatus), c->stream) != cudaSuccess) return RL_ERR_CUDA;
-  cudaMemsetAsync(logp, 0, (size_t)T * 4, c->stream);
-  if (entropy) cudaMemsetAsync(entropy, 0, (size_t)T * 4, c->stream);
-  if (lse) cudaMemsetAsync(lse, 0, (size_t)T * 4, c->stream);
   GemmShape fwd_shape;
-  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape)) != RL_OK) return s;
+  FwdPlan plan;
+  plan.out.value[0] = logp; plan.out.value[1] = entropy; plan.out.value[2] = lse;
+  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape, nullptr, plan)) != RL_OK) return s;
   LossParams p;
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
@@ -1875,8 +1912,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   p.logp_out = logp;
   p.ent_out = entropy;
   p.lse_out = lse;
-  int blocks = (int)((T + kLossThreads - 1) / kLossThreads);
-  if (blocks > 1024) blocks = 1024;
+  const int blocks = merge_blocks(T, 1);
   combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
   if (dev_status &&
       cudaMemcpyAsync(dev_status, c->dstatus, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)

@@ -9,10 +9,12 @@
 namespace rlh {
 
 // ------------------------------------------------------------------------------------------
-// Mask scan in three launches: row_map[i] = index of the i-th row with mask != 0 (ascending),
-// n_valid = their number.  Each block owns 4096 consecutive rows, each thread 16 of them (one
-// 16-byte load when the mask is 16-byte aligned): (1) per-block counts, (2) one block turns the
-// counts into exclusive offsets, (3) every block scans its rows again and writes its indices.
+// Mask scan: row_map[i] = index of the i-th row with mask != 0 (ascending), n_valid = their number, and on request
+// row_pos[t] = position of row t in the map, -1 for a masked row.  Each block owns 4096 consecutive rows, each thread 16
+// of them (one 16-byte load when the mask is 16-byte aligned): (1) per-block counts, (2) every block adds up the counts
+// before its own, scans its rows again and writes its indices.  From kScanSumBlocks blocks on, one block turns the counts
+// into offsets in a launch between the two.  Up to kPrepRows rows none of this runs: prep_rows_kernel scans for itself.
+constexpr int kScanSumBlocks = 1024;
 constexpr int kScanThreads = 256;
 constexpr int kScanRowsPerThread = 16;
 constexpr int kScanRowsPerBlock = kScanThreads * kScanRowsPerThread;
@@ -93,15 +95,48 @@ __global__ void __launch_bounds__(1024) mask_offsets_kernel(int* __restrict__ bl
   if (threadIdx.x == 0) st->n_valid = carry;
 }
 
+// sums: block_offsets holds counts (to be added up here, total -> st->n_valid) instead of offsets.
 __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t* __restrict__ mask, int T,
-                                                                  const int* __restrict__ block_offsets,
-                                                                  int* __restrict__ row_map) {
+                                                                  const int* __restrict__ block_offsets, int sums,
+                                                                  int* __restrict__ row_map, int* __restrict__ row_pos,
+                                                                  DevStatus* st) {
   __shared__ int warp_sums[32];
-  __shared__ int block_total;
+  __shared__ int block_total, before, all;
   __shared__ int staged[kScanRowsPerBlock];   // the block's valid rows, in order
   const long long base = ((long long)blockIdx.x * kScanThreads + threadIdx.x) * kScanRowsPerThread;
   unsigned bits = scan_load_bits(mask, base, T);
+  int offset;
+  if (sums) {
+    if (threadIdx.x == 0) before = all = 0;
+    __syncthreads();
+    int c = 0, a = 0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kScanThreads) {
+      const int v = block_offsets[i];
+      a += v;
+      c += i < (int)blockIdx.x ? v : 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      c += __shfl_xor_sync(0xffffffffu, c, o);
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
+    if ((threadIdx.x & 31) == 0) { atomicAdd(&before, c); atomicAdd(&all, a); }
+    __syncthreads();
+    offset = before;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->n_valid = all;
+  } else {
+    offset = block_offsets[blockIdx.x];
+  }
   int pos = block_exclusive_scan(__popc(bits), warp_sums, &block_total);
+  if (row_pos) {
+    int q = offset + pos;
+#pragma unroll
+    for (int i = 0; i < kScanRowsPerThread; ++i) {
+      const bool v = (bits >> i) & 1u;
+      if (base + i < T) row_pos[base + i] = v ? q : -1;
+      q += v;
+    }
+  }
   while (bits) {
     const int i = __ffs(bits) - 1;
     bits &= bits - 1;
@@ -109,7 +144,7 @@ __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t*
   }
   __syncthreads();
   // coalesced copy of the block's indices to their place in the map
-  int* dst = row_map + block_offsets[blockIdx.x];
+  int* dst = row_map + offset;
   for (int k = threadIdx.x; k < block_total; k += kScanThreads) dst[k] = staged[k];
 }
 
@@ -119,7 +154,9 @@ __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t*
 // token-range check.  One warp per row, 16-byte loads.  Token ids are checked against the whole
 // vocabulary [0, V) and stored relative to vocab_off, the first id of the rows of W this call
 // holds (0 unless the head is split by vocabulary): an id outside the held slice becomes a
-// negative or too large column that no tile ever matches.
+// negative or too large column that no tile ever matches.  The rows are walked in their original order, so that the
+// outputs of masked rows are zeroed in passing: nothing is cleared that is written again (a memset of dH cost as
+// much as the copy itself, and each memset a launch).
 // SweepPrep (shift2 != NULL): the one-sweep path also needs an estimate of every row's log-sum-exp before its logits are
 // formed.  The behaviour policy supplies it: lse ~ z_y - old_logp, with z_y the sampled token's logit, taken here from
 // the row that is being copied anyway (exact up to the drift between the two policies, which the codes have room for).
@@ -132,55 +169,123 @@ struct SweepPrep {
   int n_flags;
 };
 
-__global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16* __restrict__ H, long long ldH, int d,
-                                                          const int* __restrict__ row_map,
-                                                          const int* __restrict__ tokens, int V, int vocab_off,
-                                                          __nv_bfloat16* __restrict__ Hc,
-                                                          int* __restrict__ tokens_c, const SweepPrep sp,
-                                                          DevStatus* st) {
-  const int n = st->n_valid;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sp.n_flags; i += gridDim.x * blockDim.x) sp.flags[i] = 0;
-  const int n_pad = (n + 127) / 128 * 128;
-  const int lane = threadIdx.x & 31;
-  const int warps_per_block = blockDim.x >> 5;
-  const int vec_per_row = d / 8;
-  for (int i = blockIdx.x * warps_per_block + (threadIdx.x >> 5); i < n_pad; i += gridDim.x * warps_per_block) {
-    uint4* dst = reinterpret_cast<uint4*>(Hc + (size_t)i * d);
-    if (i < n) {
-      const int r = row_map[i];
-      const uint4* src = reinterpret_cast<const uint4*>(H + (size_t)r * ldH);
-      const int y = tokens[r];
-      const bool in_range = y >= 0 && y < V;
-      if (sp.shift2) {
-        const uint4* wrow = reinterpret_cast<const uint4*>(sp.W + (size_t)(in_range ? y : 0) * sp.ldW);
-        float2 acc = make_float2(0.f, 0.f);
-        for (int v = lane; v < vec_per_row; v += 32) {
-          const uint4 h = __ldg(src + v), w = __ldg(wrow + v);
-          dst[v] = h;
-          const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
-                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
-        }
-        float z = acc.x + acc.y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        if (lane == 0) {
-          const float est = z - sp.old_logp[r];
-          sp.shift2[i] = (isfinite(est) ? est : 0.f) * kLog2e;
-        }
-      } else {
-        for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
-      }
-      if (lane == 0) {
-        tokens_c[i] = in_range ? y - vocab_off : -1;
-        if (!in_range) latch_status(st, kStatusTokenRange, r);
-      }
-    } else {
-      for (int v = lane; v < vec_per_row; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
-      if (lane == 0) tokens_c[i] = -1;
+// What a call returns per original row: zeroed where the mask is 0.
+struct RowOutputs {
+  void* dH;            // [T][dH_row_bytes], or NULL
+  long long dH_row_bytes;
+  float* value[4];     // [T] each, or NULL
+  float4* stats;       // [T], or NULL
+};
+
+struct PrepParams {
+  const __nv_bfloat16* H;
+  long long ldH;
+  int d;
+  const uint8_t* mask;
+  int T;
+  int rows_per_block;     // scanning variant: multiple of 16, at most 256
+  const int* tokens;
+  int V, vocab_off;
+  __nv_bfloat16* Hc;
+  int* tokens_c;
+  int* row_map;           // written by the scanning variant
+  const int* row_pos;     // read by the other
+  SweepPrep sp;
+  RowOutputs out;
+};
+
+__device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, int lane, DevStatus* st) {
+  const int vec_per_row = p.d / 8;
+  if (pos < 0) {
+    if (p.out.dH) {
+      uint4* q = reinterpret_cast<uint4*>(static_cast<char*>(p.out.dH) + (size_t)t * p.out.dH_row_bytes);
+      const int n = (int)(p.out.dH_row_bytes / 16);
+      for (int v = lane; v < n; v += 32) __stcs(q + v, make_uint4(0, 0, 0, 0));
     }
+    if (lane < 4 && p.out.value[lane]) p.out.value[lane][t] = 0.f;
+    if (lane == 4 && p.out.stats) p.out.stats[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  uint4* dst = reinterpret_cast<uint4*>(p.Hc + (size_t)pos * p.d);
+  const uint4* src = reinterpret_cast<const uint4*>(p.H + (size_t)t * p.ldH);
+  const int y = p.tokens[t];
+  const bool in_range = y >= 0 && y < p.V;
+  if (p.sp.shift2) {
+    const uint4* wrow = reinterpret_cast<const uint4*>(p.sp.W + (size_t)(in_range ? y : 0) * p.sp.ldW);
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int v = lane; v < vec_per_row; v += 32) {
+      const uint4 h = __ldg(src + v), w = __ldg(wrow + v);
+      dst[v] = h;
+      const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
+                         __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
+    }
+    float z = acc.x + acc.y;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    if (lane == 0) {
+      const float est = z - p.sp.old_logp[t];
+      p.sp.shift2[pos] = (isfinite(est) ? est : 0.f) * kLog2e;
+    }
+  } else {
+#pragma unroll 4
+    for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
+  }
+  if (lane == 0) {
+    p.tokens_c[pos] = in_range ? y - p.vocab_off : -1;
+    if (!in_range) latch_status(st, kStatusTokenRange, t);
+  }
+}
+
+// SCAN: every block counts the mask itself (the rows before its own, and all of them), up to kPrepRows rows: one launch
+// in place of three.  At 256 to 32768 rows the mask is 0.25 to 32 KB per block out of L2.
+constexpr int kPrepRows = 32768;
+template <bool SCAN>
+__global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevStatus* st) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.sp.n_flags; i += gridDim.x * blockDim.x) p.sp.flags[i] = 0;
+  int n;
+  if constexpr (SCAN) {
+    __shared__ int warp_sums[32];
+    __shared__ int before_s, all_s;
+    __shared__ int pos_s[256];
+    const int r0 = blockIdx.x * p.rows_per_block, rows = min(p.rows_per_block, p.T - r0);
+    if (threadIdx.x == 0) before_s = all_s = 0;
+    __syncthreads();
+    int c = 0, a = 0;
+    for (int g = threadIdx.x; g * 16 < p.T; g += blockDim.x) {
+      const int k = __popc(scan_load_bits(p.mask, (long long)g * 16, p.T));
+      a += k;
+      c += g * 16 < r0 ? k : 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      c += __shfl_xor_sync(0xffffffffu, c, o);
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
+    if (lane == 0) { atomicAdd(&before_s, c); atomicAdd(&all_s, a); }
+    const int t = r0 + threadIdx.x;
+    const bool valid = (int)threadIdx.x < rows && (!p.mask || p.mask[t] != 0);
+    const int rank = block_exclusive_scan(valid ? 1 : 0, warp_sums, nullptr);
+    const int pos = valid ? before_s + rank : -1;
+    pos_s[threadIdx.x] = pos;
+    if (valid) p.row_map[pos] = t;
+    n = all_s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->n_valid = n;
+    __syncthreads();
+    for (int i = warp; i < rows; i += warps) prep_row(p, r0 + i, pos_s[i], lane, st);
+  } else {
+    n = st->n_valid;
+    for (int t = blockIdx.x * warps + warp; t < p.T; t += gridDim.x * warps) prep_row(p, t, p.row_pos[t], lane, st);
+  }
+  const int n_pad = (n + 127) / 128 * 128;
+  for (int i = n + blockIdx.x * warps + warp; i < n_pad; i += gridDim.x * warps) {
+    uint4* dst = reinterpret_cast<uint4*>(p.Hc + (size_t)i * p.d);
+    for (int v = lane; v < p.d / 8; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+    if (lane == 0) p.tokens_c[i] = -1;
   }
 }
 
@@ -374,7 +479,31 @@ __global__ void __launch_bounds__(256) batch_normalise_kernel(float* __restrict_
 // of its first row by binary search in its first sweep and from then on by a galloping search that starts
 // at the response it ended the previous sweep in, so the cost per row does not depend on how long
 // the responses are and almost all offset reads after the first sweep hit lines the block just used.
+// Fewer sweeps per block when the rows would not fill the machine with eight.
+// FUSED (few groups, at most 32 responses each): the response's advantage is worked out here, from the rewards of its
+// group, instead of being read; the block's threads also write adv_seq.  One launch in place of two.
 constexpr int kBroadcastSweeps = 8;
+
+// Advantage of response s from the rewards of its group, in double as grpo_adv_rows_kernel.
+__device__ __forceinline__ float group_advantage(const float* __restrict__ rewards, int G, int ddof, float eps_std, int s) {
+  const float* r = rewards + (size_t)(s / G) * G;
+  double sum = 0.0;
+  float mx = -CUDART_INF_F, mn = CUDART_INF_F;
+  for (int i = 0; i < G; ++i) {
+    const float x = __ldg(r + i);
+    sum += (double)x;
+    mx = fmaxf(mx, x);
+    mn = fminf(mn, x);
+  }
+  if (mx == mn) return 0.f;
+  const double mu = sum / (double)G;
+  double ss = 0.0;
+  for (int i = 0; i < G; ++i) {
+    const double c = (double)__ldg(r + i) - mu;
+    ss = fma(c, c, ss);
+  }
+  return (float)(((double)__ldg(rewards + s) - mu) * (1.0 / (sqrt(ss / (double)(G - ddof)) + (double)eps_std)));
+}
 
 // Largest s in [s_from, n_seq) with seq_offsets[s] <= t, given seq_offsets[s_from] <= t < seq_offsets[n_seq].
 __device__ __forceinline__ int seq_of_row(const int* __restrict__ seq_offsets, int n_seq, int s_from, long long t) {
@@ -388,15 +517,21 @@ __device__ __forceinline__ int seq_of_row(const int* __restrict__ seq_offsets, i
   return lo;
 }
 
-__global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restrict__ adv_seq,
-                                                            const int* __restrict__ seq_offsets, int n_seq,
-                                                            long long T, float* __restrict__ adv_tok) {
+template <bool FUSED>
+__global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restrict__ rewards, int G, int ddof, float eps_std,
+                                                            float* adv_seq, const int* __restrict__ seq_offsets, int n_seq,
+                                                            long long T, int sweeps, float* __restrict__ adv_tok) {
+  if (FUSED)
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n_seq; s += gridDim.x * blockDim.x)
+      adv_seq[s] = group_advantage(rewards, G, ddof, eps_std, s);
+  auto value = [&](int s) { return FUSED ? group_advantage(rewards, G, ddof, eps_std, s) : adv_seq[s]; };
   const int first = seq_offsets[0], last = seq_offsets[n_seq];
   const bool vec_ok = (reinterpret_cast<uintptr_t>(adv_tok) & 15) == 0;
-  const long long rows_per_block = (long long)kBroadcastSweeps * blockDim.x * 4;
+  const long long rows_per_block = (long long)sweeps * blockDim.x * 4;
   for (long long b0 = (long long)blockIdx.x * rows_per_block; b0 < T; b0 += (long long)gridDim.x * rows_per_block) {
-    int s = -1;                           // response this thread was in last, -1: not searched yet
-    for (int sweep = 0; sweep < kBroadcastSweeps; ++sweep) {
+    int s = -1, held = -1;                // response this thread was in last, -1: not searched yet; whose value a is
+    float a = 0.f;
+    for (int sweep = 0; sweep < sweeps; ++sweep) {
       const long long t0 = b0 + ((long long)sweep * blockDim.x + threadIdx.x) * 4;
       if (t0 >= T) break;
       float v[4] = {0.f, 0.f, 0.f, 0.f};
@@ -413,12 +548,13 @@ __global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restr
           s = seq_of_row(seq_offsets, n_seq, s, t_in);
         }
         int end = seq_offsets[s + 1];
-        float a = adv_seq[s];
+        if (held != s) a = value(held = s);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const long long t = t0 + i;
           if (t < first || t >= last) continue;
-          while (t >= end) { ++s; end = seq_offsets[s + 1]; a = adv_seq[s]; }   // empty ranges are skipped
+          while (t >= end) { ++s; end = seq_offsets[s + 1]; }   // empty ranges are skipped
+          if (held != s) a = value(held = s);
           v[i] = a;
         }
       }
@@ -438,39 +574,54 @@ __global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restr
 // seq_value, and the per-token value is the return-to-go ret_t = r_t + gamma ret_(next valid token).
 // kl_t is the signed log-ratio logp - ref (kind 0), exp(delta) - delta - 1 with delta = ref - logp
 // (kind 1), or a value handed in (kind 2).  Masked rows get 0 and are not a discount step.
-// One warp per response: it walks the response's rows from the end in 32-row chunks aligned to
-// 128 bytes, loads kShapeChunks chunks at a time and runs a suffix scan of the linear maps
-// x -> v + g x (valid row: g = gamma, v = r_t; masked row: the identity) with shuffles, carrying the
-// return of the first valid token of the chunks already done.  Per-token terms in fp32, sums in double.
+// A block of four warps per response: it walks the response's rows from the end, 512 rows at a time (each warp 128,
+// four 32-row chunks aligned to 128 bytes, all loaded before the first is used).  Every warp runs a suffix scan of the
+// linear maps x -> v + g x (valid row: g = gamma, v = r_t; masked row: the identity) over its rows with shuffles, the
+// warps' totals are chained through shared memory, and the return of the first valid row of the tile is carried to the
+// next.  Per-token terms in fp32, sums in double.  (One warp per response walked 512 rows as a chain of four rounds:
+// 26 us for 1024 responses; it stays for responses of less than a warp's 128 rows.)  Rows outside every response range, [0, seq_offsets[0]) and [seq_offsets[n_seq], T), get 0.
 constexpr int kShapeChunks = 4;
+constexpr int kShapeWarps = 4;
 
-__global__ void __launch_bounds__(256) kl_shaped_returns_kernel(const float* __restrict__ seq_value,
-                                                                const float* __restrict__ logp,
-                                                                const float* __restrict__ ref_logp,
-                                                                const float* __restrict__ kl_tok,
-                                                                const uint8_t* __restrict__ mask,
-                                                                const int* __restrict__ seq_offsets, int n_seq,
-                                                                float beta, float gamma, int kind,
-                                                                float* __restrict__ shaped, float* __restrict__ ret) {
-  const int lane = threadIdx.x & 31;
-  const int warps_per_block = blockDim.x >> 5;
-  for (int sq = blockIdx.x * warps_per_block + (threadIdx.x >> 5); sq < n_seq; sq += gridDim.x * warps_per_block) {
+// WARPS: warps per response, kShapeWarps or 1 (the block then works on kShapeWarps responses).
+template <int WARPS>
+__global__ void __launch_bounds__(32 * kShapeWarps) kl_shaped_returns_kernel(
+    const float* __restrict__ seq_value, const float* __restrict__ logp, const float* __restrict__ ref_logp,
+    const float* __restrict__ kl_tok, const uint8_t* __restrict__ mask, const int* __restrict__ seq_offsets, int n_seq,
+    long long T, float beta, float gamma, int kind, float* __restrict__ shaped, float* __restrict__ ret) {
+  __shared__ double g_s[WARPS], v_s[WARPS];
+  __shared__ int live_s[WARPS];
+  constexpr int kTeams = kShapeWarps / WARPS;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % WARPS, team = (threadIdx.x >> 5) / WARPS;
+  {
+    const long long first = seq_offsets[0], last = seq_offsets[n_seq];
+    const long long n_out = first + (T > last ? T - last : 0);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += (long long)gridDim.x * blockDim.x) {
+      const long long t = i < first ? i : last + (i - first);
+      ret[t] = 0.f;
+      if (shaped) shaped[t] = 0.f;
+    }
+  }
+  for (int sq = blockIdx.x * kTeams + team; sq < n_seq; sq += gridDim.x * kTeams) {
     const int lo = seq_offsets[sq], hi = seq_offsets[sq + 1];
     if (hi <= lo) continue;
     const double R = (double)seq_value[sq];
-    double carry = 0.0;            // return-to-go of the first valid token after the chunks done so far
+    double carry = 0.0;            // return-to-go of the first valid token after the tiles done so far
     bool terminal_done = false;    // the last valid token of the response has been found
     const int c_first = lo >> 5;
-    for (int c_hi = (hi - 1) >> 5; c_hi >= c_first; c_hi -= kShapeChunks) {
-      double r[kShapeChunks];
+    for (int c_hi = (hi - 1) >> 5; c_hi >= c_first; c_hi -= kShapeChunks * WARPS) {
+      const int c_warp = c_hi - warp * kShapeChunks;   // warp 0 has the last rows
+      double g[kShapeChunks], v[kShapeChunks];
+      float r[kShapeChunks];
       bool inside[kShapeChunks], valid[kShapeChunks];
+      unsigned live[kShapeChunks], any = 0;
 #pragma unroll
       for (int j = 0; j < kShapeChunks; ++j) {
-        const int t = (c_hi - j) * 32 + lane;
-        inside[j] = (c_hi - j) >= c_first && t >= lo && t < hi;
+        const int t = (c_warp - j) * 32 + lane;
+        inside[j] = (c_warp - j) >= c_first && t >= lo && t < hi;
         valid[j] = inside[j] && (!mask || mask[t] != 0);
         double kl = 0.0;
-        if (valid[j]) {
+        if (inside[j]) {
           if (kind == 2) {
             kl = (double)kl_tok[t];
           } else {
@@ -481,59 +632,91 @@ __global__ void __launch_bounds__(256) kl_shaped_returns_kernel(const float* __r
             kl = kind == 0 ? -delta : (double)expm1f(df) - delta;
           }
         }
-        r[j] = -(double)beta * kl;
+        v[j] = valid[j] ? -(double)beta * kl : 0.0;
+        live[j] = __ballot_sync(0xffffffffu, valid[j]);
+        any |= live[j];
       }
+      bool found = terminal_done, found_all = terminal_done || any != 0;
+      if constexpr (WARPS > 1) {
+        if (lane == 0) live_s[warp] = any != 0;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+          if (w < warp) found = found || live_s[w];
+          found_all = found_all || live_s[w];
+        }
+      }
+      double gw = 1.0, vw = 0.0;     // map of this warp's rows done so far, from the last row on
 #pragma unroll
       for (int j = 0; j < kShapeChunks; ++j) {
-        const unsigned live = __ballot_sync(0xffffffffu, valid[j]);
-        if (!terminal_done && live) {
-          if (lane == 31 - __clz(live)) r[j] += R;
-          terminal_done = true;
+        if (!found && live[j]) {
+          if (lane == 31 - __clz(live[j])) v[j] += R;
+          found = true;
         }
-        double g = valid[j] ? (double)gamma : 1.0, v = valid[j] ? r[j] : 0.0;
+        r[j] = (float)v[j];
+        g[j] = valid[j] ? (double)gamma : 1.0;
         if (gamma == 1.f) {
           // no discount: a plain suffix sum
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
-            const double v2 = __shfl_down_sync(0xffffffffu, v, o);
-            if (lane + o < 32) v += v2;
+            const double v2 = __shfl_down_sync(0xffffffffu, v[j], o);
+            if (lane + o < 32) v[j] += v2;
           }
+          v[j] += vw;
         } else {
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
-            const double g2 = __shfl_down_sync(0xffffffffu, g, o);
-            const double v2 = __shfl_down_sync(0xffffffffu, v, o);
-            if (lane + o < 32) { v = fma(g, v2, v); g *= g2; }
+            const double g2 = __shfl_down_sync(0xffffffffu, g[j], o);
+            const double v2 = __shfl_down_sync(0xffffffffu, v[j], o);
+            if (lane + o < 32) { v[j] = fma(g[j], v2, v[j]); g[j] *= g2; }
           }
+          v[j] = fma(g[j], vw, v[j]);
+          g[j] *= gw;
+          gw = __shfl_sync(0xffffffffu, g[j], 0);
         }
-        const double out = fma(g, carry, v);
-        carry = __shfl_sync(0xffffffffu, out, 0);
-        if (inside[j]) {
-          const int t = (c_hi - j) * 32 + lane;
-          ret[t] = valid[j] ? (float)out : 0.f;
-          if (shaped) shaped[t] = valid[j] ? (float)r[j] : 0.f;
+        vw = __shfl_sync(0xffffffffu, v[j], 0);
+      }
+      double in = carry;             // return of the first valid row behind this warp's rows
+      if constexpr (WARPS > 1) {
+        if (lane == 0) { g_s[warp] = gw; v_s[warp] = vw; }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+          if (w == warp) in = carry;
+          carry = fma(g_s[w], carry, v_s[w]);
         }
+      } else {
+        carry = fma(gw, carry, vw);
+      }
+      terminal_done = found_all;
+#pragma unroll
+      for (int j = 0; j < kShapeChunks; ++j) {
+        if (!inside[j]) continue;
+        const int t = (c_warp - j) * 32 + lane;
+        ret[t] = valid[j] ? (float)fma(g[j], in, v[j]) : 0.f;
+        if (shaped) shaped[t] = valid[j] ? r[j] : 0.f;
       }
     }
-  }
-}
-
-// Rows that lie outside every response range, [0, seq_offsets[0]) and [seq_offsets[n_seq], T), get 0.
-__global__ void __launch_bounds__(256) zero_outside_ranges_kernel(const int* __restrict__ seq_offsets, int n_seq,
-                                                                  long long T, float* __restrict__ a,
-                                                                  float* __restrict__ b) {
-  const long long first = seq_offsets[0], last = seq_offsets[n_seq];
-  const long long n_out = first + (T > last ? T - last : 0);
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += (long long)gridDim.x * blockDim.x) {
-    const long long t = i < first ? i : last + (i - first);
-    a[t] = 0.f;
-    if (b) b[t] = 0.f;
+    if (WARPS > 1) __syncthreads();   // before the next response's tiles reuse the shared words
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // Merge of the per-range statistics and the per-token loss arithmetic (Eq. 6 with the clipped
 // surrogate of section 3.1 and the k3 KL-to-reference term).
+constexpr int kLossSums = 8;  // loss, pg, kl, ent, clip, ratio, ratio_max, unused
+constexpr int kLossThreads = 256;   // eight warps: one per sum in the last stage
+
+// Where the blocks of a loss kernel leave their sums; the block that draws the last ticket adds them up in a fixed
+// order (so the result does not depend on which block that is), writes loss and metrics and returns the ticket counter to 0.
+struct LossFinish {
+  double* block_sums;     // [total][kLossSums]
+  unsigned* ticket;
+  int base, total;        // first entry of this launch, entries of all launches that share the sum
+  float* loss;
+  float* metrics;         // [8] or NULL
+};
+
 struct LossParams {
   // inputs
   const float4* partials;
@@ -549,6 +732,7 @@ struct LossParams {
   const long long* token_count;   // device scalar or NULL: divisor of the token mean (data-parallel global count)
   float eps_low, eps_high, beta, ent_coef;
   int with_loss;
+  int zero_coef;           // the coefficients are written later, and not for every row
   // full-distribution KL to the reference policy (two-product forward): second partial per
   // (range, row) = {D, Mr, Sr, 0}; outputs lse_ref, KL_t and the coefficient cb_t = w_t beta
   const float4* partials2;
@@ -567,8 +751,7 @@ struct LossParams {
   float* ent_out;
   float* lse_out;
   float* kl_out;
-  // reduction scratch: [gridDim.x][kLossSums] doubles
-  double* block_sums;
+  LossFinish fin;
   // vocabulary-parallel head: stats_out != NULL -> only merge the ranges of this call's slice and
   // write (M, S, A, z_y) per original row; ext_lse != NULL -> the statistics of the whole
   // vocabulary come from the caller ([T], original rows) instead of the partials
@@ -583,16 +766,13 @@ struct LossParams {
   int* tile_flags;   // [rows / kFlagRows], over all rows
   int* flag_count;   // non-zero: this slab has a flagged tile
 };
-constexpr int kLossSums = 8;  // loss, pg, kl, ent, clip, ratio, ratio_max, unused
-constexpr int kLossThreads = 256;
-
 // Fixed-order sum of column k of the block partials by one warp: lane l adds blocks l, l + 32, ... in order, then a
 // butterfly over the lanes; the order depends on n_blocks alone, so the result is reproducible.
 __device__ __forceinline__ double reduce_block_sums(const double* __restrict__ block_sums, int n_blocks, int k) {
   const int lane = threadIdx.x & 31;
   double v = 0.0;
   for (int b = lane; b < n_blocks; b += 32) {
-    const double u = block_sums[(size_t)b * kLossSums + k];
+    const double u = __ldcg(&block_sums[(size_t)b * kLossSums + k]);
     v = (k == 6) ? fmax(v, u) : v + u;
   }
 #pragma unroll
@@ -604,9 +784,55 @@ __device__ __forceinline__ double reduce_block_sums(const double* __restrict__ b
 }
 
 
+// Last stage of a loss kernel of kLossThreads threads: block sums, then (last block) the sums over blocks.
+__device__ __forceinline__ void finish_loss(const double (&acc)[kLossSums], const LossFinish& f, float n_metric) {
+  __shared__ double red[kLossThreads / 32][kLossSums];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kLossSums; ++k) {
+    double v = acc[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double u = __shfl_xor_sync(0xffffffffu, v, o);
+      v = (k == 6) ? fmax(v, u) : v + u;
+    }
+    if (lane == 0) red[warp][k] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < kLossSums) {
+    const int k = threadIdx.x;
+    double v = red[0][k];
+    for (int w = 1; w < kLossThreads / 32; ++w) v = (k == 6) ? fmax(v, red[w][k]) : v + red[w][k];
+    f.block_sums[(size_t)(f.base + blockIdx.x) * kLossSums + k] = v;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(f.ticket, 1u) == (unsigned)(f.total - 1);
+    if (last) *f.ticket = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  const double v = reduce_block_sums(f.block_sums, f.total, warp);
+  if (lane != 0) return;
+  if (warp == 0) f.loss[0] = (float)v;
+  if (f.metrics) {
+    if (warp >= 1 && warp <= 6) f.metrics[warp - 1] = (float)v;
+    if (warp == 7) { f.metrics[6] = n_metric; f.metrics[7] = 0.f; }
+  }
+}
+
+// A block takes 32 rows at a time, lane = row; its eight warps share the column ranges (with one thread per row a call of
+// a few hundred rows and 75 to 148 ranges was a chain of that many loads: 17 us) and warp 0 goes on with the sums.
 __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossParams p, DevStatus* st) {
+  constexpr int kW = kLossThreads / 32;
+  __shared__ float max_s[2][kW][32];
+  __shared__ float sum_s[5][kW][32];
   const int n = st->n_valid;
   const int n_ranges = p.ext_lse ? 0 : gemm_extents(p.fwd_shape, n, p.fwd_cg, p.fwd_workers).n_ranges;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[kLossSums];
 #pragma unroll
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
@@ -617,24 +843,64 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     slab_extent(n, p.slab_cap, p.slab_index, i_begin, i_end);
     i_end += i_begin;
   }
-  for (int i = i_begin + blockIdx.x * blockDim.x + threadIdx.x; i < i_end; i += gridDim.x * blockDim.x) {
-    float lse, logp, ent;
-    float M = -CUDART_INF_F, S = 0.f, A = 0.f;
+  for (int i0 = i_begin + blockIdx.x * 32; i0 < i_end; i0 += gridDim.x * 32) {
+    const int i = i0 + lane;
+    const bool in = i < i_end;
+    float lse, logp, ent, kl = 0.f;
+    float M = -CUDART_INF_F, S = 0.f, A = 0.f, Mr = -CUDART_INF_F, D = 0.f, Sr = 0.f;
     if (p.ext_lse) {
+      if (warp != 0 || !in) continue;
       const int row = p.row_map[i];
       lse = p.ext_lse[row];
       logp = p.ext_logp[row];
       ent = p.ext_ent[row];
     } else {
-      for (int r = 0; r < n_ranges; ++r) M = fmaxf(M, p.partials[(size_t)r * p.part_stride + i].x);
+      const float4* q1 = p.partials + (in ? i : i_begin);
+      const float4* q2 = p.partials2 + (in ? i : i_begin);
+#pragma unroll 4
+      for (int r = warp; r < n_ranges; r += kW) M = fmaxf(M, q1[(size_t)r * p.part_stride].x);
+      max_s[0][warp][lane] = M;
+      if (p.kl_full) {
+#pragma unroll 4
+        for (int r = warp; r < n_ranges; r += kW) Mr = fmaxf(Mr, q2[(size_t)r * p.part_stride].y);
+        max_s[1][warp][lane] = Mr;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < kW; ++w) {
+        M = fmaxf(M, max_s[0][w][lane]);
+        if (p.kl_full) Mr = fmaxf(Mr, max_s[1][w][lane]);
+      }
       float zy = 0.f;
-      for (int r = 0; r < n_ranges; ++r) {
-        const float4 q = p.partials[(size_t)r * p.part_stride + i];
+#pragma unroll 4
+      for (int r = warp; r < n_ranges; r += kW) {
+        const float4 q = q1[(size_t)r * p.part_stride];
         const float sc = exp2f((q.x - M) * kLog2e);
         S = fmaf(q.y, sc, S);
         A = fmaf(q.z, sc, A);
         zy += q.w;
+        if (p.kl_full) {
+          const float4 k = q2[(size_t)r * p.part_stride];
+          D = fmaf(k.x, sc, D);
+          Sr = fmaf(k.z, exp2f((k.y - Mr) * kLog2e), Sr);
+        }
       }
+      sum_s[0][warp][lane] = S;
+      sum_s[1][warp][lane] = A;
+      sum_s[2][warp][lane] = zy;
+      sum_s[3][warp][lane] = D;
+      sum_s[4][warp][lane] = Sr;
+      __syncthreads();
+      if (warp != 0) continue;
+#pragma unroll
+      for (int w = 1; w < kW; ++w) {
+        S += sum_s[0][w][lane];
+        A += sum_s[1][w][lane];
+        zy += sum_s[2][w][lane];
+        D += sum_s[3][w][lane];
+        Sr += sum_s[4][w][lane];
+      }
+      if (!in) continue;
       if (p.stats_out) {
         p.stats_out[p.row_map[i]] = make_float4(M, S, A, zy);
         continue;
@@ -643,16 +909,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       logp = zy - lse;
       ent = lse - A / S;
     }
-    float kl = 0.f;
     if (p.kl_full) {
-      float Mr = -CUDART_INF_F;
-      for (int r = 0; r < n_ranges; ++r) Mr = fmaxf(Mr, p.partials2[(size_t)r * p.part_stride + i].y);
-      float D = 0.f, Sr = 0.f;
-      for (int r = 0; r < n_ranges; ++r) {
-        const float4 q2 = p.partials2[(size_t)r * p.part_stride + i];
-        D = fmaf(q2.x, exp2f((p.partials[(size_t)r * p.part_stride + i].x - M) * kLog2e), D);
-        Sr = fmaf(q2.z, exp2f((q2.y - Mr) * kLog2e), Sr);
-      }
       const float lse_ref = Mr + logf(Sr);
       kl = (A - D) / S - lse + lse_ref;      // sum_j p_j (z_j - zr_j) - lse + lse_ref
       p.lse_ref_c[i] = lse_ref;
@@ -674,6 +931,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     if (p.logp_out) p.logp_out[row] = logp;
     if (p.ent_out) p.ent_out[row] = ent;
     if (p.lse_out) p.lse_out[row] = lse;
+    if (p.zero_coef) p.cp_c[i] = p.ce_c[i] = 0.f;
     if (p.with_loss) {
       const float w = p.token_weight ? p.token_weight[row] : w_mean;
       const float A_t = p.adv[row];
@@ -704,26 +962,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       acc[6] = fmax(acc[6], (double)rho);
     }
   }
-  if (!p.with_loss) return;
-  __shared__ double red[kLossThreads / 32][kLossSums];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kLossSums; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double u = __shfl_xor_sync(0xffffffffu, v, o);
-      v = (k == 6) ? fmax(v, u) : v + u;
-    }
-    if (lane == 0) red[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kLossSums) {
-    const int k = threadIdx.x;
-    double v = red[0][k];
-    for (int w = 1; w < kLossThreads / 32; ++w) v = (k == 6) ? fmax(v, red[w][k]) : v + red[w][k];
-    p.block_sums[(size_t)blockIdx.x * kLossSums + k] = v;
-  }
+  if (p.with_loss) finish_loss(acc, p.fin, (float)n);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -817,18 +1056,16 @@ __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p
 // token: works on the original rows, four consecutive rows per thread (16-byte loads and stores when
 // every array is 16-byte aligned), masked rows give zero derivatives.  Same arithmetic, in the same
 // order, as combine_loss_kernel applies to the statistics it has merged.
+constexpr int kCountBlocks = 256;   // most blocks of count_valid_kernel: one count per thread of its reader
 __global__ void __launch_bounds__(256) count_valid_kernel(const uint8_t* __restrict__ mask, long long T,
-                                                          unsigned long long* __restrict__ count) {
+                                                          unsigned* __restrict__ counts) {
   unsigned int n = 0;
   const bool vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
   const long long n16 = vec ? T / 16 : 0;
+#pragma unroll 4
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (long long)gridDim.x * blockDim.x) {
     const uint4 m = reinterpret_cast<const uint4*>(mask)[i];
-    const unsigned int w[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) n += ((w[k] >> (8 * b)) & 0xffu) != 0u;
+    n += __popc(__vsetne4(m.x, 0)) + __popc(__vsetne4(m.y, 0)) + __popc(__vsetne4(m.z, 0)) + __popc(__vsetne4(m.w, 0));
   }
   for (long long t = n16 * 16 + (long long)blockIdx.x * blockDim.x + threadIdx.x; t < T;
        t += (long long)gridDim.x * blockDim.x)
@@ -839,9 +1076,9 @@ __global__ void __launch_bounds__(256) count_valid_kernel(const uint8_t* __restr
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = n;
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned long long tot = 0;
+    unsigned tot = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    if (tot) atomicAdd(count, tot);   // integer sum: the order of the blocks does not change it
+    counts[blockIdx.x] = tot;
   }
 }
 
@@ -853,13 +1090,14 @@ struct TokenLossParams {
   const float* adv;
   const uint8_t* mask;        // or NULL: every row valid
   const float* token_weight;  // or NULL: token mean
-  const unsigned long long* count;   // divisor of the token mean (valid rows, or the caller's global count) ...
-  unsigned long long n_known;        // ... or, when count is NULL, the divisor itself
+  const unsigned* counts;            // valid rows per block of count_valid_kernel, or NULL: every row is valid
+  int n_counts;
+  const unsigned long long* token_count;   // divisor of the token mean instead of the number of valid rows, or NULL
   long long T;
   float eps_low, eps_high, beta, ent_coef;
   float* dlogp;               // or NULL
   float* dentropy;            // or NULL
-  double* block_sums;         // [gridDim.x][kLossSums]
+  LossFinish fin;
 };
 
 template <bool VEC>
@@ -867,7 +1105,18 @@ __global__ void __launch_bounds__(kLossThreads, 4) token_loss_kernel(const Token
   double acc[kLossSums];
 #pragma unroll
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
-  const unsigned long long n_mean = p.count ? *p.count : p.n_known;
+  __shared__ unsigned long long valid_s;
+  if (threadIdx.x == 0) valid_s = p.counts ? 0 : (unsigned long long)p.T;
+  __syncthreads();
+  if (p.counts) {
+    unsigned long long v = (int)threadIdx.x < p.n_counts ? p.counts[threadIdx.x] : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&valid_s, v);
+    __syncthreads();
+  }
+  const unsigned long long n_valid = valid_s;
+  const unsigned long long n_mean = p.token_count ? *p.token_count : n_valid;
   const float w_mean = n_mean > 0 ? (float)(1.0 / (double)n_mean) : 0.f;
   const long long n4 = (p.T + 3) / 4;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += (long long)gridDim.x * blockDim.x) {
@@ -945,41 +1194,7 @@ __global__ void __launch_bounds__(kLossThreads, 4) token_loss_kernel(const Token
       }
     }
   }
-  __shared__ double red[kLossThreads / 32][kLossSums];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kLossSums; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double u = __shfl_xor_sync(0xffffffffu, v, o);
-      v = (k == 6) ? fmax(v, u) : v + u;
-    }
-    if (lane == 0) red[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kLossSums) {
-    const int k = threadIdx.x;
-    double v = red[0][k];
-    for (int w = 1; w < kLossThreads / 32; ++w) v = (k == 6) ? fmax(v, red[w][k]) : v + red[w][k];
-    p.block_sums[(size_t)blockIdx.x * kLossSums + k] = v;
-  }
-}
-
-// Fixed-order sum of the block partials of token_loss_kernel -> loss[1], metrics[8].  One warp per sum.
-__global__ void __launch_bounds__(32 * kLossSums) finalize_token_loss_kernel(const double* __restrict__ block_sums,
-                                                                             int n_blocks, float* __restrict__ loss,
-                                                                             float* __restrict__ metrics,
-                                                                             const unsigned long long* __restrict__ count,
-                                                                             unsigned long long n_rows_valid_known) {
-  const int k = threadIdx.x >> 5;
-  const double v = reduce_block_sums(block_sums, n_blocks, k);
-  if ((threadIdx.x & 31) != 0) return;
-  if (k == 0) loss[0] = (float)v;
-  if (metrics) {
-    if (k >= 1 && k <= 6) metrics[k - 1] = (float)v;
-    if (k == 7) { metrics[6] = (float)(count ? *count : n_rows_valid_known); metrics[7] = 0.f; }
-  }
+  finish_loss(acc, p.fin, (float)n_valid);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -987,8 +1202,9 @@ __global__ void __launch_bounds__(32 * kLossSums) finalize_token_loss_kernel(con
 // (the length normalisation by token weights of section 2.2) and the sequence-level importance
 // ratio (the GSPO variant named in section 4.2; reading: rho_i = exp of the mean
 // token log-ratio over the valid tokens of response i, used by every token of the response).
-// One warp per response; its valid tokens are the compact rows [lo, hi) found by binary search
-// in the ascending row map.
+// One team of threads per response - a block, or a warp where responses are short; its valid tokens are the compact rows
+// [lo, hi) found by binary search in the ascending row map.  (One warp per response always: 8 responses of 345 rows took
+// 50 us in one block.)
 struct SeqParams {
   const int* seq_offsets;   // [n_seq + 1] row range of each response
   int n_seq;
@@ -1005,7 +1221,7 @@ struct SeqParams {
   int* l_max;               // device scalar: longest row range
   float* cp_c;
   float* ce_c;
-  double* block_sums;       // [gridDim.x][kLossSums]
+  LossFinish fin;
 };
 
 __global__ void __launch_bounds__(1024) seq_lmax_kernel(const int* __restrict__ seq_offsets, int n_seq, int* l_max) {
@@ -1031,10 +1247,28 @@ __device__ __forceinline__ int lower_bound_rows(const int* __restrict__ row_map,
   return lo;
 }
 
+// Sum over the TEAM threads of a team, the same value for all of them; every thread of the block calls it.
+template <int TEAM>
+__device__ __forceinline__ float team_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (TEAM > 32) {
+    __shared__ float part[TEAM / 32];
+    __syncthreads();   // the previous sum has been read
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.f;
+#pragma unroll
+    for (int w = 0; w < TEAM / 32; ++w) v += part[w];
+  }
+  return v;
+}
+
+template <int TEAM>
 __global__ void __launch_bounds__(kLossThreads) seq_loss_kernel(const SeqParams p, DevStatus* st) {
   const int n = st->n_valid;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int warps_per_block = kLossThreads / 32;
+  const int lane = threadIdx.x % TEAM, team = threadIdx.x / TEAM;
+  constexpr int teams = kLossThreads / TEAM;
   double acc[kLossSums];
 #pragma unroll
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
@@ -1042,7 +1276,7 @@ __global__ void __launch_bounds__(kLossThreads) seq_loss_kernel(const SeqParams 
   const int n_part = p.agg_mode == 0 ? lower_bound_rows(p.row_map, n, p.seq_offsets[p.n_seq]) -
                                            lower_bound_rows(p.row_map, n, p.seq_offsets[0])
                                      : 0;
-  for (int sq = blockIdx.x * warps_per_block + warp; sq < p.n_seq; sq += gridDim.x * warps_per_block) {
+  for (int sq = blockIdx.x * teams + team; sq < p.n_seq; sq += gridDim.x * teams) {
     const int lo = lower_bound_rows(p.row_map, n, p.seq_offsets[sq]);
     const int hi = lower_bound_rows(p.row_map, n, p.seq_offsets[sq + 1]);
     const int len = hi - lo;
@@ -1054,22 +1288,20 @@ __global__ void __launch_bounds__(kLossThreads) seq_loss_kernel(const SeqParams 
     float rho_seq = 1.f, seq_sum = 0.f;
     if (p.sequence_level) {
       float lr = 0.f;
-      for (int k = lo + lane; k < hi; k += 32) lr += p.logp_c[k] - p.old_logp[p.row_map[k]];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lr += __shfl_xor_sync(0xffffffffu, lr, o);
+      for (int k = lo + lane; k < hi; k += TEAM) lr += p.logp_c[k] - p.old_logp[p.row_map[k]];
+      lr = team_sum<TEAM>(lr);
       rho_seq = expf(lr / (float)len);
       const float clipped = fminf(fmaxf(rho_seq, 1.f - p.eps_low), 1.f + p.eps_high);
-      for (int k = lo + lane; k < hi; k += 32) {
+      for (int k = lo + lane; k < hi; k += TEAM) {
         const int row = p.row_map[k];
         const float w = p.token_weight ? p.token_weight[row] : w_seq;
         const float A_t = p.adv[row];
         const bool active = rho_seq * A_t <= clipped * A_t;
         seq_sum += active ? w * A_t : 0.f;
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) seq_sum += __shfl_xor_sync(0xffffffffu, seq_sum, o);
+      seq_sum = team_sum<TEAM>(seq_sum);
     }
-    for (int k = lo + lane; k < hi; k += 32) {
+    for (int k = lo + lane; k < hi; k += TEAM) {
       const int row = p.row_map[k];
       const float w = p.token_weight ? p.token_weight[row] : w_seq;
       const float A_t = p.adv[row];
@@ -1101,38 +1333,7 @@ __global__ void __launch_bounds__(kLossThreads) seq_loss_kernel(const SeqParams 
       acc[6] = fmax(acc[6], (double)rho);
     }
   }
-  __shared__ double red[kLossThreads / 32][kLossSums];
-#pragma unroll
-  for (int k = 0; k < kLossSums; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double u = __shfl_xor_sync(0xffffffffu, v, o);
-      v = (k == 6) ? fmax(v, u) : v + u;
-    }
-    if (lane == 0) red[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kLossSums) {
-    const int k = threadIdx.x;
-    double v = red[0][k];
-    for (int w = 1; w < kLossThreads / 32; ++w) v = (k == 6) ? fmax(v, red[w][k]) : v + red[w][k];
-    p.block_sums[(size_t)blockIdx.x * kLossSums + k] = v;
-  }
-}
-
-// Second stage: fixed-order sum of the block partials -> loss[1] and metrics[8].  One warp per sum.
-__global__ void __launch_bounds__(32 * kLossSums) finalize_loss_kernel(const double* __restrict__ block_sums, int n_blocks,
-                                                                       float* __restrict__ loss, float* __restrict__ metrics,
-                                                                       const DevStatus* st) {
-  const int k = threadIdx.x >> 5;
-  const double v = reduce_block_sums(block_sums, n_blocks, k);
-  if ((threadIdx.x & 31) != 0) return;
-  if (k == 0) loss[0] = (float)v;
-  if (metrics) {
-    if (k >= 1 && k <= 6) metrics[k - 1] = (float)v;
-    if (k == 7) { metrics[6] = (float)st->n_valid; metrics[7] = 0.f; }
-  }
+  finish_loss(acc, p.fin, (float)n);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -1,0 +1,74 @@
+"""The kernels around the tensor-core passes at the sizes where they change form: row preparation (scans for itself up
+to 32768 rows), loss per response (a block or a warp each), advantages worked out in the broadcast."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import grpo_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _np64(t):
+    return t.detach().double().cpu().numpy()
+
+
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 2367, 2369, 32767, 32768, 32769, 70001])
+@pytest.mark.parametrize("shift", [0, 1])   # mask pointer 16-byte aligned or not
+def test_rows_are_scored_in_place_and_masked_rows_are_zero(T, shift):
+    from paper_2512_21450_b200 import Context
+    d, V = 64, 300
+    g = torch.Generator(device="cuda").manual_seed(T)
+    H = torch.randn(T, d, generator=g, device="cuda").to(torch.bfloat16)
+    W = (torch.randn(V, d, generator=g, device="cuda") * 0.1).to(torch.bfloat16)
+    tok = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    backing = torch.zeros(T + 16, dtype=torch.uint8, device="cuda")
+    mask = backing[shift:shift + T]
+    c = Context(0)
+    try:
+        for p in (0.5, 0.0, 1.0):
+            mask.copy_((torch.rand(T, generator=g, device="cuda") < p).to(torch.uint8) * 3)
+            c.ensure_workspace(T, d, V)
+            c._ws.fill_(0xFF)
+            lp, ent, lse = c.rl_token_logprobs(H, W, tok, mask)
+            assert c.last_device_status()[0] == 0
+            z = H.double() @ W.double().T
+            ref = z.gather(1, tok.long()[:, None])[:, 0] - torch.logsumexp(z, 1)
+            m = mask.bool()
+            assert (lp[m].double() - ref[m]).abs().max().item() <= 2e-3 if m.any() else True
+            assert not lp[~m].any() and not ent[~m].any() and not lse[~m].any()
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("L_max", [7, 63, 64, 150])    # a warp per response below 64 rows each, a block from there on
+@pytest.mark.parametrize("agg_mode,sequence_level", [(0, True), (1, False), (2, True)])
+def test_loss_per_response(L_max, agg_mode, sequence_level):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    from tests.test_gpu_parity import _check_against_oracle
+    c = Context(0)
+    try:
+        _check_against_oracle(c, make_workload(1, prompts=3, L_max=L_max, d=64, V=500, seed=6000 + L_max, sigma_old=0.3),
+                              agg_mode=agg_mode, sequence_level=sequence_level)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("n_groups,G", [(1, 2), (2047, 3), (2048, 3), (40, 32), (40, 33)])
+def test_advantages_in_the_broadcast(n_groups, G):
+    from paper_2512_21450_b200 import Context
+    rng = np.random.default_rng(G)
+    r = (10 + rng.uniform(size=n_groups * G)).astype(np.float32)
+    r[:G] = r[0]
+    off = np.concatenate([[3], 3 + np.cumsum(rng.integers(0, 9, size=r.size))]).astype(np.int32)
+    c = Context(0)
+    try:
+        seq, tok = c.rl_grpo_advantages(torch.from_numpy(r).cuda(), G, seq_offsets=torch.from_numpy(off).cuda(), T=int(off[-1]) + 5)
+        assert c.last_device_status()[0] == 0
+    finally:
+        c.close()
+    assert np.abs(_np64(seq) - O.grpo_advantages(r, G)).max() <= 1e-6
+    want = np.zeros(int(off[-1]) + 5)
+    want[3:off[-1]] = np.repeat(_np64(seq), np.diff(off))
+    assert np.array_equal(_np64(tok), want)
