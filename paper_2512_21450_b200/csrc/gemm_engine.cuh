@@ -430,7 +430,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
             const typename Epi::Params ep, DevStatus* status) {
-  if (Epi::kTileFlags && sh.flag_count && *sh.flag_count == 0) return;   // no flagged row tile
+  if (Epi::kTileFlags && sh.flag_count) {
+    chain_wait();
+    if (*sh.flag_count == 0) return;   // no flagged row tile
+  }
   static_assert(MODE != kTileWide || CG == 2, "wide tiles run on CTA pairs");
   static_assert(MODE != kTileDual || (A_MN == 0 && B_MN == 0), "the two-product mode takes K-major operands");
   using Cfg = StageCfg<CG, MODE, Epi::kStagingBytes>;
@@ -470,6 +473,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   __syncthreads();
   if (CG == 2) cluster_sync_all();   // the peer's barriers exist before anything signals them
   tc_fence_after();
+  chain_wait();
   const uint32_t tmem_base = tmem_base_smem;
   volatile int* abort_p = &abort_flag;
 
@@ -714,6 +718,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     Epi::finish(st);   // e.g. wait for bulk stores that still read this warp's staging memory
   }
 
+  chain_release();
   tc_fence_before();
   __syncthreads();
   if (CG == 2) cluster_sync_all();   // the pair's UMMAs have retired and both epilogues are done

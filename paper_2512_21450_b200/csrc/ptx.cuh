@@ -18,6 +18,19 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+// Programmatic dependent launch.  Every kernel of this library is launched with stream serialisation relaxed: the next
+// launch may be scheduled once all blocks of this one have called chain_release(), and waits in chain_wait() until
+// everything before it has completed and is visible.  No kernel touches global memory before chain_wait(), so that
+// completion of a kernel implies completion of all kernels before it.  The small kernels do both at once; the tensor-core
+// kernels wait after setting up barriers and tensor memory and release at the end (released at the start, the next
+// launch's blocks cost a 77-row scoring call 2 %).  Tiny step 81.4 -> 66.3 us, per-token values 42.5 -> 38.6 us.
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_begin() {
+  chain_release();
+  chain_wait();
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

@@ -312,6 +312,22 @@ void prof_end(rl_ctx* c, int i, int kind) {
   c->prof_used = i + 1;
 }
 
+// One kernel launch on the context's stream that may be scheduled while the launch before it still runs (chain_begin()).
+template <class... P, class... A>
+void launch(rl_ctx* c, void (*kernel)(P...), int grid, int block, A&&... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = c->stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // One launch of the tensor-core engine in tile mode MODE on the context's persistent grid (CTA pairs
 // when cta_group is 2; wide tiles exist for pairs only).  a2 / b2 / k2_len: second product (kTileDual).
 template <class Epi, int A_MN, int B_MN, int MODE>
@@ -319,24 +335,25 @@ void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUten
                   const CUtensorMap& b2, const CUtensorMap& out, const GemmShape& sh, int k2_len,
                   const typename Epi::Params& ep) {
   const int prof = prof_begin(c, kind);
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(c->grid[cg]);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = kGemmSmemBytes;
+  cfg.stream = c->stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cg == 2 ? 2 : 1;
   if (cg == 2) {
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(c->grid[2]);
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = kGemmSmemBytes;
-    cfg.stream = c->stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, gemm_kernel<Epi, A_MN, B_MN, 2, MODE>, a, b, a2, b2, out, sh, k2_len, ep, c->dstatus);
   } else if constexpr (MODE != kTileWide) {
-    gemm_kernel<Epi, A_MN, B_MN, 1, MODE><<<c->grid[1], kGemmThreads, kGemmSmemBytes, c->stream>>>(
-        a, b, a2, b2, out, sh, k2_len, ep, c->dstatus);
+    cudaLaunchKernelEx(&cfg, gemm_kernel<Epi, A_MN, B_MN, 1, MODE>, a, b, a2, b2, out, sh, k2_len, ep, c->dstatus);
   }
   c->launches++;
   prof_end(c, prof, kind);
@@ -403,9 +420,9 @@ void launch_mask_scan(rl_ctx* c, const uint8_t* mask, int64_t T, int* block_coun
   const int pr = prof_begin(c, 4);
   const int n_blocks = (int)((T + kScanRowsPerBlock - 1) / kScanRowsPerBlock);
   const int sums = n_blocks <= kScanSumBlocks ? 1 : 0;
-  mask_count_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts);
-  if (!sums) mask_offsets_kernel<<<1, 1024, 0, c->stream>>>(block_counts, n_blocks, c->dstatus);
-  mask_write_kernel<<<n_blocks, kScanThreads, 0, c->stream>>>(mask, (int)T, block_counts, sums, row_map, row_pos, c->dstatus);
+  launch(c, mask_count_kernel, n_blocks, kScanThreads, mask, (int)T, block_counts);
+  if (!sums) launch(c, mask_offsets_kernel, 1, 1024, block_counts, n_blocks, c->dstatus);
+  launch(c, mask_write_kernel, n_blocks, kScanThreads, mask, (int)T, block_counts, sums, row_map, row_pos, c->dstatus);
   prof_end(c, pr, 4);
   c->launches += sums ? 2 : 3;
 }
@@ -456,14 +473,14 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     int rows = (int)align_up((size_t)(T + c->n_sm * 4 - 1) / (c->n_sm * 4), 16);   // at most 256: kPrepRows / (4 n_sm)
     if (rows > 256) rows = 256;
     pp.rows_per_block = rows;
-    prep_rows_kernel<true><<<(int)((T + rows - 1) / rows), 256, 0, c->stream>>>(pp, c->dstatus);
+    launch(c, prep_rows_kernel<true>, (int)((T + rows - 1) / rows), 256, pp, c->dstatus);
     prof_end(c, pr, 5);
   } else {
     int* row_pos = reinterpret_cast<int*>(ws + L.row_pos);
     if (plan.scan) launch_mask_scan(c, mask, T, reinterpret_cast<int*>(ws + L.scan_counts), row_map, row_pos);
     pp.row_pos = row_pos;
     const int pr = prof_begin(c, 5);
-    prep_rows_kernel<false><<<c->n_sm * 8, 256, 0, c->stream>>>(pp, c->dstatus);
+    launch(c, prep_rows_kernel<false>, c->n_sm * 8, 256, pp, c->dstatus);
     prof_end(c, pr, 5);
   }
   c->launches += 1;
@@ -496,8 +513,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     // full KL: compact the reference hidden states with the same row map and form both logit
     // tiles per output tile
     __nv_bfloat16* Hc_ref = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc_ref);
-    gather_plain_kernel<<<c->n_sm * 4, 256, 0, c->stream>>>(static_cast<const __nv_bfloat16*>(kl->H_ref), kl->ldH_ref,
-                                                            (int)kl->d_ref, row_map, Hc_ref, c->dstatus);
+    launch(c, gather_plain_kernel, c->n_sm * 4, 256, static_cast<const __nv_bfloat16*>(kl->H_ref), kl->ldH_ref, (int)kl->d_ref, row_map, Hc_ref, c->dstatus);
     c->launches++;
     CUtensorMap tmA2, tmB2;
     if (!map_kmajor(c, &tmA2, Hc_ref, (uint64_t)L.Tpad, (uint64_t)kl->d_ref, (uint64_t)kl->d_ref, BM)) return RL_ERR_CUDA;
@@ -818,18 +834,17 @@ rl_status rl_grpo_advantages_ex(rl_ctx* c, const float* rewards, int64_t n_seq, 
     const float4* r4 = reinterpret_cast<const float4*>(rewards);
     float4* a4 = reinterpret_cast<float4*>(adv_seq);
     switch (group_size / 4) {
-      case 1: grpo_adv_rows_kernel<1><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 2: grpo_adv_rows_kernel<2><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 3: grpo_adv_rows_kernel<3><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 4: grpo_adv_rows_kernel<4><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 5: grpo_adv_rows_kernel<5><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 6: grpo_adv_rows_kernel<6><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      case 7: grpo_adv_rows_kernel<7><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
-      default: grpo_adv_rows_kernel<8><<<blocks, 256, 0, c->stream>>>(r4, n_groups, ddof, eps_std, a4); break;
+      case 1: launch(c, grpo_adv_rows_kernel<1>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 2: launch(c, grpo_adv_rows_kernel<2>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 3: launch(c, grpo_adv_rows_kernel<3>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 4: launch(c, grpo_adv_rows_kernel<4>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 5: launch(c, grpo_adv_rows_kernel<5>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 6: launch(c, grpo_adv_rows_kernel<6>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      case 7: launch(c, grpo_adv_rows_kernel<7>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
+      default: launch(c, grpo_adv_rows_kernel<8>, blocks, 256, r4, n_groups, ddof, eps_std, a4); break;
     }
   } else {
-    grpo_adv_kernel<<<(n_groups + groups_per_block - 1) / groups_per_block, warps * 32, 0, c->stream>>>(
-        rewards, n_groups, group_size, ddof, eps_std, adv_seq);
+    launch(c, grpo_adv_kernel, (n_groups + groups_per_block - 1) / groups_per_block, warps * 32, rewards, n_groups, group_size, ddof, eps_std, adv_seq);
   }
   c->launches += fused ? 0 : 1;
   if (adv_tok && T > 0) {
@@ -838,11 +853,9 @@ rl_status rl_grpo_advantages_ex(rl_ctx* c, const float* rewards, int64_t n_seq, 
     long long blocks = (T + sweeps * 1024 - 1) / (sweeps * 1024);
     if (blocks > (long long)c->n_sm * 32) blocks = (long long)c->n_sm * 32;
     if (fused)
-      broadcast_adv_kernel<true><<<(int)blocks, 256, 0, c->stream>>>(rewards, group_size, ddof, eps_std, adv_seq, seq_offsets,
-                                                                     (int)n_seq, (long long)T, (int)sweeps, adv_tok);
+      launch(c, broadcast_adv_kernel<true>, (int)blocks, 256, rewards, group_size, ddof, eps_std, adv_seq, seq_offsets, (int)n_seq, (long long)T, (int)sweeps, adv_tok);
     else
-      broadcast_adv_kernel<false><<<(int)blocks, 256, 0, c->stream>>>(rewards, group_size, ddof, eps_std, adv_seq, seq_offsets,
-                                                                      (int)n_seq, (long long)T, (int)sweeps, adv_tok);
+      launch(c, broadcast_adv_kernel<false>, (int)blocks, 256, rewards, group_size, ddof, eps_std, adv_seq, seq_offsets, (int)n_seq, (long long)T, (int)sweeps, adv_tok);
     c->launches++;
   }
   prof_end(c, pr_adv, 8);
@@ -862,15 +875,14 @@ rl_status rl_advantages(rl_ctx* c, int estimator, const float* rewards, const in
   const int n_groups = (int)(n_seq / group_size);
   const int warps = 8;
   const int pr = prof_begin(c, 8);
-  group_baseline_kernel<<<(n_groups + warps - 1) / warps, warps * 32, 0, c->stream>>>(rewards, lengths, n_groups,
-                                                                                      group_size, estimator, adv_seq);
+  launch(c, group_baseline_kernel, (n_groups + warps - 1) / warps, warps * 32, rewards, lengths, n_groups, group_size, estimator, adv_seq);
   c->launches++;
   if (estimator == RL_ADV_REINFORCE_PP) {
     double* stats = reinterpret_cast<double*>(reinterpret_cast<char*>(c->dstatus) + 64);
-    batch_stats_kernel<<<1, 1024, 0, c->stream>>>(adv_seq, (long long)n_seq, stats);
+    launch(c, batch_stats_kernel, 1, 1024, adv_seq, (long long)n_seq, stats);
     int blocks = (int)((n_seq + 255) / 256);
     if (blocks > 4096) blocks = 4096;
-    batch_normalise_kernel<<<blocks, 256, 0, c->stream>>>(adv_seq, (long long)n_seq, stats, eps_std);
+    launch(c, batch_normalise_kernel, blocks, 256, adv_seq, (long long)n_seq, stats, eps_std);
     c->launches += 2;
   }
   prof_end(c, pr, 8);
@@ -901,7 +913,7 @@ rl_status rl_token_loss(rl_ctx* c, const float* logp, const float* entropy, cons
   if (mask) {
     cb = (T / 16 + 255) / 256 + 1;
     if (cb > kCountBlocks) cb = kCountBlocks;
-    count_valid_kernel<<<(int)cb, 256, 0, st>>>(mask, (long long)T, counts);
+    launch(c, count_valid_kernel, (int)cb, 256, mask, (long long)T, counts);
     c->launches++;
   }
   TokenLossParams p;
@@ -928,8 +940,8 @@ rl_status rl_token_loss(rl_ctx* c, const float* logp, const float* entropy, cons
   p.fin.total = (int)blocks;
   p.fin.loss = loss;
   p.fin.metrics = metrics_out;
-  if (vec) token_loss_kernel<true><<<(int)blocks, kLossThreads, 0, st>>>(p);
-  else     token_loss_kernel<false><<<(int)blocks, kLossThreads, 0, st>>>(p);
+  if (vec) launch(c, token_loss_kernel<true>, (int)blocks, kLossThreads, p);
+  else     launch(c, token_loss_kernel<false>, (int)blocks, kLossThreads, p);
   c->launches += 1;
   prof_end(c, pr, 6);
   return cuda_ok();
@@ -958,12 +970,12 @@ rl_status rl_kl_shaped_returns(rl_ctx* c, const float* seq_value, const float* l
   int64_t blocks = by_block ? n_seq : (n_seq + kShapeWarps - 1) / kShapeWarps;
   if (blocks > (int64_t)c->n_sm * 64) blocks = (int64_t)c->n_sm * 64;
   const int pr = prof_begin(c, 8);
-  auto launch = [&](auto kernel) {
-    kernel<<<(int)blocks, 32 * kShapeWarps, 0, c->stream>>>(seq_value, logp, ref_logp, kl_tok, mask, seq_offsets, (int)n_seq,
+  auto shape = [&](auto kernel) {
+    launch(c, kernel, (int)blocks, 32 * kShapeWarps, seq_value, logp, ref_logp, kl_tok, mask, seq_offsets, (int)n_seq,
                                                             (long long)T, beta, gamma, kl_estimate, shaped_reward, returns);
   };
-  if (by_block) launch(kl_shaped_returns_kernel<kShapeWarps>);
-  else          launch(kl_shaped_returns_kernel<1>);
+  if (by_block) shape(kl_shaped_returns_kernel<kShapeWarps>);
+  else          shape(kl_shaped_returns_kernel<1>);
   prof_end(c, pr, 8);
   c->launches += 1;
   return cuda_ok();
@@ -1011,7 +1023,7 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   p.ent_out = entropy;
   p.lse_out = lse;
   const int blocks = merge_blocks(T, 1);
-  combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
+  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
   c->launches++;
   return cuda_ok();
 }
@@ -1156,14 +1168,14 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       p.fin = fin;
       p.fin.base = r * nb;
       p.fin.total = slabs * nb;
-      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(p, c->dstatus);
+      launch(c, combine_loss_kernel, nb, kLossThreads, p, c->dstatus);
       c->launches++;
     } else {
       // merge the statistics first, then one team per response forms weights, ratios and the loss; valid rows that lie
       // outside every response range take no part: their coefficients stay 0
       p.with_loss = 0;
       p.zero_coef = 1;
-      combine_loss_kernel<<<nb, kLossThreads, 0, st>>>(p, c->dstatus);
+      launch(c, combine_loss_kernel, nb, kLossThreads, p, c->dstatus);
       SeqParams q;
       memset(&q, 0, sizeof(q));
       q.seq_offsets = o.seq_offsets;
@@ -1184,15 +1196,15 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       q.fin = fin;
       q.fin.base = 0;
       if (q.agg_mode == 2) {
-        seq_lmax_kernel<<<1, 1024, 0, st>>>(o.seq_offsets, (int)o.n_seq, q.l_max);
+        launch(c, seq_lmax_kernel, 1, 1024, o.seq_offsets, (int)o.n_seq, q.l_max);
         c->launches++;
       }
       // a block per response unless that would be mostly idle threads
       const bool by_block = T >= 64 * o.n_seq;
       const int64_t teams = by_block ? o.n_seq : (o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32);
       q.fin.total = (int)(teams < 1024 ? teams : 1024);
-      if (by_block) seq_loss_kernel<kLossThreads><<<q.fin.total, kLossThreads, 0, st>>>(q, c->dstatus);
-      else          seq_loss_kernel<32><<<q.fin.total, kLossThreads, 0, st>>>(q, c->dstatus);
+      if (by_block) launch(c, seq_loss_kernel<kLossThreads>, q.fin.total, kLossThreads, q, c->dstatus);
+      else          launch(c, seq_loss_kernel<32>, q.fin.total, kLossThreads, q, c->dstatus);
       c->launches += 2;
     }
     prof_end(c, pr_loss, 6);
@@ -1283,7 +1295,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.shift2 = ep.shift2;
           lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
           const int pr_lg = prof_begin(c, 1);
-          logit_grad_kernel<<<c->n_sm * 8, 256, 0, st>>>(lg, c->dstatus);
+          launch(c, logit_grad_kernel, c->n_sm * 8, 256, lg, c->dstatus);
           prof_end(c, pr_lg, 1);
           c->launches++;
         }
@@ -1377,8 +1389,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     src.slots = dH_slots;
     src.tile_rows = dh_tile_rows;
     src.tile_cols = dh_cols;
-    if (o.dH_dtype) scatter_dH_kernel<true><<<c->n_sm * 8, 256, 0, st>>>(src, row_map, dH, c->dstatus);
-    else            scatter_dH_kernel<false><<<c->n_sm * 8, 256, 0, st>>>(src, row_map, dH, c->dstatus);
+    if (o.dH_dtype) launch(c, scatter_dH_kernel<true>, c->n_sm * 8, 256, src, row_map, dH, c->dstatus);
+    else            launch(c, scatter_dH_kernel<false>, c->n_sm * 8, 256, src, row_map, dH, c->dstatus);
     prof_end(c, pr_sc, 7);
     c->launches++;
   }
@@ -1441,7 +1453,7 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   p.stats_out = reinterpret_cast<float4*>(stats);
   const int blocks = merge_blocks(T, 1);
   const int pr = prof_begin(c, 6);
-  combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
+  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
   prof_end(c, pr, 6);
   c->launches++;
   return cuda_ok();
@@ -1456,8 +1468,7 @@ rl_status rl_merge_logit_stats(rl_ctx* c, const float* stats, int n_shards, cons
   int blocks = (int)((T + 255) / 256);
   if (blocks > 4096) blocks = 4096;
   const int pr = prof_begin(c, 6);
-  merge_shard_stats_kernel<<<blocks, 256, 0, c->stream>>>(reinterpret_cast<const float4*>(stats), n_shards,
-                                                          (long long)T, mask, logp, entropy, lse);
+  launch(c, merge_shard_stats_kernel, blocks, 256, reinterpret_cast<const float4*>(stats), n_shards, (long long)T, mask, logp, entropy, lse);
   prof_end(c, pr, 6);
   c->launches++;
   return cuda_ok();
@@ -1502,7 +1513,7 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
     p.logp_out = logp[i];
     p.ent_out = entropy ? entropy[i] : nullptr;
     const int blocks = merge_blocks(T, 1);
-    combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
+    launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
     c->launches++;
   }
   return cuda_ok();
@@ -1913,7 +1924,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   p.ent_out = entropy;
   p.lse_out = lse;
   const int blocks = merge_blocks(T, 1);
-  combine_loss_kernel<<<blocks, kLossThreads, 0, c->stream>>>(p, c->dstatus);
+  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
   if (dev_status &&
       cudaMemcpyAsync(dev_status, c->dstatus, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
     return RL_ERR_CUDA;

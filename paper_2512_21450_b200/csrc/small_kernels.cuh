@@ -65,6 +65,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int* 
 
 __global__ void __launch_bounds__(kScanThreads) mask_count_kernel(const uint8_t* __restrict__ mask, int T,
                                                                   int* __restrict__ block_counts) {
+  chain_begin();
   __shared__ int warp_sums[32];
   const long long base = ((long long)blockIdx.x * kScanThreads + threadIdx.x) * kScanRowsPerThread;
   int c = __popc(scan_load_bits(mask, base, T));
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(kScanThreads) mask_count_kernel(const uint8_t*
 
 // One block: block_counts[0..n) -> exclusive offsets in place, total -> st->n_valid.
 __global__ void __launch_bounds__(1024) mask_offsets_kernel(int* __restrict__ block_counts, int n, DevStatus* st) {
+  chain_begin();
   __shared__ int warp_sums[32];
   __shared__ int chunk_total;
   int carry = 0;
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t*
                                                                   const int* __restrict__ block_offsets, int sums,
                                                                   int* __restrict__ row_map, int* __restrict__ row_pos,
                                                                   DevStatus* st) {
+  chain_begin();
   __shared__ int warp_sums[32];
   __shared__ int block_total, before, all;
   __shared__ int staged[kScanRowsPerBlock];   // the block's valid rows, in order
@@ -245,6 +248,7 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
 constexpr int kPrepRows = 32768;
 template <bool SCAN>
 __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevStatus* st) {
+  chain_begin();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.sp.n_flags; i += gridDim.x * blockDim.x) p.sp.flags[i] = 0;
   int n;
@@ -293,6 +297,7 @@ __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevS
 __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* __restrict__ H, long long ldH, int d,
                                                            const int* __restrict__ row_map,
                                                            __nv_bfloat16* __restrict__ Hc, const DevStatus* st) {
+  chain_begin();
   const int n = st->n_valid;
   const int n_pad = (n + 127) / 128 * 128;
   const int lane = threadIdx.x & 31;
@@ -317,6 +322,7 @@ __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* 
 // stay inside the segment.  For power-of-two G a warp reads and writes 128 contiguous bytes.
 __global__ void __launch_bounds__(256) grpo_adv_kernel(const float* __restrict__ rewards, int n_groups, int G,
                                                        int ddof, float eps_std, float* __restrict__ adv_seq) {
+  chain_begin();
   int seg = 32;
   while (seg > 1 && (seg >> 1) >= G) seg >>= 1;
   const int groups_per_warp = 32 / seg;
@@ -363,6 +369,7 @@ __global__ void __launch_bounds__(256) grpo_adv_kernel(const float* __restrict__
 template <int G4>
 __global__ void __launch_bounds__(256) grpo_adv_rows_kernel(const float4* __restrict__ rewards, int n_groups, int ddof,
                                                             float eps_std, float4* __restrict__ adv_seq) {
+  chain_begin();
   constexpr int G = 4 * G4;
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= n_groups) return;
@@ -408,6 +415,7 @@ __global__ void __launch_bounds__(256) grpo_adv_rows_kernel(const float4* __rest
 __global__ void __launch_bounds__(256) group_baseline_kernel(const float* __restrict__ rewards,
                                                              const int* __restrict__ lengths, int n_groups, int G,
                                                              int est, float* __restrict__ adv_seq) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (g >= n_groups) return;
@@ -439,6 +447,7 @@ __global__ void __launch_bounds__(256) group_baseline_kernel(const float* __rest
 // Batch statistics of c[n] in double, fixed order (one block): stats[0] = mean, stats[1] = population std.
 __global__ void __launch_bounds__(1024) batch_stats_kernel(const float* __restrict__ c, long long n,
                                                            double* __restrict__ stats) {
+  chain_begin();
   __shared__ double red[32];
   __shared__ double mean_s;
   double acc = 0.0;
@@ -465,6 +474,7 @@ __global__ void __launch_bounds__(1024) batch_stats_kernel(const float* __restri
 
 __global__ void __launch_bounds__(256) batch_normalise_kernel(float* __restrict__ c, long long n,
                                                               const double* __restrict__ stats, float eps_std) {
+  chain_begin();
   const double mu = stats[0];
   const double inv = 1.0 / (stats[1] + (double)eps_std);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -521,6 +531,7 @@ template <bool FUSED>
 __global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restrict__ rewards, int G, int ddof, float eps_std,
                                                             float* adv_seq, const int* __restrict__ seq_offsets, int n_seq,
                                                             long long T, int sweeps, float* __restrict__ adv_tok) {
+  chain_begin();
   if (FUSED)
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n_seq; s += gridDim.x * blockDim.x)
       adv_seq[s] = group_advantage(rewards, G, ddof, eps_std, s);
@@ -589,6 +600,7 @@ __global__ void __launch_bounds__(32 * kShapeWarps) kl_shaped_returns_kernel(
     const float* __restrict__ seq_value, const float* __restrict__ logp, const float* __restrict__ ref_logp,
     const float* __restrict__ kl_tok, const uint8_t* __restrict__ mask, const int* __restrict__ seq_offsets, int n_seq,
     long long T, float beta, float gamma, int kind, float* __restrict__ shaped, float* __restrict__ ret) {
+  chain_begin();
   __shared__ double g_s[WARPS], v_s[WARPS];
   __shared__ int live_s[WARPS];
   constexpr int kTeams = kShapeWarps / WARPS;
@@ -827,6 +839,7 @@ __device__ __forceinline__ void finish_loss(const double (&acc)[kLossSums], cons
 // A block takes 32 rows at a time, lane = row; its eight warps share the column ranges (with one thread per row a call of
 // a few hundred rows and 75 to 148 ranges was a chain of that many loads: 17 us) and warp 0 goes on with the sums.
 __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossParams p, DevStatus* st) {
+  chain_begin();
   constexpr int kW = kLossThreads / 32;
   __shared__ float max_s[2][kW][32];
   __shared__ float sum_s[5][kW][32];
@@ -988,6 +1001,7 @@ struct LogitGradParams {
 };
 
 __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
+  chain_begin();
   int off, rows;
   slab_extent(st->n_valid, p.slab_cap, p.slab_index, off, rows);
   const int rows_pad = (rows + 127) / 128 * 128;
@@ -1059,6 +1073,7 @@ __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p
 constexpr int kCountBlocks = 256;   // most blocks of count_valid_kernel: one count per thread of its reader
 __global__ void __launch_bounds__(256) count_valid_kernel(const uint8_t* __restrict__ mask, long long T,
                                                           unsigned* __restrict__ counts) {
+  chain_begin();
   unsigned int n = 0;
   const bool vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
   const long long n16 = vec ? T / 16 : 0;
@@ -1102,6 +1117,7 @@ struct TokenLossParams {
 
 template <bool VEC>
 __global__ void __launch_bounds__(kLossThreads, 4) token_loss_kernel(const TokenLossParams p) {
+  chain_begin();
   double acc[kLossSums];
 #pragma unroll
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
@@ -1225,6 +1241,7 @@ struct SeqParams {
 };
 
 __global__ void __launch_bounds__(1024) seq_lmax_kernel(const int* __restrict__ seq_offsets, int n_seq, int* l_max) {
+  chain_begin();
   __shared__ int red[32];
   int m = 0;
   for (int i = threadIdx.x; i < n_seq; i += blockDim.x) m = max(m, seq_offsets[i + 1] - seq_offsets[i]);
@@ -1266,6 +1283,7 @@ __device__ __forceinline__ float team_sum(float v) {
 
 template <int TEAM>
 __global__ void __launch_bounds__(kLossThreads) seq_loss_kernel(const SeqParams p, DevStatus* st) {
+  chain_begin();
   const int n = st->n_valid;
   const int lane = threadIdx.x % TEAM, team = threadIdx.x / TEAM;
   constexpr int teams = kLossThreads / TEAM;
@@ -1345,6 +1363,7 @@ __global__ void __launch_bounds__(256) merge_shard_stats_kernel(const float4* __
                                                                 long long T, const uint8_t* __restrict__ mask,
                                                                 float* __restrict__ logp, float* __restrict__ ent,
                                                                 float* __restrict__ lse) {
+  chain_begin();
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += (long long)gridDim.x * blockDim.x) {
     float o_logp = 0.f, o_ent = 0.f, o_lse = 0.f;
     if (!mask || mask[t]) {
@@ -1399,6 +1418,7 @@ __device__ __forceinline__ void add_piece(float4 (&x)[4], const float* q, int co
 template <bool F32>
 __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const int* __restrict__ row_map,
                                                          void* __restrict__ dH, const DevStatus* st) {
+  chain_begin();
   int slab_base, rows;
   slab_extent(st->n_valid, s.shape.slab_cap, s.shape.slab_index, slab_base, rows);
   const GemmExtents ex = gemm_extents(s.shape, st->n_valid, s.cg, s.workers);
