@@ -65,8 +65,8 @@ const char* rl_status_string(rl_status s);
  * size does not grow with T*V: the gradient with respect to the logits (and the 16-bit codes it is
  * made from) only ever exists for a bounded slab of rows x vocabulary columns. */
 rl_status rl_workspace_bytes(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, size_t* bytes);
-/* The same for calls that set rl_loss_opts.kl_full with a reference model of hidden size d_ref
- * (adds the compacted reference rows and five per-row arrays). */
+/* The same for calls that set rl_loss_opts.kl_full with a reference model of hidden size d_ref (adds the
+ * compacted reference rows, seven per-row arrays and, from d + d_ref = 1536 on, 4 bytes per slab entry). */
 rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, int64_t d_ref, size_t* bytes);
 /* Size of the slab the backward pass works in: at most max_rows token rows x max_cols vocabulary
  * columns of the gradient with respect to the logits exist at a time (bf16, in the workspace).
@@ -282,8 +282,8 @@ typedef struct {
                               /* KL(pi_theta(.|s_t) || pi_ref(.|s_t)) = sum_j p_j (log p_j -   */
                               /* log q_j) over the vocabulary, as sections 2.2 and 3.1 print   */
                               /* it, instead of the sampled-token k3 estimate; q = softmax(    */
-                              /* W_ref h_ref_t) is recomputed tile by tile next to p, never    */
-                              /* stored.  ref_logp is then unused (may be NULL).  Not          */
+                              /* W_ref h_ref_t) exists for a bounded slab of rows at a time,   */
+                              /* as p does.  ref_logp is then unused (may be NULL).  Not          */
                               /* combined with sequence_level / agg_mode 1, 2 (INVALID_ARG).   */
   const void* H_ref;          /* [T, d_ref] bf16 device, row stride ldH_ref: hidden states of  */
   int64_t ldH_ref;            /* the frozen reference model for the same rows                  */

@@ -94,6 +94,11 @@ inline int merge_blocks(int64_t rows, int slabs) {
 }
 // Neither option set: the tiles of the dH pass's ragged last wave are cut into parts that lie in slots.
 inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_slices == 1; }
+// Full-distribution KL: two single-product passes that leave 6 bytes per logit pair behind, or two-product tiles formed
+// twice.  The former trades 4 d + 4 d_ref tensor flops for 14 bytes of traffic per entry.  4096 rows, V = 151936: logits and
+// their gradient take 3.3 / 3.7 / 4.9 / 8.3 ms against 2.8 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
+constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
+inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
 // tile that is half empty costs as much as a full one.
 inline bool use_wide(const rl_ctx* c, int64_t d) {
@@ -116,6 +121,7 @@ struct WsLayout {
   size_t dH_slots;                                   // parts of cut dH tiles (0: none)
   int n_row_slabs, n_flags;                          // n_flags: row tiles, then one count per row slab
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
+  size_t words, zy_c, centre;                        // its one-sweep form (words 0: two-product tiles)
 };
 
 // Reference-model operands of the full-distribution KL (all NULL / 0 when it is not used).
@@ -163,7 +169,8 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   long long rows = c->slab_rows;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
   if (c->slab_auto) {
-    const long long whole = kSlabElements / Vpad / 256 * 256;
+    // as many rows as kSlabElements allows (half where slab entries take 6 bytes)
+    const long long whole = kSlabElements / (kl_one_sweep(d, d_ref) ? 2 : 1) / Vpad / 256 * 256;
     if (whole >= kSlabRowsMin || whole >= L.Tpad) {
       rows = whole < kSlabRowsMax ? whole : kSlabRowsMax;
       L.Vs = Vpad;
@@ -206,13 +213,18 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
   L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
   L.flags = take((size_t)L.n_flags * 4);
-  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = 0;
+  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.words = L.zy_c = L.centre = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
     L.partials2 = take((size_t)n_part_ranges * L.Tpad * sizeof(float4));
     L.lse_ref_c = take((size_t)L.Tpad * 4);
     L.kl_c = take((size_t)L.Tpad * 4);
     L.cb_c = take((size_t)L.Tpad * 4);
+    if (L.Vs == Vpad && kl_one_sweep(d, d_ref)) {
+      L.words = take((size_t)L.Ts * L.Vs * 4);
+      L.zy_c = take((size_t)L.Tpad * 4);
+      L.centre = take((size_t)L.Tpad * 4);
+    }
   }
   L.staging = o;
   o += (size_t)host_slots * carve_stage(nullptr, T, d, nullptr);
@@ -455,6 +467,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     sp.shift2 = reinterpret_cast<float*>(ws + L.shift2);
     sp.flags = reinterpret_cast<int*>(ws + L.flags);
     sp.n_flags = L.n_flags;
+    if (kl) sp.zy = reinterpret_cast<float*>(ws + L.zy_c);
   }
   pp.H = static_cast<const __nv_bfloat16*>(H);
   pp.ldH = ldH;
@@ -484,6 +497,13 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     prof_end(c, pr, 5);
   }
   c->launches += 1;
+  __nv_bfloat16* Hc_ref = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc_ref);
+  if (kl) {   // full KL: compact the reference hidden states with the same row map
+    launch(c, gather_plain_kernel, c->n_sm * 4, 256, static_cast<const __nv_bfloat16*>(kl->H_ref), kl->ldH_ref, (int)kl->d_ref,
+           row_map, Hc_ref, static_cast<const __nv_bfloat16*>(kl->W_ref), kl->ldW_ref, tokens_c, sp.zy,
+           sp.zy ? reinterpret_cast<float*>(ws + L.centre) : nullptr, c->dstatus);
+    c->launches++;
+  }
   if (!plan.stats) {
     memset(shape_out, 0, sizeof(*shape_out));
     return cuda_ok();
@@ -510,11 +530,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   if (!kl) {
     launch_gemm<EpiStats, 0, 0>(c, cg, 0, tmA, tmB, tmA, tmA, sh, ep);   // no output map
   } else {
-    // full KL: compact the reference hidden states with the same row map and form both logit
-    // tiles per output tile
-    __nv_bfloat16* Hc_ref = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc_ref);
-    launch(c, gather_plain_kernel, c->n_sm * 4, 256, static_cast<const __nv_bfloat16*>(kl->H_ref), kl->ldH_ref, (int)kl->d_ref, row_map, Hc_ref, c->dstatus);
-    c->launches++;
+    // both logit tiles per output tile
     CUtensorMap tmA2, tmB2;
     if (!map_kmajor(c, &tmA2, Hc_ref, (uint64_t)L.Tpad, (uint64_t)kl->d_ref, (uint64_t)kl->d_ref, BM)) return RL_ERR_CUDA;
     if (!map_kmajor(c, &tmB2, kl->W_ref, (uint64_t)V, (uint64_t)kl->d_ref, (uint64_t)kl->ldW_ref, b_box_rows(c)))
@@ -595,7 +611,8 @@ rl_status rl_create(rl_ctx** out, int device) {
   if (cudaMalloc(&c->dstatus, kStatusBytes) != cudaSuccess) { delete c; return RL_ERR_CUDA; }
   cudaMemset(c->dstatus, 0, kStatusBytes);
   bool ok = set_smem_attr<EpiStats, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad, 0, 0>() == cudaSuccess &&
-            set_smem_attr<EpiSweep, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiSweep, 0, 0>() == cudaSuccess && set_smem_attr<EpiRefSweep, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiSweepKL, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
@@ -1091,7 +1108,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   // rows' coefficients are known.  Not where the coefficients of a row need rows of another slab, nor where the
   // statistics come from elsewhere: those paths form the logits a second time.
   const int Vpad = (int)align_up((size_t)V, 256);
-  const bool sweep = L.Vs == Vpad && !shard && !o.kl_full &&
+  const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.words) &&
                      (L.n_row_slabs == 1 || (L.Ts % kFlagRows == 0 && !seq_path));
   GemmShape fwd_shape;
   FwdPlan plan;
@@ -1146,8 +1163,10 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   }
   if (o.kl_full) {
     p.kl_full = 1;
-    p.fwd_cg = c->cta_group;   // two-product tiles
-    p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+    if (!sweep) {   // two-product tiles
+      p.fwd_cg = c->cta_group;
+      p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
+    }
     p.partials2 = reinterpret_cast<const float4*>(ws + L.partials2);
     p.lse_ref_c = reinterpret_cast<float*>(ws + L.lse_ref_c);
     p.kl_c = reinterpret_cast<float*>(ws + L.kl_c);
@@ -1217,7 +1236,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int* row_map = reinterpret_cast<const int*>(ws + L.row_map);
   const int* n_valid = &c->dstatus->n_valid;
 
-  CUtensorMap tmHc_k, tmW_k, tmG_k, tmW_mn, tmG_mn, tmHc_mn, tm_dH, tm_dW, tm_G_out, tmHr_k, tmWr_k, tm_slots, tmW_fwd;
+  CUtensorMap tmHc_k, tmW_k, tmG_k, tmW_mn, tmG_mn, tmHc_mn, tm_dH, tm_dW, tm_G_out, tmHr_k, tmWr_k, tm_slots, tmW_fwd,
+      tmWr_fwd;
   if (o.kl_full) {
     if (!map_kmajor(c, &tmHr_k, ws + L.Hc_ref, (uint64_t)L.Tpad, (uint64_t)o.d_ref, (uint64_t)o.d_ref, BM) ||
         !map_kmajor(c, &tmWr_k, o.W_ref, (uint64_t)V, (uint64_t)o.d_ref, (uint64_t)o.ldW_ref, b_box_rows(c)))
@@ -1243,6 +1263,9 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   tmW_fwd = tmW_k;
   if (cg_fwd != c->cta_group)
     ok = ok && map_kmajor(c, &tmW_fwd, W, (uint64_t)V, (uint64_t)d, (uint64_t)ldW, b_box_rows(cg_fwd));
+  tmWr_fwd = tmWr_k;
+  if (o.kl_full && cg_fwd != c->cta_group)
+    ok = ok && map_kmajor(c, &tmWr_fwd, o.W_ref, (uint64_t)V, (uint64_t)o.d_ref, (uint64_t)o.ldW_ref, b_box_rows(cg_fwd));
   if (!ok) return RL_ERR_CUDA;
 
   const int n_row_slabs = L.n_row_slabs;
@@ -1272,13 +1295,38 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sw.n_split_max = L.part_ranges;
           sw.a_mn_slab = 1;
           sw.m_group = row_group_tiles(c, d);
+          const float* centre = reinterpret_cast<const float*>(ws + L.centre);
+          float* words = reinterpret_cast<float*>(ws + L.words);
+          if (o.kl_full) {
+            GemmShape sr = sw;
+            sr.k_cap = (int)o.d_ref;
+            sr.m_group = row_group_tiles(c, o.d_ref);
+            EpiRefSweep::Params er;
+            er.partials2 = reinterpret_cast<float4*>(ws + L.partials2);
+            er.part_stride = L.Tpad;
+            er.V = (int)V;
+            er.slab = words;
+            er.ld = L.Vs;
+            launch_gemm<EpiRefSweep, 0, 0>(c, cg_fwd, 0, tmHr_k, tmWr_fwd, tm_G_out, tm_G_out, sr, er);
+          }
           EpiSweep::Params ep;
           ep.stats.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.stats.partials = reinterpret_cast<float4*>(ws + L.partials);
           ep.stats.part_stride = L.Tpad;
           ep.stats.V = (int)V;
           ep.shift2 = reinterpret_cast<const float*>(ws + L.shift2);
-          launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
+          if (o.kl_full) {
+            EpiSweepKL::Params ek;
+            ek.stats = ep.stats;
+            ek.partials2 = reinterpret_cast<float4*>(ws + L.partials2);
+            ek.shift2 = ep.shift2;
+            ek.centre = centre;
+            ek.slab = words;
+            ek.ld = L.Vs;
+            launch_gemm<EpiSweepKL, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ek);
+          } else {
+            launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
+          }
           p.fwd_shape = sw;
           p.slab_cap = L.Ts;
           p.slab_index = r;
@@ -1295,7 +1343,11 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.shift2 = ep.shift2;
           lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
           const int pr_lg = prof_begin(c, 1);
-          launch(c, logit_grad_kernel, c->n_sm * 8, 256, lg, c->dstatus);
+          lg.words = reinterpret_cast<const uint32_t*>(words);
+          lg.centre = centre;
+          lg.lse_ref = p.lse_ref_c; lg.kl = p.kl_c; lg.cb = p.cb_c;
+          if (o.kl_full) launch(c, logit_grad_kl_kernel, c->n_sm * 8, 256, lg, c->dstatus);
+          else           launch(c, logit_grad_kernel, c->n_sm * 8, 256, lg, c->dstatus);
           prof_end(c, pr_lg, 1);
           c->launches++;
         }
@@ -1325,7 +1377,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           ep.lse = p.lse_c; ep.lse_ref = p.lse_ref_c; ep.ent = p.ent_c; ep.kl = p.kl_c;
           ep.cp = p.cp_c; ep.cb = p.cb_c; ep.ce = p.ce_c;
           ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_dual<EpiGradKL>(c, 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
+          launch_dual<EpiGradKL>(c, sweep ? -1 : 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
         }
       }
       // (2) dH_slab (+)= G * W_slab        [rows x d], K = vocabulary columns of the slab

@@ -168,6 +168,7 @@ struct SweepPrep {
   long long ldW;
   const float* old_logp;   // [T] original rows
   float* shift2;           // [rows] compact: the estimate in units of log 2, or NULL
+  float* zy;               // [rows] compact: the logit itself, or NULL
   int* flags;              // words cleared for the launches that follow
   int n_flags;
 };
@@ -232,6 +233,7 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
     if (lane == 0) {
       const float est = z - p.sp.old_logp[t];
       p.sp.shift2[pos] = (isfinite(est) ? est : 0.f) * kLog2e;
+      if (p.sp.zy) p.sp.zy[pos] = z;
     }
   } else {
 #pragma unroll 4
@@ -293,10 +295,14 @@ __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevS
   }
 }
 
-// Row compaction of a second hidden-state matrix (the reference model's) with the same row map.
+// Row compaction of a second hidden-state matrix (the reference model's) with the same row map.  centre != NULL: also the
+// difference of the sampled token's two logits, which the words of the one-sweep KL are centred on.
 __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* __restrict__ H, long long ldH, int d,
                                                            const int* __restrict__ row_map,
-                                                           __nv_bfloat16* __restrict__ Hc, const DevStatus* st) {
+                                                           __nv_bfloat16* __restrict__ Hc,
+                                                           const __nv_bfloat16* __restrict__ W, long long ldW,
+                                                           const int* __restrict__ tokens_c, const float* __restrict__ zy,
+                                                           float* __restrict__ centre, const DevStatus* st) {
   chain_begin();
   const int n = st->n_valid;
   const int n_pad = (n + 127) / 128 * 128;
@@ -307,7 +313,27 @@ __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* 
     uint4* dst = reinterpret_cast<uint4*>(Hc + (size_t)i * d);
     if (i < n) {
       const uint4* src = reinterpret_cast<const uint4*>(H + (size_t)row_map[i] * ldH);
-      for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
+      const uint4* wrow = centre ? reinterpret_cast<const uint4*>(W + (size_t)max(tokens_c[i], 0) * ldW) : nullptr;
+      float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+      for (int v = lane; v < vec_per_row; v += 32) {
+        const uint4 h = __ldg(src + v);
+        dst[v] = h;
+        if (centre) {
+          const uint4 w = __ldg(wrow + v);
+          const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
+                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
+        }
+      }
+      if (centre) {
+        float z = acc.x + acc.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (lane == 0) centre[i] = zy[i] - z;
+      }
     } else {
       for (int v = lane; v < vec_per_row; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
     }
@@ -998,7 +1024,74 @@ struct LogitGradParams {
   const float* ent;
   const float* cp;
   const float* ce;
+  // full-distribution KL: words of code and fp16 (z - zr - centre), read from here; the slab is only written
+  const uint32_t* words;
+  const float* centre;
+  const float* lse_ref;
+  const float* kl;
+  const float* cb;
 };
+
+// The same with the regulariser's term: g_tj = cp_t (p_tj - 1[j = y_t]) + cb_t p_tj (log p_tj - log q_tj - KL_t)
+// + ce_t p_tj (log p_tj + Ent_t).  4 bytes in and 2 out per entry.
+__global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParams p, const DevStatus* st) {
+  chain_begin();
+  int off, rows;
+  slab_extent(st->n_valid, p.slab_cap, p.slab_index, off, rows);
+  const int rows_pad = (rows + 127) / 128 * 128;
+  const int units_per_row = (p.ld + kGradUnit - 1) / kGradUnit;
+  const long long n_units = (long long)rows_pad * units_per_row;
+  const int lane = threadIdx.x & 31;
+  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
+    const int r = (int)(u / units_per_row);
+    const int c0 = (int)(u - (long long)r * units_per_row) * kGradUnit;
+    uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
+    if (r >= rows) {
+#pragma unroll
+      for (int k = 0; k < kGradVecs; ++k)
+        if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
+      continue;
+    }
+    const uint4* src = reinterpret_cast<const uint4*>(p.words + (size_t)r * p.ld + c0) + 2 * lane;
+    uint4 q[2 * kGradVecs];
+#pragma unroll
+    for (int k = 0; k < kGradVecs; ++k)
+      if (c0 + k * 256 < p.ld) { q[2 * k] = __ldcs(src + k * 64); q[2 * k + 1] = __ldcs(src + k * 64 + 1); }
+    const int i = off + r;
+    const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i], cb = p.cb[i];
+    const int y = p.tokens_c[i];
+    const float shift = fmaf(-lse, kLog2e, p.shift2[i]);   // log2 p = exponent of the code + shift
+    // g = p (kc + kl log2 p + cb delta), delta = the fp16 half: z - zr - centre
+    const float kc = fmaf(ce, ent, cp) + cb * (p.centre[i] - lse + p.lse_ref[i] - p.kl[i]), kl = ce * kLn2;
+    const float py = ex2_approx(logp * kLog2e);
+#pragma unroll
+    for (int k = 0; k < kGradVecs; ++k) {
+      const int c = c0 + k * 256 + lane * 8;
+      if (c0 + k * 256 >= p.ld) break;
+      const uint32_t w[8] = {q[2 * k].x, q[2 * k].y, q[2 * k].z, q[2 * k].w,
+                             q[2 * k + 1].x, q[2 * k + 1].y, q[2 * k + 1].z, q[2 * k + 1].w};
+      float g[8];
+      const unsigned rel = (unsigned)(y - c);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float t = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5410))) + shift;
+        const float dl = __half2float(__ushort_as_half((unsigned short)(w[j] >> 16)));
+        const bool at = rel == (unsigned)j;
+        const float f = fmaf(cb, dl, fmaf(kl, at ? logp * kLog2e : t, kc));
+        g[j] = at ? fmaf(py, f, -cp) : ex2_approx(t) * f;
+        if (c + j >= p.V) g[j] = 0.f;
+      }
+      uint32_t o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
+        o[j] = *reinterpret_cast<const uint32_t*>(&b);
+      }
+      base[k * 32] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
 
 __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
   chain_begin();

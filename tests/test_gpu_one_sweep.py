@@ -86,3 +86,42 @@ def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
     assert torch.allclose(a["loss"], b["loss"], rtol=1e-5)
     # two roundings to bf16 (2^-9 each) of the same gradient
     assert _rel(_np64(a["dH"]), _np64(b["dH"])) <= 4e-3 and _rel(_np64(a["dW"]), _np64(b["dW"])) <= 4e-3
+
+
+# full-distribution KL with the logits of both models formed once: hidden sizes on both sides of the rule that chooses it,
+# slabs of one and several row tiles, a single-CTA case (at most 128 rows), ragged vocabulary, an entropy term, and rows
+# whose codes cannot hold their logits; regulariser alone (adv = 0) so that its own term is what is compared
+@pytest.mark.parametrize("d,d_ref,V,L_max,rows,off,ent", [
+    (768, 768, 1025, 150, 256, 0.0, 0.01), (1472, 64, 2085, 150, 512, 0.0, 0.0), (1408, 64, 2085, 150, 512, 0.0, 0.0),
+    (64, 1536, 300, 15, 0, 0.0, 0.0), (768, 1024, 1536, 150, 0, 20.0, 0.0),
+])
+def test_one_sweep_full_kl(d, d_ref, V, L_max, rows, off, ent):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_reference_model, make_workload
+    w = make_workload(1, prompts=1, L_max=L_max, d=d, V=V, seed=2000 + V)
+    H_ref, W_ref = make_reference_model(w, d_ref=d_ref, drift=0.3)
+    valid = torch.nonzero(w.mask)[:, 0]
+    hit = valid[::max(1, valid.numel() // 3)]
+    w.old_logp[hit[0::2]] += off
+    w.old_logp[hit[1::2]] -= off
+    c = Context(0)
+    try:
+        if rows:
+            c.set_slab_limits(rows, -(-V // 256) * 256)
+        c.ensure_workspace(w.T, d, V, d_ref=d_ref)
+        c._ws.fill_(0xFF)
+        for scale in (0.0, 0.1):
+            adv = torch.rand(w.T, device="cuda") * scale
+            out = c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, None, adv, w.mask, w.eps_low, w.eps_high, 0.05,
+                                           ent_coef=ent, dH_fp32=True, H_ref=H_ref, W_ref=W_ref)
+            status, detail = c.last_device_status()
+            assert status == 0, (status, hex(detail & 0xffffffff))
+            oo = O.policy_loss_fwd_bwd(_np64(w.H), _np64(w.W), w.tokens.cpu().numpy(), _np64(w.old_logp), None, _np64(adv),
+                                       w.mask.cpu().numpy(), w.eps_low, w.eps_high, 0.05, ent_coef=ent,
+                                       H_ref=_np64(H_ref), W_ref=_np64(W_ref))
+            # KL_t is a difference of fp32 quantities of the size of lse (about 10): a few ulp of that
+            assert abs(out["metrics"][1].item() - oo["kl_mean"]) <= 2e-3 * abs(oo["kl_mean"]) + 2e-5
+            assert abs(out["loss"].item() - oo["loss"]) <= 1e-3 * abs(oo["loss"]) + 1e-6
+            assert _rel(_np64(out["dH"]), oo["dH"]) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
+    finally:
+        c.close()
