@@ -72,8 +72,8 @@ rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, in
  * columns of the gradient with respect to the logits exist at a time (bf16, in the workspace).
  * max_rows a multiple of 128, max_cols a multiple of 256, max_rows * max_cols at most 2^31; 0 for one of
  * them is 32768 rows or 37888 columns.  (0, 0) restores the default: rows over the whole vocabulary, at most
- * 2^31 entries (14080 rows at 152 K words, 4.3 GB), or 32768 x 37888 for vocabularies of which fewer than
- * 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary, max_rows at least 256)
+ * 2^31 entries and 58 MB of hidden states (14080 rows at d = 2048 and 152 K words, 4.3 GB), or 32768 x 37888 for
+ * vocabularies of which fewer than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary, max_rows at least 256)
  * the loss calls form the logits once instead of twice: 13-20 % of a step.  Changes what
  * rl_workspace_bytes() returns: call it first. */
 rl_status rl_set_slab_limits(rl_ctx* ctx, int max_rows, int max_cols);

@@ -61,11 +61,14 @@ namespace {
 
 constexpr long long kRowGroupBytes = 36ll << 20;   // A panels walked together by the rows-first passes (L2 is 126 MB)
 constexpr int kSlabRowsMax = 32768;        // rows of one gradient slab
-// Slab shape when the caller sets none: rows over the WHOLE vocabulary, as many as kSlabElements allows (14080 rows at
-// 152 K words, 4.3 GB).  A row that is complete in the slab needs its logits formed only once.  Fewer rows per slab mean
-// more passes over dW (8 bytes per entry and slab, beside 10 bytes per entry of the slab itself); below
-// kSlabRowsMin rows a slab is cut by columns instead.
+// Slab shape when the caller sets none: rows over the WHOLE vocabulary, at most kSlabElements entries, and no more than
+// kSlabRowBytes of compact hidden rows (14080 rows at d = 2048 and 152 K words, 4.3 GB).  A row that is complete in the slab
+// needs its logits formed only once.  Fewer rows per slab mean more passes over dW (8 bytes per entry and slab, beside 10
+// bytes per entry of the slab itself); more rows than L2 keeps make the dW pass re-read them from DRAM (7B-class step:
+// 208 ms with 85 MB of rows per slab, 200 with 57; d = 2560: 178 ms with 70 MB, 173 with 60; 48 MB instead of 58 at d =
+// 2048: 1 % slower; twice the slab: 1-3 % slower on every large step).  Below kSlabRowsMin rows a slab is cut by columns.
 constexpr long long kSlabElements = 1ll << 31;
+constexpr long long kSlabRowBytes = 58ll << 20;
 constexpr int kSlabRowsMin = 2048;
 // Device words a context owns besides the workspace: the status record, a few scalars of the small kernels
 // (byte 64: batch statistics, 96: longest response, kTicketOffset: ticket counter of the loss kernels), the valid-row
@@ -169,8 +172,12 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   long long rows = c->slab_rows;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
   if (c->slab_auto) {
-    // as many rows as kSlabElements allows (half where slab entries take 6 bytes)
-    const long long whole = kSlabElements / (kl_one_sweep(d, d_ref) ? 2 : 1) / Vpad / 256 * 256;
+    // as many rows as kSlabElements allows (half where slab entries take 6 bytes), and no more than
+    // keep the compact rows, which the dW pass reads once per row panel of dW, in L2 beside the streamed slab
+    long long whole = kSlabElements / (kl_one_sweep(d, d_ref) ? 2 : 1) / Vpad / 256 * 256;
+    long long resident = kSlabRowBytes / (d * 2) / 256 * 256;
+    if (resident < kSlabRowsMin) resident = kSlabRowsMin;
+    if (whole > resident) whole = resident;
     if (whole >= kSlabRowsMin || whole >= L.Tpad) {
       rows = whole < kSlabRowsMax ? whole : kSlabRowsMax;
       L.Vs = Vpad;
