@@ -115,10 +115,10 @@ struct GemmShape {
   int skip_if_k0;   // nothing to do at all when K is empty (otherwise the epilogue sees zeros)
   int n_fastest;    // 1: consecutive units walk the column ranges of one row tile first
   // Row slabs of the backward pass: when slab_cap > 0 the valid rows are cut into
-  // ceil(n_valid / slab_cap) slabs of equal size (a multiple of 256, at most slab_cap) and this
+  // ceil(n_valid / slab_cap) slabs of equal size (a multiple of 256; one slab up to slab_one rows) and this
   // launch works on slab slab_index: its row offset replaces m_dyn_off / k_dyn_off, and is added
   // to the A row coordinate (a_mn_slab) or the B k coordinate (b_k_slab).
-  int slab_cap, slab_index, a_mn_slab, b_k_slab;
+  int slab_cap, slab_one, slab_index, a_mn_slab, b_k_slab;
   // K split: when k_split_max > 1 every output tile may be cut into up to k_split_max slices of
   // the K range, each a work unit of its own that adds into its own output buffer (the epilogue
   // gets the slice index); the slice count is chosen on the device to even out the last wave.
@@ -208,11 +208,11 @@ __host__ __device__ inline int choose_k_split(long tiles, int n_workers, int sma
 }
 
 // Offset and row count of slab `index` when n_valid rows are cut into equal slabs of at most cap rows.
-__host__ __device__ inline void slab_extent(int n_valid, int cap, int index, int& off, int& rows) {
-  int n_slabs = (n_valid + cap - 1) / cap;
-  if (n_slabs < 1) n_slabs = 1;
+// Up to `one` rows (at least cap) stay in one slab: two half slabs would be worse than one that is a little long.
+__host__ __device__ inline void slab_extent(int n_valid, int cap, int one, int index, int& off, int& rows) {
+  int n_slabs = n_valid <= one ? 1 : (n_valid + cap - 1) / cap;
   int per = ((n_valid + n_slabs - 1) / n_slabs + 255) / 256 * 256;
-  if (per > cap) per = cap;
+  if (per > one) per = one;
   off = index * per;
   rows = n_valid - off;
   rows = rows < 0 ? 0 : (rows > per ? per : rows);
@@ -258,7 +258,7 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
   e.slab_off = 0;
   int m, k;
   if (sh.slab_cap > 0) {
-    slab_extent(n_valid, sh.slab_cap, sh.slab_index, e.slab_off, m);
+    slab_extent(n_valid, sh.slab_cap, sh.slab_one, sh.slab_index, e.slab_off, m);
     k = m;
   } else {
     m = n_valid - sh.m_dyn_off;

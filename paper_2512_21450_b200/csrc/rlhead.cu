@@ -116,7 +116,8 @@ inline size_t dh_slot_bytes(const rl_ctx* c, int64_t d) {
 }
 
 struct WsLayout {
-  int Tpad, Ts, Vs;
+  int Tpad, Ts, Vs;   // rows; most rows and columns of a slab
+  int Tc;             // rows of a slab when there are several
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
   size_t row_pos;                                    // position of every row in the row map (large T)
   size_t shift2, flags;                              // one-sweep path: log-sum-exp estimates, row-tile flags
@@ -169,7 +170,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   WsLayout L;
   L.Tpad = (int)align_up((size_t)(T > 0 ? T : 1), 128);
   const int Vpad = (int)align_up((size_t)V, 256);
-  long long rows = c->slab_rows;
+  long long rows = c->slab_rows, one = 0;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
   if (c->slab_auto) {
     // as many rows as kSlabElements allows (half where slab entries take 6 bytes), and no more than
@@ -177,14 +178,17 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
     long long whole = kSlabElements / (kl_one_sweep(d, d_ref) ? 2 : 1) / Vpad / 256 * 256;
     long long resident = kSlabRowBytes / (d * 2) / 256 * 256;
     if (resident < kSlabRowsMin) resident = kSlabRowsMin;
-    if (whole > resident) whole = resident;
     if (whole >= kSlabRowsMin || whole >= L.Tpad) {
-      rows = whole < kSlabRowsMax ? whole : kSlabRowsMax;
+      if (whole > kSlabRowsMax) whole = kSlabRowsMax;
+      rows = whole < resident ? whole : resident;
+      one = whole < resident * 3 / 2 ? whole : resident * 3 / 512 * 256;
       L.Vs = Vpad;
     }
   }
-  L.Ts = L.Tpad < rows ? L.Tpad : (int)rows;
-  L.n_row_slabs = (L.Tpad + L.Ts - 1) / L.Ts;
+  if (one < rows) one = rows;
+  L.Ts = L.Tpad < one ? L.Tpad : (int)one;
+  L.Tc = L.Tpad < rows ? L.Tpad : (int)rows;
+  L.n_row_slabs = L.Tpad <= L.Ts ? 1 : (L.Tpad + L.Tc - 1) / L.Tc;
   size_t o = 0;
   size_t n_part_ranges = kMaxSplit;
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 1024); return at; };
@@ -1116,7 +1120,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   // statistics come from elsewhere: those paths form the logits a second time.
   const int Vpad = (int)align_up((size_t)V, 256);
   const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.words) &&
-                     (L.n_row_slabs == 1 || (L.Ts % kFlagRows == 0 && !seq_path));
+                     (L.n_row_slabs == 1 || (L.Tc % kFlagRows == 0 && !seq_path));
   GemmShape fwd_shape;
   FwdPlan plan;
   plan.out.dH = dH;
@@ -1296,7 +1300,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           GemmShape sw;
           memset(&sw, 0, sizeof(sw));
           sw.n_valid = n_valid;
-          sw.m_rows_cap = rows_cap; sw.m_dyn = 1; sw.slab_cap = L.Ts; sw.slab_index = r;
+          sw.m_rows_cap = rows_cap; sw.m_dyn = 1; sw.slab_cap = L.Tc; sw.slab_one = L.Ts; sw.slab_index = r;
           sw.k_cap = (int)d;
           sw.n_tiles = (cols + BN - 1) / BN;
           sw.n_split_max = L.part_ranges;
@@ -1335,7 +1339,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
           }
           p.fwd_shape = sw;
-          p.slab_cap = L.Ts;
+          p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;
           p.shift2 = ep.shift2;
           p.tile_flags = flags;
@@ -1345,7 +1349,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.slab = reinterpret_cast<uint16_t*>(G);
           lg.ld = L.Vs;
           lg.V = (int)V;
-          lg.slab_cap = L.Ts; lg.slab_index = r;
+          lg.slab_cap = L.Tc; lg.slab_one = L.Ts; lg.slab_index = r;
           lg.tokens_c = ep.stats.tokens_c;
           lg.shift2 = ep.shift2;
           lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
@@ -1353,15 +1357,21 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.words = reinterpret_cast<const uint32_t*>(words);
           lg.centre = centre;
           lg.lse_ref = p.lse_ref_c; lg.kl = p.kl_c; lg.cb = p.cb_c;
-          if (o.kl_full) launch(c, logit_grad_kl_kernel, c->n_sm * 8, 256, lg, c->dstatus);
-          else           launch(c, logit_grad_kernel, c->n_sm * 8, 256, lg, c->dstatus);
+          const long long padded = (long long)align_up(rows_cap, 128);
+          const bool few = o.kl_full || padded * ((L.Vs + 256 * kGradVecs - 1) / (256 * kGradVecs)) < kGradFewUnits;
+          const int unit = 256 * (few ? kGradVecsFew : kGradVecs);
+          long long grad_blocks = (padded * ((L.Vs + unit - 1) / unit) + 7) / 8;   // a warp each
+          if (grad_blocks > c->n_sm * 64) grad_blocks = c->n_sm * 64;
+          if (o.kl_full) launch(c, logit_grad_kl_kernel, (int)grad_blocks, 256, lg, c->dstatus);
+          else if (few)  launch(c, logit_grad_kernel<kGradVecsFew>, (int)grad_blocks, 256, lg, c->dstatus);
+          else           launch(c, logit_grad_kernel<kGradVecs>, (int)grad_blocks, 256, lg, c->dstatus);
           prof_end(c, pr_lg, 1);
           c->launches++;
         }
         GemmShape sh;
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
-        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
+        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
         sh.k_cap = (int)d;
         sh.n_tiles = (cols + BN - 1) / BN;
         sh.n_range = 0; sh.n_range_lo = 1; sh.n_range_hi = kFwdRange; sh.n_range_always = 1;   // chosen on the device
@@ -1392,7 +1402,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         GemmShape sh;
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
-        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
+        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
         sh.k_cap = cols;
         sh.n_tiles = (int)((d + dh_cols - 1) / dh_cols);
         sh.n_range = 1;
@@ -1417,7 +1427,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
         sh.m_rows_cap = cols - c0 < step ? cols - c0 : step;
-        sh.k_cap = rows_cap; sh.k_dyn = 1; sh.slab_cap = L.Ts; sh.slab_index = r;
+        sh.k_cap = rows_cap; sh.k_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
         const bool wide = use_wide(c, d) && L.Ts >= kWideMinRows;
         sh.n_tiles = wide ? (int)((d + 2 * BN - 1) / (2 * BN)) : d_tiles;
         sh.n_range = 1;

@@ -799,7 +799,7 @@ struct LossParams {
   const float* ext_lse;
   // one row slab of the one-sweep path (slab_cap > 0): only its rows are merged, and the row tiles whose estimated
   // log-sum-exp lies too far from the true one for the 16-bit codes are flagged
-  int slab_cap, slab_index;
+  int slab_cap, slab_one, slab_index;
   const float* shift2;
   int* tile_flags;   // [rows / kFlagRows], over all rows
   int* flag_count;   // non-zero: this slab has a flagged tile
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
   const float w_mean = n_mean > 0 ? (float)(1.0 / (double)n_mean) : 0.f;
   int i_begin = 0, i_end = n;
   if (p.slab_cap > 0) {
-    slab_extent(n, p.slab_cap, p.slab_index, i_begin, i_end);
+    slab_extent(n, p.slab_cap, p.slab_one, p.slab_index, i_begin, i_end);
     i_end += i_begin;
   }
   for (int i0 = i_begin + blockIdx.x * 32; i0 < i_end; i0 += gridDim.x * 32) {
@@ -1009,14 +1009,16 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
 //   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),  log p_tj = code exponent + (estimate - lse_t),
 // rows past the slab's valid rows (up to a multiple of 128) and columns past V become zero.  The sampled token's own
 // entry uses its exact log-probability.  Bound by memory: 2 bytes in and 2 out per entry and nothing read twice.  A
-// warp takes kGradUnit consecutive columns of one row, all its 16-byte loads in flight before the first is used.
-constexpr int kGradVecs = 4;                       // 16-byte words per lane and unit
-constexpr int kGradUnit = 32 * 8 * kGradVecs;      // columns per warp and unit
+// warp takes VECS * 256 consecutive columns of one row, all its 16-byte loads in flight before the first is used.  18947 rows
+// x 152064 columns: 2.13 ms, 5.4 TB/s (four loads instead of eight, and one wave of blocks instead of many: 2.32 ms).
+constexpr int kGradVecs = 8;         // 16-byte words per lane and unit of VECS * 256 columns
+constexpr int kGradVecsFew = 4;      // the same with few rows (twice the warps), and for the KL kernel, which loads two per output
+constexpr long long kGradFewUnits = 65536;   // units of kGradVecs below which it is few: 276 rows 35 us instead of 37
 struct LogitGradParams {
   uint16_t* slab;          // [slab rows][ld]
   int ld;                  // multiple of 256
   int V;
-  int slab_cap, slab_index;
+  int slab_cap, slab_one, slab_index;
   const int* tokens_c;     // per compact row, as the arrays below
   const float* shift2;
   const float* lse;
@@ -1037,26 +1039,26 @@ struct LogitGradParams {
 __global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParams p, const DevStatus* st) {
   chain_begin();
   int off, rows;
-  slab_extent(st->n_valid, p.slab_cap, p.slab_index, off, rows);
+  slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
   const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + kGradUnit - 1) / kGradUnit;
+  const int units_per_row = (p.ld + (kGradVecsFew * 256) - 1) / (kGradVecsFew * 256);
   const long long n_units = (long long)rows_pad * units_per_row;
   const int lane = threadIdx.x & 31;
   const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
     const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * kGradUnit;
+    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecsFew * 256);
     uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
     if (r >= rows) {
 #pragma unroll
-      for (int k = 0; k < kGradVecs; ++k)
+      for (int k = 0; k < kGradVecsFew; ++k)
         if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
       continue;
     }
     const uint4* src = reinterpret_cast<const uint4*>(p.words + (size_t)r * p.ld + c0) + 2 * lane;
-    uint4 q[2 * kGradVecs];
+    uint4 q[2 * kGradVecsFew];
 #pragma unroll
-    for (int k = 0; k < kGradVecs; ++k)
+    for (int k = 0; k < kGradVecsFew; ++k)
       if (c0 + k * 256 < p.ld) { q[2 * k] = __ldcs(src + k * 64); q[2 * k + 1] = __ldcs(src + k * 64 + 1); }
     const int i = off + r;
     const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i], cb = p.cb[i];
@@ -1066,7 +1068,7 @@ __global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParam
     const float kc = fmaf(ce, ent, cp) + cb * (p.centre[i] - lse + p.lse_ref[i] - p.kl[i]), kl = ce * kLn2;
     const float py = ex2_approx(logp * kLog2e);
 #pragma unroll
-    for (int k = 0; k < kGradVecs; ++k) {
+    for (int k = 0; k < kGradVecsFew; ++k) {
       const int c = c0 + k * 256 + lane * 8;
       if (c0 + k * 256 >= p.ld) break;
       const uint32_t w[8] = {q[2 * k].x, q[2 * k].y, q[2 * k].z, q[2 * k].w,
@@ -1093,28 +1095,29 @@ __global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParam
   }
 }
 
+template <int VECS>
 __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
   chain_begin();
   int off, rows;
-  slab_extent(st->n_valid, p.slab_cap, p.slab_index, off, rows);
+  slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
   const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + kGradUnit - 1) / kGradUnit;
+  const int units_per_row = (p.ld + (VECS * 256) - 1) / (VECS * 256);
   const long long n_units = (long long)rows_pad * units_per_row;
   const int lane = threadIdx.x & 31;
   const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
     const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * kGradUnit;
+    const int c0 = (int)(u - (long long)r * units_per_row) * (VECS * 256);
     uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
     if (r >= rows) {
 #pragma unroll
-      for (int k = 0; k < kGradVecs; ++k)
+      for (int k = 0; k < VECS; ++k)
         if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
       continue;
     }
-    uint4 q[kGradVecs];
+    uint4 q[VECS];
 #pragma unroll
-    for (int k = 0; k < kGradVecs; ++k)
+    for (int k = 0; k < VECS; ++k)
       if (c0 + k * 256 < p.ld) q[k] = base[k * 32];
     const int i = off + r;
     const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i];
@@ -1124,7 +1127,7 @@ __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p
     // the sampled token's entry from its exact log-probability
     const float gy = fmaf(ex2_approx(logp * kLog2e), fmaf(ce, logp, kc), -cp);
 #pragma unroll
-    for (int k = 0; k < kGradVecs; ++k) {
+    for (int k = 0; k < VECS; ++k) {
       const int c = c0 + k * 256 + lane * 8;
       if (c0 + k * 256 >= p.ld) break;
       const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
@@ -1513,7 +1516,7 @@ __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const
                                                          void* __restrict__ dH, const DevStatus* st) {
   chain_begin();
   int slab_base, rows;
-  slab_extent(st->n_valid, s.shape.slab_cap, s.shape.slab_index, slab_base, rows);
+  slab_extent(st->n_valid, s.shape.slab_cap, s.shape.slab_one, s.shape.slab_index, slab_base, rows);
   const GemmExtents ex = gemm_extents(s.shape, st->n_valid, s.cg, s.workers);
   const int slices = s.shape.stream_k == 1 ? 2 : ex.k_split;   // stream-K launches always keep two buffers
   const int lane = threadIdx.x & 31;
