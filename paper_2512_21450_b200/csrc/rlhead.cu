@@ -436,6 +436,14 @@ inline int row_group_tiles(const rl_ctx* c, int64_t k) {
   return n < 1 ? 1 : (n > (1 << 20) ? (1 << 20) : (int)n);
 }
 
+// Compute capability and SM count (cudaGetDeviceProperties takes 2.5 ms, these two queries a microsecond).
+rl_status device_facts(int device, int* major, int* n_sm) {
+  if (cudaDeviceGetAttribute(major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return RL_ERR_CUDA;
+  return *major == 10 ? RL_OK : RL_ERR_UNSUPPORTED_ARCH;
+}
+
 inline rl_status cuda_ok() { return cudaGetLastError() == cudaSuccess ? RL_OK : RL_ERR_CUDA; }
 
 // Mask scan of T rows in two launches (three for very many), row_pos may be NULL.
@@ -580,14 +588,14 @@ const char* rl_status_string(rl_status s) {
 rl_status rl_create(rl_ctx** out, int device) {
   if (!out) return RL_ERR_INVALID_ARG;
   *out = nullptr;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return RL_ERR_CUDA;
-  if (prop.major != 10) return RL_ERR_UNSUPPORTED_ARCH;
+  int major = 0, n_sm = 0;
+  rl_status sd = device_facts(device, &major, &n_sm);
+  if (sd != RL_OK) return sd;
   if (cudaSetDevice(device) != cudaSuccess) return RL_ERR_CUDA;
   rl_ctx* c = new (std::nothrow) rl_ctx();
   if (!c) return RL_ERR_CUDA;
   c->device = device;
-  c->n_sm = prop.multiProcessorCount;
+  c->n_sm = n_sm;
   c->stream = nullptr;
   c->ws = nullptr;
   c->ws_bytes = 0;
@@ -1930,9 +1938,8 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   if (!slot.ready) {
     // once per device, with that device current: the array's name is only a host-side handle;
     // the address kernels and memsets can use comes from cudaGetSymbolAddress
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return RL_ERR_CUDA;
-    if (prop.major != 10) return RL_ERR_UNSUPPORTED_ARCH;
+    int major = 0, n_sm = 0;
+    if ((s = device_facts(device, &major, &n_sm)) != RL_OK) return s;
     unsigned char* base = nullptr;
     if (cudaGetSymbolAddress(reinterpret_cast<void**>(&base), g_static_scratch) != cudaSuccess || !base)
       return RL_ERR_CUDA;
@@ -1945,7 +1952,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
     rl_ctx& c = slot.ctx;
     memset(&c, 0, sizeof(c));
     c.device = device;
-    c.n_sm = prop.multiProcessorCount;
+    c.n_sm = n_sm;
     c.encode = reinterpret_cast<EncodeTiledFn>(fn);
     c.dstatus = reinterpret_cast<DevStatus*>(base);
     c.ws = base + kStaticHeaderBytes;
