@@ -22,7 +22,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // Forward statistics (policy over the vocabulary, section 2.2): for its row and the vocabulary
 // range of the work unit, keeps the running maximum M, S = sum exp(z-M), A = sum exp(z-M) z and
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
-struct EpiStats {
+struct RowStats {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 0;
@@ -97,11 +97,34 @@ struct EpiStats {
       st.zy = z;
     }
   }
+  // the two column halves of a row: as the merge of two vocabulary ranges
+  static constexpr int kMerge = 4;
+  __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) {
+    x[0] = st.m; x[1] = st.s; x[2] = st.a; x[3] = st.zy;
+  }
+  __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) {
+    const float m = fmaxf(st.m, x[0]);
+    // a half that saw no column inside the vocabulary has m = -inf and sums of 0
+    const float a = st.m == m ? 1.f : ex2_approx((st.m - m) * kLog2e), b = x[0] == m ? 1.f : ex2_approx((x[0] - m) * kLog2e);
+    st.s = fmaf(st.s, a, x[1] * b);
+    st.a = fmaf(st.a, a, x[2] * b);
+    st.zy += x[3];
+    st.m = m;
+  }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int m_tile, int nr, int row_in_tile,
                                                   int m_rows) {
     const int row = m_tile * BM + row_in_tile;
     if (row < m_rows) p.partials[(size_t)nr * p.part_stride + row] = make_float4(st.m, st.s, st.a, st.zy);
   }
+};
+
+// With four epilogue warps (one per scheduler) their latencies are exposed and a tile's epilogue takes 3.8 us; with
+// eight it takes 2.7, but they slow the MMA issuer down.  So eight where K is short: 8192 rows x 151936 words, score pass
+// 908 / 1072 / 1377 / 1608 / 3072 us with four, 752 / 949 / 1250 / 1668 / 3718 with eight at d = 256 / 512 / 768 / 1024 / 2048.
+constexpr int kEightWarpsMaxK = 896;
+template <int W>
+struct EpiStats : RowStats {
+  static constexpr int kWarps = W;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -123,13 +146,14 @@ __device__ __forceinline__ float code_exponent(float f) {
 
 // 32 rows x 32 columns of 16-bit values (two per word, one row per lane) into one half of a 128-byte-swizzled 32 x 64
 // box; c = index of the 32-column chunk.  The second half hands the box to the TMA unit.
+template <int BUFS>   // boxes per warp
 __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, uint32_t staging, uint32_t& n_issued,
                                                const CUtensorMap* map, int col, int row0) {
   const int lane = threadIdx.x & 31;
-  const uint32_t buf = staging + (n_issued & 1u) * 4096u;
+  const uint32_t buf = staging + (n_issued % BUFS) * kBoxBytes;
   if ((c & 1) == 0) {
-    // first half of a new box: the store issued from this buffer two boxes ago must have read it
-    if (lane == 0) bulk_wait_group_read<1>();
+    // first half of a new box: the last store issued from this buffer must have read it
+    if (lane == 0) bulk_wait_group_read<BUFS - 1>();
     __syncwarp();
   }
   // row `lane` of the box is 128 bytes = 8 chunks of 8 values; chunk j sits at position j ^ (row & 7)
@@ -156,16 +180,22 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // place the gradient with respect to the logits then takes).  Forming the logits once instead of twice (statistics,
 // then recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  At d = 2048 the extra
 // arithmetic (about 3 instructions per logit on top of the statistics' 3) still hides behind the next tile's MMAs.
+// Eight warps pay up to d = 1280 here: 1438 / 1449 / 1706 / 1946 / 2471 / 3391 us with four, 1073 / 1279 / 1560 / 1839 /
+// 2225 / 3613 with eight at d = 256 / 512 / 768 / 1024 / 1280 / 2048.
+constexpr int kEightWarpsMaxKSweep = 1280;
+struct SweepParams {
+  RowStats::Params stats;
+  const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
+};
+template <int W>
 struct EpiSweep {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
-  static constexpr int kStagingBytes = 4 * kStagingPerWarp;
-  struct Params {
-    EpiStats::Params stats;
-    const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
-  };
+  static constexpr int kWarps = W;
+  static constexpr int kStagingBytes = kEpiStaging;
+  using Params = SweepParams;
   struct State {
-    EpiStats::State s;
+    RowStats::State s;
     float k1, k2;
     uint32_t n_issued;
     int grow;   // compact row
@@ -194,7 +224,7 @@ struct EpiSweep {
                                                const CUtensorMap* map, uint32_t staging) {
     // a CTA pair may own a 128-row tile that lies wholly past the slab's rows: nothing to write
     if (m_tile * BM >= ((m_rows + BM - 1) / BM) * BM) return;
-    EpiStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
+    RowStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
     const float2 a1 = make_float2(kLog2e * kCodeSlope1, kLog2e * kCodeSlope1), b1 = make_float2(st.k1, st.k1);
     const float2 a2 = make_float2(kLog2e * kCodeSlope2, kLog2e * kCodeSlope2), b2 = make_float2(st.k2, st.k2);
     const float2 magic = make_float2(8388608.f, 8388608.f);   // low 16 bits of 2^23 + x are round(x)
@@ -207,8 +237,11 @@ struct EpiSweep {
       w[i] = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x5410);
     }
     const int lane = threadIdx.x & 31;
-    stage_half_box(w, c, staging, st.n_issued, map, n_tile * BN + c * 32, m_tile * BM + (row_in_tile - lane));
+    stage_half_box<kStagingBytes / kWarps / kBoxBytes>(w, c, staging, st.n_issued, map, n_tile * BN + c * 32, m_tile * BM + (row_in_tile - lane));
   }
+  static constexpr int kMerge = RowStats::kMerge;
+  __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) { RowStats::pack(st.s, x); }
+  __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) { RowStats::merge(st.s, x); }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int, int nr, int, int) {
     if (st.grow >= 0)
       p.stats.partials[(size_t)nr * p.stats.part_stride + st.grow] = make_float4(st.s.m, st.s.s, st.s.a, st.s.zy);
@@ -223,19 +256,25 @@ struct EpiSweep {
 //   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),  p_tj = exp(z_tj - lse_t)
 // cp_t = -w_t dloss_t/dlogp_t and ce_t = w_t ent_coef come from the per-token loss kernel.
 // Rows past the valid rows of the slab and columns past V are written as zero.
+// Eight warps as in EpiStats: 708 / 661 / 772 / 894 us with four, 484 / 588 / 727 / 903 with eight at d = 256 / 512 / 768 / 1024
+// (8192 rows x 75968 words).
+struct GradParams {
+  const int* tokens_c;
+  const float* lse;
+  const float* ent;
+  const float* cp;
+  const float* ce;
+  int V;
+  int vocab_base;  // global column of the slab's column 0
+};
+template <int W>
 struct EpiGrad {
   static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
   static constexpr bool kParts = false;
-  static constexpr int kStagingBytes = 4 * kStagingPerWarp;
-  struct Params {
-    const int* tokens_c;
-    const float* lse;
-    const float* ent;
-    const float* cp;
-    const float* ce;
-    int V;
-    int vocab_base;  // global column of the slab's column 0
-  };
+  static constexpr int kWarps = W;
+  static constexpr int kMerge = 0;
+  static constexpr int kStagingBytes = kEpiStaging;
+  using Params = GradParams;
   struct State {
     float lse, ent, cp, ce;
     int y;
@@ -317,7 +356,7 @@ struct EpiGrad {
       w[i] = *reinterpret_cast<const uint32_t*>(&b);
     }
     const int lane = threadIdx.x & 31;
-    stage_half_box(w, c, staging, st.n_issued, tmG, col_l, m_tile * BM + (row_in_tile - lane));
+    stage_half_box<kStagingBytes / kWarps / kBoxBytes>(w, c, staging, st.n_issued, tmG, col_l, m_tile * BM + (row_in_tile - lane));
   }
   __device__ static __forceinline__ void end_unit(const Params&, State&, int, int, int, int) {}
 };
@@ -332,7 +371,9 @@ struct EpiGrad {
 struct EpiAcc {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = true;
-  static constexpr int kStagingBytes = 4 * kStagingPerWarp;
+  static constexpr int kWarps = 4;
+  static constexpr int kMerge = 0;
+  static constexpr int kStagingBytes = kEpiStaging;
   struct Params {
     int n_cols;
     int accumulate;
@@ -361,9 +402,10 @@ struct EpiAcc {
     const int col0 = n_tile * BN + c * 32;
     if (row0 >= m_rows || col0 >= p.n_cols) return;        // warp-uniform
     const bool part = p.tile_cols > 0 && st.k_slice > 0;
-    const uint32_t buf = staging + (st.n_issued & 1u) * 4096u;
-    // the store issued from this buffer two chunks ago must have finished reading it
-    if (lane == 0) bulk_wait_group_read<1>();
+    constexpr int kBufs = kStagingBytes / kWarps / kBoxBytes;
+    const uint32_t buf = staging + (st.n_issued % kBufs) * kBoxBytes;
+    // the last store issued from this buffer must have finished reading it
+    if (lane == 0) bulk_wait_group_read<kBufs - 1>();
     __syncwarp();
     // row `lane` of the box: 8 chunks of 16 bytes, chunk j stored at position j ^ (row & 7)
 #pragma unroll

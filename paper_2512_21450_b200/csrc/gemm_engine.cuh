@@ -6,9 +6,10 @@
 //                 shared-memory ring, 128-byte swizzled; a ring stage holds one k-slice, or two for
 //                 the 256-column pair tiles (see StageCfg::kKSub).
 //   warp 1      : allocates tensor memory; one lane issues tcgen05.mma.
-//   warps 2..5  : epilogue - each warp owns the 32 tensor-memory lanes (tile rows) that its
-//                 rank modulo 4 may read, pulls the accumulator out in 32-column chunks and
-//                 hands them to the epilogue functor.
+//   warps 2..   : epilogue, four or eight warps (Epi::kWarps) - each warp owns the 32 tensor-memory lanes (tile rows)
+//                 that its rank modulo 4 may read, pulls its columns of the accumulator (all, or one half of
+//                 them) out in 32-column chunks and hands them to the epilogue functor.  With eight, the functor's
+//                 per-row state of the second half is merged into the first's at the end of a unit.
 //
 // Tile modes (per CTA 128 accumulator rows):
 //   kTileSquare : a tile is 256 columns wide and lives in ONE accumulator; tile t uses accumulator
@@ -54,10 +55,11 @@ constexpr int BM = 128;   // accumulator rows per CTA
 constexpr int BN = 256;   // accumulator columns
 constexpr int BK = 64;
 constexpr int kAStageBytes = BM * BK * 2;
-constexpr int kGemmThreads = 192;
+constexpr int gemm_threads(int epi_warps) { return 64 + 32 * epi_warps; }
 constexpr int kTileSmemBytes = 224 * 1024;             // operand ring + epilogue staging
-constexpr int kGemmSmemBytes = kTileSmemBytes + 1024;  // + slack for 1024-byte alignment
-constexpr int kStagingPerWarp = 8192;                  // two 32x32 fp32 boxes per epilogue warp
+constexpr int kMaxSmemBytes = 227 * 1024;              // static + dynamic shared memory of a block
+constexpr int kBoxBytes = 4096;                        // one 32 x 32 fp32 or 32 x 64 bf16 box
+constexpr int kEpiStaging = 8 * kBoxBytes;             // of an epilogue that stores boxes: two per warp, or one of eight
 constexpr int kTmemCols = 512;
 constexpr int kMaxSplit = 16;   // most column ranges per row tile unless GemmShape::n_split_max says otherwise
 constexpr int kFewRowTiles = 16;   // row tiles up to which the column split is chosen by waves (choose_split)
@@ -85,6 +87,14 @@ struct StageCfg {
   static constexpr uint32_t kTxBytes = uint32_t(kStageBytes) * CG;  // bytes counted on the issuing CTA's barrier
 };
 constexpr int kMaxStages = 7;
+
+// Dynamic shared memory of a kernel whose static part is static_bytes: ring and staging, which start on a multiple of 1024
+// behind the static part (the window itself is aligned; the kernel checks), and slack where there is room.
+template <int CG, int MODE, int kStaging>
+constexpr int gemm_smem_bytes(int static_bytes) {
+  const int need = StageCfg<CG, MODE, kStaging>::kRingBytes + kStaging + 1024;
+  return need < kMaxSmemBytes - static_bytes ? need : kMaxSmemBytes - static_bytes;
+}
 
 // Device status word shared by all kernels of a context.
 struct DevStatus {
@@ -411,13 +421,16 @@ struct UnitWalk {
   }
 };
 
-// Epilogue functor contract (all methods run in the 128 epilogue threads, one tile row each):
+// Epilogue functor contract (all methods run in the epilogue threads, one tile row each):
 //   struct Epi { struct Params; struct State;
 //     static void begin_unit(const Params&, State&, int m_tile, int n_range_idx, int row_in_tile, int m_rows, int slab_off, int k_slice);
 //     static void chunk(const Params&, State&, int m_tile, int n_tile, int chunk, int row_in_tile, int m_rows, const float (&v)[32],
 //                       const CUtensorMap* out_map, uint32_t staging);
 //     static void end_unit(const Params&, State&, int m_tile, int n_range_idx, int row_in_tile, int m_rows);
 //     static void init(State&); static void finish(State&);     // once per kernel, per thread
+//     static constexpr int kWarps;                             // epilogue warps, 4 or 8 (two per 32 rows)
+//     static constexpr int kMerge;                             // floats of state that pack() hands to the other half's
+//     static void pack(const State&, float (&)[kMerge]); static void merge(State&, const float (&)[kMerge]);   // if > 0
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
 //     static constexpr bool kTileFlags;                        // launches may be restricted by GemmShape::tile_flags
 //     static constexpr bool kParts; };                         // knows what to do with parts of tiles (stream_k == 2)
@@ -425,7 +438,7 @@ struct UnitWalk {
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
 // sh.n_tiles then counts 512-wide tiles).  tmA2 / tmB2 / k2_len are read by kTileDual only.
 template <class Epi, int A_MN, int B_MN, int CG, int MODE>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(Epi::kWarps), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
@@ -446,18 +459,30 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   __shared__ __align__(8) uint64_t bar_acc_empty[2];
   __shared__ __align__(8) uint64_t bar_drain;
   __shared__ uint32_t tmem_base_smem;
+  // state of the second column half, on its way to the warp that has the first (one producer and one consumer warp each)
+  constexpr int kHalves = Epi::kWarps / 4;
+  constexpr bool kMerges = kHalves > 1 && Epi::kMerge > 0;
+  __shared__ float merge_s[kMerges ? Epi::kMerge : 1][kMerges ? BM : 1];
+  __shared__ __align__(8) uint64_t bar_merge[2][4];   // full, empty
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  if (tiles_base + Cfg::kRingBytes + Epi::kStagingBytes > smem_u32(smem_raw) + dynamic_smem_bytes()) {
+    // cannot happen with the sizes gemm_smem_bytes() gives; every block of the launch would leave here
+    chain_wait();
+    if (threadIdx.x == 0) latch_status(status, kStatusTimeout, 7 << 28);
+    return;
+  }
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;   // position in the CTA pair
   const int worker = blockIdx.x / CG;
   const int n_workers = gridDim.x / CG;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&bar_full[s]), 1); mbar_init(smem_u32(&bar_empty[s]), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&bar_acc_full[a]), 1); mbar_init(smem_u32(&bar_acc_empty[a]), 4 * CG); }
+    for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&bar_acc_full[a]), 1); mbar_init(smem_u32(&bar_acc_empty[a]), Epi::kWarps * CG); }
+    for (int w = 0; w < 4; ++w) { mbar_init(smem_u32(&bar_merge[0][w]), 1); mbar_init(smem_u32(&bar_merge[1][w]), 1); }
     mbar_init(smem_u32(&bar_drain), 1);
     abort_flag = 0;
     fence_mbar_init();
@@ -647,8 +672,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   } else {
     // ------------------------------------------------------------- epilogue warps (both CTAs)
     const int q = warp & 3;
+    const int half = (warp - 2) >> 2;             // which part of every accumulator's columns is this warp's
+    constexpr int kChunks = BN / 32 / kHalves;    // 32-column chunks per accumulator and warp
+    uint32_t units = 0;
     const int row_in_tile = q * 32 + lane;
-    const uint32_t staging = tiles_base + Cfg::kRingBytes + q * kStagingPerWarp;   // this warp's epilogue staging
+    const uint32_t staging = tiles_base + Cfg::kRingBytes + (half * 4 + q) * (Epi::kStagingBytes / Epi::kWarps);   // this warp's epilogue staging
     typename Epi::State st;
     Epi::init(st);
     uint32_t t = 0;
@@ -677,7 +705,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           const uint32_t acc_i = a + (uint32_t)s;   // accumulator this half of the tile sits in
           const uint32_t taddr = tmem_base + acc_i * BN + (uint32_t(q * 32) << 16);
 #pragma unroll 1
-          for (int c = 0; c < BN / 32; ++c) {
+          for (int c = half * kChunks; c < (half + 1) * kChunks; ++c) {
             float v[32];
             if constexpr (MODE == kTileDual) {
               uint32_t r[32], r2[32];
@@ -713,7 +741,32 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
         }
       }
-      if (ok) Epi::end_unit(ep, st, m, nr, row_in_tile, ex.m_rows);
+      if constexpr (kMerges) {
+        // every lane waits for itself: the other warp's writes are then visible to it
+        const uint32_t full = smem_u32(&bar_merge[0][q]), empty = smem_u32(&bar_merge[1][q]);
+        float x[Epi::kMerge];
+        if (half == 1) {
+          if (ok && !mbar_wait_bounded(empty, (units & 1u) ^ 1u, abort_p)) ok = false;
+          if (ok) {
+            Epi::pack(st, x);
+#pragma unroll
+            for (int i = 0; i < Epi::kMerge; ++i) merge_s[i][row_in_tile] = x[i];
+          }
+        } else {
+          if (ok && !mbar_wait_bounded(full, units & 1u, abort_p)) ok = false;
+          if (ok) {
+#pragma unroll
+            for (int i = 0; i < Epi::kMerge; ++i) x[i] = merge_s[i][row_in_tile];
+            Epi::merge(st, x);
+          }
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        __syncwarp();   // all lanes have written (or read) before one of them says so
+        if (!ok && lane == 0) latch_status(status, kStatusTimeout, (6 << 28) | (blockIdx.x << 8) | q);
+        if (ok && lane == 0) mbar_arrive(half == 1 ? full : empty);
+        ++units;
+      }
+      if (ok && half == 0) Epi::end_unit(ep, st, m, nr, row_in_tile, ex.m_rows);
     }
     Epi::finish(st);   // e.g. wait for bulk stores that still read this warp's staging memory
   }

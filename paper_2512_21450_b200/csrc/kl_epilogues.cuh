@@ -12,9 +12,12 @@ namespace rlh {
 //   D  = sum_j exp(z_j - M) zr_j          (so that sum_j p_j (z_j - zr_j) = (A - D) / S)
 //   Mr, Sr = running max and sum exp(zr - Mr) of the reference logits (for lse_ref).
 // Two float4 per (range, row): {M, S, A, z_y} and {D, Mr, Sr, 0}.
+// Eight epilogue warps in all passes of the full KL: their epilogues are the heavy ones (d = d_ref = 256 / 512 / 704 / 2048:
+// statistics 1200 / 1474 / 1858 / 4775 us with four, 985 / 1246 / 1607 / 4395 with eight).
 struct EpiStatsKL {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
+  static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;
@@ -75,6 +78,23 @@ struct EpiStatsKL {
       st.zy = z;
     }
   }
+  static constexpr int kMerge = 7;
+  __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) {
+    x[0] = st.m; x[1] = st.s; x[2] = st.a; x[3] = st.zy; x[4] = st.dsum; x[5] = st.mr; x[6] = st.sr;
+  }
+  __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) {
+    const float m = fmaxf(st.m, x[0]), mr = fmaxf(st.mr, x[5]);
+    // a half that saw no column inside the vocabulary has maxima of -inf and sums of 0
+    const float a = st.m == m ? 1.f : ex2_approx((st.m - m) * kLog2e), b = x[0] == m ? 1.f : ex2_approx((x[0] - m) * kLog2e);
+    const float ar = st.mr == mr ? 1.f : ex2_approx((st.mr - mr) * kLog2e), br = x[5] == mr ? 1.f : ex2_approx((x[5] - mr) * kLog2e);
+    st.s = fmaf(st.s, a, x[1] * b);
+    st.a = fmaf(st.a, a, x[2] * b);
+    st.zy += x[3];
+    st.dsum = fmaf(st.dsum, a, x[4] * b);
+    st.sr = fmaf(st.sr, ar, x[6] * br);
+    st.m = m;
+    st.mr = mr;
+  }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int m_tile, int nr, int row_in_tile,
                                                   int m_rows) {
     const int row = m_tile * BM + row_in_tile;
@@ -110,6 +130,7 @@ __device__ __forceinline__ void st_global_v8(float* p, const float* v) {
 struct EpiRefSweep {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
+  static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
     float4* partials2;
@@ -119,7 +140,7 @@ struct EpiRefSweep {
     int ld;
   };
   struct State {
-    EpiStats::State s;
+    RowStats::State s;
     float* row;
     int grow;
   };
@@ -136,15 +157,18 @@ struct EpiRefSweep {
   }
   __device__ static __forceinline__ void chunk(const Params& p, State& st, int, int n_tile, int c, int, int,
                                                const float (&v)[32], const CUtensorMap* map, uint32_t staging) {
-    EpiStats::Params ps;
+    RowStats::Params ps;
     ps.V = p.V;
-    EpiStats::chunk(ps, st.s, 0, n_tile, c, 0, 0, v, map, staging);
+    RowStats::chunk(ps, st.s, 0, n_tile, c, 0, 0, v, map, staging);
     if (st.row) {
       float* q = st.row + n_tile * BN + c * 32;
 #pragma unroll
       for (int j = 0; j < 4; ++j) st_global_v8(q + 8 * j, v + 8 * j);
     }
   }
+  static constexpr int kMerge = RowStats::kMerge;
+  __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) { RowStats::pack(st.s, x); }
+  __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) { RowStats::merge(st.s, x); }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int, int nr, int, int) {
     if (st.grow >= 0) p.partials2[(size_t)nr * p.part_stride + st.grow] = make_float4(0.f, st.s.m, st.s.s, 0.f);
   }
@@ -155,9 +179,10 @@ struct EpiRefSweep {
 struct EpiSweepKL {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
+  static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
-    EpiStats::Params stats;
+    RowStats::Params stats;
     float4* partials2;
     const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
     const float* centre;   // [rows] compact: c
@@ -165,7 +190,7 @@ struct EpiSweepKL {
     int ld;                // whole tiles: columns past V are read and written as well
   };
   struct State {
-    EpiStats::State s;
+    RowStats::State s;
     float d, k1, k2, centre;
     float* row;
     int grow;
@@ -204,13 +229,15 @@ struct EpiSweepKL {
 #pragma unroll
       for (int j = 0; j < 32; ++j) zr[j] = st.next[j];
     }
-    if (col + 32 < p.ld) {
+    // this warp's next columns: four chunks in a row, then the other half's four are passed over
+    const int ahead = (c & 3) == 3 ? 32 + BN / 2 : 32;
+    if (col + ahead < p.ld) {
 #pragma unroll
-      for (int j = 0; j < 32; j += 8) ld_global_v8(q + 32, st.next, j);
+      for (int j = 0; j < 32; j += 8) ld_global_v8(q + ahead, st.next, j);
     }
     const int nvalid = p.stats.V - col;
     const float m_old = st.s.m;
-    EpiStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
+    RowStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
     if (nvalid > 0) {
       // D with the same weights as A (the sum that EpiStats keeps), rescaled as A is
       const float mL = st.s.m * kLog2e;
@@ -242,6 +269,16 @@ struct EpiSweepKL {
 #pragma unroll
     for (int j = 0; j < 4; ++j) st_global_v8(q + 8 * j, w + 8 * j);
   }
+  static constexpr int kMerge = RowStats::kMerge + 1;
+  __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) {
+    x[0] = st.s.m; x[1] = st.s.s; x[2] = st.s.a; x[3] = st.s.zy; x[4] = st.d;
+  }
+  __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) {
+    const float y[RowStats::kMerge] = {x[0], x[1], x[2], x[3]}, m = fmaxf(st.s.m, x[0]);
+    st.d = fmaf(st.d, st.s.m == m ? 1.f : ex2_approx((st.s.m - m) * kLog2e),
+                x[4] * (x[0] == m ? 1.f : ex2_approx((x[0] - m) * kLog2e)));
+    RowStats::merge(st.s, y);
+  }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int, int nr, int, int) {
     if (st.grow < 0) return;
     const size_t i = (size_t)nr * p.stats.part_stride + st.grow;
@@ -257,7 +294,9 @@ struct EpiSweepKL {
 struct EpiGradKL {
   static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
   static constexpr bool kParts = false;
-  static constexpr int kStagingBytes = 4 * kStagingPerWarp;
+  static constexpr int kWarps = 8;
+  static constexpr int kMerge = 0;
+  static constexpr int kStagingBytes = kEpiStaging;
   struct Params {
     const int* tokens_c;
     const float* lse;
@@ -326,9 +365,10 @@ struct EpiGradKL {
       }
     }
     const int lane = threadIdx.x & 31;
-    const uint32_t buf = staging + (st.n_issued & 1u) * 4096u;
+    constexpr int kBufs = kStagingBytes / kWarps / kBoxBytes;
+    const uint32_t buf = staging + (st.n_issued % kBufs) * kBoxBytes;
     if ((c & 1) == 0) {
-      if (lane == 0) bulk_wait_group_read<1>();
+      if (lane == 0) bulk_wait_group_read<kBufs - 1>();
       __syncwarp();
     }
 #pragma unroll

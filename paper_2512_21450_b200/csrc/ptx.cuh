@@ -18,6 +18,12 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+__device__ __forceinline__ uint32_t dynamic_smem_bytes() {
+  uint32_t n;
+  asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(n));
+  return n;
+}
+
 // Programmatic dependent launch.  Every kernel of this library is launched with stream serialisation relaxed: the next
 // launch may be scheduled once all blocks of this one have called chain_release(), and waits in chain_wait() until
 // everything before it has completed and is visible.  No kernel touches global memory before chain_wait(), so that

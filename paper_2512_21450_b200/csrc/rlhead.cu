@@ -99,7 +99,7 @@ inline int merge_blocks(int64_t rows, int slabs) {
 inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_slices == 1; }
 // Full-distribution KL: two single-product passes that leave 6 bytes per logit pair behind, or two-product tiles formed
 // twice.  The former trades 4 d + 4 d_ref tensor flops for 14 bytes of traffic per entry.  4096 rows, V = 151936: logits and
-// their gradient take 3.3 / 3.7 / 4.9 / 8.3 ms against 2.8 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
+// their gradient take 3.3 / 3.5 / 4.9 / 8.3 ms against 2.5 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
 constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
 inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
@@ -291,10 +291,17 @@ bool map_out_bf16(rl_ctx* c, CUtensorMap* m, const void* base, uint64_t rows, ui
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Dynamic shared memory of an instantiation: a constant of the build, known once its static size was asked for.
+template <class Epi, int A_MN, int B_MN, int CG, int MODE>
+int g_smem_bytes = 0;
 template <class Epi, int A_MN, int B_MN, int CG, int MODE>
 cudaError_t set_smem_attr_one() {
-  return cudaFuncSetAttribute(gemm_kernel<Epi, A_MN, B_MN, CG, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kGemmSmemBytes);
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, gemm_kernel<Epi, A_MN, B_MN, CG, MODE>);
+  if (e != cudaSuccess) return e;
+  const int bytes = gemm_smem_bytes<CG, MODE, Epi::kStagingBytes>((int)fa.sharedSizeBytes);
+  g_smem_bytes<Epi, A_MN, B_MN, CG, MODE> = bytes;
+  return cudaFuncSetAttribute(gemm_kernel<Epi, A_MN, B_MN, CG, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 // square tiles, single CTAs and CTA pairs
 template <class Epi, int A_MN, int B_MN>
@@ -361,8 +368,7 @@ void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUten
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(c->grid[cg]);
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = kGemmSmemBytes;
+  cfg.blockDim = dim3(gemm_threads(Epi::kWarps));
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -374,8 +380,10 @@ void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUten
   cfg.attrs = attr;
   cfg.numAttrs = cg == 2 ? 2 : 1;
   if (cg == 2) {
+    cfg.dynamicSmemBytes = g_smem_bytes<Epi, A_MN, B_MN, 2, MODE>;
     cudaLaunchKernelEx(&cfg, gemm_kernel<Epi, A_MN, B_MN, 2, MODE>, a, b, a2, b2, out, sh, k2_len, ep, c->dstatus);
   } else if constexpr (MODE != kTileWide) {
+    cfg.dynamicSmemBytes = g_smem_bytes<Epi, A_MN, B_MN, 1, MODE>;
     cudaLaunchKernelEx(&cfg, gemm_kernel<Epi, A_MN, B_MN, 1, MODE>, a, b, a2, b2, out, sh, k2_len, ep, c->dstatus);
   }
   c->launches++;
@@ -541,13 +549,14 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   sh.n_range = 0;  // split chosen on the device from the number of valid rows
   sh.n_split_max = L.part_ranges;
   sh.m_group = row_group_tiles(c, d + (kl ? kl->d_ref : 0));
-  EpiStats::Params ep;
+  RowStats::Params ep;
   ep.tokens_c = tokens_c;
   ep.partials = reinterpret_cast<float4*>(ws + L.partials);
   ep.part_stride = L.Tpad;
   ep.V = (int)V;
   if (!kl) {
-    launch_gemm<EpiStats, 0, 0>(c, cg, 0, tmA, tmB, tmA, tmA, sh, ep);   // no output map
+    if (d <= kEightWarpsMaxK) launch_gemm<EpiStats<8>, 0, 0>(c, cg, 0, tmA, tmB, tmA, tmA, sh, ep);
+    else                      launch_gemm<EpiStats<4>, 0, 0>(c, cg, 0, tmA, tmB, tmA, tmA, sh, ep);   // no output map
   } else {
     // both logit tiles per output tile
     CUtensorMap tmA2, tmB2;
@@ -629,8 +638,9 @@ rl_status rl_create(rl_ctx** out, int device) {
   // device block: status word, then two doubles for batch statistics
   if (cudaMalloc(&c->dstatus, kStatusBytes) != cudaSuccess) { delete c; return RL_ERR_CUDA; }
   cudaMemset(c->dstatus, 0, kStatusBytes);
-  bool ok = set_smem_attr<EpiStats, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad, 0, 0>() == cudaSuccess &&
-            set_smem_attr<EpiSweep, 0, 0>() == cudaSuccess && set_smem_attr<EpiRefSweep, 0, 0>() == cudaSuccess &&
+  bool ok = set_smem_attr<EpiStats<4>, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad<4>, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiStats<8>, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad<8>, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiSweep<4>, 0, 0>() == cudaSuccess && set_smem_attr<EpiSweep<8>, 0, 0>() == cudaSuccess && set_smem_attr<EpiRefSweep, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiSweepKL, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
@@ -646,8 +656,8 @@ rl_status rl_create(rl_ctx** out, int device) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(c->grid[2]);
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = kGemmSmemBytes;
+    cfg.blockDim = dim3(gemm_threads(EpiAcc::kWarps));
+    cfg.dynamicSmemBytes = g_smem_bytes<EpiAcc, 0, 0, 2, kTileSquare>;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 2;
@@ -1328,7 +1338,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             er.ld = L.Vs;
             launch_gemm<EpiRefSweep, 0, 0>(c, cg_fwd, 0, tmHr_k, tmWr_fwd, tm_G_out, tm_G_out, sr, er);
           }
-          EpiSweep::Params ep;
+          SweepParams ep;
           ep.stats.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.stats.partials = reinterpret_cast<float4*>(ws + L.partials);
           ep.stats.part_stride = L.Tpad;
@@ -1343,8 +1353,10 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             ek.slab = words;
             ek.ld = L.Vs;
             launch_gemm<EpiSweepKL, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ek);
+          } else if (d <= kEightWarpsMaxKSweep) {
+            launch_gemm<EpiSweep<8>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
           } else {
-            launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
+            launch_gemm<EpiSweep<4>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
           }
           p.fwd_shape = sw;
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
@@ -1391,11 +1403,14 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sh.flag_count = flag_count;
         }
         if (!o.kl_full) {
-          EpiGrad::Params ep;
+          GradParams ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.lse = p.lse_c; ep.ent = p.ent_c; ep.cp = p.cp_c; ep.ce = p.ce_c;
           ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_gemm<EpiGrad, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
+          if (d <= kEightWarpsMaxK)
+            launch_gemm<EpiGrad<8>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
+          else
+            launch_gemm<EpiGrad<4>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
         } else {
           EpiGradKL::Params ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
@@ -1948,7 +1963,8 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn ||
         qres != cudaDriverEntryPointSuccess)
       return RL_ERR_CUDA;
-    if (set_smem_attr<EpiStats, 0, 0>() != cudaSuccess) return RL_ERR_CUDA;
+    if (set_smem_attr<EpiStats<4>, 0, 0>() != cudaSuccess || set_smem_attr<EpiStats<8>, 0, 0>() != cudaSuccess)
+      return RL_ERR_CUDA;
     rl_ctx& c = slot.ctx;
     memset(&c, 0, sizeof(c));
     c.device = device;

@@ -125,3 +125,30 @@ def test_one_sweep_full_kl(d, d_ref, V, L_max, rows, off, ent):
             assert _rel(_np64(out["dH"]), oo["dH"]) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
     finally:
         c.close()
+
+
+# hidden sizes on both sides of the rules for eight epilogue warps (each has half of a tile's columns, merged per unit):
+# vocabularies whose second half of the only tile is empty, holds one column, or is ragged; K-major passes of every kind
+@pytest.mark.parametrize("d", [64, 896, 960, 1280, 1344])
+@pytest.mark.parametrize("V", [100, 128, 129, 700])
+def test_column_halves(d, V):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    w = make_workload(1, prompts=1, L_max=40, d=d, V=V, seed=3000 + V + d)
+    adv = torch.randn(w.T, device="cuda")
+    oo = O.policy_loss_fwd_bwd(_np64(w.H), _np64(w.W), w.tokens.cpu().numpy(), _np64(w.old_logp), _np64(w.ref_logp),
+                               _np64(adv), w.mask.cpu().numpy(), w.eps_low, w.eps_high, w.beta, ent_coef=0.01)
+    olp, oent, _ = O.token_logprobs(_np64(w.H), _np64(w.W), w.tokens.cpu().numpy(), w.mask.cpu().numpy())
+    c = Context(0)
+    try:
+        lp, ent, _ = c.rl_token_logprobs(w.H, w.W, w.tokens, w.mask)
+        assert np.abs(_np64(lp) - olp).max() <= 2e-3 and np.abs(_np64(ent) - oent).max() <= 2e-3
+        for cols in (1024, 256):          # whole rows (one sweep), and column slabs (logits formed twice) where V > 256
+            c.set_slab_limits(256, cols)
+            out = c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, w.ref_logp, adv, w.mask, w.eps_low, w.eps_high,
+                                           w.beta, ent_coef=0.01, dH_fp32=True)
+            assert c.last_device_status()[0] == 0
+            assert abs(out["loss"].item() - oo["loss"]) <= 1e-3 * abs(oo["loss"]) + 1e-6
+            assert _rel(_np64(out["dH"]), oo["dH"]) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
+    finally:
+        c.close()
