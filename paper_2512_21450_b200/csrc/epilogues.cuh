@@ -130,18 +130,25 @@ struct EpiStats : RowStats {
 // ---------------------------------------------------------------------------------------------
 // 16-bit logarithmic code of exp(z - m): what the one-sweep path keeps of a logit between the pass that forms it and the
 // point where the row's log-sum-exp and loss coefficients are known.  With t = (z - m) log2(e) and m an estimate of
-// the log-sum-exp of the row, code = round(max(1024 t + 57344, 512 t + 38912)) clamped at 0: steps of 2^-10 of an
-// octave down to t = -36 (relative error of p at most 2^-11.5, an eighth of the bf16 rounding that follows; rms of
-// the two together 0.7 % above bf16 alone), 2^-9 of an octave down to t = -76.  t reaches up to 8 before the code
-// leaves 16 bits: rows whose estimate is that far off are recomputed (kCodeTop, kCodeLow below).
-constexpr float kCodeSlope1 = 1024.f, kCodeBase1 = 57344.f, kCodeSlope2 = 512.f, kCodeBase2 = 38912.f;
+// the log-sum-exp of the row, code = round(1024 t + 57344) clamped at 0: steps of 2^-10 of an octave (relative error of p
+// at most 2^-11.5, an eighth of the bf16 rounding that follows; rms of the two together 0.7 % above bf16 alone) down to
+// t = -56, where p stays at 2^-56 (the floors of a whole vocabulary add up to less than one fp32 rounding of the row's sum).  t
+// reaches up to 8 before the code leaves 16 bits: rows whose estimate is that far off are recomputed (kCodeTop, kCodeLow
+// below).  One multiply-add puts 2^23 + code into the low bits of a float, the clamp is one maximum.
+constexpr float kCodeSlope = 1024.f, kCodeBase = 57344.f, kCodeMagic = 8388608.f;
 constexpr float kCodeTop = 7.9f;    // largest t of a row that its codes can hold
-constexpr float kCodeLow = -14.f;   // least log2 of the row's sum of exp(z - m): below, too little of the fine range is left
+constexpr float kCodeLow = -14.f;   // least log2 of the row's sum of exp(z - m): below, too little of the range is left
 
 // p's exponent t of the code in the low 16 bits of the float 2^23 + code.
 __device__ __forceinline__ float code_exponent(float f) {
-  return fminf(fmaf(f, 1.f / kCodeSlope1, -(8388608.f + kCodeBase1) / kCodeSlope1),
-               fmaf(f, 1.f / kCodeSlope2, -(8388608.f + kCodeBase2) / kCodeSlope2));
+  return fmaf(f, 1.f / kCodeSlope, -(kCodeMagic + kCodeBase) / kCodeSlope);
+}
+// The offset of the multiply-add for a row whose estimate is shift2 (in units of log 2).
+__device__ __forceinline__ float code_offset(float shift2) { return fmaf(-kCodeSlope, shift2, kCodeBase) + kCodeMagic; }
+// 2^23 + code of two logits.
+__device__ __forceinline__ float2 code_words(float2 z, float offset) {
+  const float2 x = __ffma2_rn(z, make_float2(kLog2e * kCodeSlope, kLog2e * kCodeSlope), make_float2(offset, offset));
+  return make_float2(fmaxf(x.x, kCodeMagic), fmaxf(x.y, kCodeMagic));
 }
 
 // 32 rows x 32 columns of 16-bit values (two per word, one row per lane) into one half of a 128-byte-swizzled 32 x 64
@@ -179,7 +186,7 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // Forward statistics of EpiStats for one slab of rows, plus the code of every logit written to the slab scratch (the
 // place the gradient with respect to the logits then takes).  Forming the logits once instead of twice (statistics,
 // then recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  At d = 2048 the extra
-// arithmetic (about 3 instructions per logit on top of the statistics' 3) still hides behind the next tile's MMAs.
+// arithmetic (2 instructions per logit on top of the statistics' 3.5) still hides behind the next tile's MMAs.
 // Eight warps pay up to d = 1280 here: 1438 / 1449 / 1706 / 1946 / 2471 / 3391 us with four, 1073 / 1279 / 1560 / 1839 /
 // 2225 / 3613 with eight at d = 256 / 512 / 768 / 1024 / 1280 / 2048.
 constexpr int kEightWarpsMaxKSweep = 1280;
@@ -196,7 +203,7 @@ struct EpiSweep {
   using Params = SweepParams;
   struct State {
     RowStats::State s;
-    float k1, k2;
+    float offset;
     uint32_t n_issued;
     int grow;   // compact row
   };
@@ -216,8 +223,7 @@ struct EpiSweep {
     st.s.zy = 0.f;
     st.s.y = valid ? p.stats.tokens_c[st.grow] : -1;
     const float sh = valid ? p.shift2[st.grow] : 0.f;
-    st.k1 = fmaf(-kCodeSlope1, sh, kCodeBase1);
-    st.k2 = fmaf(-kCodeSlope2, sh, kCodeBase2);
+    st.offset = code_offset(sh);
   }
   __device__ static __forceinline__ void chunk(const Params& p, State& st, int m_tile, int n_tile, int c,
                                                int row_in_tile, int m_rows, const float (&v)[32],
@@ -225,15 +231,10 @@ struct EpiSweep {
     // a CTA pair may own a 128-row tile that lies wholly past the slab's rows: nothing to write
     if (m_tile * BM >= ((m_rows + BM - 1) / BM) * BM) return;
     RowStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
-    const float2 a1 = make_float2(kLog2e * kCodeSlope1, kLog2e * kCodeSlope1), b1 = make_float2(st.k1, st.k1);
-    const float2 a2 = make_float2(kLog2e * kCodeSlope2, kLog2e * kCodeSlope2), b2 = make_float2(st.k2, st.k2);
-    const float2 magic = make_float2(8388608.f, 8388608.f);   // low 16 bits of 2^23 + x are round(x)
     uint32_t w[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const float2 z2 = make_float2(v[2 * i], v[2 * i + 1]);
-      const float2 x = __ffma2_rn(z2, a1, b1), y = __ffma2_rn(z2, a2, b2);
-      const float2 q = __fadd2_rn(make_float2(fmaxf(fmaxf(x.x, y.x), 0.f), fmaxf(fmaxf(x.y, y.y), 0.f)), magic);
+      const float2 q = code_words(make_float2(v[2 * i], v[2 * i + 1]), st.offset);
       w[i] = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x5410);
     }
     const int lane = threadIdx.x & 31;

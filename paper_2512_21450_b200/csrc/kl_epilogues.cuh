@@ -191,7 +191,7 @@ struct EpiSweepKL {
   };
   struct State {
     RowStats::State s;
-    float d, k1, k2, centre;
+    float d, offset, centre;
     float* row;
     int grow;
     bool fresh;      // nothing loaded ahead yet
@@ -210,8 +210,7 @@ struct EpiSweepKL {
     st.d = 0.f;
     st.s.y = valid ? p.stats.tokens_c[st.grow] : -1;
     const float sh = valid ? p.shift2[st.grow] : 0.f;
-    st.k1 = fmaf(-kCodeSlope1, sh, kCodeBase1);
-    st.k2 = fmaf(-kCodeSlope2, sh, kCodeBase2);
+    st.offset = code_offset(sh);
     st.centre = valid ? p.centre[st.grow] : 0.f;
     st.fresh = true;
   }
@@ -251,15 +250,12 @@ struct EpiSweepKL {
       }
       st.d = fmaf(st.d, ex2_approx((m_old - st.s.m) * kLog2e), cd2.x + cd2.y);
     }
-    const float2 a1 = make_float2(kLog2e * kCodeSlope1, kLog2e * kCodeSlope1), b1 = make_float2(st.k1, st.k1);
-    const float2 a2 = make_float2(kLog2e * kCodeSlope2, kLog2e * kCodeSlope2), b2 = make_float2(st.k2, st.k2);
-    const float2 magic = make_float2(8388608.f, 8388608.f), nc2 = make_float2(-st.centre, -st.centre);
+    const float2 nc2 = make_float2(-st.centre, -st.centre);
     float w[32];
 #pragma unroll
     for (int i = 0; i < 32; i += 2) {
       const float2 z2 = make_float2(v[i], v[i + 1]);
-      const float2 x = __ffma2_rn(z2, a1, b1), y = __ffma2_rn(z2, a2, b2);
-      const float2 f = __fadd2_rn(make_float2(fmaxf(fmaxf(x.x, y.x), 0.f), fmaxf(fmaxf(x.y, y.y), 0.f)), magic);
+      const float2 f = code_words(z2, st.offset);
       const float2 dl = __fadd2_rn(__fadd2_rn(z2, make_float2(-zr[i], -zr[i + 1])), nc2);
       const __half2 h = __floats2half2_rn(fminf(fmaxf(dl.x, -65504.f), 65504.f), fminf(fmaxf(dl.y, -65504.f), 65504.f));
       const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);

@@ -232,7 +232,8 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
     for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
     if (lane == 0) {
       const float est = z - p.sp.old_logp[t];
-      p.sp.shift2[pos] = (isfinite(est) ? est : 0.f) * kLog2e;
+      // a whole number of code steps, so that the offset the codes are formed with is exact
+      p.sp.shift2[pos] = rintf((isfinite(est) ? est : 0.f) * (kLog2e * kCodeSlope)) * (1.f / kCodeSlope);
       if (p.sp.zy) p.sp.zy[pos] = z;
     }
   } else {
