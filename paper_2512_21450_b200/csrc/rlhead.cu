@@ -79,7 +79,6 @@ constexpr size_t kSumsOffset = kCountOffset + kCountBlocks * sizeof(unsigned);
 constexpr size_t kStatusBytes = kSumsOffset + (size_t)kTokenLossBlocks * kLossSums * sizeof(double);
 constexpr int kAdvRowsMinGroups = 2048;     // from this many groups on, GRPO advantages run one thread per group
 constexpr int kWideGain = 96;              // time of a 256 x 512 tile, in % of two 256 x 256 tiles of the same K
-constexpr int kWideMinRows = 8192;         // rows of a slab (K of the dW pass) from which its tiles are 512 wide
 constexpr int kMergeBlocks = 512;          // blocks per merge launch when a call makes several (kLossThreads threads each)
 constexpr size_t kTicketOffset = 192;      // in the device block: blocks of a loss kernel that are done (0 between calls)
 constexpr int kDhSplitMax = 4;             // most K slices (separate fp32 accumulators) of the dH pass
@@ -103,7 +102,9 @@ inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_s
 constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
 inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
-// tile that is half empty costs as much as a full one.
+// tile that is half empty costs as much as a full one.  For dH, whose K is the vocabulary: 7 % of the pass (8.59 / 53.1 /
+// 58.9 ms against 9.35 / 57.3 / 63.1 at d = 2048 / 2560 / 3584).  Not for dW, whose K is a slab of rows: 256 x 256 tiles
+// take 54.5 / 62.1 / 133.6 ms against 56.3 / 63.7 / 137.0 at 10 / 8 / 14 thousand rows per slab.
 inline bool use_wide(const rl_ctx* c, int64_t d) {
   const int64_t wide = (d + 2 * BN - 1) / (2 * BN) * 2, square = (d + BN - 1) / BN;
   return c->wide_tiles && c->cta_group == 2 && wide * kWideGain <= square * 100;
@@ -1451,8 +1452,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.n_valid = n_valid;
         sh.m_rows_cap = cols - c0 < step ? cols - c0 : step;
         sh.k_cap = rows_cap; sh.k_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
-        const bool wide = use_wide(c, d) && L.Ts >= kWideMinRows;
-        sh.n_tiles = wide ? (int)((d + 2 * BN - 1) / (2 * BN)) : d_tiles;
+        sh.n_tiles = d_tiles;
         sh.n_range = 1;
         sh.skip_if_k0 = (r > 0 || o.accumulate_dW) ? 1 : 0;
         sh.a_mn_off = c0;
@@ -1461,8 +1461,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         EpiAcc::Params ep;
         ep.n_cols = (int)d; ep.accumulate = (r > 0 || o.accumulate_dW) ? 1 : 0;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
-        if (wide) launch_wide<EpiAcc, 1, 1>(c, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
-        else launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
+        launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
         // these rows of dW are complete once the last row slab has added to them
         if (report) {
           const int64_t row0 = (int64_t)vocab_base + c0;
