@@ -101,7 +101,7 @@ struct DevStatus {
   int code;    // rl_status value, 0 = ok (first error wins)
   int detail;  // where it happened
   int n_valid; // number of rows with mask != 0, written by the mask scan
-  int pad;
+  int n_ranges;   // column ranges per row of the last pass that left row statistics (GemmShape::leaves_ranges)
 };
 constexpr int kStatusTokenRange = 7;
 constexpr int kStatusTimeout = 8;
@@ -121,6 +121,7 @@ struct GemmShape {
   // With n_range == 0 and n_range_hi > 0 the range length is chosen in [n_range_lo, n_range_hi] by choose_range():
   // always (n_range_always != 0) or only when there is plenty of work (otherwise the split that fills the SMs).
   int n_range_lo, n_range_hi, n_range_always;
+  int leaves_ranges;  // the pass leaves statistics per (row, column range): note how many ranges for their merge
   int n_split_max;  // most column ranges per row tile (what the partials have room for); 0: kMaxSplit
   int skip_if_k0;   // nothing to do at all when K is empty (otherwise the epilogue sees zeros)
   int n_fastest;    // 1: consecutive units walk the column ranges of one row tile first
@@ -159,6 +160,13 @@ struct GemmShape {
   int a_mn_off, a_k_off, b_mn_off, b_k_off;
 };
 
+// a / b for a >= 0, b > 0.  The schedule below is worked out by every thread at the start of a launch, as a chain of a few
+// dozen divisions, and a 64-bit division takes several times as long as a 32-bit one; the operands nearly always fit.
+__host__ __device__ inline long long div_floor(long long a, int b) {
+  return a < (1ll << 31) ? (long long)((unsigned)a / (unsigned)b) : a / b;
+}
+__host__ __device__ inline long long div_up(long long a, int b) { return div_floor(a + b - 1, b); }
+
 // Number of vocabulary ranges each row tile is split into so that (row tiles x ranges) fills the
 // machine: minimises waves * (tiles-per-range, and 5 % of a tile for what the roles do between units).  m_units = row
 // tiles of 128*CG rows, n_workers = CTAs (CG = 1) or CTA pairs (CG = 2).  For a given number of waves the best split is
@@ -166,17 +174,19 @@ struct GemmShape {
 // d = 2560: 478 us when no more than 16 ranges (16 of 74 pairs) were allowed, 172 us with 148 on single CTAs.
 __host__ __device__ inline int choose_split(int m_units, int n_tiles, int n_workers, int smax) {
   int best = 1;
-  long best_cost = -1;
+  long long best_cost = -1;
+  if (m_units < 1) return best;
   const int w0 = (m_units + n_workers - 1) / n_workers;
   for (int waves = w0; waves < w0 + 5; ++waves) {
-    long sp = m_units > 0 ? (long)waves * n_workers / m_units : 1;
+    int sp = waves * n_workers / m_units;
     if (sp > smax) sp = smax;
     if (sp > n_tiles) sp = n_tiles;
     if (sp < 1) sp = 1;
-    const int per = (int)((n_tiles + sp - 1) / sp);
+    const int per = (n_tiles + sp - 1) / sp;
     const int ranges = (n_tiles + per - 1) / per;
-    const long cost = ((long)m_units * ranges + n_workers - 1) / n_workers * (100L * per + 5);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = (int)sp; }
+    const long long cost = div_up((long long)m_units * ranges, n_workers) * (100ll * per + 5);
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = sp; }
+    if (sp == n_tiles) break;   // more waves cannot split further
   }
   return best;
 }
@@ -188,11 +198,10 @@ __host__ __device__ inline int choose_split(int m_units, int n_tiles, int n_work
 // tiles take 8.02 / 7.86 / 7.80 / 7.90 ms.
 __host__ __device__ inline int choose_range(int m_units, int n_tiles, int n_workers, int lo, int hi) {
   int best = lo;
-  long best_cost = -1;
+  long long best_cost = -1;
   for (int nr = lo; nr <= hi; ++nr) {
-    const long ranges = (n_tiles + nr - 1) / nr;
-    const long waves = ((long)m_units * ranges + n_workers - 1) / n_workers;
-    const long cost = waves * (100 * nr + 5);
+    const int ranges = (n_tiles + nr - 1) / nr;
+    const long long cost = div_up((long long)m_units * ranges, n_workers) * (100 * nr + 5);
     if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = nr; }
   }
   return best;
@@ -241,7 +250,7 @@ __host__ __device__ inline void cut_tiles(GemmExtents& e, int n_workers) {
   if (S > e.k_blocks / kMinShare) S = e.k_blocks / kMinShare;
   if (S < 1) return;
   const int len = e.k_blocks / S;   // shortest range
-  const int fair = (int)(((long long)R * e.k_blocks + n_workers - 1) / n_workers);
+  const int fair = (int)div_up((long long)R * e.k_blocks, n_workers);
   e.cut_len = S == n_workers / R && R * S < n_workers && S <= kHelpSplit && len - fair >= kMinShare ? fair : 0;
   if (S == 1 && e.cut_len == 0) return;
   e.cut = R;
@@ -249,7 +258,7 @@ __host__ __device__ inline void cut_tiles(GemmExtents& e, int n_workers) {
 }
 // First k-block of range s of a cut tile, and the position of the end of part s in the list of its tile's ends.
 __host__ __device__ inline int cut_begin(const GemmExtents& e, int s) {
-  return (int)((long long)e.k_blocks * s / e.cut_parts);
+  return (int)div_floor((long long)e.k_blocks * s, e.cut_parts);
 }
 __host__ __device__ inline int cut_end_pos(const GemmExtents& e, int s) { return cut_begin(e, s) - s * e.cut_len; }
 // k-blocks in all ends of one tile, and in those of all tiles.
@@ -259,7 +268,8 @@ __host__ __device__ inline int cut_tile_ends(const GemmExtents& e) { return e.k_
 // Helper that does block `pos` of the list of all ends.
 __host__ __device__ inline int cut_helper(const GemmExtents& e, int n_workers, long long pos) {
   const long long total = (long long)e.cut * cut_tile_ends(e);
-  return (int)(((pos + 1) * (n_workers - e.cut * e.cut_parts) - 1) / total);
+  const long long x = (pos + 1) * (n_workers - e.cut * e.cut_parts) - 1;
+  return (int)(total < (1ll << 31) ? div_floor(x, (int)total) : x / total);
 }
 
 // cg = CTAs per output row tile, n_workers = gridDim.x / cg.
@@ -363,8 +373,8 @@ struct UnitWalk {
         it_end = 1;
       } else if (ex.cut_len > 0) {
         const long long total = (long long)ex.cut * cut_tile_ends(ex);
-        it = total * (worker - mains) / helpers;
-        it_end = total * (worker - mains + 1) / helpers;
+        it = div_floor(total * (worker - mains), helpers);
+        it_end = div_floor(total * (worker - mains + 1), helpers);
       }
     } else if (ex.stream_k) {
       plain_units = (ex.n_units / n_workers - 1) * n_workers;
@@ -405,7 +415,7 @@ struct UnitWalk {
       it = it_end;
     } else {
       const int ends = cut_tile_ends(ex);
-      r = (int)(it / ends);
+      r = (int)div_floor(it, ends);
       const int pos = (int)(it - (long long)r * ends);
       for (s = 0; s + 1 < S && cut_end_pos(ex, s + 1) <= pos; ++s) {}
       kb0 = cut_begin(ex, s) + ex.cut_len + pos - cut_end_pos(ex, s);
@@ -505,6 +515,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   // parts of cut tiles go to slots, seen through the second map of operand A (one-product passes only)
   const CUtensorMap* part_map = MODE == kTileDual ? &tmC : &tmA2;
   const GemmExtents ex = gemm_extents(sh, sh.n_valid ? *sh.n_valid : 0, CG, n_workers);
+  if (sh.leaves_ranges && blockIdx.x == 0 && threadIdx.x == 0) status->n_ranges = ex.n_ranges;
   const int k2_blocks = MODE == kTileDual ? (k2_len + BK - 1) / BK : 0;
   // the two-product mode has nothing to do unless both products have a K range
   const bool run = MODE != kTileDual || (ex.k_blocks > 0 && k2_blocks > 0);

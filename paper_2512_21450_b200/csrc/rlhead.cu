@@ -325,7 +325,6 @@ inline uint32_t b_box_panels(const rl_ctx* c) { return BN / 64 / c->cta_group; }
 // CTAs per row tile of the passes that form logits: a pair would spend half its tensor work on padding when at most 128
 // rows exist, and with so few rows the pass is a stream of W.
 inline int fwd_cta_group(const rl_ctx* c, const WsLayout& L) { return L.Tpad <= BM ? 1 : c->cta_group; }
-inline int fwd_workers(const rl_ctx* c, const WsLayout& L) { const int cg = fwd_cta_group(c, L); return c->grid[cg] / cg; }
 
 // Optional timing of a group of launches: event pair on the context's stream, tagged with a kind.
 int prof_begin(rl_ctx* c, int kind) {
@@ -480,7 +479,7 @@ struct FwdPlan {
 // Mask scan + row compaction + forward statistics.  Leaves per-range partials in the workspace.
 rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, const void* W, int64_t ldW,
                       const int32_t* tokens, const uint8_t* mask, int64_t T, int64_t d, int64_t V,
-                      GemmShape* shape_out, const KlRef* kl = nullptr, const FwdPlan& plan = FwdPlan()) {
+                      const KlRef* kl = nullptr, const FwdPlan& plan = FwdPlan()) {
   char* ws = static_cast<char*>(c->ws);
   int* row_map = reinterpret_cast<int*>(ws + L.row_map);
   int* tokens_c = reinterpret_cast<int*>(ws + L.tokens_c);
@@ -511,7 +510,8 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   pp.out = plan.out;
   if (T <= kPrepRows) {
     const int pr = prof_begin(c, 5);
-    int rows = (int)align_up((size_t)(T + c->n_sm * 4 - 1) / (c->n_sm * 4), 16);   // at most 256: kPrepRows / (4 n_sm)
+    // a row per warp while that takes no more than four blocks per SM; at most 256: kPrepRows / (4 n_sm)
+    int rows = (int)align_up((size_t)(T + c->n_sm * 4 - 1) / (c->n_sm * 4), 8);
     if (rows > 256) rows = 256;
     pp.rows_per_block = rows;
     launch(c, prep_rows_kernel<true>, (int)((T + rows - 1) / rows), 256, pp, c->dstatus);
@@ -533,7 +533,6 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     c->launches++;
   }
   if (!plan.stats) {
-    memset(shape_out, 0, sizeof(*shape_out));
     return cuda_ok();
   }
   const int cg = kl ? c->cta_group : fwd_cta_group(c, L);
@@ -549,6 +548,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   sh.n_tiles = (int)((V + BN - 1) / BN);
   sh.n_range = 0;  // split chosen on the device from the number of valid rows
   sh.n_split_max = L.part_ranges;
+  sh.leaves_ranges = 1;
   sh.m_group = row_group_tiles(c, d + (kl ? kl->d_ref : 0));
   RowStats::Params ep;
   ep.tokens_c = tokens_c;
@@ -572,7 +572,6 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     ek.V = (int)V;
     launch_dual<EpiStatsKL>(c, 0, tmA, tmB, tmA2, tmB2, tmA, sh, (int)kl->d_ref, ek);
   }
-  *shape_out = sh;
   return cuda_ok();
 }
 
@@ -1051,17 +1050,13 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   const WsLayout L = ws_layout(c, T, d, V, false);
   if ((s = check_ws(c, L)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
-  GemmShape fwd_shape;
   FwdPlan plan;
   plan.out.value[0] = logp; plan.out.value[1] = entropy; plan.out.value[2] = lse;
-  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape, nullptr, plan)) != RL_OK) return s;
+  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, nullptr, plan)) != RL_OK) return s;
   LossParams p;
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
-  p.fwd_shape = fwd_shape;
-  p.fwd_cg = fwd_cta_group(c, L);
-  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.with_loss = 0;
   p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);
@@ -1140,7 +1135,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int Vpad = (int)align_up((size_t)V, 256);
   const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.words) &&
                      (L.n_row_slabs == 1 || (L.Tc % kFlagRows == 0 && !seq_path));
-  GemmShape fwd_shape;
   FwdPlan plan;
   plan.out.dH = dH;
   plan.out.dH_row_bytes = (long long)d * (o.dH_dtype ? 4 : 2);
@@ -1156,7 +1150,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     plan.vocab_off = shard->vocab_off;
     plan.V_total = shard->V_total;
   }
-  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape, o.kl_full ? &klref : nullptr, plan)) !=
+  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, o.kl_full ? &klref : nullptr, plan)) !=
       RL_OK)
     return s;
 
@@ -1165,9 +1159,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
-  p.fwd_shape = fwd_shape;
-  p.fwd_cg = fwd_cta_group(c, L);
-  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.old_logp = old_logp;
   p.ref_logp = ref_logp;
@@ -1193,10 +1184,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   }
   if (o.kl_full) {
     p.kl_full = 1;
-    if (!sweep) {   // two-product tiles
-      p.fwd_cg = c->cta_group;
-      p.fwd_workers = c->grid[c->cta_group] / c->cta_group;
-    }
     p.partials2 = reinterpret_cast<const float4*>(ws + L.partials2);
     p.lse_ref_c = reinterpret_cast<float*>(ws + L.lse_ref_c);
     p.kl_c = reinterpret_cast<float*>(ws + L.kl_c);
@@ -1323,6 +1310,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sw.k_cap = (int)d;
           sw.n_tiles = (cols + BN - 1) / BN;
           sw.n_split_max = L.part_ranges;
+          sw.leaves_ranges = 1;
           sw.a_mn_slab = 1;
           sw.m_group = row_group_tiles(c, d);
           const float* centre = reinterpret_cast<const float*>(ws + L.centre);
@@ -1359,7 +1347,6 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           } else {
             launch_gemm<EpiSweep<4>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
           }
-          p.fwd_shape = sw;
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;
           p.shift2 = ep.shift2;
@@ -1526,20 +1513,16 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   const WsLayout L = ws_layout(c, T, d, V_shard, false);
   if ((s = check_ws(c, L)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
-  GemmShape fwd_shape;
   FwdPlan plan;
   plan.vocab_off = vocab_offset;
   plan.V_total = V_total;
   plan.out.stats = reinterpret_cast<float4*>(stats);
-  if ((s = run_forward(c, L, H, ldH, W_shard, ldW, tokens, mask, T, d, V_shard, &fwd_shape, nullptr, plan)) != RL_OK)
+  if ((s = run_forward(c, L, H, ldH, W_shard, ldW, tokens, mask, T, d, V_shard, nullptr, plan)) != RL_OK)
     return s;
   LossParams p;
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
-  p.fwd_shape = fwd_shape;
-  p.fwd_cg = fwd_cta_group(c, L);
-  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.stats_out = reinterpret_cast<float4*>(stats);
   const int blocks = merge_blocks(T, 1);
@@ -1585,19 +1568,15 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
   if (s != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
   for (int i = 0; i < n_models; ++i) {
-    GemmShape fwd_shape;
     FwdPlan plan;
     plan.out.value[0] = logp[i]; plan.out.value[1] = entropy ? entropy[i] : nullptr;
     plan.scan = i == 0;   // the mask is scanned once; every model reuses the row map
-    if ((s = run_forward(c, L, H[i], ldH[i], W[i], ldW[i], tokens, mask, T, d[i], V, &fwd_shape, nullptr, plan)) != RL_OK)
+    if ((s = run_forward(c, L, H[i], ldH[i], W[i], ldW[i], tokens, mask, T, d[i], V, nullptr, plan)) != RL_OK)
       return s;
     LossParams p;
     memset(&p, 0, sizeof(p));
     p.partials = reinterpret_cast<const float4*>(ws + L.partials);
     p.part_stride = L.Tpad;
-    p.fwd_shape = fwd_shape;
-    p.fwd_cg = fwd_cta_group(c, L);
-    p.fwd_workers = fwd_workers(c, L);
     p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
     p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);
     p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
@@ -1996,17 +1975,13 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   char* ws = static_cast<char*>(c->ws);
   // the array keeps the previous call's contents: the status word and the valid-row count start at zero
   if (cudaMemsetAsync(c->dstatus, 0, sizeof(DevStatus), c->stream) != cudaSuccess) return RL_ERR_CUDA;
-  GemmShape fwd_shape;
   FwdPlan plan;
   plan.out.value[0] = logp; plan.out.value[1] = entropy; plan.out.value[2] = lse;
-  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, &fwd_shape, nullptr, plan)) != RL_OK) return s;
+  if ((s = run_forward(c, L, H, ldH, W, ldW, tokens, mask, T, d, V, nullptr, plan)) != RL_OK) return s;
   LossParams p;
   memset(&p, 0, sizeof(p));
   p.partials = reinterpret_cast<const float4*>(ws + L.partials);
   p.part_stride = L.Tpad;
-  p.fwd_shape = fwd_shape;
-  p.fwd_cg = fwd_cta_group(c, L);
-  p.fwd_workers = fwd_workers(c, L);
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.with_loss = 0;
   p.lse_c = reinterpret_cast<float*>(ws + L.lse_c);

@@ -187,7 +187,7 @@ struct PrepParams {
   int d;
   const uint8_t* mask;
   int T;
-  int rows_per_block;     // scanning variant: multiple of 16, at most 256
+  int rows_per_block;     // scanning variant: at most 256
   const int* tokens;
   int V, vocab_off;
   __nv_bfloat16* Hc;
@@ -217,7 +217,7 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
   if (p.sp.shift2) {
     const uint4* wrow = reinterpret_cast<const uint4*>(p.sp.W + (size_t)(in_range ? y : 0) * p.sp.ldW);
     float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 4
+#pragma unroll 8
     for (int v = lane; v < vec_per_row; v += 32) {
       const uint4 h = __ldg(src + v), w = __ldg(wrow + v);
       dst[v] = h;
@@ -237,7 +237,7 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
       if (p.sp.zy) p.sp.zy[pos] = z;
     }
   } else {
-#pragma unroll 4
+#pragma unroll 8
     for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
   }
   if (lane == 0) {
@@ -264,9 +264,10 @@ __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevS
     __syncthreads();
     int c = 0, a = 0;
     for (int g = threadIdx.x; g * 16 < p.T; g += blockDim.x) {
-      const int k = __popc(scan_load_bits(p.mask, (long long)g * 16, p.T));
-      a += k;
-      c += g * 16 < r0 ? k : 0;
+      const unsigned bits = scan_load_bits(p.mask, (long long)g * 16, p.T);
+      const int before = r0 - g * 16;   // rows of this group that lie before the block's
+      a += __popc(bits);
+      c += before >= 16 ? __popc(bits) : (before > 0 ? __popc(bits & ((1u << before) - 1u)) : 0);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -577,6 +578,12 @@ __global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restr
         const long long t_in = t0 < first ? first : t0;
         if (s < 0) {
           int lo = 0, hi = n_seq;         // seq_offsets[lo] <= t_in < seq_offsets[hi]
+          // responses padded to one length: the first guess is right, and ten dependent loads are saved
+          const int guess = (int)((float)(t_in - first) / (float)(last - first) * (float)n_seq);
+          if (guess < n_seq) {
+            const int o0 = seq_offsets[guess], o1 = seq_offsets[guess + 1];
+            if (o0 <= t_in && t_in < o1) { lo = guess; hi = guess + 1; }
+          }
           while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (seq_offsets[mid] <= t_in) lo = mid; else hi = mid;
@@ -760,9 +767,6 @@ struct LossParams {
   // inputs
   const float4* partials;
   int part_stride;
-  GemmShape fwd_shape;  // shape of the forward pass: together with its grid it fixes the vocabulary split
-  int fwd_cg;           // CTAs per row tile of the forward pass
-  int fwd_workers;      // grid of the forward pass / fwd_cg
   const int* row_map;
   const float* old_logp;   // [T] original rows; NULL in log-prob-only mode
   const float* ref_logp;   // [T] or NULL
@@ -864,14 +868,14 @@ __device__ __forceinline__ void finish_loss(const double (&acc)[kLossSums], cons
 }
 
 // A block takes 32 rows at a time, lane = row; its eight warps share the column ranges (with one thread per row a call of
-// a few hundred rows and 75 to 148 ranges was a chain of that many loads: 17 us) and warp 0 goes on with the sums.
+// a few hundred rows and 75 to 148 ranges was a chain of that many loads: 17 us) and warp 0 goes on with the sums.  What
+// the loss needs besides is loaded before the merge, one round trip instead of three.
 __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossParams p, DevStatus* st) {
   chain_begin();
   constexpr int kW = kLossThreads / 32;
-  __shared__ float max_s[2][kW][32];
-  __shared__ float sum_s[5][kW][32];
+  __shared__ float part_s[2][7][kW][32];
   const int n = st->n_valid;
-  const int n_ranges = p.ext_lse ? 0 : gemm_extents(p.fwd_shape, n, p.fwd_cg, p.fwd_workers).n_ranges;
+  const int n_ranges = p.ext_lse ? 0 : st->n_ranges;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[kLossSums];
 #pragma unroll
@@ -883,14 +887,26 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     slab_extent(n, p.slab_cap, p.slab_one, p.slab_index, i_begin, i_end);
     i_end += i_begin;
   }
-  for (int i0 = i_begin + blockIdx.x * 32; i0 < i_end; i0 += gridDim.x * 32) {
+  int turn = 0;
+  for (int i0 = i_begin + blockIdx.x * 32; i0 < i_end; i0 += gridDim.x * 32, turn ^= 1) {
     const int i = i0 + lane;
     const bool in = i < i_end;
     float lse, logp, ent, kl = 0.f;
-    float M = -CUDART_INF_F, S = 0.f, A = 0.f, Mr = -CUDART_INF_F, D = 0.f, Sr = 0.f;
+    float M = -CUDART_INF_F, S = 0.f, A = 0.f, zy = 0.f, Mr = -CUDART_INF_F, D = 0.f, Sr = 0.f;
+    int row = 0;
+    float A_t = 0.f, old_lp = 0.f, ref_lp = 0.f, tw = 0.f, shift2 = 0.f;
+    if (warp == 0 && in) {
+      row = p.row_map[i];
+      if (p.shift2) shift2 = p.shift2[i];
+      if (p.with_loss) {
+        A_t = p.adv[row];
+        old_lp = p.old_logp[row];
+        if (p.token_weight) tw = p.token_weight[row];
+        if (p.beta != 0.f && !p.kl_full) ref_lp = p.ref_logp[row];
+      }
+    }
     if (p.ext_lse) {
       if (warp != 0 || !in) continue;
-      const int row = p.row_map[i];
       lse = p.ext_lse[row];
       logp = p.ext_logp[row];
       ent = p.ext_ent[row];
@@ -898,51 +914,57 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       const float4* q1 = p.partials + (in ? i : i_begin);
       const float4* q2 = p.partials2 + (in ? i : i_begin);
 #pragma unroll 4
-      for (int r = warp; r < n_ranges; r += kW) M = fmaxf(M, q1[(size_t)r * p.part_stride].x);
-      max_s[0][warp][lane] = M;
-      if (p.kl_full) {
-#pragma unroll 4
-        for (int r = warp; r < n_ranges; r += kW) Mr = fmaxf(Mr, q2[(size_t)r * p.part_stride].y);
-        max_s[1][warp][lane] = Mr;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int w = 0; w < kW; ++w) {
-        M = fmaxf(M, max_s[0][w][lane]);
-        if (p.kl_full) Mr = fmaxf(Mr, max_s[1][w][lane]);
-      }
-      float zy = 0.f;
-#pragma unroll 4
       for (int r = warp; r < n_ranges; r += kW) {
         const float4 q = q1[(size_t)r * p.part_stride];
-        const float sc = exp2f((q.x - M) * kLog2e);
-        S = fmaf(q.y, sc, S);
-        A = fmaf(q.z, sc, A);
+        const float m = fmaxf(M, q.x), a = exp2f((M - m) * kLog2e), b = exp2f((q.x - m) * kLog2e);
+        S = fmaf(S, a, q.y * b);
+        A = fmaf(A, a, q.z * b);
         zy += q.w;
         if (p.kl_full) {
           const float4 k = q2[(size_t)r * p.part_stride];
-          D = fmaf(k.x, sc, D);
-          Sr = fmaf(k.z, exp2f((k.y - Mr) * kLog2e), Sr);
+          const float mr = fmaxf(Mr, k.y);
+          D = fmaf(D, a, k.x * b);
+          Sr = fmaf(Sr, exp2f((Mr - mr) * kLog2e), k.z * exp2f((k.y - mr) * kLog2e));
+          Mr = mr;
         }
+        M = m;
       }
-      sum_s[0][warp][lane] = S;
-      sum_s[1][warp][lane] = A;
-      sum_s[2][warp][lane] = zy;
-      sum_s[3][warp][lane] = D;
-      sum_s[4][warp][lane] = Sr;
+      float (*ps)[kW][32] = part_s[turn];   // the other buffer may still be read by warp 0
+      ps[0][warp][lane] = M;
+      ps[1][warp][lane] = S;
+      ps[2][warp][lane] = A;
+      ps[3][warp][lane] = zy;
+      if (p.kl_full) {
+        ps[4][warp][lane] = D;
+        ps[5][warp][lane] = Mr;
+        ps[6][warp][lane] = Sr;
+      }
       __syncthreads();
       if (warp != 0) continue;
+      float Mt = M, Mrt = Mr;
 #pragma unroll
       for (int w = 1; w < kW; ++w) {
-        S += sum_s[0][w][lane];
-        A += sum_s[1][w][lane];
-        zy += sum_s[2][w][lane];
-        D += sum_s[3][w][lane];
-        Sr += sum_s[4][w][lane];
+        Mt = fmaxf(Mt, ps[0][w][lane]);
+        if (p.kl_full) Mrt = fmaxf(Mrt, ps[5][w][lane]);
       }
+      S = A = zy = D = Sr = 0.f;
+#pragma unroll
+      for (int w = 0; w < kW; ++w) {
+        const float m = ps[0][w][lane], b = m == -CUDART_INF_F ? 0.f : exp2f((m - Mt) * kLog2e);   // -inf: no range
+        S = fmaf(ps[1][w][lane], b, S);
+        A = fmaf(ps[2][w][lane], b, A);
+        zy += ps[3][w][lane];
+        if (p.kl_full) {
+          const float mr = ps[5][w][lane];
+          D = fmaf(ps[4][w][lane], b, D);
+          Sr = fmaf(ps[6][w][lane], mr == -CUDART_INF_F ? 0.f : exp2f((mr - Mrt) * kLog2e), Sr);
+        }
+      }
+      M = Mt;
+      Mr = Mrt;
       if (!in) continue;
       if (p.stats_out) {
-        p.stats_out[p.row_map[i]] = make_float4(M, S, A, zy);
+        p.stats_out[row] = make_float4(M, S, A, zy);
         continue;
       }
       lse = M + logf(S);
@@ -956,14 +978,12 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       p.kl_c[i] = kl;
     }
     if (p.shift2) {
-      const float shift2 = p.shift2[i];
       // (the comparison is written so that a NaN counts as too far)
       if (!(fmaf(M, kLog2e, -shift2) <= kCodeTop && fmaf(lse, kLog2e, -shift2) >= kCodeLow)) {
         p.tile_flags[i / kFlagRows] = 1;
         *p.flag_count = 1;
       }
     }
-    const int row = p.row_map[i];
     if (p.kl_out) p.kl_out[row] = kl;
     p.lse_c[i] = lse;
     p.ent_c[i] = ent;
@@ -973,9 +993,8 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     if (p.lse_out) p.lse_out[row] = lse;
     if (p.zero_coef) p.cp_c[i] = p.ce_c[i] = 0.f;
     if (p.with_loss) {
-      const float w = p.token_weight ? p.token_weight[row] : w_mean;
-      const float A_t = p.adv[row];
-      const float rho = expf(logp - p.old_logp[row]);
+      const float w = p.token_weight ? tw : w_mean;
+      const float rho = expf(logp - old_lp);
       const float clipped = fminf(fmaxf(rho, 1.f - p.eps_low), 1.f + p.eps_high);
       const float su = rho * A_t, sc = clipped * A_t;
       const bool active = su <= sc;          // unclipped branch is the minimum (ties: unclipped)
@@ -985,7 +1004,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
         k3 = kl;                              // its gradient is applied per vocabulary entry (cb)
         p.cb_c[i] = w * p.beta;
       } else if (p.beta != 0.f) {
-        const float delta = p.ref_logp[row] - logp;
+        const float delta = ref_lp - logp;
         const float ed = expf(delta);
         k3 = ed - delta - 1.f;
         dk3 = 1.f - ed;
