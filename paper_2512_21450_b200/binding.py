@@ -176,6 +176,7 @@ class Context:
         self._ws = None
         self._ws_key = None
         self._slot_busy = [False, False]
+        self._stream = None
 
     def close(self):
         if self.handle:
@@ -189,9 +190,12 @@ class Context:
             pass
 
     def _bind_stream(self):
-        # the raw handle of torch's current stream, without building a Stream object for every call
-        _check(self.lib.rl_set_stream(self.handle, torch._C._cuda_getCurrentRawStream(self.device.index)),
-               "rl_set_stream")
+        # the raw handle of torch's current stream, without building a Stream object for every call; the context keeps the
+        # one it was given last
+        stream = torch._C._cuda_getCurrentRawStream(self.device.index)
+        if stream != self._stream:
+            _check(self.lib.rl_set_stream(self.handle, stream), "rl_set_stream")
+            self._stream = stream
 
     def workspace_bytes(self, T, d, V, host=False, d_ref=0):
         n = c_size_t()
@@ -386,14 +390,11 @@ class Context:
             assert x is None or (x.dtype == torch.float32 and x.is_contiguous() and x.numel() == T)
         assert mask is None or (mask.dtype == torch.uint8 and mask.numel() == T)
         assert token_count is None or token_count.dtype == torch.int64
-        dev = logp.device
         out = dict(out or {})
-        out.setdefault("loss", torch.empty(1, dtype=torch.float32, device=dev))
-        if want_grads:
-            out.setdefault("dlogp", torch.empty(T, dtype=torch.float32, device=dev))
-            out.setdefault("dentropy", torch.empty(T, dtype=torch.float32, device=dev))
-        if want_metrics:
-            out.setdefault("metrics", torch.empty(8, dtype=torch.float32, device=dev))
+        for key, n in (("loss", 1),) + ((("dlogp", T), ("dentropy", T)) if want_grads else ()) + \
+                ((("metrics", 8),) if want_metrics else ()):
+            if key not in out:
+                out[key] = logp.new_empty(n)
         _check(self.lib.rl_token_loss(self.handle, _ptr(logp), _ptr(entropy), _ptr(old_logp), _ptr(ref_logp), _ptr(adv),
                                       _ptr(mask), T, eps_low, eps_high, beta, ent_coef, _ptr(token_weight),
                                       _ptr(token_count), _ptr(out["loss"]), _ptr(out.get("dlogp")),
