@@ -23,7 +23,7 @@ if ROOT not in sys.path:
 
 METRIC = "fused LM-head logprob+GRPO loss fwd+bwd tokens/s; % of bf16 tensor peak"
 KIND_NAMES = ["gemm_kernel<EpiSweep,square> (logits: statistics and codes)", "logit_grad_kernel (codes -> dlogits, HBM bound)",
-              "gemm_kernel<EpiAcc,K,MN,wide> (dH)", "gemm_kernel<EpiAcc,MN,MN,wide> (dW)"]
+              "gemm_kernel<EpiAcc,K,MN,wide> (dH)", "gemm_kernel<EpiAcc,MN,MN,square> (dW)"]
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the tensor-core kernels from one ncu capture
 # of a whole config-1 step (profiles/gemm_kernel_dram_config1.md; these three metrics take one pass), valid only
