@@ -1,5 +1,5 @@
-// Epilogue functors of the GEMM engine.  Each of the 128 epilogue threads owns one row of the
-// 128x256 accumulator tile and receives it in chunks of 32 consecutive columns.
+// Epilogue functors of the GEMM engine.  An epilogue thread owns one row of the 128x256 accumulator
+// tile (with eight warps: one row of one half of its columns) and receives it in chunks of 32 columns.
 #pragma once
 #include <math_constants.h>
 

@@ -14,12 +14,12 @@
 // Tile modes (per CTA 128 accumulator rows):
 //   kTileSquare : a tile is 256 columns wide and lives in ONE accumulator; tile t uses accumulator
 //                 t & 1, so the MMAs of tile t + 1 overlap the epilogue of tile t.  Used where K is
-//                 short and the epilogue heavy (forward statistics, gradient of the logits).
+//                 short and the epilogue heavy (logit passes) and for dW = G^T H, whose K is a slab of rows.
 //   kTileWide   : a tile is 512 columns wide and fills BOTH accumulators; a stage holds A and two B
 //                 boxes, every k-slice of A feeds two UMMAs, so a CTA pulls a quarter fewer operand
 //                 bytes from L2 per flop; the epilogue of a tile no longer overlaps the next main
-//                 loop (about 1 % of a tile at K of 17-19 thousand).  CTA pairs only.  Used for the
-//                 two long-K gradient products dH = G W and dW = G^T H.
+//                 loop (about 1 % of a tile at K of 17-19 thousand).  CTA pairs only.  Used for
+//                 dH = G W, whose K is the whole vocabulary.
 //   kTileDual   : a tile is 256 columns wide and BOTH accumulators hold it, one per product:
 //                 Z = A B^T (K = k_len) and Z2 = A2 B2^T (K = k2_len) of the same rows and columns,
 //                 whose 32-column chunks reach the epilogue side by side.  Used for the

@@ -20,7 +20,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 constexpr int kProfMax = 1 << 16;   // timed launch groups kept between two rl_profile_read calls
-constexpr int kProfKinds = 9;    // 0 forward statistics, 1 dlogits, 2 dH, 3 dW, 4 mask scan, 5 row gather,
+constexpr int kProfKinds = 9;    // 0 logits, 1 dlogits, 2 dH, 3 dW, 4 mask scan, 5 row preparation,
                                  // 6 merge + loss, 7 dH scatter, 8 advantages
 
 struct rl_ctx {
