@@ -64,6 +64,7 @@ constexpr int kTmemCols = 512;
 constexpr int kMaxSplit = 16;   // most column ranges per row tile unless GemmShape::n_split_max says otherwise
 constexpr int kFewRowTiles = 16;   // row tiles up to which the column split is chosen by waves (choose_split)
 constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
+constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
 constexpr int kFlagRows = 256;  // rows one entry of GemmShape::tile_flags stands for
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
@@ -242,7 +243,11 @@ __host__ __device__ inline void slab_extent(int n_valid, int cap, int one, int i
 // operand panels through L2 (one contiguous run of (tile, k) per worker, the usual stream-K, lost that: 640 rows against
 // 152 K words at d = 2048 took 405 us, bound by 2.8 GB of DRAM reads).  When n - R S workers would be left idle and S is
 // small enough for that to matter, each part stops after cut_len k-blocks and the ends of the parts, in order of
-// (tile, range), are shared equally among the remaining workers.  A wave that is nearly full is left alone.
+// (tile, range), are shared equally among the remaining workers.  An end costs its helper kPartCost k-blocks beyond its
+// length (128 or 256 KB of fp32 per CTA: 10 us), so cut_len is what makes parts and helpers end together with that counted, and two
+// helpers of 72 parts get nothing.  Without the cost / with 8 / 20 / 32 blocks, dH against 152 K words: 679 / 326 / 320 / 318 us for
+// 600 rows at d = 2048, 1014 / 809 / 654 / 662 for 1536; 311 / 168 / 166 / 157 for 100 rows at d = 2560; 540 / 442 / 390 / 389 for
+// 400 rows at d = 3584; 444 / 346 / 294 / 293 for 1280 rows at d = 896; no size slower.  A wave that is nearly full is left alone.
 __host__ __device__ inline void cut_tiles(GemmExtents& e, int n_workers) {
   const int R = e.n_units % n_workers, waves = e.n_units / n_workers + 1;
   if (R == 0 || e.k_blocks == 0 || (n_workers - R) * 20 < n_workers * waves) return;
@@ -250,7 +255,7 @@ __host__ __device__ inline void cut_tiles(GemmExtents& e, int n_workers) {
   if (S > e.k_blocks / kMinShare) S = e.k_blocks / kMinShare;
   if (S < 1) return;
   const int len = e.k_blocks / S;   // shortest range
-  const int fair = (int)div_up((long long)R * e.k_blocks, n_workers);
+  const int fair = (int)div_up((long long)R * e.k_blocks + (long long)R * S * kPartCost, n_workers);
   e.cut_len = S == n_workers / R && R * S < n_workers && S <= kHelpSplit && len - fair >= kMinShare ? fair : 0;
   if (S == 1 && e.cut_len == 0) return;
   e.cut = R;

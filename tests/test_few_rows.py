@@ -32,6 +32,22 @@ def test_cut_tiles_cover_every_block_once(cta_group, workers):
             assert work.max() <= 1.08 * even + 8, (rows, k_len, n_tiles, work.max(), even)
 
 
+# 12, 24 and 7 tiles leave 2 or 4 of 74 workers over (too few for the ends of 70 parts), 8 tiles 2; 32 leave 10, 48 leave 26
+@pytest.mark.parametrize("rows,n_tiles,k_len,helped", [(600, 4, 151936, False), (1536, 4, 151936, False), (100, 5, 151936, False),
+                                                       (400, 2, 152064, False), (1800, 4, 151936, True), (3072, 4, 151936, True)])
+def test_helpers_end_with_the_parts(rows, n_tiles, k_len, helped):
+    from paper_2512_21450_b200.binding import debug_schedule
+    u = debug_schedule(rows, 32768, k_len, n_tiles, n_range=1, n_fastest=1, stream_k=2, cta_group=2, n_workers=74)
+    pieces, work = np.zeros(74, dtype=np.int64), np.zeros(74, dtype=np.int64)
+    for w, *_, kb0, kb1, _ in u:
+        pieces[w] += 1
+        work[w] += kb1 - kb0
+    assert (pieces.max() > 1) == helped
+    # with 20 k-blocks for the output of each part, nobody is later than a part by more than one more
+    cost = work + 20 * pieces
+    assert cost.max() <= cost[pieces == 1].max() + 20
+
+
 @pytest.mark.parametrize("rows,n_tiles,most,expect", [(77, 594, 148, 0.88), (276, 594, 118, 0.9), (2757, 594, 75, 0.9),
                                                       (60, 16, 16, 0.0), (1, 1, 16, 0.0), (4096, 594, 75, 0.9)])
 def test_column_ranges_fill_the_machine(rows, n_tiles, most, expect):
