@@ -624,7 +624,8 @@ __global__ void __launch_bounds__(256) broadcast_adv_kernel(const float* __restr
 // linear maps x -> v + g x (valid row: g = gamma, v = r_t; masked row: the identity) over its rows with shuffles, the
 // warps' totals are chained through shared memory, and the return of the first valid row of the tile is carried to the
 // next.  Per-token terms in fp32, sums in double.  (One warp per response walked 512 rows as a chain of four rounds:
-// 26 us for 1024 responses; it stays for responses of less than a warp's 128 rows.)  Rows outside every response range, [0, seq_offsets[0]) and [seq_offsets[n_seq], T), get 0.
+// 26 us for 1024 responses; it stays for responses of less than a warp's 128 rows, and for many whose last 512 rows would be
+// mostly empty.)  Rows outside every response range, [0, seq_offsets[0]) and [seq_offsets[n_seq], T), get 0.
 constexpr int kShapeChunks = 4;
 constexpr int kShapeWarps = 4;
 

@@ -72,3 +72,30 @@ def test_advantages_in_the_broadcast(n_groups, G):
     want = np.zeros(int(off[-1]) + 5)
     want[3:off[-1]] = np.repeat(_np64(seq), np.diff(off))
     assert np.array_equal(_np64(tok), want)
+
+
+# few responses and many (from 1185 on), a block each or a warp each: 150 and 600 rows leave a block's last 512 mostly empty, 420 and
+# 900 do not; 127 rows are always a warp's
+@pytest.mark.parametrize("n_seq", [1184, 1400])
+@pytest.mark.parametrize("mean", [127, 150, 420, 600, 900])
+def test_shaped_returns_of_many_responses(n_seq, mean):
+    from paper_2512_21450_b200 import Context
+    rng = np.random.default_rng(n_seq + mean)
+    lengths = np.full(n_seq, mean)
+    lengths[0::2] -= rng.integers(0, 100, size=len(lengths[0::2]))
+    lengths[1] += mean * n_seq - lengths.sum()   # the mean is what decides
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    T = int(off[-1])
+    logp, ref, R = (rng.standard_normal(s).astype(np.float32) for s in (T, T, n_seq))
+    mask = (rng.random(T) < 0.7).astype(np.uint8)
+    t = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    c = Context(0)
+    try:
+        sh, ret = c.rl_kl_shaped_returns(t(R), t(logp), t(ref), t(mask), t(off), T, 0.25)
+        assert c.last_device_status()[0] == 0
+        o_sh, o_ret = O.kl_shaped_returns(*(a.astype(np.float64) for a in (R, logp, ref)), mask, off, 0.25, gamma=1.0, kind="k3")
+        # fp32 k3 terms (exp within 2 ulp of up to e^6) summed in double over the rows of a response
+        for got, want in ((sh, o_sh), (ret, o_ret)):
+            assert np.all(np.abs(_np64(got) - want) <= 1e-6 + 1e-6 * np.abs(want))
+    finally:
+        c.close()
