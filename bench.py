@@ -30,7 +30,7 @@ KIND_NAMES = ["gemm_kernel<EpiSweep,square> (logits: statistics and codes)", "lo
 # for the sources of those kernels (main loop, epilogues, PTX wrappers, small kernels) whose hash is recorded with it.  Bytes
 # per AVERAGE launch of a step.
 KERNEL_SOURCES = ("epilogues.cuh", "gemm_engine.cuh", "ptx.cuh", "small_kernels.cuh")
-NCU_TRAFFIC = {"sources_sha256": "6476307f7b8a690bf2a1704d3c4824159463db69258340d2376cea1a2fcd1ae1", "config": 1,
+NCU_TRAFFIC = {"sources_sha256": "90e82871bb4e166aad8732371092da458a6bfc1d1b3abea8f69c4bf9a0538974", "config": 1,
                "bytes_per_avg_launch": {0: 2608919000, 1: 3383986000, 2: 6038128000, 3: 4450700000}}
 
 
