@@ -66,7 +66,7 @@ const char* rl_status_string(rl_status s);
  * made from) only ever exists for a bounded slab of rows x vocabulary columns. */
 rl_status rl_workspace_bytes(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, size_t* bytes);
 /* The same for calls that set rl_loss_opts.kl_full with a reference model of hidden size d_ref (adds the
- * compacted reference rows, seven per-row arrays and, from d + d_ref = 1536 on, 4 bytes per slab entry). */
+ * compacted reference rows, five per-row arrays and, from d + d_ref = 1536 on, 6 bytes per slab entry). */
 rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, int64_t d_ref, size_t* bytes);
 /* Size of the slab the backward pass works in: at most max_rows token rows x max_cols vocabulary
  * columns of the gradient with respect to the logits exist at a time (bf16, in the workspace).

@@ -1,8 +1,6 @@
 // Epilogues of the two-product tile mode of the GEMM engine: full-distribution KL(pi_theta || pi_ref) per token
 // (section 2.2 "KL-to-reference", section 3.1 Omega) and its gradient with respect to the logits.
 #pragma once
-#include <cuda_fp16.h>
-
 #include "epilogues.cuh"
 
 namespace rlh {
@@ -107,11 +105,10 @@ struct EpiStatsKL {
 
 // ---------------------------------------------------------------------------------------------
 // One-sweep form: the reference logits and the policy logits of a slab of whole rows are formed once each, in two
-// single-product passes whose epilogues overlap the next tile's MMAs.  The slab holds one 32-bit word per entry: first the
-// reference logit zr in fp32, then (policy pass) the 16-bit code of exp(z - m) and z - zr - c in fp16, with c the
-// sampled token's own difference, so that what is rounded is of the size of the spread of z - zr under the policy.
-// Forming both logits side by side (two-product tiles) left the epilogue exposed and had to be done twice: 4.2 + 4.0 ms
-// at 4096 rows, d = d_ref = 2048, V = 151936.  All statistics, KL_t among them, are taken from the fp32 logits.
+// single-product passes whose epilogues overlap the next tile's MMAs, and both stay in the slab in fp32 until the rows'
+// log-sum-exps and loss coefficients are known: the reference logits as they are, the policy logits as two 16-bit planes,
+// so that the gradient can take the place of the upper halves.  Forming both logits side by side (two-product tiles) left
+// the epilogue exposed and had to be done twice: 4.2 + 4.0 ms at 4096 rows, d = d_ref = 2048, V = 151936.
 __device__ __forceinline__ void ld_global_v8(const float* p, float (&v)[32], int i) {
   asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3]), "=f"(v[i + 4]), "=f"(v[i + 5]), "=f"(v[i + 6]),
@@ -123,6 +120,22 @@ __device__ __forceinline__ void st_global_v8(float* p, const float* v) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
                "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
                : "memory");
+}
+
+// Upper and lower 16-bit halves of 32 consecutive logits of a row, to the two planes (32-byte stores, every sector whole).
+__device__ __forceinline__ void st_planes(const float (&v)[32], uint16_t* hi, uint16_t* lo) {
+  float h[16], l[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint32_t a = __float_as_uint(v[2 * i]), b = __float_as_uint(v[2 * i + 1]);
+    h[i] = __uint_as_float(__byte_perm(a, b, 0x7632));
+    l[i] = __uint_as_float(__byte_perm(a, b, 0x5410));
+  }
+#pragma unroll
+  for (int j = 0; j < 16; j += 8) {
+    st_global_v8(reinterpret_cast<float*>(hi) + j, h + j);
+    st_global_v8(reinterpret_cast<float*>(lo) + j, l + j);
+  }
 }
 
 // Reference pass: zr to the slab, running max and sum of exp of the reference logits to partials2 = {-, Mr, Sr, -}.
@@ -174,8 +187,8 @@ struct EpiRefSweep {
   }
 };
 
-// Policy pass: statistics of EpiStats, D = sum_j exp(z_j - M) zr_j (to partials2.x), and the slab's words.  The words of
-// the next 32 columns are loaded while these are worked on; nobody else touches this thread's part of its row.
+// Policy pass: statistics of EpiStats, D = sum_j exp(z_j - M) zr_j (to partials2.x), and the planes of z.  The reference
+// logits of the next 32 columns are loaded while these are worked on.
 struct EpiSweepKL {
   static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
@@ -184,15 +197,15 @@ struct EpiSweepKL {
   struct Params {
     RowStats::Params stats;
     float4* partials2;
-    const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
-    const float* centre;   // [rows] compact: c
-    float* slab;
+    const float* zr;       // reference logits of the slab
+    uint16_t* hi;          // planes of the policy logits
+    uint16_t* lo;
     int ld;                // whole tiles: columns past V are read and written as well
   };
   struct State {
     RowStats::State s;
-    float d, offset, centre;
-    float* row;
+    float d;
+    long long at;    // start of this thread's row in the slab, -1: past the valid rows
     int grow;
     bool fresh;      // nothing loaded ahead yet
     float next[32];
@@ -204,21 +217,18 @@ struct EpiSweepKL {
     const int rl = m_tile * BM + row_in_tile;
     const bool valid = rl < m_rows;
     st.grow = valid ? slab_off + rl : -1;
-    st.row = valid ? p.slab + (size_t)rl * p.ld : nullptr;
+    st.at = valid ? (long long)rl * p.ld : -1;
     st.s.m = -CUDART_INF_F;
     st.s.s = st.s.a = st.s.zy = 0.f;
     st.d = 0.f;
     st.s.y = valid ? p.stats.tokens_c[st.grow] : -1;
-    const float sh = valid ? p.shift2[st.grow] : 0.f;
-    st.offset = code_offset(sh);
-    st.centre = valid ? p.centre[st.grow] : 0.f;
     st.fresh = true;
   }
   __device__ static __forceinline__ void chunk(const Params& p, State& st, int, int n_tile, int c, int, int,
                                                const float (&v)[32], const CUtensorMap* map, uint32_t staging) {
-    if (!st.row) return;
+    if (st.at < 0) return;
     const int col = n_tile * BN + c * 32;
-    float* q = st.row + col;
+    const float* q = p.zr + st.at + col;
     float zr[32];
     if (st.fresh) {
 #pragma unroll
@@ -250,20 +260,7 @@ struct EpiSweepKL {
       }
       st.d = fmaf(st.d, ex2_approx((m_old - st.s.m) * kLog2e), cd2.x + cd2.y);
     }
-    const float2 nc2 = make_float2(-st.centre, -st.centre);
-    float w[32];
-#pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-      const float2 z2 = make_float2(v[i], v[i + 1]);
-      const float2 f = code_words(z2, st.offset);
-      const float2 dl = __fadd2_rn(__fadd2_rn(z2, make_float2(-zr[i], -zr[i + 1])), nc2);
-      const __half2 h = __floats2half2_rn(fminf(fmaxf(dl.x, -65504.f), 65504.f), fminf(fmaxf(dl.y, -65504.f), 65504.f));
-      const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
-      w[i] = __uint_as_float(__byte_perm(__float_as_uint(f.x), hb, 0x5410));
-      w[i + 1] = __uint_as_float(__byte_perm(__float_as_uint(f.y), hb, 0x7610));
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) st_global_v8(q + 8 * j, w + 8 * j);
+    st_planes(v, p.hi + st.at + col, p.lo + st.at + col);
   }
   static constexpr int kMerge = RowStats::kMerge + 1;
   __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) {
@@ -288,7 +285,7 @@ struct EpiSweepKL {
 //                  + ce_t p_tj (log p_tj + Ent_t),   cb_t = w_t beta,
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
-  static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
+  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = 8;
   static constexpr int kMerge = 0;

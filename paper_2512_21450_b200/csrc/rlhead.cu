@@ -100,6 +100,7 @@ inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_s
 // twice.  The former trades 4 d + 4 d_ref tensor flops for 14 bytes of traffic per entry.  4096 rows, V = 151936: logits and
 // their gradient take 3.3 / 3.5 / 4.9 / 8.3 ms against 2.5 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
 constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
+constexpr int kKlEntryBytes = 8;         // two fp32 logits per slab entry
 inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
 // tile that is half empty costs as much as a full one.  For dH, whose K is the vocabulary: 7 % of the pass (8.59 / 53.1 /
@@ -126,7 +127,7 @@ struct WsLayout {
   size_t dH_slots;                                   // parts of cut dH tiles (0: none)
   int n_row_slabs, n_flags;                          // n_flags: row tiles, then one count per row slab
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
-  size_t words, zy_c, centre;                        // its one-sweep form (words 0: two-product tiles)
+  size_t zr, z_lo;                                   // its one-sweep form (0: two-product tiles)
 };
 
 // Reference-model operands of the full-distribution KL (all NULL / 0 when it is not used).
@@ -174,9 +175,9 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   long long rows = c->slab_rows, one = 0;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
   if (c->slab_auto) {
-    // as many rows as kSlabElements allows (half where slab entries take 6 bytes), and no more than
+    // as many rows as kSlabElements allows (a quarter where a slab entry takes 8 bytes), and no more than
     // keep the compact rows, which the dW pass reads once per row panel of dW, in L2 beside the streamed slab
-    long long whole = kSlabElements / (kl_one_sweep(d, d_ref) ? 2 : 1) / Vpad / 256 * 256;
+    long long whole = kSlabElements * 2 / (kl_one_sweep(d, d_ref) ? kKlEntryBytes : 2) / Vpad / 256 * 256;
     long long resident = kSlabRowBytes / (d * 2) / 256 * 256;
     if (resident < kSlabRowsMin) resident = kSlabRowsMin;
     if (whole >= kSlabRowsMin || whole >= L.Tpad) {
@@ -225,7 +226,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
   L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
   L.flags = take((size_t)L.n_flags * 4);
-  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.words = L.zy_c = L.centre = 0;
+  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = L.z_lo = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
     L.partials2 = take((size_t)n_part_ranges * L.Tpad * sizeof(float4));
@@ -233,9 +234,8 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
     L.kl_c = take((size_t)L.Tpad * 4);
     L.cb_c = take((size_t)L.Tpad * 4);
     if (L.Vs == Vpad && kl_one_sweep(d, d_ref)) {
-      L.words = take((size_t)L.Ts * L.Vs * 4);
-      L.zy_c = take((size_t)L.Tpad * 4);
-      L.centre = take((size_t)L.Tpad * 4);
+      L.zr = take((size_t)L.Ts * L.Vs * 4);
+      L.z_lo = take((size_t)L.Ts * L.Vs * 2);
     }
   }
   L.staging = o;
@@ -494,7 +494,6 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
     sp.shift2 = reinterpret_cast<float*>(ws + L.shift2);
     sp.flags = reinterpret_cast<int*>(ws + L.flags);
     sp.n_flags = L.n_flags;
-    if (kl) sp.zy = reinterpret_cast<float*>(ws + L.zy_c);
   }
   pp.H = static_cast<const __nv_bfloat16*>(H);
   pp.ldH = ldH;
@@ -528,8 +527,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   __nv_bfloat16* Hc_ref = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc_ref);
   if (kl) {   // full KL: compact the reference hidden states with the same row map
     launch(c, gather_plain_kernel, c->n_sm * 4, 256, static_cast<const __nv_bfloat16*>(kl->H_ref), kl->ldH_ref, (int)kl->d_ref,
-           row_map, Hc_ref, static_cast<const __nv_bfloat16*>(kl->W_ref), kl->ldW_ref, tokens_c, sp.zy,
-           sp.zy ? reinterpret_cast<float*>(ws + L.centre) : nullptr, c->dstatus);
+           row_map, Hc_ref, c->dstatus);
     c->launches++;
   }
   if (!plan.stats) {
@@ -1139,7 +1137,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   // rows' coefficients are known.  Not where the coefficients of a row need rows of another slab, nor where the
   // statistics come from elsewhere: those paths form the logits a second time.
   const int Vpad = (int)align_up((size_t)V, 256);
-  const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.words) &&
+  const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.zr) &&
                      (L.n_row_slabs == 1 || (L.Tc % kFlagRows == 0 && !seq_path));
   FwdPlan plan;
   plan.out.dH = dH;
@@ -1148,7 +1146,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   plan.out.value[2] = o.kl_full ? o.kl_out : nullptr;
   if (sweep) {
     plan.stats = false;
-    plan.old_logp = old_logp;
+    plan.old_logp = o.kl_full ? nullptr : old_logp;
   }
   if (shard) {
     // the statistics of the whole vocabulary are given: only the row compaction is needed
@@ -1319,8 +1317,9 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sw.leaves_ranges = 1;
           sw.a_mn_slab = 1;
           sw.m_group = row_group_tiles(c, d);
-          const float* centre = reinterpret_cast<const float*>(ws + L.centre);
-          float* words = reinterpret_cast<float*>(ws + L.words);
+          float* zr = reinterpret_cast<float*>(ws + L.zr);
+          uint16_t* z_hi = reinterpret_cast<uint16_t*>(G);
+          uint16_t* z_lo = reinterpret_cast<uint16_t*>(ws + L.z_lo);
           if (o.kl_full) {
             GemmShape sr = sw;
             sr.k_cap = (int)o.d_ref;
@@ -1329,7 +1328,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             er.partials2 = reinterpret_cast<float4*>(ws + L.partials2);
             er.part_stride = L.Tpad;
             er.V = (int)V;
-            er.slab = words;
+            er.slab = zr;
             er.ld = L.Vs;
             launch_gemm<EpiRefSweep, 0, 0>(c, cg_fwd, 0, tmHr_k, tmWr_fwd, tm_G_out, tm_G_out, sr, er);
           }
@@ -1343,9 +1342,9 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             EpiSweepKL::Params ek;
             ek.stats = ep.stats;
             ek.partials2 = reinterpret_cast<float4*>(ws + L.partials2);
-            ek.shift2 = ep.shift2;
-            ek.centre = centre;
-            ek.slab = words;
+            ek.zr = zr;
+            ek.hi = z_hi;
+            ek.lo = z_lo;
             ek.ld = L.Vs;
             launch_gemm<EpiSweepKL, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ek);
           } else if (d <= kEightWarpsMaxKSweep) {
@@ -1355,12 +1354,14 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           }
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;
-          p.shift2 = ep.shift2;
-          p.tile_flags = flags;
-          p.flag_count = flag_count;
+          if (!o.kl_full) {
+            p.shift2 = ep.shift2;
+            p.tile_flags = flags;
+            p.flag_count = flag_count;
+          }
           merge_and_loss(r);
           LogitGradParams lg;
-          lg.slab = reinterpret_cast<uint16_t*>(G);
+          lg.slab = z_hi;
           lg.ld = L.Vs;
           lg.V = (int)V;
           lg.slab_cap = L.Tc; lg.slab_one = L.Ts; lg.slab_index = r;
@@ -1368,12 +1369,12 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.shift2 = ep.shift2;
           lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
           const int pr_lg = prof_begin(c, 1);
-          lg.words = reinterpret_cast<const uint32_t*>(words);
-          lg.centre = centre;
+          lg.lo = z_lo;
+          lg.zr = zr;
           lg.lse_ref = p.lse_ref_c; lg.kl = p.kl_c; lg.cb = p.cb_c;
           const long long padded = (long long)align_up(rows_cap, 128);
-          const bool few = o.kl_full || padded * ((L.Vs + 256 * kGradVecs - 1) / (256 * kGradVecs)) < kGradFewUnits;
-          const int unit = 256 * (few ? kGradVecsFew : kGradVecs);
+          const bool few = padded * ((L.Vs + 256 * kGradVecs - 1) / (256 * kGradVecs)) < kGradFewUnits;
+          const int unit = 256 * (o.kl_full ? kGradVecsKL : few ? kGradVecsFew : kGradVecs);
           long long grad_blocks = (padded * ((L.Vs + unit - 1) / unit) + 7) / 8;   // a warp each
           if (grad_blocks > c->n_sm * 64) grad_blocks = c->n_sm * 64;
           if (o.kl_full) launch(c, logit_grad_kl_kernel, (int)grad_blocks, 256, lg, c->dstatus);
@@ -1405,13 +1406,13 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             launch_gemm<EpiGrad<8>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
           else
             launch_gemm<EpiGrad<4>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
-        } else {
+        } else if (!sweep) {
           EpiGradKL::Params ep;
           ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
           ep.lse = p.lse_c; ep.lse_ref = p.lse_ref_c; ep.ent = p.ent_c; ep.kl = p.kl_c;
           ep.cp = p.cp_c; ep.cb = p.cb_c; ep.ce = p.ce_c;
           ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_dual<EpiGradKL>(c, sweep ? -1 : 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
+          launch_dual<EpiGradKL>(c, 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
         }
       }
       // (2) dH_slab (+)= G * W_slab        [rows x d], K = vocabulary columns of the slab

@@ -168,7 +168,6 @@ struct SweepPrep {
   long long ldW;
   const float* old_logp;   // [T] original rows
   float* shift2;           // [rows] compact: the estimate in units of log 2, or NULL
-  float* zy;               // [rows] compact: the logit itself, or NULL
   int* flags;              // words cleared for the launches that follow
   int n_flags;
 };
@@ -234,7 +233,6 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
       const float est = z - p.sp.old_logp[t];
       // a whole number of code steps, so that the offset the codes are formed with is exact
       p.sp.shift2[pos] = rintf((isfinite(est) ? est : 0.f) * (kLog2e * kCodeSlope)) * (1.f / kCodeSlope);
-      if (p.sp.zy) p.sp.zy[pos] = z;
     }
   } else {
 #pragma unroll 8
@@ -297,14 +295,10 @@ __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevS
   }
 }
 
-// Row compaction of a second hidden-state matrix (the reference model's) with the same row map.  centre != NULL: also the
-// difference of the sampled token's two logits, which the words of the one-sweep KL are centred on.
+// Row compaction of a second hidden-state matrix (the reference model's) with the same row map.
 __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* __restrict__ H, long long ldH, int d,
                                                            const int* __restrict__ row_map,
-                                                           __nv_bfloat16* __restrict__ Hc,
-                                                           const __nv_bfloat16* __restrict__ W, long long ldW,
-                                                           const int* __restrict__ tokens_c, const float* __restrict__ zy,
-                                                           float* __restrict__ centre, const DevStatus* st) {
+                                                           __nv_bfloat16* __restrict__ Hc, const DevStatus* st) {
   chain_begin();
   const int n = st->n_valid;
   const int n_pad = (n + 127) / 128 * 128;
@@ -315,27 +309,8 @@ __global__ void __launch_bounds__(256) gather_plain_kernel(const __nv_bfloat16* 
     uint4* dst = reinterpret_cast<uint4*>(Hc + (size_t)i * d);
     if (i < n) {
       const uint4* src = reinterpret_cast<const uint4*>(H + (size_t)row_map[i] * ldH);
-      const uint4* wrow = centre ? reinterpret_cast<const uint4*>(W + (size_t)max(tokens_c[i], 0) * ldW) : nullptr;
-      float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 4
-      for (int v = lane; v < vec_per_row; v += 32) {
-        const uint4 h = __ldg(src + v);
-        dst[v] = h;
-        if (centre) {
-          const uint4 w = __ldg(wrow + v);
-          const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
-                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
-        }
-      }
-      if (centre) {
-        float z = acc.x + acc.y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        if (lane == 0) centre[i] = zy[i] - z;
-      }
+      for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
     } else {
       for (int v = lane; v < vec_per_row; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
     }
@@ -1033,7 +1008,8 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
 // warp takes VECS * 256 consecutive columns of one row, all its 16-byte loads in flight before the first is used.  18947 rows
 // x 152064 columns: 2.13 ms, 5.4 TB/s (four loads instead of eight, and one wave of blocks instead of many: 2.32 ms).
 constexpr int kGradVecs = 8;         // 16-byte words per lane and unit of VECS * 256 columns
-constexpr int kGradVecsFew = 4;      // the same with few rows (twice the warps), and for the KL kernel, which loads two per output
+constexpr int kGradVecsFew = 4;      // the same with few rows (twice the warps)
+constexpr int kGradVecsKL = 2;       // the KL kernel loads four of them per output
 constexpr long long kGradFewUnits = 65536;   // units of kGradVecs below which it is few: 276 rows 35 us instead of 37
 struct LogitGradParams {
   uint16_t* slab;          // [slab rows][ld]
@@ -1047,62 +1023,67 @@ struct LogitGradParams {
   const float* ent;
   const float* cp;
   const float* ce;
-  // full-distribution KL: words of code and fp16 (z - zr - centre), read from here; the slab is only written
-  const uint32_t* words;
-  const float* centre;
+  // full-distribution KL: the slab holds the upper halves of the policy logits, `lo` the lower ones, `zr` the reference's
+  const uint16_t* lo;
+  const float* zr;
   const float* lse_ref;
   const float* kl;
   const float* cb;
 };
 
-// The same with the regulariser's term: g_tj = cp_t (p_tj - 1[j = y_t]) + cb_t p_tj (log p_tj - log q_tj - KL_t)
-// + ce_t p_tj (log p_tj + Ent_t).  4 bytes in and 2 out per entry.
+// The same with the regulariser's term, from the fp32 logits of both models, in the arithmetic of EpiGradKL:
+//   g_tj = cp_t (p_tj - 1[j = y_t]) + cb_t p_tj (log p_tj - log q_tj - KL_t) + ce_t p_tj (log p_tj + Ent_t).
+// 8 bytes in and 2 out per entry.
 __global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParams p, const DevStatus* st) {
   chain_begin();
   int off, rows;
   slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
   const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + (kGradVecsFew * 256) - 1) / (kGradVecsFew * 256);
+  const int units_per_row = (p.ld + (kGradVecsKL * 256) - 1) / (kGradVecsKL * 256);
   const long long n_units = (long long)rows_pad * units_per_row;
   const int lane = threadIdx.x & 31;
   const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
     const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecsFew * 256);
-    uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
+    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecsKL * 256);
+    const size_t at = (size_t)r * p.ld + c0;
+    uint4* base = reinterpret_cast<uint4*>(p.slab + at) + lane;
     if (r >= rows) {
 #pragma unroll
-      for (int k = 0; k < kGradVecsFew; ++k)
+      for (int k = 0; k < kGradVecsKL; ++k)
         if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
       continue;
     }
-    const uint4* src = reinterpret_cast<const uint4*>(p.words + (size_t)r * p.ld + c0) + 2 * lane;
-    uint4 q[2 * kGradVecsFew];
+    const uint4* low = reinterpret_cast<const uint4*>(p.lo + at) + lane;
+    const float4* ref = reinterpret_cast<const float4*>(p.zr + at) + 2 * lane;
+    uint4 h[kGradVecsKL], l[kGradVecsKL];
+    float4 z0[kGradVecsKL], z1[kGradVecsKL];
 #pragma unroll
-    for (int k = 0; k < kGradVecsFew; ++k)
-      if (c0 + k * 256 < p.ld) { q[2 * k] = __ldcs(src + k * 64); q[2 * k + 1] = __ldcs(src + k * 64 + 1); }
+    for (int k = 0; k < kGradVecsKL; ++k)
+      if (c0 + k * 256 < p.ld) {
+        h[k] = base[k * 32];
+        l[k] = __ldcs(low + k * 32);
+        z0[k] = __ldcs(ref + k * 64);
+        z1[k] = __ldcs(ref + k * 64 + 1);
+      }
     const int i = off + r;
-    const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i], cb = p.cb[i];
+    const float lse = p.lse[i], lse_ref = p.lse_ref[i], cp = p.cp[i], ce = p.ce[i], cb = p.cb[i];
+    const float rest = cp + ce * p.ent[i] - cb * p.kl[i];   // terms that do not depend on j
+    const float k_lp = cb + ce;                             // coefficient of log p_j
     const int y = p.tokens_c[i];
-    const float shift = fmaf(-lse, kLog2e, p.shift2[i]);   // log2 p = exponent of the code + shift
-    // g = p (kc + kl log2 p + cb delta), delta = the fp16 half: z - zr - centre
-    const float kc = fmaf(ce, ent, cp) + cb * (p.centre[i] - lse + p.lse_ref[i] - p.kl[i]), kl = ce * kLn2;
-    const float py = ex2_approx(logp * kLog2e);
 #pragma unroll
-    for (int k = 0; k < kGradVecsFew; ++k) {
+    for (int k = 0; k < kGradVecsKL; ++k) {
       const int c = c0 + k * 256 + lane * 8;
       if (c0 + k * 256 >= p.ld) break;
-      const uint32_t w[8] = {q[2 * k].x, q[2 * k].y, q[2 * k].z, q[2 * k].w,
-                             q[2 * k + 1].x, q[2 * k + 1].y, q[2 * k + 1].z, q[2 * k + 1].w};
+      const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, lw[4] = {l[k].x, l[k].y, l[k].z, l[k].w};
+      const float zr[8] = {z0[k].x, z0[k].y, z0[k].z, z0[k].w, z1[k].x, z1[k].y, z1[k].z, z1[k].w};
       float g[8];
       const unsigned rel = (unsigned)(y - c);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float t = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5410))) + shift;
-        const float dl = __half2float(__ushort_as_half((unsigned short)(w[j] >> 16)));
-        const bool at = rel == (unsigned)j;
-        const float f = fmaf(cb, dl, fmaf(kl, at ? logp * kLog2e : t, kc));
-        g[j] = at ? fmaf(py, f, -cp) : ex2_approx(t) * f;
+        const float lp = __uint_as_float(__byte_perm(lw[j / 2], hw[j / 2], j & 1 ? 0x7632 : 0x5410)) - lse;
+        g[j] = ex2_approx(lp * kLog2e) * (fmaf(k_lp, lp, rest) - cb * (zr[j] - lse_ref));
+        if (rel == (unsigned)j) g[j] -= cp;
         if (c + j >= p.V) g[j] = 0.f;
       }
       uint32_t o[4];

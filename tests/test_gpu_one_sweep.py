@@ -152,3 +152,33 @@ def test_column_halves(d, V):
             assert _rel(_np64(out["dH"]), oo["dH"]) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
     finally:
         c.close()
+
+
+# rows whose sampled token is an outlier: the reference gives it 5 nats more than the policy, all other words nearly the same
+# logit.  The regulariser's gradient of such a row is made of differences of logits a hundred times smaller than the
+# sampled token's own, which a difference held to less than fp32 loses.
+def test_one_sweep_full_kl_outlier_rows():
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    d, V = 768, 40001
+    w = make_workload(1, prompts=1, L_max=40, d=d, V=V, seed=2600)
+    H_ref = w.H
+    W_ref = (w.W.float() * (1.0 + 0.05 * torch.randn(V, d, device="cuda"))).to(torch.bfloat16)
+    valid = torch.nonzero(w.mask)[:, 0]
+    h, y = w.H[valid].float(), w.tokens[valid].long()
+    W_ref[y] = (W_ref[y].float() + 5.0 * h / h.square().sum(1, keepdim=True)).to(torch.bfloat16)
+    adv = torch.zeros(w.T, device="cuda")
+    c = Context(0)
+    try:
+        out = c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, None, adv, w.mask, w.eps_low, w.eps_high, 0.05,
+                                       dH_fp32=True, H_ref=H_ref, W_ref=W_ref)
+        assert c.last_device_status()[0] == 0
+    finally:
+        c.close()
+    oo = O.policy_loss_fwd_bwd(_np64(w.H), _np64(w.W), w.tokens.cpu().numpy(), _np64(w.old_logp), None, _np64(adv),
+                               w.mask.cpu().numpy(), w.eps_low, w.eps_high, 0.05, H_ref=_np64(H_ref), W_ref=_np64(W_ref))
+    m = w.mask.cpu().numpy().astype(bool)
+    err = np.linalg.norm(_np64(out["dH"])[m] - oo["dH"][m], axis=1) / np.linalg.norm(oo["dH"][m], axis=1)
+    # an entry of G is rounded to bf16 once (2^-9 at most, 1.7e-3 rms over a row of many entries), and a row of dH is the sum
+    # of its entries times random rows of W, which keeps the ratio up to 1/sqrt(d)
+    assert err.max() <= 4e-3, np.sort(err)[-5:]
