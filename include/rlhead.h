@@ -62,19 +62,19 @@ rl_status rl_set_stream(rl_ctx* ctx, void* cuda_stream);
 const char* rl_status_string(rl_status s);
 
 /* Bytes of scratch needed by any call with at most T rows, hidden size d, vocabulary V.  The
- * size does not grow with T*V: the gradient with respect to the logits (and the 16-bit codes it is
- * made from) only ever exists for a bounded slab of rows x vocabulary columns. */
+ * size does not grow with T*V beyond one slab: the gradient with respect to the logits, and the fp32
+ * logits it is made from, only ever exist for a bounded slab of rows x vocabulary columns. */
 rl_status rl_workspace_bytes(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, size_t* bytes);
 /* The same for calls that set rl_loss_opts.kl_full with a reference model of hidden size d_ref (adds the
- * compacted reference rows, five per-row arrays and, from d + d_ref = 1536 on, 6 bytes per slab entry). */
+ * compacted reference rows, five per-row arrays and, from d + d_ref = 1536 on, 4 bytes more per slab entry). */
 rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, int64_t d_ref, size_t* bytes);
 /* Size of the slab the backward pass works in: at most max_rows token rows x max_cols vocabulary
  * columns of the gradient with respect to the logits exist at a time (bf16, in the workspace).
  * max_rows a multiple of 128, max_cols a multiple of 256, max_rows * max_cols at most 2^31; 0 for one of
  * them is 32768 rows or 37888 columns.  (0, 0) restores the default: rows over the whole vocabulary, at most
- * 2^31 entries and 58 MB of hidden states (14080 rows at d = 2048 and 152 K words, 4.3 GB), or 32768 x 37888 for
- * vocabularies of which fewer than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary, max_rows at least 256)
- * the loss calls form the logits once instead of twice: 13-20 % of a step.  Changes what
+ * 4.3 GB and 58 MB of hidden states (6912 rows at 152 K words), or 32768 x 37888 for vocabularies of which fewer
+ * than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary) the loss calls keep the fp32
+ * logits there, 4 bytes per entry, and form them once instead of twice: 13-18 % of a step.  Changes what
  * rl_workspace_bytes() returns: call it first. */
 rl_status rl_set_slab_limits(rl_ctx* ctx, int max_rows, int max_cols);
 /* Tile shape of the tensor-core passes: 1 = one CTA per 128x256 output tile, 2 = CTA pairs
@@ -439,7 +439,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
  * rl_set_profiling(on): when on, every kernel (or group of small kernels) is bracketed by a pair of CUDA events
  * on the context's stream (at most 65536 launch groups are kept between two reads; later ones go untimed).
  * rl_profile_read: synchronises the stream and returns, per kernel kind (0 logits (statistics, and
- * codes where the logits are formed once), 1 gradient-of-logits slab, 2 dH, 3 dW, 4 mask scan, 5 row preparation, 6 merge + loss,
+ * the logits themselves where they are formed once), 1 gradient-of-logits slab, 2 dH, 3 dW, 4 mask scan, 5 row preparation, 6 merge + loss,
  * 7 dH scatter, 8 advantages), the summed device time in milliseconds ms[9] (host) and the number
  * of timed launch groups launches[9] (host) since the previous read.  The paper has no
  * counterpart; these exist so that a benchmark can report per-kernel roofline figures. */

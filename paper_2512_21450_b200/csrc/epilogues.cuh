@@ -23,7 +23,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // range of the work unit, keeps the running maximum M, S = sum exp(z-M), A = sum exp(z-M) z and
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
 struct RowStats {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -128,29 +127,6 @@ struct EpiStats : RowStats {
 };
 
 // ---------------------------------------------------------------------------------------------
-// 16-bit logarithmic code of exp(z - m): what the one-sweep path keeps of a logit between the pass that forms it and the
-// point where the row's log-sum-exp and loss coefficients are known.  With t = (z - m) log2(e) and m an estimate of
-// the log-sum-exp of the row, code = round(1024 t + 57344) clamped at 0: steps of 2^-10 of an octave (relative error of p
-// at most 2^-11.5, an eighth of the bf16 rounding that follows; rms of the two together 0.7 % above bf16 alone) down to
-// t = -56, where p stays at 2^-56 (the floors of a whole vocabulary add up to less than one fp32 rounding of the row's sum).  t
-// reaches up to 8 before the code leaves 16 bits: rows whose estimate is that far off are recomputed (kCodeTop, kCodeLow
-// below).  One multiply-add puts 2^23 + code into the low bits of a float, the clamp is one maximum.
-constexpr float kCodeSlope = 1024.f, kCodeBase = 57344.f, kCodeMagic = 8388608.f;
-constexpr float kCodeTop = 7.9f;    // largest t of a row that its codes can hold
-constexpr float kCodeLow = -14.f;   // least log2 of the row's sum of exp(z - m): below, too little of the range is left
-
-// p's exponent t of the code in the low 16 bits of the float 2^23 + code.
-__device__ __forceinline__ float code_exponent(float f) {
-  return fmaf(f, 1.f / kCodeSlope, -(kCodeMagic + kCodeBase) / kCodeSlope);
-}
-// The offset of the multiply-add for a row whose estimate is shift2 (in units of log 2).
-__device__ __forceinline__ float code_offset(float shift2) { return fmaf(-kCodeSlope, shift2, kCodeBase) + kCodeMagic; }
-// 2^23 + code of two logits.
-__device__ __forceinline__ float2 code_words(float2 z, float offset) {
-  const float2 x = __ffma2_rn(z, make_float2(kLog2e * kCodeSlope, kLog2e * kCodeSlope), make_float2(offset, offset));
-  return make_float2(fmaxf(x.x, kCodeMagic), fmaxf(x.y, kCodeMagic));
-}
-
 // 32 rows x 32 columns of 16-bit values (two per word, one row per lane) into one half of a 128-byte-swizzled 32 x 64
 // box; c = index of the 32-column chunk.  The second half hands the box to the TMA unit.
 template <int BUFS>   // boxes per warp
@@ -183,27 +159,20 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
   }
 }
 
-// Forward statistics of EpiStats for one slab of rows, plus the code of every logit written to the slab scratch (the
-// place the gradient with respect to the logits then takes).  Forming the logits once instead of twice (statistics,
-// then recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  At d = 2048 the extra
-// arithmetic (2 instructions per logit on top of the statistics' 3.5) still hides behind the next tile's MMAs.
-// Eight warps pay up to d = 1280 here: 1438 / 1449 / 1706 / 1946 / 2471 / 3391 us with four, 1073 / 1279 / 1560 / 1839 /
-// 2225 / 3613 with eight at d = 256 / 512 / 768 / 1024 / 1280 / 2048.
+// Forward statistics of EpiStats for one slab of rows, plus the logits themselves: kept in fp32 in the slab between the
+// pass that forms them and the point where the row's log-sum-exp and loss coefficients are known, as two 16-bit planes so
+// that the gradient can take the place of the upper halves.  Forming the logits once instead of twice (statistics, then
+// recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  Both planes are seen through one map
+// {columns, rows, planes} with boxes of 32 x 32, 64-byte swizzled.
 constexpr int kEightWarpsMaxKSweep = 1280;
-struct SweepParams {
-  RowStats::Params stats;
-  const float* shift2;   // [rows] compact: estimated log-sum-exp in units of log 2
-};
 template <int W>
 struct EpiSweep {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = W;
   static constexpr int kStagingBytes = kEpiStaging;
-  using Params = SweepParams;
+  using Params = RowStats::Params;
   struct State {
     RowStats::State s;
-    float offset;
     uint32_t n_issued;
     int grow;   // compact row
   };
@@ -221,31 +190,51 @@ struct EpiSweep {
     st.s.s = 0.f;
     st.s.a = 0.f;
     st.s.zy = 0.f;
-    st.s.y = valid ? p.stats.tokens_c[st.grow] : -1;
-    const float sh = valid ? p.shift2[st.grow] : 0.f;
-    st.offset = code_offset(sh);
+    st.s.y = valid ? p.tokens_c[st.grow] : -1;
   }
   __device__ static __forceinline__ void chunk(const Params& p, State& st, int m_tile, int n_tile, int c,
                                                int row_in_tile, int m_rows, const float (&v)[32],
                                                const CUtensorMap* map, uint32_t staging) {
     // a CTA pair may own a 128-row tile that lies wholly past the slab's rows: nothing to write
     if (m_tile * BM >= ((m_rows + BM - 1) / BM) * BM) return;
-    RowStats::chunk(p.stats, st.s, 0, n_tile, c, 0, 0, v, map, staging);
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float2 q = code_words(make_float2(v[2 * i], v[2 * i + 1]), st.offset);
-      w[i] = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x5410);
-    }
+    RowStats::chunk(p, st.s, 0, n_tile, c, 0, 0, v, map, staging);
     const int lane = threadIdx.x & 31;
-    stage_half_box<kStagingBytes / kWarps / kBoxBytes>(w, c, staging, st.n_issued, map, n_tile * BN + c * 32, m_tile * BM + (row_in_tile - lane));
+    constexpr int kBufs = kStagingBytes / kWarps / kBoxBytes;
+    const uint32_t buf = staging + (st.n_issued % kBufs) * kBoxBytes;   // 2 KB of upper halves, 2 KB of lower ones
+    // the last stores issued from this buffer must have read it
+    if (lane == 0) bulk_wait_group_read<kBufs - 1>();
+    __syncwarp();
+    // row `lane` of a box is 64 bytes = 4 chunks of 8 values; chunk j sits at position j ^ ((row >> 1) & 3)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint32_t h[4], l[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t a = __float_as_uint(v[8 * j + 2 * k]), b = __float_as_uint(v[8 * j + 2 * k + 1]);
+        h[k] = __byte_perm(a, b, 0x7632);
+        l[k] = __byte_perm(a, b, 0x5410);
+      }
+      const uint32_t addr = buf + lane * 64u + ((uint32_t(j) ^ (uint32_t(lane >> 1) & 3u)) << 4);
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr + kBoxBytes / 2), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3])
+                   : "memory");
+    }
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      const int col = n_tile * BN + c * 32, row0 = m_tile * BM + (row_in_tile - lane);
+      tma_store_3d(map, buf, col, row0, 0);
+      tma_store_3d(map, buf + kBoxBytes / 2, col, row0, 1);
+      bulk_commit_group();
+    }
+    st.n_issued++;
   }
   static constexpr int kMerge = RowStats::kMerge;
   __device__ static __forceinline__ void pack(const State& st, float (&x)[kMerge]) { RowStats::pack(st.s, x); }
   __device__ static __forceinline__ void merge(State& st, const float (&x)[kMerge]) { RowStats::merge(st.s, x); }
   __device__ static __forceinline__ void end_unit(const Params& p, State& st, int, int nr, int, int) {
     if (st.grow >= 0)
-      p.stats.partials[(size_t)nr * p.stats.part_stride + st.grow] = make_float4(st.s.m, st.s.s, st.s.a, st.s.zy);
+      p.partials[(size_t)nr * p.part_stride + st.grow] = make_float4(st.s.m, st.s.s, st.s.a, st.s.zy);
   }
 };
 
@@ -270,7 +259,6 @@ struct GradParams {
 };
 template <int W>
 struct EpiGrad {
-  static constexpr bool kTileFlags = true;   // redoes single row tiles of the one-sweep path
   static constexpr bool kParts = false;
   static constexpr int kWarps = W;
   static constexpr int kMerge = 0;
@@ -370,7 +358,6 @@ struct EpiGrad {
 // also clips rows past the tensor.  Every element is written by exactly one tile per launch, so
 // the result does not depend on timing.
 struct EpiAcc {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = true;
   static constexpr int kWarps = 4;
   static constexpr int kMerge = 0;

@@ -66,7 +66,6 @@ constexpr int kFewRowTiles = 16;   // row tiles up to which the column split is 
 constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
 constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
-constexpr int kFlagRows = 256;  // rows one entry of GemmShape::tile_flags stands for
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
 
 enum TileMode { kTileSquare = 0, kTileWide = 1, kTileDual = 2 };
@@ -153,10 +152,6 @@ struct GemmShape {
   // walked for one group before the next group starts, so that the A panels the CTAs running at any
   // moment keep re-reading stay in L2; B is then fetched once per group instead of once per launch.
   int m_group;
-  // Row-tile selection: when tile_flags is set, only row tiles whose flag (indexed from the slab's first row, one per
-  // kFlagRows rows) is non-zero are walked, and the launch returns at once when *flag_count is 0.
-  const int* tile_flags;
-  const int* flag_count;
   // coordinate offsets into the operands' global tensors
   int a_mn_off, a_k_off, b_mn_off, b_k_off;
 };
@@ -209,7 +204,6 @@ __host__ __device__ inline int choose_range(int m_units, int n_tiles, int n_work
 }
 
 struct GemmExtents {
-  int tile_rows;   // rows of one row tile (BM x CTAs per tile)
   int m_rows, m_units, k_blocks, n_range, n_ranges, n_units, slab_off, k_split, kb_per, stream_k, m_group;
   int cut, cut_parts, cut_len;   // stream_k == 2: tiles that are cut, parts each, k-blocks of a part (0: all of its range)
 };
@@ -293,7 +287,6 @@ __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_v
   e.m_rows = sh.m_dyn ? m : sh.m_rows_cap;
   k = k < 0 ? 0 : (k > sh.k_cap ? sh.k_cap : k);
   const int k_len = sh.k_dyn ? k : sh.k_cap;
-  e.tile_rows = BM * cg;
   e.m_units = (e.m_rows + BM * cg - 1) / (BM * cg);
   e.k_blocks = (k_len + BK - 1) / BK;
   const int smax = sh.n_split_max > 0 ? sh.n_split_max : kMaxSplit;
@@ -361,8 +354,6 @@ __host__ __device__ inline void unit_coords(const GemmShape& sh, const GemmExten
 // tile-major, are cut into one contiguous share per worker, one unit per tile a share touches; ks
 // is then the output slice of the part: 0 when it starts at k-block 0, else 1.  stream_k == 2: full waves, then this
 // worker's parts of cut tiles (cut_tiles); ks is 0 for a whole tile, else 1 + the slot of the part.
-// FLAGS: row tiles whose GemmShape::tile_flags entry is zero are passed over.
-template <bool FLAGS = false>
 struct UnitWalk {
   const GemmShape& sh;
   const GemmExtents& ex;
@@ -389,10 +380,9 @@ struct UnitWalk {
     }
   }
   __host__ __device__ inline bool next(int& mu, int& nr, int& ks, int& kb0, int& kb1) {
-    while (u < plain_units) {
+    if (u < plain_units) {
       unit_coords(sh, ex, u, mu, nr, ks, kb0, kb1);
       u += n_workers;
-      if (FLAGS && sh.tile_flags && !sh.tile_flags[(ex.slab_off + mu * ex.tile_rows) / kFlagRows]) continue;
       return true;
     }
     if (it >= it_end) return false;
@@ -447,7 +437,6 @@ struct UnitWalk {
 //     static constexpr int kMerge;                             // floats of state that pack() hands to the other half's
 //     static void pack(const State&, float (&)[kMerge]); static void merge(State&, const float (&)[kMerge]);   // if > 0
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
-//     static constexpr bool kTileFlags;                        // launches may be restricted by GemmShape::tile_flags
 //     static constexpr bool kParts; };                         // knows what to do with parts of tiles (stream_k == 2)
 //   kTileDual: chunk receives the chunk of the second product as well (..., v, v2, out_map, staging).
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
@@ -458,10 +447,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
             const typename Epi::Params ep, DevStatus* status) {
-  if (Epi::kTileFlags && sh.flag_count) {
-    chain_wait();
-    if (*sh.flag_count == 0) return;   // no flagged row tile
-  }
   static_assert(MODE != kTileWide || CG == 2, "wide tiles run on CTA pairs");
   static_assert(MODE != kTileDual || (A_MN == 0 && B_MN == 0), "the two-product mode takes K-major operands");
   using Cfg = StageCfg<CG, MODE, Epi::kStagingBytes>;
@@ -531,7 +516,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
+      UnitWalk walk(sh, ex, worker, n_workers);
       int mu, nr, ks, kb0, kb1;
       while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
         const int m = mu * CG + (int)rank;
@@ -618,7 +603,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       uint32_t t = 0;   // tiles issued so far
       bool ok = true;
       if (run && ex.k_blocks > 0) {
-        UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
+        UnitWalk walk(sh, ex, worker, n_workers);
         int mu, nr, ks, kb0, kb1;
         while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
           if (kb1 <= kb0) continue;   // empty K slice: the epilogue handles it without an accumulator
@@ -697,7 +682,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     Epi::init(st);
     uint32_t t = 0;
     bool ok = true;
-    UnitWalk<Epi::kTileFlags> walk(sh, ex, worker, n_workers);
+    UnitWalk walk(sh, ex, worker, n_workers);
     int mu, nr, ks, kb0, kb1;
     while (ok && run && walk.next(mu, nr, ks, kb0, kb1)) {
       const bool has_k = kb1 > kb0;   // an empty K slice contributes zeros

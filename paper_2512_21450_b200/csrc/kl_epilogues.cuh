@@ -13,7 +13,6 @@ namespace rlh {
 // Eight epilogue warps in all passes of the full KL: their epilogues are the heavy ones (d = d_ref = 256 / 512 / 704 / 2048:
 // statistics 1200 / 1474 / 1858 / 4775 us with four, 985 / 1246 / 1607 / 4395 with eight).
 struct EpiStatsKL {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
@@ -141,7 +140,6 @@ __device__ __forceinline__ void st_planes(const float (&v)[32], uint16_t* hi, ui
 // Reference pass: zr to the slab, running max and sum of exp of the reference logits to partials2 = {-, Mr, Sr, -}.
 // A thread holds 32 consecutive columns of its row: four 32-byte stores, every sector written whole.
 struct EpiRefSweep {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
@@ -190,7 +188,6 @@ struct EpiRefSweep {
 // Policy pass: statistics of EpiStats, D = sum_j exp(z_j - M) zr_j (to partials2.x), and the planes of z.  The reference
 // logits of the next 32 columns are loaded while these are worked on.
 struct EpiSweepKL {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
@@ -285,7 +282,6 @@ struct EpiSweepKL {
 //                  + ce_t p_tj (log p_tj + Ent_t),   cb_t = w_t beta,
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
-  static constexpr bool kTileFlags = false;
   static constexpr bool kParts = false;
   static constexpr int kWarps = 8;
   static constexpr int kMerge = 0;

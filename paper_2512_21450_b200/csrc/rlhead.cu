@@ -61,13 +61,13 @@ namespace {
 
 constexpr long long kRowGroupBytes = 36ll << 20;   // A panels walked together by the rows-first passes (L2 is 126 MB)
 constexpr int kSlabRowsMax = 32768;        // rows of one gradient slab
-// Slab shape when the caller sets none: rows over the WHOLE vocabulary, at most kSlabElements entries, and no more than
-// kSlabRowBytes of compact hidden rows (14080 rows at d = 2048 and 152 K words, 4.3 GB).  A row that is complete in the slab
-// needs its logits formed only once.  Fewer rows per slab mean more passes over dW (8 bytes per entry and slab, beside 10
-// bytes per entry of the slab itself); more rows than L2 keeps make the dW pass re-read them from DRAM (7B-class step:
-// 208 ms with 85 MB of rows per slab, 200 with 57; d = 2560: 178 ms with 70 MB, 173 with 60; 48 MB instead of 58 at d =
-// 2048: 1 % slower; twice the slab: 1-3 % slower on every large step).  Below kSlabRowsMin rows a slab is cut by columns.
-constexpr long long kSlabElements = 1ll << 31;
+// Slab shape when the caller sets none: rows over the WHOLE vocabulary, at most kSlabBytes of them at 4 bytes an entry (8 with
+// the full-distribution KL), and no more than kSlabRowBytes of compact hidden rows.  A row that is complete in the slab
+// needs its logits formed only once.  Fewer rows per slab mean more passes over dW (8 bytes per entry and slab, beside 14
+// bytes per entry of the slab itself): twice kSlabBytes takes 1.5 % off 16896 rows at d = 2048 and adds 1.3 % to 67244 rows
+// at d = 3584.  More rows than L2 keeps make the dW pass re-read them from DRAM (7B-class step: 208 ms with 85 MB of rows
+// per slab, 200 with 57; d = 2560: 178 ms with 70 MB, 173 with 60).  Below kSlabRowsMin rows a slab is cut by columns.
+constexpr long long kSlabBytes = 1ll << 32;
 constexpr long long kSlabRowBytes = 58ll << 20;
 constexpr int kSlabRowsMin = 2048;
 // Device words a context owns besides the workspace: the status record, a few scalars of the small kernels
@@ -100,8 +100,10 @@ inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_s
 // twice.  The former trades 4 d + 4 d_ref tensor flops for 14 bytes of traffic per entry.  4096 rows, V = 151936: logits and
 // their gradient take 3.3 / 3.5 / 4.9 / 8.3 ms against 2.5 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
 constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
-constexpr int kKlEntryBytes = 8;         // two fp32 logits per slab entry
 inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
+// Bytes of a slab entry: fp32 logits that wait for the loss (two of them with the full KL) and leave room for the bf16
+// gradient, or the gradient alone.
+inline int slab_entry_bytes(int64_t d, int64_t d_ref) { return d_ref == 0 ? 4 : kl_one_sweep(d, d_ref) ? 8 : 2; }
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
 // tile that is half empty costs as much as a full one.  For dH, whose K is the vocabulary: 7 % of the pass (8.59 / 53.1 /
 // 58.9 ms against 9.35 / 57.3 / 63.1 at d = 2048 / 2560 / 3584).  Not for dW, whose K is a slab of rows: 256 x 256 tiles
@@ -122,12 +124,13 @@ struct WsLayout {
   int Tc;             // rows of a slab when there are several
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
   size_t row_pos;                                    // position of every row in the row map (large T)
-  size_t shift2, flags;                              // one-sweep path: log-sum-exp estimates, row-tile flags
+  bool keeps_logits;                                 // one-sweep path: G's place first holds the upper halves of fp32 logits,
+                                                     // the plane behind it their lower halves
   int part_ranges;                                   // column ranges per row that the partials have room for
   size_t dH_slots;                                   // parts of cut dH tiles (0: none)
-  int n_row_slabs, n_flags;                          // n_flags: row tiles, then one count per row slab
+  int n_row_slabs;
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
-  size_t zr, z_lo;                                   // its one-sweep form (0: two-product tiles)
+  size_t zr;                                         // the reference's logits of the slab (one-sweep form)
 };
 
 // Reference-model operands of the full-distribution KL (all NULL / 0 when it is not used).
@@ -175,9 +178,9 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   long long rows = c->slab_rows, one = 0;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
   if (c->slab_auto) {
-    // as many rows as kSlabElements allows (a quarter where a slab entry takes 8 bytes), and no more than
-    // keep the compact rows, which the dW pass reads once per row panel of dW, in L2 beside the streamed slab
-    long long whole = kSlabElements * 2 / (kl_one_sweep(d, d_ref) ? kKlEntryBytes : 2) / Vpad / 256 * 256;
+    // as many rows as kSlabBytes allows, and no more than keep the compact rows, which the dW pass reads once per row
+    // panel of dW, in L2 beside the streamed slab
+    long long whole = kSlabBytes / slab_entry_bytes(d, d_ref) / Vpad / 256 * 256;
     long long resident = kSlabRowBytes / (d * 2) / 256 * 256;
     if (resident < kSlabRowsMin) resident = kSlabRowsMin;
     if (whole >= kSlabRowsMin || whole >= L.Tpad) {
@@ -219,24 +222,19 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   }
   L.block_sums = take((size_t)kMergeBlocks * (1 + L.n_row_slabs) * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
-  L.G = take((size_t)L.Ts * L.Vs * 2);
+  L.keeps_logits = L.Vs == Vpad && slab_entry_bytes(d, d_ref) >= 4;
+  L.G = take((size_t)L.Ts * L.Vs * (L.keeps_logits ? 4 : 2));
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
   L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
-  L.shift2 = take((size_t)L.Tpad * 4);
   L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
-  L.n_flags = L.Tpad / kFlagRows + 1 + L.n_row_slabs;
-  L.flags = take((size_t)L.n_flags * 4);
-  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = L.z_lo = 0;
+  L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
     L.partials2 = take((size_t)n_part_ranges * L.Tpad * sizeof(float4));
     L.lse_ref_c = take((size_t)L.Tpad * 4);
     L.kl_c = take((size_t)L.Tpad * 4);
     L.cb_c = take((size_t)L.Tpad * 4);
-    if (L.Vs == Vpad && kl_one_sweep(d, d_ref)) {
-      L.zr = take((size_t)L.Ts * L.Vs * 4);
-      L.z_lo = take((size_t)L.Ts * L.Vs * 2);
-    }
+    if (L.keeps_logits) L.zr = take((size_t)L.Ts * L.Vs * 4);
   }
   L.staging = o;
   o += (size_t)host_slots * carve_stage(nullptr, T, d, nullptr);
@@ -289,6 +287,17 @@ bool map_out_bf16(rl_ctx* c, CUtensorMap* m, const void* base, uint64_t rows, ui
   cuuint32_t es[2] = {1, 1};
   return c->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The slab's two 16-bit planes of fp32 logits, rows * ld elements apart, written by the logit pass in 32 x 32 boxes, 64-byte swizzled.
+bool map_out_planes(rl_ctx* c, CUtensorMap* m, const void* base, uint64_t rows, uint64_t ld) {
+  cuuint64_t dims[3] = {ld, rows, 2};
+  cuuint64_t strides[2] = {ld * 2, rows * ld * 2};
+  cuuint32_t box[3] = {32, 32, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return c->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -472,7 +481,6 @@ struct FwdPlan {
   bool stats = true;         // tensor-core pass that leaves per-range statistics in the workspace
   int64_t vocab_off = 0;     // first vocabulary id of W's rows (vocabulary-parallel head)
   int64_t V_total = 0;       // size of the whole vocabulary for the token-range check (0: V)
-  const float* old_logp = nullptr;   // one-sweep path: estimate every row's log-sum-exp while its row is copied
   RowOutputs out = {};       // per-row outputs of the call, zeroed where the mask is 0
 };
 
@@ -486,15 +494,6 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   __nv_bfloat16* Hc = reinterpret_cast<__nv_bfloat16*>(ws + L.Hc);
   PrepParams pp;
   memset(&pp, 0, sizeof(pp));
-  SweepPrep& sp = pp.sp;
-  if (plan.old_logp) {
-    sp.W = static_cast<const __nv_bfloat16*>(W);
-    sp.ldW = ldW;
-    sp.old_logp = plan.old_logp;
-    sp.shift2 = reinterpret_cast<float*>(ws + L.shift2);
-    sp.flags = reinterpret_cast<int*>(ws + L.flags);
-    sp.n_flags = L.n_flags;
-  }
   pp.H = static_cast<const __nv_bfloat16*>(H);
   pp.ldH = ldH;
   pp.d = (int)d;
@@ -1133,21 +1132,16 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   }
 
   // ---- forward: statistics per (row, vocabulary range).  One sweep: a slab that holds whole rows lets the pass that
-  // forms their logits leave them there as 16-bit codes, which an elementwise pass turns into the gradient once the
-  // rows' coefficients are known.  Not where the coefficients of a row need rows of another slab, nor where the
+  // forms their logits leave them there in fp32, and an elementwise pass turns them into the gradient once the rows'
+  // coefficients are known.  Not where the coefficients of a row need rows of another slab, nor where the
   // statistics come from elsewhere: those paths form the logits a second time.
-  const int Vpad = (int)align_up((size_t)V, 256);
-  const bool sweep = L.Vs == Vpad && !shard && (!o.kl_full || L.zr) &&
-                     (L.n_row_slabs == 1 || (L.Tc % kFlagRows == 0 && !seq_path));
+  const bool sweep = L.keeps_logits && !shard && (L.n_row_slabs == 1 || !seq_path);
   FwdPlan plan;
   plan.out.dH = dH;
   plan.out.dH_row_bytes = (long long)d * (o.dH_dtype ? 4 : 2);
   plan.out.value[0] = o.logp_out; plan.out.value[1] = o.entropy_out;
   plan.out.value[2] = o.kl_full ? o.kl_out : nullptr;
-  if (sweep) {
-    plan.stats = false;
-    plan.old_logp = o.kl_full ? nullptr : old_logp;
-  }
+  if (sweep) plan.stats = false;
   if (shard) {
     // the statistics of the whole vocabulary are given: only the row compaction is needed
     plan.stats = false;
@@ -1178,7 +1172,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
   p.cp_c = reinterpret_cast<float*>(ws + L.cp_c);
   p.ce_c = reinterpret_cast<float*>(ws + L.ce_c);
-  if (sweep || seq_path) p.logp_c = reinterpret_cast<float*>(ws + L.logp_c);
+  if (seq_path) p.logp_c = reinterpret_cast<float*>(ws + L.logp_c);
   p.logp_out = o.logp_out;
   p.ent_out = o.entropy_out;
   if (shard) {
@@ -1258,7 +1252,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int* n_valid = &c->dstatus->n_valid;
 
   CUtensorMap tmHc_k, tmW_k, tmG_k, tmW_mn, tmG_mn, tmHc_mn, tm_dH, tm_dW, tm_G_out, tmHr_k, tmWr_k, tm_slots, tmW_fwd,
-      tmWr_fwd;
+      tmWr_fwd, tm_planes;
   if (o.kl_full) {
     if (!map_kmajor(c, &tmHr_k, ws + L.Hc_ref, (uint64_t)L.Tpad, (uint64_t)o.d_ref, (uint64_t)o.d_ref, BM) ||
         !map_kmajor(c, &tmWr_k, o.W_ref, (uint64_t)V, (uint64_t)o.d_ref, (uint64_t)o.ldW_ref, b_box_rows(c)))
@@ -1287,6 +1281,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   tmWr_fwd = tmWr_k;
   if (o.kl_full && cg_fwd != c->cta_group)
     ok = ok && map_kmajor(c, &tmWr_fwd, o.W_ref, (uint64_t)V, (uint64_t)o.d_ref, (uint64_t)o.ldW_ref, b_box_rows(cg_fwd));
+  tm_planes = tm_G_out;
+  if (sweep) ok = ok && map_out_planes(c, &tm_planes, G, (uint64_t)L.Ts, (uint64_t)L.Vs);
   if (!ok) return RL_ERR_CUDA;
 
   const int n_row_slabs = L.n_row_slabs;
@@ -1302,10 +1298,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     for (int cs = 0; cs < n_col_slabs; ++cs) {
       const int vocab_base = cs * L.Vs;
       const int cols = (int)((V - vocab_base) < L.Vs ? (V - vocab_base) : L.Vs);
-      // (1) the slab's G = dloss/dlogits as bf16: from the codes of a first pass, or by forming the logits again
+      // (1) the slab's G = dloss/dlogits as bf16: from the logits of a first pass, or by forming them again
       {
-        int* flags = reinterpret_cast<int*>(ws + L.flags);
-        int* flag_count = flags + (L.n_flags - n_row_slabs) + r;
         if (sweep) {
           GemmShape sw;
           memset(&sw, 0, sizeof(sw));
@@ -1319,7 +1313,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           sw.m_group = row_group_tiles(c, d);
           float* zr = reinterpret_cast<float*>(ws + L.zr);
           uint16_t* z_hi = reinterpret_cast<uint16_t*>(G);
-          uint16_t* z_lo = reinterpret_cast<uint16_t*>(ws + L.z_lo);
+          uint16_t* z_lo = z_hi + (size_t)L.Ts * L.Vs;
           if (o.kl_full) {
             GemmShape sr = sw;
             sr.k_cap = (int)o.d_ref;
@@ -1332,15 +1326,14 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             er.ld = L.Vs;
             launch_gemm<EpiRefSweep, 0, 0>(c, cg_fwd, 0, tmHr_k, tmWr_fwd, tm_G_out, tm_G_out, sr, er);
           }
-          SweepParams ep;
-          ep.stats.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
-          ep.stats.partials = reinterpret_cast<float4*>(ws + L.partials);
-          ep.stats.part_stride = L.Tpad;
-          ep.stats.V = (int)V;
-          ep.shift2 = reinterpret_cast<const float*>(ws + L.shift2);
+          RowStats::Params ep;
+          ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
+          ep.partials = reinterpret_cast<float4*>(ws + L.partials);
+          ep.part_stride = L.Tpad;
+          ep.V = (int)V;
           if (o.kl_full) {
             EpiSweepKL::Params ek;
-            ek.stats = ep.stats;
+            ek.stats = ep;
             ek.partials2 = reinterpret_cast<float4*>(ws + L.partials2);
             ek.zr = zr;
             ek.hi = z_hi;
@@ -1348,26 +1341,20 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             ek.ld = L.Vs;
             launch_gemm<EpiSweepKL, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ek);
           } else if (d <= kEightWarpsMaxKSweep) {
-            launch_gemm<EpiSweep<8>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
+            launch_gemm<EpiSweep<8>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_planes, tm_planes, sw, ep);
           } else {
-            launch_gemm<EpiSweep<4>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ep);
+            launch_gemm<EpiSweep<4>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_planes, tm_planes, sw, ep);
           }
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;
-          if (!o.kl_full) {
-            p.shift2 = ep.shift2;
-            p.tile_flags = flags;
-            p.flag_count = flag_count;
-          }
           merge_and_loss(r);
           LogitGradParams lg;
           lg.slab = z_hi;
           lg.ld = L.Vs;
           lg.V = (int)V;
           lg.slab_cap = L.Tc; lg.slab_one = L.Ts; lg.slab_index = r;
-          lg.tokens_c = ep.stats.tokens_c;
-          lg.shift2 = ep.shift2;
-          lg.lse = p.lse_c; lg.logp = p.logp_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
+          lg.tokens_c = ep.tokens_c;
+          lg.lse = p.lse_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
           const int pr_lg = prof_begin(c, 1);
           lg.lo = z_lo;
           lg.zr = zr;
@@ -1382,37 +1369,34 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           else           launch(c, logit_grad_kernel<kGradVecs>, (int)grad_blocks, 256, lg, c->dstatus);
           prof_end(c, pr_lg, 1);
           c->launches++;
-        }
-        GemmShape sh;
-        memset(&sh, 0, sizeof(sh));
-        sh.n_valid = n_valid;
-        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
-        sh.k_cap = (int)d;
-        sh.n_tiles = (cols + BN - 1) / BN;
-        sh.n_range = 0; sh.n_range_lo = 1; sh.n_range_hi = kFwdRange; sh.n_range_always = 1;   // chosen on the device
-        sh.a_mn_slab = 1;
-        sh.b_mn_off = vocab_base;
-        sh.m_group = row_group_tiles(c, d + (o.kl_full ? o.d_ref : 0));
-        if (sweep) {   // only row tiles whose codes could not hold their logits (none as a rule)
-          sh.tile_flags = flags;
-          sh.flag_count = flag_count;
-        }
-        if (!o.kl_full) {
-          GradParams ep;
-          ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
-          ep.lse = p.lse_c; ep.ent = p.ent_c; ep.cp = p.cp_c; ep.ce = p.ce_c;
-          ep.V = (int)V; ep.vocab_base = vocab_base;
-          if (d <= kEightWarpsMaxK)
-            launch_gemm<EpiGrad<8>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
-          else
-            launch_gemm<EpiGrad<4>, 0, 0>(c, c->cta_group, sweep ? -1 : 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
-        } else if (!sweep) {
-          EpiGradKL::Params ep;
-          ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
-          ep.lse = p.lse_c; ep.lse_ref = p.lse_ref_c; ep.ent = p.ent_c; ep.kl = p.kl_c;
-          ep.cp = p.cp_c; ep.cb = p.cb_c; ep.ce = p.ce_c;
-          ep.V = (int)V; ep.vocab_base = vocab_base;
-          launch_dual<EpiGradKL>(c, 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
+        } else {
+          GemmShape sh;
+          memset(&sh, 0, sizeof(sh));
+          sh.n_valid = n_valid;
+          sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
+          sh.k_cap = (int)d;
+          sh.n_tiles = (cols + BN - 1) / BN;
+          sh.n_range = 0; sh.n_range_lo = 1; sh.n_range_hi = kFwdRange; sh.n_range_always = 1;   // chosen on the device
+          sh.a_mn_slab = 1;
+          sh.b_mn_off = vocab_base;
+          sh.m_group = row_group_tiles(c, d + (o.kl_full ? o.d_ref : 0));
+          if (!o.kl_full) {
+            GradParams ep;
+            ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
+            ep.lse = p.lse_c; ep.ent = p.ent_c; ep.cp = p.cp_c; ep.ce = p.ce_c;
+            ep.V = (int)V; ep.vocab_base = vocab_base;
+            if (d <= kEightWarpsMaxK)
+              launch_gemm<EpiGrad<8>, 0, 0>(c, c->cta_group, 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
+            else
+              launch_gemm<EpiGrad<4>, 0, 0>(c, c->cta_group, 1, tmHc_k, tmW_k, tm_G_out, tm_G_out, sh, ep);
+          } else {
+            EpiGradKL::Params ep;
+            ep.tokens_c = reinterpret_cast<const int*>(ws + L.tokens_c);
+            ep.lse = p.lse_c; ep.lse_ref = p.lse_ref_c; ep.ent = p.ent_c; ep.kl = p.kl_c;
+            ep.cp = p.cp_c; ep.cb = p.cb_c; ep.ce = p.ce_c;
+            ep.V = (int)V; ep.vocab_base = vocab_base;
+            launch_dual<EpiGradKL>(c, 1, tmHc_k, tmW_k, tmHr_k, tmWr_k, tm_G_out, sh, (int)o.d_ref, ep);
+          }
         }
       }
       // (2) dH_slab (+)= G * W_slab        [rows x d], K = vocabulary columns of the slab
@@ -1795,7 +1779,7 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
   const GemmExtents ex = gemm_extents(sh, nv, cta_group, n_workers);
   int64_t n = 0;
   for (int worker = 0; worker < n_workers; ++worker) {
-    UnitWalk<> walk(sh, ex, worker, n_workers);
+    UnitWalk walk(sh, ex, worker, n_workers);
     int mu, nr, ks, kb0, kb1;
     while (walk.next(mu, nr, ks, kb0, kb1)) {
       if (n < max_units) {

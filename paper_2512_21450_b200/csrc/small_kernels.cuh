@@ -160,18 +160,6 @@ __global__ void __launch_bounds__(kScanThreads) mask_write_kernel(const uint8_t*
 // negative or too large column that no tile ever matches.  The rows are walked in their original order, so that the
 // outputs of masked rows are zeroed in passing: nothing is cleared that is written again (a memset of dH cost as
 // much as the copy itself, and each memset a launch).
-// SweepPrep (shift2 != NULL): the one-sweep path also needs an estimate of every row's log-sum-exp before its logits are
-// formed.  The behaviour policy supplies it: lse ~ z_y - old_logp, with z_y the sampled token's logit, taken here from
-// the row that is being copied anyway (exact up to the drift between the two policies, which the codes have room for).
-struct SweepPrep {
-  const __nv_bfloat16* W;
-  long long ldW;
-  const float* old_logp;   // [T] original rows
-  float* shift2;           // [rows] compact: the estimate in units of log 2, or NULL
-  int* flags;              // words cleared for the launches that follow
-  int n_flags;
-};
-
 // What a call returns per original row: zeroed where the mask is 0.
 struct RowOutputs {
   void* dH;            // [T][dH_row_bytes], or NULL
@@ -193,7 +181,6 @@ struct PrepParams {
   int* tokens_c;
   int* row_map;           // written by the scanning variant
   const int* row_pos;     // read by the other
-  SweepPrep sp;
   RowOutputs out;
 };
 
@@ -211,34 +198,11 @@ __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, in
   }
   uint4* dst = reinterpret_cast<uint4*>(p.Hc + (size_t)pos * p.d);
   const uint4* src = reinterpret_cast<const uint4*>(p.H + (size_t)t * p.ldH);
-  const int y = p.tokens[t];
-  const bool in_range = y >= 0 && y < p.V;
-  if (p.sp.shift2) {
-    const uint4* wrow = reinterpret_cast<const uint4*>(p.sp.W + (size_t)(in_range ? y : 0) * p.sp.ldW);
-    float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 8
-    for (int v = lane; v < vec_per_row; v += 32) {
-      const uint4 h = __ldg(src + v), w = __ldg(wrow + v);
-      dst[v] = h;
-      const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        acc = __ffma2_rn(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[k])),
-                         __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[k])), acc);
-    }
-    float z = acc.x + acc.y;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if (lane == 0) {
-      const float est = z - p.sp.old_logp[t];
-      // a whole number of code steps, so that the offset the codes are formed with is exact
-      p.sp.shift2[pos] = rintf((isfinite(est) ? est : 0.f) * (kLog2e * kCodeSlope)) * (1.f / kCodeSlope);
-    }
-  } else {
-#pragma unroll 8
-    for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
-  }
+  for (int v = lane; v < vec_per_row; v += 32) dst[v] = __ldg(src + v);
   if (lane == 0) {
+    const int y = p.tokens[t];
+    const bool in_range = y >= 0 && y < p.V;
     p.tokens_c[pos] = in_range ? y - p.vocab_off : -1;
     if (!in_range) latch_status(st, kStatusTokenRange, t);
   }
@@ -251,7 +215,6 @@ template <bool SCAN>
 __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevStatus* st) {
   chain_begin();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.sp.n_flags; i += gridDim.x * blockDim.x) p.sp.flags[i] = 0;
   int n;
   if constexpr (SCAN) {
     __shared__ int warp_sums[32];
@@ -778,12 +741,8 @@ struct LossParams {
   const float* ext_logp;
   const float* ext_ent;
   const float* ext_lse;
-  // one row slab of the one-sweep path (slab_cap > 0): only its rows are merged, and the row tiles whose estimated
-  // log-sum-exp lies too far from the true one for the 16-bit codes are flagged
+  // one row slab of the one-sweep path (slab_cap > 0): only its rows are merged
   int slab_cap, slab_one, slab_index;
-  const float* shift2;
-  int* tile_flags;   // [rows / kFlagRows], over all rows
-  int* flag_count;   // non-zero: this slab has a flagged tile
 };
 // Fixed-order sum of column k of the block partials by one warp: lane l adds blocks l, l + 32, ... in order, then a
 // butterfly over the lanes; the order depends on n_blocks alone, so the result is reproducible.
@@ -870,10 +829,9 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     float lse, logp, ent, kl = 0.f;
     float M = -CUDART_INF_F, S = 0.f, A = 0.f, zy = 0.f, Mr = -CUDART_INF_F, D = 0.f, Sr = 0.f;
     int row = 0;
-    float A_t = 0.f, old_lp = 0.f, ref_lp = 0.f, tw = 0.f, shift2 = 0.f;
+    float A_t = 0.f, old_lp = 0.f, ref_lp = 0.f, tw = 0.f;
     if (warp == 0 && in) {
       row = p.row_map[i];
-      if (p.shift2) shift2 = p.shift2[i];
       if (p.with_loss) {
         A_t = p.adv[row];
         old_lp = p.old_logp[row];
@@ -953,13 +911,6 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
       p.lse_ref_c[i] = lse_ref;
       p.kl_c[i] = kl;
     }
-    if (p.shift2) {
-      // (the comparison is written so that a NaN counts as too far)
-      if (!(fmaf(M, kLog2e, -shift2) <= kCodeTop && fmaf(lse, kLog2e, -shift2) >= kCodeLow)) {
-        p.tile_flags[i / kFlagRows] = 1;
-        *p.flag_count = 1;
-      }
-    }
     if (p.kl_out) p.kl_out[row] = kl;
     p.lse_c[i] = lse;
     p.ent_c[i] = ent;
@@ -1001,30 +952,27 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
 }
 
 // ------------------------------------------------------------------------------------------
-// One-sweep path: the 16-bit codes of a slab's logits become, in place, the bf16 gradient with respect to the logits
-//   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),  log p_tj = code exponent + (estimate - lse_t),
-// rows past the slab's valid rows (up to a multiple of 128) and columns past V become zero.  The sampled token's own
-// entry uses its exact log-probability.  Bound by memory: 2 bytes in and 2 out per entry and nothing read twice.  A
-// warp takes VECS * 256 consecutive columns of one row, all its 16-byte loads in flight before the first is used.  18947 rows
-// x 152064 columns: 2.13 ms, 5.4 TB/s (four loads instead of eight, and one wave of blocks instead of many: 2.32 ms).
-constexpr int kGradVecs = 8;         // 16-byte words per lane and unit of VECS * 256 columns
-constexpr int kGradVecsFew = 4;      // the same with few rows (twice the warps)
-constexpr int kGradVecsKL = 2;       // the KL kernel loads four of them per output
-constexpr long long kGradFewUnits = 65536;   // units of kGradVecs below which it is few: 276 rows 35 us instead of 37
+// One-sweep path: the fp32 logits of a slab become the bf16 gradient with respect to the logits, in the arithmetic of EpiGrad:
+//   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),
+// written in place of their upper halves; rows past the slab's valid rows (up to a multiple of 128) and columns past V
+// become zero.  Bound by memory: 4 bytes in and 2 out per entry and nothing read twice.  A warp takes VECS * 256
+// consecutive columns of one row, all its 16-byte loads in flight before the first is used.
+constexpr int kGradVecs = 4;         // pairs of 16-byte words per lane and unit of VECS * 256 columns
+constexpr int kGradVecsFew = 2;      // the same with few rows (twice the warps)
+constexpr int kGradVecsKL = 2;       // the KL kernel loads four words per output
+constexpr long long kGradFewUnits = 65536;   // units of kGradVecs below which it is few
 struct LogitGradParams {
-  uint16_t* slab;          // [slab rows][ld]
+  uint16_t* slab;          // [slab rows][ld] upper halves of the logits, then the gradient
+  const uint16_t* lo;      // lower halves
   int ld;                  // multiple of 256
   int V;
   int slab_cap, slab_one, slab_index;
   const int* tokens_c;     // per compact row, as the arrays below
-  const float* shift2;
   const float* lse;
-  const float* logp;
   const float* ent;
   const float* cp;
   const float* ce;
-  // full-distribution KL: the slab holds the upper halves of the policy logits, `lo` the lower ones, `zr` the reference's
-  const uint16_t* lo;
+  // full-distribution KL: the reference's logits
   const float* zr;
   const float* lse_ref;
   const float* kl;
@@ -1117,35 +1065,33 @@ __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p
         if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
       continue;
     }
-    uint4 q[VECS];
+    const uint4* low = reinterpret_cast<const uint4*>(p.lo + (size_t)r * p.ld + c0) + lane;
+    uint4 h[VECS], l[VECS];
 #pragma unroll
     for (int k = 0; k < VECS; ++k)
-      if (c0 + k * 256 < p.ld) q[k] = base[k * 32];
+      if (c0 + k * 256 < p.ld) {
+        h[k] = base[k * 32];
+        l[k] = __ldcs(low + k * 32);
+      }
     const int i = off + r;
-    const float lse = p.lse[i], logp = p.logp[i], ent = p.ent[i], cp = p.cp[i], ce = p.ce[i];
+    const float lse = p.lse[i], cp = p.cp[i], ce = p.ce[i], kc = fmaf(ce, p.ent[i], cp);
     const int y = p.tokens_c[i];
-    const float shift = fmaf(-lse, kLog2e, p.shift2[i]);   // log2 p = exponent of the code + shift
-    const float kc = fmaf(ce, ent, cp), kl = ce * kLn2;     // g = p (kc + kl log2 p)
-    // the sampled token's entry from its exact log-probability
-    const float gy = fmaf(ex2_approx(logp * kLog2e), fmaf(ce, logp, kc), -cp);
 #pragma unroll
     for (int k = 0; k < VECS; ++k) {
       const int c = c0 + k * 256 + lane * 8;
       if (c0 + k * 256 >= p.ld) break;
-      const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+      const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, lw[4] = {l[k].x, l[k].y, l[k].z, l[k].w};
       float g[8];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // 0x4B00 above a 16-bit code is the float 2^23 + code
-        const float t0 = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5410))) + shift;
-        const float t1 = code_exponent(__uint_as_float(__byte_perm(w[j], 0x4B00u, 0x5432))) + shift;
-        g[2 * j] = ex2_approx(t0) * fmaf(kl, t0, kc);
-        g[2 * j + 1] = ex2_approx(t1) * fmaf(kl, t1, kc);
+      for (int j = 0; j < 8; ++j) {
+        const float z = __uint_as_float(__byte_perm(lw[j / 2], hw[j / 2], j & 1 ? 0x7632 : 0x5410));
+        const float e = ex2_approx(fmaf(z, kLog2e, -lse * kLog2e));
+        g[j] = ce == 0.f ? e * cp : e * fmaf(ce, z - lse, kc);
       }
       const unsigned rel = (unsigned)(y - c);
       if (rel < 8u) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) g[j] = rel == (unsigned)j ? gy : g[j];
+        for (int j = 0; j < 8; ++j) g[j] = rel == (unsigned)j ? g[j] - cp : g[j];
       }
       if (c + 8 > p.V) {
 #pragma unroll

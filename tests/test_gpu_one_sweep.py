@@ -1,6 +1,6 @@
-"""The one-sweep backward (logits formed once per slab of whole rows, kept as 16-bit codes until the loss coefficients are
-known) where it can go wrong: slab edges, ragged vocabulary tails, and rows whose log-sum-exp is badly estimated by
-their behaviour log-probability, which have to be recomputed.  Oracle and tolerances of the parity tests."""
+"""The one-sweep backward (logits formed once per slab of whole rows and kept in fp32 until the loss coefficients are
+known) where it can go wrong: slab edges, ragged vocabulary tails, rows whose behaviour log-probability is far off.
+Oracle and tolerances of the parity tests; and against the form that makes the logits twice, which holds nothing."""
 import numpy as np
 import pytest
 import torch
@@ -18,14 +18,15 @@ def _rel(a, b):
     return np.linalg.norm(a - b) / np.linalg.norm(b)
 
 
-# the codes hold estimates that are 5.4 nats too low to 9.7 nats too high; beyond that the row tile is recomputed
 @pytest.mark.parametrize("cta_group", [2, 1])
 @pytest.mark.parametrize("rows,V,d,ent,off", [
     (256, 300, 64, 0.0, 0.0),        # slabs of one row tile, one ragged column tile
     (256, 1024, 128, 0.01, 0.0),     # entropy term, vocabulary a whole number of warp units
-    (512, 2085, 192, 0.0, 5.0),      # estimates off by up to 5 nats: still within the codes
-    (512, 1025, 64, 0.01, 20.0),     # single rows far off in both directions: those tiles are recomputed
-    (0, 70001, 64, 0.0, 12.0),       # default limits: one slab, several row tiles of it recomputed
+    (512, 2085, 192, 0.0, 5.0),      # behaviour policy off by 5 nats
+    (512, 1025, 64, 0.01, 20.0),     # single rows far off in both directions
+    (0, 70001, 64, 0.0, 12.0),       # default limits: one slab
+    (128, 1500, 64, 0.01, 0.0),      # slabs of half a row tile
+    (384, 700, 128, 0.0, 0.0),       # slabs of one row tile and a half
 ])
 def test_one_sweep_matches_oracle(cta_group, rows, V, d, ent, off):
     from paper_2512_21450_b200 import Context
@@ -59,15 +60,39 @@ def test_one_sweep_matches_oracle(cta_group, rows, V, d, ent, off):
     m = w.mask.cpu().numpy().astype(bool)
     got, want = _np64(out["dH"]), oo["dH"]
     assert not got[~m].any()
-    # every row by itself: one bf16 rounding per factor, a row that kept wrong codes would be off by its own size
+    # every row by itself: one bf16 rounding per factor
     err, size = np.linalg.norm(got[m] - want[m], axis=1), np.linalg.norm(want[m], axis=1)
     assert (err <= 1e-2 * size + 1e-2 * np.median(size)).all()
     assert _rel(got, want) <= 1e-2 and _rel(_np64(out["dW"]), oo["dW"]) <= 1e-2
 
 
+# What the slab holds between the logit pass and the gradient is the fp32 logits: the gradient is that of the form that makes
+# the logits again from the same operands.  Entropy term alone, so that no entry is larger than its row's others together.
+# The log-sum-exp of a row may differ by its last bits (2e-6 of about 10: another split into column ranges), which turns
+# over the bf16 rounding (spacing 2^-8 to 2^-7) of 2e-6 / 0.0055 = 4e-4 of the entries: sqrt(4e-4) * 0.0055 = 1.1e-4 of G.
+@pytest.mark.parametrize("d,V", [(256, 9000), (1344, 5001)])
+def test_one_sweep_keeps_fp32_logits(d, V):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    w = make_workload(1, prompts=1, L_max=150, d=d, V=V, seed=78)
+    adv = torch.zeros(w.T, device="cuda")
+    outs = []
+    for cols in (0, 2048):
+        c = Context(0)
+        try:
+            c.set_slab_limits(0, cols)
+            outs.append(c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, None, adv, w.mask, 0.2, 0.2, 0.0,
+                                                 ent_coef=0.01, dH_fp32=True))
+            assert c.last_device_status()[0] == 0
+        finally:
+            c.close()
+    a, b = outs
+    assert _rel(_np64(a["dH"]), _np64(b["dH"])) <= 2e-4 and _rel(_np64(a["dW"]), _np64(b["dW"])) <= 2e-4
+
+
 def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
     # the coefficients of a response's rows need all its rows: with more than one row slab the logits are recomputed, and
-    # the result is that of one slab up to fp32 summation order and the rounding of the codes
+    # the result is that of one slab up to fp32 summation order
     from paper_2512_21450_b200 import Context
     from paper_2512_21450_b200.workloads import make_workload
     w = make_workload(1, prompts=1, L_max=150, d=128, V=2000, seed=77)
@@ -90,7 +115,7 @@ def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
 
 # full-distribution KL with the logits of both models formed once: hidden sizes on both sides of the rule that chooses it,
 # slabs of one and several row tiles, a single-CTA case (at most 128 rows), ragged vocabulary, an entropy term, and rows
-# whose codes cannot hold their logits; regulariser alone (adv = 0) so that its own term is what is compared
+# whose behaviour log-probability is far off; regulariser alone (adv = 0) so that its own term is what is compared
 @pytest.mark.parametrize("d,d_ref,V,L_max,rows,off,ent", [
     (768, 768, 1025, 150, 256, 0.0, 0.01), (1472, 64, 2085, 150, 512, 0.0, 0.0), (1408, 64, 2085, 150, 512, 0.0, 0.0),
     (64, 1536, 300, 15, 0, 0.0, 0.0), (768, 1024, 1536, 150, 0, 20.0, 0.0),
