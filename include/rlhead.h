@@ -414,8 +414,8 @@ rl_status rl_policy_loss_fwd_bwd_host_wait(rl_ctx* ctx, int slot, float* loss_ho
  * rl_token_logprobs; everything in between (compacted rows, row map, per-range softmax
  * statistics, the status word) lives in a fixed 16 MiB device array that is part of the library
  * image, so every GPU on which the library is loaded holds those 16 MiB until the process exits.
- *   Limit: the forward scratch, about Tpad*(2*d + 28 + 16*R) + 70 KB bytes with Tpad = T rounded up
- *   to 128 and R = max(16, ceil(ceil(V/256)/8)) vocabulary ranges, must fit in 16 MiB - 256 B (e.g.
+ *   Limit: the forward scratch, about Tpad*(2*d + 28 + 16*R) + 70 KB bytes (and 4*T more from T = 32769
+ *   on) with Tpad = T rounded up to 128 and R = max(16, ceil(ceil(V/256)/8)) vocabulary ranges, must fit in 16 MiB - 256 B (e.g.
  *   T <= 3712 at d = 2048 for V <= 32768; T <= 3072 at d = 2048 and T <= 1664 at d = 4096 for the
  *   151936-word vocabulary, where R = 75); larger
  *   sizes are rejected with RL_ERR_WORKSPACE before anything is enqueued.
@@ -486,6 +486,12 @@ rl_status rl_selftest_cluster_exchange(rl_ctx* ctx, int mode, int cluster_size, 
 rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, int64_t n_tiles, int n_range,
                             int n_fastest, int m_group, int stream_k, int k_split_max, int cta_group,
                             int n_workers, int32_t* units, int64_t max_units, int64_t* n_units);
+/* Host-only view of the workspace layout (works without a GPU; the paper has no counterpart) with default
+ * options on a GPU of n_sm SMs: bytes[0] = what rl_workspace_bytes[_kl] returns (d_ref = 0: no reference model),
+ * bytes[1] = where the arrays that forming log-probabilities uses end, bytes[2] = where the row positions, which only
+ * calls of more than 32768 rows have, end.  static_scratch != 0: as rl_token_logprobs_static lays out its array. */
+rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int n_sm, int static_scratch,
+                             int64_t* bytes);
 
 /* Self-test of the bounded waits every kernel of this library uses: launches one warp that waits,
  * for at most limit_ms (1..1000) milliseconds, on a barrier nothing ever signals.  The kernel

@@ -122,6 +122,8 @@ def load_library():
     lib.rl_debug_schedule.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, c_int, c_int, c_int, c_int, c_int,
                                       P, c_int64, POINTER(c_int64)]
     lib.rl_debug_schedule.restype = c_int
+    lib.rl_debug_workspace.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, POINTER(c_int64)]
+    lib.rl_debug_workspace.restype = c_int
     lib.rl_selftest_cluster_exchange.argtypes = [P, c_int, c_int, c_int, c_int, c_int, POINTER(c_float), POINTER(c_int)]
     lib.rl_selftest_cluster_exchange.restype = c_int
     lib.rl_mask_scan.argtypes = [P, P, c_int64, P, P]
@@ -589,6 +591,13 @@ class Context:
         _check(self.lib.rl_selftest_gemm(self.handle, _ptr(A), _ptr(B), _ptr(C), M, N, K, int(a_mn_major),
                                          int(b_mn_major), int(accumulate)), "rl_selftest_gemm")
         return C
+
+
+def debug_workspace(T, d, V, d_ref=0, n_sm=148, static_scratch=False):
+    """Host-only workspace layout: (bytes of any call, end of the forward arrays, end of the row positions)."""
+    out = (c_int64 * 3)()
+    _check(load_library().rl_debug_workspace(T, d, V, d_ref, n_sm, int(static_scratch), out), "rl_debug_workspace")
+    return tuple(out)
 
 
 def debug_schedule(n_valid, rows_cap, k_len, n_tiles, n_range=1, n_fastest=0, m_group=0, stream_k=0, k_split_max=1,

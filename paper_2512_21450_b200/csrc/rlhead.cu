@@ -123,7 +123,7 @@ struct WsLayout {
   int Tpad, Ts, Vs;   // rows; most rows and columns of a slab
   int Tc;             // rows of a slab when there are several
   size_t scan_counts, row_map, tokens_c, logp_c, lse_c, ent_c, cp_c, ce_c, partials, block_sums, Hc, G, dH_acc, staging, total;
-  size_t row_pos;                                    // position of every row in the row map (large T)
+  size_t row_pos;                                    // position of every row in the row map (T > kPrepRows)
   bool keeps_logits;                                 // one-sweep path: G's place first holds the upper halves of fp32 logits,
                                                      // the plane behind it their lower halves
   int part_ranges;                                   // column ranges per row that the partials have room for
@@ -199,6 +199,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 1024); return at; };
   L.scan_counts = take(((size_t)L.Tpad / 4096 + 2) * 4);
   L.row_map = take((size_t)L.Tpad * 4);
+  L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
   L.tokens_c = take((size_t)L.Tpad * 4);
   L.logp_c = take((size_t)L.Tpad * 4);
   L.lse_c = take((size_t)L.Tpad * 4);
@@ -223,10 +224,10 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.block_sums = take((size_t)kMergeBlocks * (1 + L.n_row_slabs) * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
   L.keeps_logits = L.Vs == Vpad && slab_entry_bytes(d, d_ref) >= 4;
+  // what run_forward() touches lies before this point (without a reference model)
   L.G = take((size_t)L.Ts * L.Vs * (L.keeps_logits ? 4 : 2));
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
   L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
-  L.row_pos = take(T > kPrepRows ? (size_t)T * 4 : 0);
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
@@ -1792,6 +1793,26 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
     }
   }
   *n_units = n;
+  return RL_OK;
+}
+
+rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int n_sm, int static_scratch, int64_t* bytes) {
+  if (!bytes || T < 0 || d <= 0 || V <= 0 || d_ref < 0 || n_sm < 2) return RL_ERR_INVALID_ARG;
+  rl_ctx c = {};
+  c.n_sm = n_sm;
+  c.slab_rows = kSlabRowsMax;
+  c.slab_cols = kSlabColsMax;
+  c.slab_auto = static_scratch ? 0 : 1;
+  c.cta_group = static_scratch ? 1 : 2;
+  c.dh_k_slices = 1;
+  c.wide_tiles = static_scratch ? 0 : 1;
+  c.fixed_scratch = static_scratch ? 1 : 0;
+  c.grid_full[1] = n_sm;
+  c.grid_full[2] = n_sm / 2 * 2;
+  const WsLayout L = ws_layout(&c, T, d, V, 0, d_ref);
+  bytes[0] = (int64_t)L.total;
+  bytes[1] = (int64_t)L.G;
+  bytes[2] = (int64_t)(L.row_pos + (T > kPrepRows ? (size_t)T * 4 : 0));
   return RL_OK;
 }
 

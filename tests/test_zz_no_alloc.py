@@ -110,3 +110,33 @@ def test_static_entry_with_no_rows_clears_the_status_words():
                              torch.zeros(0, device="cuda"), dev_status=st)
     torch.cuda.synchronize()
     assert st.cpu().tolist() == [0, 0]
+
+
+def test_static_entry_with_a_mask_scan_of_its_own():
+    # more than 32768 rows of a small head fit the fixed scratch; their row positions must as well
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.binding import debug_workspace, rl_token_logprobs_static
+    T, d, V = 32769, 64, 300
+    _, forward, row_pos_end = debug_workspace(T, d, V, static_scratch=True)
+    assert row_pos_end <= forward <= 2 ** 24 - 256
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    H = torch.randn(T, d, generator=gen, device="cuda").to(torch.bfloat16)
+    W = (0.05 * torch.randn(V, d, generator=gen, device="cuda")).to(torch.bfloat16)
+    tok = torch.randint(0, V, (T,), generator=gen, device="cuda", dtype=torch.int32)
+    mask = (torch.rand(T, generator=gen, device="cuda") < 0.7).to(torch.uint8)
+    ctx = Context(0)
+    try:
+        ref_lp, ref_ent, ref_lse = ctx.rl_token_logprobs(H, W, tok, mask)
+        assert ctx.last_device_status()[0] == 0
+    finally:
+        ctx.close()
+    lp, ent, lse = (torch.full((T,), 7.0, device="cuda") for _ in range(3))
+    st = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+    rl_token_logprobs_static(H, W, tok, mask, lp, ent, lse, st)
+    torch.cuda.synchronize()
+    assert st.cpu().tolist() == [0, 0]
+    for a, b in ((lp, ref_lp), (ent, ref_ent), (lse, ref_lse)):
+        assert (a - b).abs().max().item() <= TOL
+    z = H.double() @ W.double().T
+    want = (z.gather(1, tok[:, None].long())[:, 0] - torch.logsumexp(z, 1)) * mask
+    assert (lp - want).abs().max().item() <= TOL
