@@ -183,7 +183,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
     long long whole = kSlabBytes / slab_entry_bytes(d, d_ref) / Vpad / 256 * 256;
     long long resident = kSlabRowBytes / (d * 2) / 256 * 256;
     if (resident < kSlabRowsMin) resident = kSlabRowsMin;
-    if (whole >= kSlabRowsMin || whole >= L.Tpad) {
+    if (whole >= kSlabRowsMin) {   // whatever T is: a smaller batch must not need more than a larger one
       if (whole > kSlabRowsMax) whole = kSlabRowsMax;
       rows = whole < resident ? whole : resident;
       one = whole < resident * 3 / 2 ? whole : resident * 3 / 512 * 256;
@@ -195,7 +195,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.Tc = L.Tpad < rows ? L.Tpad : (int)rows;
   L.n_row_slabs = L.Tpad <= L.Ts ? 1 : (L.Tpad + L.Tc - 1) / L.Tc;
   size_t o = 0;
-  size_t n_part_ranges = kMaxSplit;
+  size_t n_part_ranges = kMaxSplit, n_partials;
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 1024); return at; };
   L.scan_counts = take(((size_t)L.Tpad / 4096 + 2) * 4);
   L.row_map = take((size_t)L.Tpad * 4);
@@ -212,14 +212,17 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
     const size_t tiles = (size_t)((V + BN - 1) / BN);
     const size_t by_range = (tiles + kFwdRange - 1) / kFwdRange;
     n_part_ranges = by_range > (size_t)kMaxSplit ? by_range : (size_t)kMaxSplit;
+    n_partials = n_part_ranges * L.Tpad;
     if (!c->fixed_scratch) {
-      size_t fill = (size_t)c->n_sm * 512 / L.Tpad;
-      if (fill > (size_t)c->n_sm) fill = c->n_sm;
-      if (fill > tiles) fill = tiles;
+      const size_t most = tiles < (size_t)c->n_sm ? tiles : (size_t)c->n_sm, room = (size_t)c->n_sm * 512;
+      const size_t fill = most * L.Tpad < room ? most : room / L.Tpad;
       if (n_part_ranges < fill) n_part_ranges = fill;
+      // (sized by the room, not by the whole number of ranges that fit it, so that the size does not fall as T grows)
+      const size_t n = most * L.Tpad < room ? most * L.Tpad : room;
+      if (n_partials < n) n_partials = n;
     }
     L.part_ranges = (int)n_part_ranges;
-    L.partials = take(n_part_ranges * L.Tpad * sizeof(float4));
+    L.partials = take(n_partials * sizeof(float4));
   }
   L.block_sums = take((size_t)kMergeBlocks * (1 + L.n_row_slabs) * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
@@ -231,7 +234,7 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
-    L.partials2 = take((size_t)n_part_ranges * L.Tpad * sizeof(float4));
+    L.partials2 = take(n_partials * sizeof(float4));
     L.lse_ref_c = take((size_t)L.Tpad * 4);
     L.kl_c = take((size_t)L.Tpad * 4);
     L.cb_c = take((size_t)L.Tpad * 4);

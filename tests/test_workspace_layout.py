@@ -12,3 +12,18 @@ def test_forward_arrays_end_where_the_slab_starts(T, d, V, static_scratch):
     total, forward, row_pos_end = debug_workspace(T, d, V, static_scratch=static_scratch)
     assert 0 < row_pos_end <= forward <= total
     assert forward >= T * (2 * d + 28 + 16 * 16) + (4 * T if T > 32768 else 0)
+
+
+# the size is promised for any call with at most T rows: it must not fall as T grows, whatever the slab's shape is
+@pytest.mark.parametrize("d,V,d_ref", [(64, 300, 0), (256, 4096, 0), (2048, 151936, 0), (3584, 152064, 0), (2048, 400000, 0),
+                                       (2048, 600000, 0), (2048, 1100000, 0), (64, 5000000, 0), (2048, 151936, 2048),
+                                       (64, 9000, 64), (2048, 300000, 2048), (2048, 600000, 2048), (896, 151936, 0)])
+def test_size_does_not_fall_with_more_rows(d, V, d_ref):
+    from paper_2512_21450_b200.binding import debug_workspace
+    rows = sorted(set(list(range(1, 9000, 61)) + list(range(128, 60000, 1280)) + [32768, 32769, 100000, 2 ** 20]))
+    for n_sm in (148, 132):
+        last = (0, 0)
+        for T in rows:
+            now = debug_workspace(T, d, V, d_ref, n_sm=n_sm)[:2]
+            assert now[0] >= last[0] and now[1] >= last[1], (T, now, last)
+            last = now
