@@ -65,6 +65,10 @@ const char* rl_status_string(rl_status s);
  * size does not grow with T*V beyond one slab: the gradient with respect to the logits, and the fp32
  * logits it is made from, only ever exist for a bounded slab of rows x vocabulary columns. */
 rl_status rl_workspace_bytes(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, size_t* bytes);
+/* What the calls that only score need of it: rl_token_logprobs, rl_token_logprobs_multi (d = the largest of the models')
+ * and rl_shard_logit_stats (V = the rows of W held).  They leave the slab and everything behind it alone: 0.18 GB of
+ * 4.5 at T = 32768, d = 2048, V = 151936. */
+rl_status rl_workspace_bytes_logprobs(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, size_t* bytes);
 /* The same for calls that set rl_loss_opts.kl_full with a reference model of hidden size d_ref (adds the
  * compacted reference rows, five per-row arrays and, from d + d_ref = 1536 on, 4 bytes more per slab entry). */
 rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, int64_t d_ref, size_t* bytes);
@@ -488,7 +492,7 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
                             int n_workers, int32_t* units, int64_t max_units, int64_t* n_units);
 /* Host-only view of the workspace layout (works without a GPU; the paper has no counterpart) with default
  * options on a GPU of n_sm SMs: bytes[0] = what rl_workspace_bytes[_kl] returns (d_ref = 0: no reference model),
- * bytes[1] = where the arrays that forming log-probabilities uses end, bytes[2] = where the row positions, which only
+ * bytes[1] = what rl_workspace_bytes_logprobs returns, where the arrays that forming log-probabilities uses end, bytes[2] = where the row positions, which only
  * calls of more than 32768 rows have, end.  static_scratch != 0: as rl_token_logprobs_static lays out its array. */
 rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int n_sm, int static_scratch,
                              int64_t* bytes);

@@ -74,6 +74,7 @@ def load_library():
     lib.rl_set_stream.argtypes = [P, P]
     lib.rl_workspace_bytes.argtypes = [P, c_int64, c_int64, c_int64, POINTER(c_size_t)]
     lib.rl_workspace_bytes_host.argtypes = [P, c_int64, c_int64, c_int64, POINTER(c_size_t)]
+    lib.rl_workspace_bytes_logprobs.argtypes = [P, c_int64, c_int64, c_int64, POINTER(c_size_t)]
     lib.rl_workspace_bytes_kl.argtypes = [P, c_int64, c_int64, c_int64, c_int64, POINTER(c_size_t)]
     lib.rl_set_workspace.argtypes = [P, P, c_size_t]
     lib.rl_set_slab_limits.argtypes = [P, c_int, c_int]
@@ -145,7 +146,7 @@ def load_library():
                                              POINTER(rl_loss_opts)]
     lib.rl_policy_loss_shard_bwd.restype = c_int
     for name in ("rl_create", "rl_destroy", "rl_set_stream", "rl_workspace_bytes", "rl_workspace_bytes_host",
-                 "rl_workspace_bytes_kl",
+                 "rl_workspace_bytes_kl", "rl_workspace_bytes_logprobs",
                  "rl_set_workspace", "rl_set_slab_limits", "rl_last_device_status", "rl_grpo_advantages", "rl_grpo_advantages_ex",
                  "rl_token_logprobs", "rl_policy_loss_fwd_bwd", "rl_policy_loss_fwd_bwd_ex",
                  "rl_policy_loss_fwd_bwd_host", "rl_selftest_gemm", "rl_launch_count", "rl_set_profiling",
@@ -199,17 +200,18 @@ class Context:
             _check(self.lib.rl_set_stream(self.handle, stream), "rl_set_stream")
             self._stream = stream
 
-    def workspace_bytes(self, T, d, V, host=False, d_ref=0):
+    def workspace_bytes(self, T, d, V, host=False, d_ref=0, scoring=False):
         n = c_size_t()
         if d_ref:
             _check(self.lib.rl_workspace_bytes_kl(self.handle, T, d, V, d_ref, byref(n)), "rl_workspace_bytes_kl")
             return n.value
-        fn = self.lib.rl_workspace_bytes_host if host else self.lib.rl_workspace_bytes
+        fn = (self.lib.rl_workspace_bytes_logprobs if scoring else
+              self.lib.rl_workspace_bytes_host if host else self.lib.rl_workspace_bytes)
         _check(fn(self.handle, T, d, V, byref(n)), "rl_workspace_bytes")
         return n.value
 
-    def ensure_workspace(self, T, d, V, host=False, d_ref=0):
-        need = self.workspace_bytes(T, d, V, host, d_ref)
+    def ensure_workspace(self, T, d, V, host=False, d_ref=0, scoring=False):
+        need = self.workspace_bytes(T, d, V, host, d_ref, scoring)
         if self._ws is None or self._ws.numel() < need:
             self._ws = None
             self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
@@ -287,7 +289,7 @@ class Context:
         V = W.shape[0]
         assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and tokens.dtype == torch.int32
         assert H.stride(1) == 1 and W.stride(1) == 1
-        self.ensure_workspace(T, d, V)
+        self.ensure_workspace(T, d, V, scoring=True)
         logp = torch.empty(T, dtype=torch.float32, device=H.device)
         ent = torch.empty_like(logp)
         lse = torch.empty_like(logp)
@@ -429,7 +431,7 @@ class Context:
             assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and H.shape[0] == T and W.shape[0] == V
             assert H.stride(1) == 1 and W.stride(1) == 1 and H.shape[1] == W.shape[1]
         assert tokens.dtype == torch.int32
-        self.ensure_workspace(T, max(W.shape[1] for W in Ws), V)
+        self.ensure_workspace(T, max(W.shape[1] for W in Ws), V, scoring=True)
         dev = Ws[0].device
         logp = [torch.empty(T, dtype=torch.float32, device=dev) for _ in range(n)]
         ent = [torch.empty(T, dtype=torch.float32, device=dev) for _ in range(n)] if want_entropy else None
@@ -449,7 +451,7 @@ class Context:
         Vs = W_shard.shape[0]
         assert H.dtype == torch.bfloat16 and W_shard.dtype == torch.bfloat16 and tokens.dtype == torch.int32
         assert H.stride(1) == 1 and W_shard.stride(1) == 1
-        self.ensure_workspace(T, d, Vs)
+        self.ensure_workspace(T, d, Vs, scoring=True)
         if stats is None:
             stats = torch.empty(T, 4, dtype=torch.float32, device=H.device)
         assert stats.dtype == torch.float32 and stats.is_contiguous() and stats.numel() == 4 * T

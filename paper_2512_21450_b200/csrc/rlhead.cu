@@ -435,8 +435,8 @@ rl_status check_hw(const void* H, int64_t ldH, const void* W, int64_t ldW, int64
   return RL_OK;
 }
 
-rl_status check_ws(rl_ctx* c, const WsLayout& L) {
-  if (!c->ws || c->ws_bytes < L.total) return RL_ERR_WORKSPACE;
+rl_status check_ws(rl_ctx* c, size_t bytes) {
+  if (!c->ws || c->ws_bytes < bytes) return RL_ERR_WORKSPACE;
   return RL_OK;
 }
 
@@ -715,6 +715,12 @@ rl_status rl_set_stream(rl_ctx* c, void* s) {
 rl_status rl_workspace_bytes(rl_ctx* c, int64_t T, int64_t d, int64_t V, size_t* bytes) {
   if (!c || !bytes || T < 0 || d <= 0 || V <= 0) return RL_ERR_INVALID_ARG;
   *bytes = ws_layout(c, T, d, V, false).total;
+  return RL_OK;
+}
+
+rl_status rl_workspace_bytes_logprobs(rl_ctx* c, int64_t T, int64_t d, int64_t V, size_t* bytes) {
+  if (!c || !bytes || T < 0 || d <= 0 || V <= 0) return RL_ERR_INVALID_ARG;
+  *bytes = ws_layout(c, T, d, V, false).G;
   return RL_OK;
 }
 
@@ -1055,7 +1061,7 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   if (T == 0) return RL_OK;
   if (!tokens || !logp) return RL_ERR_INVALID_ARG;
   const WsLayout L = ws_layout(c, T, d, V, false);
-  if ((s = check_ws(c, L)) != RL_OK) return s;
+  if ((s = check_ws(c, L.G)) != RL_OK) return s;   // the forward arrays
   char* ws = static_cast<char*>(c->ws);
   FwdPlan plan;
   plan.out.value[0] = logp; plan.out.value[1] = entropy; plan.out.value[2] = lse;
@@ -1124,7 +1130,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     klref.d_ref = o.d_ref;
   }
   const WsLayout L = ws_layout(c, T, d, V, false, o.kl_full ? o.d_ref : 0);
-  if ((s = check_ws(c, L)) != RL_OK) return s;
+  if ((s = check_ws(c, L.total)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
   cudaStream_t st = c->stream;
 
@@ -1506,7 +1512,7 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   if (!tokens || !stats) return RL_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(stats) & 15) return RL_ERR_ALIGNMENT;
   const WsLayout L = ws_layout(c, T, d, V_shard, false);
-  if ((s = check_ws(c, L)) != RL_OK) return s;
+  if ((s = check_ws(c, L.G)) != RL_OK) return s;   // the forward arrays
   char* ws = static_cast<char*>(c->ws);
   FwdPlan plan;
   plan.vocab_off = vocab_offset;
@@ -1559,7 +1565,7 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
   if (!tokens) return RL_ERR_INVALID_ARG;
   // one layout for all models: the compacted rows of the widest model fix the offsets
   const WsLayout L = ws_layout(c, T, d_max, V, false);
-  rl_status s = check_ws(c, L);
+  rl_status s = check_ws(c, L.G);   // the forward arrays
   if (s != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
   for (int i = 0; i < n_models; ++i) {
@@ -1680,7 +1686,7 @@ rl_status rl_policy_loss_fwd_bwd_host(rl_ctx* c, const void* H_host, int64_t ldH
   rl_status s = host_step_check(c, a);
   if (s != RL_OK) return s;
   const WsLayout L = ws_layout(c, T, d, V, 1);
-  if ((s = check_ws(c, L)) != RL_OK) return s;
+  if ((s = check_ws(c, L.total)) != RL_OK) return s;
   HostStage hs;
   carve_stage(static_cast<char*>(c->ws) + L.staging, T, d, &hs);
   if ((s = host_step_enqueue(c, hs, c->stream, nullptr, a)) != RL_OK) return s;
@@ -1711,7 +1717,7 @@ rl_status rl_policy_loss_fwd_bwd_host_submit(rl_ctx* c, int slot, const void* H_
   if (s != RL_OK) return s;
   if (slot < 0 || slot > 1 || c->slot_busy[slot]) return RL_ERR_INVALID_ARG;
   const WsLayout L = ws_layout(c, T, d, V, 2);
-  if ((s = check_ws(c, L)) != RL_OK) return s;
+  if ((s = check_ws(c, L.total)) != RL_OK) return s;
   if (!c->copy_stream) {
     // first pipelined call on this context: the copy stream, two events and 64 pinned bytes per slot;
     // all of it or none of it, so that a later call never finds a half-made set

@@ -27,3 +27,41 @@ def test_size_does_not_fall_with_more_rows(d, V, d_ref):
             now = debug_workspace(T, d, V, d_ref, n_sm=n_sm)[:2]
             assert now[0] >= last[0] and now[1] >= last[1], (T, now, last)
             last = now
+
+
+# scoring touches the forward arrays alone: a workspace of just those, with a guard behind it, is enough and stays whole
+@pytest.mark.gpu
+def test_scoring_needs_the_forward_arrays_alone():
+    import torch
+    from paper_2512_21450_b200 import Context, RLHeadError
+    from paper_2512_21450_b200.binding import debug_workspace
+    T, V, d = 300, 5000, (256, 512)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    H = [torch.randn(T, k, generator=gen, device="cuda").to(torch.bfloat16) for k in d]
+    W = [(0.05 * torch.randn(V, k, generator=gen, device="cuda")).to(torch.bfloat16) for k in d]
+    tok = torch.randint(0, V, (T,), generator=gen, device="cuda", dtype=torch.int32)
+    ctx = Context(0)
+    try:
+        need = ctx.workspace_bytes(T, d[1], V, scoring=True)
+        assert need == debug_workspace(T, d[1], V)[1] < ctx.workspace_bytes(T, d[1], V)
+        ws = torch.full((need + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        ctx._ws = ws[:need]
+        logp, _ = ctx.rl_token_logprobs_multi(H, W, tok)
+        one, _, lse = ctx.rl_token_logprobs(H[1], W[1], tok)
+        stats = ctx.rl_shard_logit_stats(H[1], W[1], tok, None, 0, V)
+        assert ctx.last_device_status()[0] == 0 and ctx._ws.data_ptr() == ws.data_ptr()
+        assert (ws[need:] == 0xA5).all()
+        for h, w, lp in zip(H, W, logp):
+            z = h.double() @ w.double().T
+            want = z.gather(1, tok[:, None].long())[:, 0] - torch.logsumexp(z, 1)
+            assert (lp - want).abs().max().item() <= 2e-3
+        assert torch.equal(one, logp[1])
+        assert (stats[:, 0] + stats[:, 1].log() - lse).abs().max().item() <= 1e-5      # fp32, a few last bits of about 10
+        ctx._ws = ws[:need - 1024]
+        ctx.lib.rl_set_workspace(ctx.handle, ws.data_ptr(), need - 1024)
+        with pytest.raises(RLHeadError) as e:                                           # a little less is refused
+            ctx.ensure_workspace = lambda *a, **k: None
+            ctx.rl_token_logprobs(H[1], W[1], tok)
+        assert e.value.status == 4
+    finally:
+        ctx.close()
