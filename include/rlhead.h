@@ -490,6 +490,11 @@ rl_status rl_selftest_cluster_exchange(rl_ctx* ctx, int mode, int cluster_size, 
 rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, int64_t n_tiles, int n_range,
                             int n_fastest, int m_group, int stream_k, int k_split_max, int cta_group,
                             int n_workers, int32_t* units, int64_t max_units, int64_t* n_units);
+/* The reader's side of the same for stream_k = 2 (n_range = 1, n_fastest = 1): the slots that are added up for every cut
+ * tile, in that order, as pairs {tile = row tile * n_tiles + column tile, slot} of int32; slots may be NULL when
+ * max_slots = 0, *n_slots = number of pairs. */
+rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers,
+                              int32_t* slots, int64_t max_slots, int64_t* n_slots);
 /* Host-only view of the workspace layout (works without a GPU; the paper has no counterpart) with default
  * options on a GPU of n_sm SMs: bytes[0] = what rl_workspace_bytes[_kl] returns (d_ref = 0: no reference model),
  * bytes[1] = what rl_workspace_bytes_logprobs returns, where the arrays that forming log-probabilities uses end, bytes[2] = where the row positions, which only

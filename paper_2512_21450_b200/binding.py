@@ -123,6 +123,8 @@ def load_library():
     lib.rl_debug_schedule.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, c_int, c_int, c_int, c_int, c_int,
                                       P, c_int64, POINTER(c_int64)]
     lib.rl_debug_schedule.restype = c_int
+    lib.rl_debug_tile_slots.argtypes = [c_int64, c_int64, c_int64, c_int, c_int, P, c_int64, POINTER(c_int64)]
+    lib.rl_debug_tile_slots.restype = c_int
     lib.rl_debug_workspace.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, POINTER(c_int64)]
     lib.rl_debug_workspace.restype = c_int
     lib.rl_selftest_cluster_exchange.argtypes = [P, c_int, c_int, c_int, c_int, c_int, POINTER(c_float), POINTER(c_int)]
@@ -593,6 +595,17 @@ class Context:
         _check(self.lib.rl_selftest_gemm(self.handle, _ptr(A), _ptr(B), _ptr(C), M, N, K, int(a_mn_major),
                                          int(b_mn_major), int(accumulate)), "rl_selftest_gemm")
         return C
+
+
+def debug_tile_slots(n_valid, k_len, n_tiles, cta_group=2, n_workers=74):
+    """Host-only: pairs (tile, slot) that whoever reads the output of a pass with cut tiles adds up, in order."""
+    import numpy as np
+    lib, n = load_library(), c_int64()
+    args = (n_valid, k_len, n_tiles, cta_group, n_workers)
+    _check(lib.rl_debug_tile_slots(*args, None, 0, byref(n)), "rl_debug_tile_slots")
+    out = np.empty((n.value, 2), dtype=np.int32)
+    _check(lib.rl_debug_tile_slots(*args, out.ctypes.data_as(c_void_p), n.value, byref(n)), "rl_debug_tile_slots")
+    return out
 
 
 def debug_workspace(T, d, V, d_ref=0, n_sm=148, static_scratch=False):

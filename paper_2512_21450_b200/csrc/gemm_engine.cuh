@@ -271,6 +271,19 @@ __host__ __device__ inline int cut_helper(const GemmExtents& e, int n_workers, l
   return (int)(total < (1ll << 31) ? div_floor(x, (int)total) : x / total);
 }
 
+// Where part s of cut tile r lies: slot `main`, and the pieces of its end in slots first .. last (none: first > last).
+struct CutSlots { int main, first, last; };
+__host__ __device__ inline CutSlots cut_slots(const GemmExtents& e, int n_workers, int r, int s) {
+  CutSlots c = {r * e.cut_parts + s, 1, 0};
+  if (e.cut_len > 0) {
+    const long long pos = (long long)r * cut_tile_ends(e);
+    const int base = e.cut * e.cut_parts + c.main;
+    c.first = base + cut_helper(e, n_workers, pos + cut_end_pos(e, s));
+    c.last = base + cut_helper(e, n_workers, pos + cut_end_pos(e, s + 1) - 1);
+  }
+  return c;
+}
+
 // cg = CTAs per output row tile, n_workers = gridDim.x / cg.
 __host__ __device__ inline GemmExtents gemm_extents(const GemmShape& sh, int n_valid, int cg, int n_workers) {
   GemmExtents e;

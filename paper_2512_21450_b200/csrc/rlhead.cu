@@ -1805,6 +1805,39 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
   return RL_OK;
 }
 
+rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers, int32_t* slots,
+                              int64_t max_slots, int64_t* n_slots) {
+  if (!n_slots || n_valid <= 0 || k_len <= 0 || n_tiles <= 0 || n_workers <= 0 || max_slots < 0 ||
+      (cta_group != 1 && cta_group != 2) || (max_slots > 0 && !slots))
+    return RL_ERR_INVALID_ARG;
+  const int nv = (int)n_valid;
+  GemmShape sh;
+  memset(&sh, 0, sizeof(sh));
+  sh.n_valid = &nv;
+  sh.m_rows_cap = nv;
+  sh.m_dyn = 1;
+  sh.k_cap = (int)k_len;
+  sh.n_tiles = (int)n_tiles;
+  sh.n_range = 1;
+  sh.n_fastest = 1;
+  sh.k_split_max = 1;
+  sh.stream_k = 2;
+  const GemmExtents ex = gemm_extents(sh, nv, cta_group, n_workers);
+  int64_t n = 0;
+  auto put = [&](int tile, int slot) {
+    if (n < max_slots) { slots[2 * n] = tile; slots[2 * n + 1] = slot; }
+    ++n;
+  };
+  for (int r = 0; r < ex.cut; ++r)
+    for (int s = 0; s < ex.cut_parts; ++s) {
+      const CutSlots c = cut_slots(ex, n_workers, r, s);
+      put(ex.n_units - ex.cut + r, c.main);
+      for (int h = c.first; h <= c.last; ++h) put(ex.n_units - ex.cut + r, h);
+    }
+  *n_slots = n;
+  return RL_OK;
+}
+
 rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int n_sm, int static_scratch, int64_t* bytes) {
   if (!bytes || T < 0 || d <= 0 || V <= 0 || d_ref < 0 || n_sm < 2) return RL_ERR_INVALID_ARG;
   rl_ctx c = {};

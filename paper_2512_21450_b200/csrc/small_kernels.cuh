@@ -1480,20 +1480,16 @@ __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const
     for (int k = 0; k < 4; ++k) x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int r = i / s.tile_rows * ex.n_ranges + nt - (ex.n_units - ex.cut);
     if (ex.stream_k == 2 && r >= 0) {
-      const int S = ex.cut_parts, mains = ex.cut * S;
+      const int S = ex.cut_parts;
       const size_t slot = (size_t)s.tile_rows * s.tile_cols;
       const float* base = s.slots + (size_t)(i % s.tile_rows) * s.tile_cols;
-      int h0 = 1, h1 = 0;   // lane s: helpers that did the end of part s
-      if (ex.cut_len > 0 && lane < S) {
-        const long long pos = (long long)r * cut_tile_ends(ex);
-        h0 = cut_helper(ex, s.workers, pos + cut_end_pos(ex, lane));
-        h1 = cut_helper(ex, s.workers, pos + cut_end_pos(ex, lane + 1) - 1);
-      }
+      CutSlots at = {0, 1, 0};   // lane s: of part s
+      if (ex.cut_len > 0 && lane < S) at = cut_slots(ex, s.workers, r, lane);
       for (int p = 0; p < S; ++p) {
         add_piece(x, base + slot * (r * S + p), cols, lane);
         if (ex.cut_len > 0) {
-          const int a = __shfl_sync(0xffffffffu, h0, p), b = __shfl_sync(0xffffffffu, h1, p);
-          for (int h = a; h <= b; ++h) add_piece(x, base + slot * (mains + r * S + p + h), cols, lane);
+          const int a = __shfl_sync(0xffffffffu, at.first, p), b = __shfl_sync(0xffffffffu, at.last, p);
+          for (int h = a; h <= b; ++h) add_piece(x, base + slot * h, cols, lane);
         }
       }
     } else {
