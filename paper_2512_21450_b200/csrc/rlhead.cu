@@ -71,7 +71,7 @@ constexpr long long kSlabBytes = 1ll << 32;
 constexpr long long kSlabRowBytes = 58ll << 20;
 constexpr int kSlabRowsMin = 2048;
 // Device words a context owns besides the workspace: the status record, a few scalars of the small kernels
-// (byte 64: batch statistics, 96: longest response, kTicketOffset: ticket counter of the loss kernels), the valid-row
+// (byte 64: batch statistics, 96: longest response, kTicketOffset: ticket counters), the valid-row
 // counts of rl_token_loss and, behind them, its block partials.
 constexpr int kTokenLossBlocks = 1024;
 constexpr size_t kCountOffset = 256;
@@ -80,7 +80,8 @@ constexpr size_t kStatusBytes = kSumsOffset + (size_t)kTokenLossBlocks * kLossSu
 constexpr int kAdvRowsMinGroups = 2048;     // from this many groups on, GRPO advantages run one thread per group
 constexpr int kWideGain = 96;              // time of a 256 x 512 tile, in % of two 256 x 256 tiles of the same K
 constexpr int kMergeBlocks = 512;          // blocks per merge launch when a call makes several (kLossThreads threads each)
-constexpr size_t kTicketOffset = 192;      // in the device block: blocks of a loss kernel that are done (0 between calls)
+constexpr size_t kTicketOffset = 192;      // in the device block: blocks that are done, of the loss kernels of a step (cleared by
+                                           // its row preparation) and of rl_token_loss (one launch: 0 whenever none runs)
 constexpr int kDhSplitMax = 4;             // most K slices (separate fp32 accumulators) of the dH pass
 constexpr int kSlabColsMax = 148 * 256;    // vocabulary columns of one gradient slab (148 tiles of 256: two per SM pair)
 
@@ -510,6 +511,7 @@ rl_status run_forward(rl_ctx* c, const WsLayout& L, const void* H, int64_t ldH, 
   pp.tokens_c = tokens_c;
   pp.row_map = row_map;
   pp.out = plan.out;
+  pp.ticket = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(c->dstatus) + kTicketOffset);
   if (T <= kPrepRows) {
     const int pr = prof_begin(c, 5);
     // a row per warp while that takes no more than four blocks per SM; at most 256: kPrepRows / (4 n_sm)
@@ -988,7 +990,7 @@ rl_status rl_token_loss(rl_ctx* c, const float* logp, const float* entropy, cons
                   reinterpret_cast<uintptr_t>(dentropy);
   const bool vec = (all & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0;
   p.fin.block_sums = block_sums;
-  p.fin.ticket = reinterpret_cast<unsigned*>(base + kTicketOffset);
+  p.fin.ticket = reinterpret_cast<unsigned*>(base + kTicketOffset) + 1;
   p.fin.base = 0;
   p.fin.total = (int)blocks;
   p.fin.loss = loss;

@@ -182,6 +182,7 @@ struct PrepParams {
   int* row_map;           // written by the scanning variant
   const int* row_pos;     // read by the other
   RowOutputs out;
+  unsigned* ticket;       // of the loss kernels that follow: cleared, whatever became of the call before
 };
 
 __device__ __forceinline__ void prep_row(const PrepParams& p, int t, int pos, int lane, DevStatus* st) {
@@ -215,6 +216,7 @@ template <bool SCAN>
 __global__ void __launch_bounds__(256) prep_rows_kernel(const PrepParams p, DevStatus* st) {
   chain_begin();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0;
   int n;
   if constexpr (SCAN) {
     __shared__ int warp_sums[32];

@@ -99,3 +99,34 @@ def test_shaped_returns_of_many_responses(n_seq, mean):
             assert np.all(np.abs(_np64(got) - want) <= 1e-6 + 1e-6 * np.abs(want))
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(agg_mode=1), dict(sequence_level=True)])
+def test_loss_after_a_call_that_failed_half_way(kw):
+    # the block that finishes last is found by a ticket counter in the context's device block; a call of which only some
+    # launches happened leaves it at some count, and the next call's loss must not depend on that
+    import ctypes
+    from cuda.bindings import runtime
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    w = make_workload(1, prompts=1, L_max=150, d=64, V=700, seed=91)
+    adv = torch.randn(w.T, device="cuda")
+    c = Context(0)
+    try:
+        c.set_slab_limits(256, 768)
+        outs = []
+        for left in (0, 3):
+            torch.cuda.synchronize()
+            # the context's fourth member after two ints and the stream: its device block; the counter is 192 bytes in
+            block = ctypes.cast(c.handle, ctypes.POINTER(ctypes.c_void_p))[2]
+            ticket = (ctypes.c_uint * 1)(left)
+            (err,) = runtime.cudaMemcpy(block + 192, ctypes.addressof(ticket), 4, runtime.cudaMemcpyKind.cudaMemcpyHostToDevice)
+            assert int(err) == 0
+            loss = torch.full((1,), float("nan"), device="cuda")
+            outs.append(c.rl_policy_loss_fwd_bwd(w.H, w.W, w.tokens, w.old_logp, w.ref_logp, adv, w.mask, 0.2, 0.2, 0.04,
+                                                 loss=loss, seq_offsets=w.seq_offsets if kw else None, **kw))
+            assert c.last_device_status()[0] == 0
+        assert torch.equal(outs[0]["loss"], outs[1]["loss"]) and torch.equal(outs[0]["metrics"], outs[1]["metrics"])
+        assert torch.isfinite(outs[1]["loss"]).all()
+    finally:
+        c.close()
