@@ -454,7 +454,7 @@ rl_status rl_profile_read(rl_ctx* ctx, double* ms, int64_t* launches);
 /* Self-test of the tensor-core GEMM engine the calls above are built from: C[M,N] (fp32,
  * row-major, ldc = N) = A * B with bf16 operands.  a_mn_major = 0: A is [M,K] row-major;
  * 1: A is stored [K,M] row-major.  b_mn_major = 0: B is stored [N,K] row-major; 1: B is stored
- * [K,N] row-major.  M, N multiples of 64, K a multiple of 8.  The paper has no counterpart; this
+ * [K,N] row-major.  M a multiple of 128, N of 256, K of 8.  The paper has no counterpart; this
  * entry exists so that the operand layouts can be checked against a library product. */
 rl_status rl_selftest_gemm(rl_ctx* ctx, const void* A, const void* B, float* C,
                            int64_t M, int64_t N, int64_t K, int a_mn_major, int b_mn_major,

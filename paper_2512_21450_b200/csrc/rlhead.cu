@@ -648,10 +648,7 @@ rl_status rl_create(rl_ctx** out, int device) {
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
-            set_smem_attr_one<EpiAcc, 0, 0, 2, kTileWide>() == cudaSuccess &&
-            set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess &&
-            set_smem_attr_one<EpiAcc, 1, 0, 2, kTileWide>() == cudaSuccess &&
-            set_smem_attr_one<EpiAcc, 1, 1, 2, kTileWide>() == cudaSuccess;
+            set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess;
   if (!ok) { cudaFree(c->dstatus); delete c; return RL_ERR_CUDA; }
   {
     // how many CTA pairs can be resident at once (pairs must share a TPC): the persistent grid
@@ -1943,12 +1940,9 @@ rl_status rl_selftest_gemm(rl_ctx* c, const void* A, const void* B, float* C, in
   if (!map_out_f32(c, &tc, C, (uint64_t)M, (uint64_t)N, (uint64_t)N, 1, (uint64_t)M)) return RL_ERR_CUDA;
   EpiAcc::Params ep;
   ep.n_cols = (int)N; ep.accumulate = accumulate; ep.row_base = 0; ep.slice_add = 0; ep.tile_cols = 0;
-  if (c->wide_tiles && c->cta_group == 2) {
+  if (c->wide_tiles && c->cta_group == 2 && !a_mn && b_mn) {   // the operand layout of dH, the one pass that has wide tiles
     sh.n_tiles = (int)((N + 2 * BN - 1) / (2 * BN));
-    if (!a_mn && !b_mn) launch_wide<EpiAcc, 0, 0>(c, -1, ta, tb, tc, tc, sh, ep);
-    else if (!a_mn && b_mn) launch_wide<EpiAcc, 0, 1>(c, -1, ta, tb, tc, tc, sh, ep);
-    else if (a_mn && !b_mn) launch_wide<EpiAcc, 1, 0>(c, -1, ta, tb, tc, tc, sh, ep);
-    else launch_wide<EpiAcc, 1, 1>(c, -1, ta, tb, tc, tc, sh, ep);
+    launch_wide<EpiAcc, 0, 1>(c, -1, ta, tb, tc, tc, sh, ep);
   } else if (!a_mn && !b_mn) launch_gemm<EpiAcc, 0, 0>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
   else if (!a_mn && b_mn) launch_gemm<EpiAcc, 0, 1>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
   else if (a_mn && !b_mn) launch_gemm<EpiAcc, 1, 0>(c, c->cta_group, -1, ta, tb, tc, tc, sh, ep);
