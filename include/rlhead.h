@@ -77,8 +77,9 @@ rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, in
  * max_rows a multiple of 128, max_cols a multiple of 256, max_rows * max_cols at most 2^31; 0 for one of
  * them is 32768 rows or 37888 columns.  (0, 0) restores the default: rows over the whole vocabulary, at most
  * 4.3 GB and 58 MB of hidden states (6912 rows at 152 K words), or 32768 x 37888 for vocabularies of which fewer
- * than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary) the loss calls keep the fp32
- * logits there, 4 bytes per entry, and form them once instead of twice: 13-18 % of a step.  Changes what
+ * than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary) and d >= 896 the loss calls keep
+ * the fp32 logits there, 4 bytes per entry, and form them once instead of twice: 13-18 % of a step.  Below that the slab
+ * takes 2 bytes per entry and 4.3 GB hold 14080 rows.  Changes what
  * rl_workspace_bytes() returns: call it first. */
 rl_status rl_set_slab_limits(rl_ctx* ctx, int max_rows, int max_cols);
 /* Tile shape of the tensor-core passes: 1 = one CTA per 128x256 output tile, 2 = CTA pairs

@@ -163,12 +163,12 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // pass that forms them and the point where the row's log-sum-exp and loss coefficients are known, as two 16-bit planes so
 // that the gradient can take the place of the upper halves.  Forming the logits once instead of twice (statistics, then
 // recomputation for the gradient) leaves 6 d V tensor flops per token of 8 d V.  Both planes are seen through one map
-// {columns, rows, planes} with boxes of 32 x 32, 64-byte swizzled.
-constexpr int kEightWarpsMaxKSweep = 1280;
-template <int W>
+// {columns, rows, planes} with boxes of 32 x 32, 64-byte swizzled.  6912 rows x 151936 words: 1.97 / 2.17 / 3.34 / 5.63 ms at
+// d = 896 / 1024 / 2048 / 3584 (eight epilogue warps 1.94 / 2.17 / 3.52 / 5.98; stores straight from registers 1.96 / - / 3.48 / 5.75;
+// the statistics alone 1.36 / 1.65 / 2.85 / 5.16).
 struct EpiSweep {
   static constexpr bool kParts = false;
-  static constexpr int kWarps = W;
+  static constexpr int kWarps = 4;
   static constexpr int kStagingBytes = kEpiStaging;
   using Params = RowStats::Params;
   struct State {

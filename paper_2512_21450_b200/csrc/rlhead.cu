@@ -62,7 +62,7 @@ namespace {
 constexpr long long kRowGroupBytes = 36ll << 20;   // A panels walked together by the rows-first passes (L2 is 126 MB)
 constexpr int kSlabRowsMax = 32768;        // rows of one gradient slab
 // Slab shape when the caller sets none: rows over the WHOLE vocabulary, at most kSlabBytes of them at 4 bytes an entry (8 with
-// the full-distribution KL), and no more than kSlabRowBytes of compact hidden rows.  A row that is complete in the slab
+// the full-distribution KL, 2 for a narrow head), and no more than kSlabRowBytes of compact hidden rows.  A row that is complete in the slab
 // needs its logits formed only once.  Fewer rows per slab mean more passes over dW (8 bytes per entry and slab, beside 14
 // bytes per entry of the slab itself): twice kSlabBytes takes 1.5 % off 16896 rows at d = 2048 and adds 1.3 % to 67244 rows
 // at d = 3584.  More rows than L2 keeps make the dW pass re-read them from DRAM (7B-class step: 208 ms with 85 MB of rows
@@ -102,9 +102,15 @@ inline bool dh_cuts_tiles(const rl_ctx* c) { return !c->dh_stream_k && c->dh_k_s
 // their gradient take 3.3 / 3.5 / 4.9 / 8.3 ms against 2.5 / 4.3 / 8.2 / 17.2 ms at d = d_ref = 512 / 1024 / 2048 / 4096.
 constexpr int64_t kKlSweepMinK = 1536;   // d + d_ref
 inline bool kl_one_sweep(int64_t d, int64_t d_ref) { return d_ref > 0 && d + d_ref >= kKlSweepMinK; }
+// Keeping the logits of a model takes 8 bytes of traffic per entry and a heavier epilogue, forming them again 2 d flops.
+// Logits and their gradient, 6912 rows x 151936 words, kept against formed twice: 1.92 / 2.38 / 2.75 / 2.90 / 3.04 / 3.14 /
+// 3.36 ms against 1.40 / 1.98 / 2.62 / 2.96 / 3.17 / 3.50 / 3.66 at d = 256 / 512 / 768 / 896 / 960 / 1024 / 1152.
+constexpr int64_t kSweepMinK = 896;
 // Bytes of a slab entry: fp32 logits that wait for the loss (two of them with the full KL) and leave room for the bf16
 // gradient, or the gradient alone.
-inline int slab_entry_bytes(int64_t d, int64_t d_ref) { return d_ref == 0 ? 4 : kl_one_sweep(d, d_ref) ? 8 : 2; }
+inline int slab_entry_bytes(int64_t d, int64_t d_ref) {
+  return d_ref > 0 ? (kl_one_sweep(d, d_ref) ? 8 : 2) : (d >= kSweepMinK ? 4 : 2);
+}
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
 // tile that is half empty costs as much as a full one.  For dH, whose K is the vocabulary: 7 % of the pass (8.59 / 53.1 /
 // 58.9 ms against 9.35 / 57.3 / 63.1 at d = 2048 / 2560 / 3584).  Not for dW, whose K is a slab of rows: 256 x 256 tiles
@@ -643,7 +649,7 @@ rl_status rl_create(rl_ctx** out, int device) {
   cudaMemset(c->dstatus, 0, kStatusBytes);
   bool ok = set_smem_attr<EpiStats<4>, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad<4>, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiStats<8>, 0, 0>() == cudaSuccess && set_smem_attr<EpiGrad<8>, 0, 0>() == cudaSuccess &&
-            set_smem_attr<EpiSweep<4>, 0, 0>() == cudaSuccess && set_smem_attr<EpiSweep<8>, 0, 0>() == cudaSuccess && set_smem_attr<EpiRefSweep, 0, 0>() == cudaSuccess &&
+            set_smem_attr<EpiSweep, 0, 0>() == cudaSuccess && set_smem_attr<EpiRefSweep, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiSweepKL, 0, 0>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
@@ -1349,10 +1355,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
             ek.lo = z_lo;
             ek.ld = L.Vs;
             launch_gemm<EpiSweepKL, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_G_out, tm_G_out, sw, ek);
-          } else if (d <= kEightWarpsMaxKSweep) {
-            launch_gemm<EpiSweep<8>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_planes, tm_planes, sw, ep);
           } else {
-            launch_gemm<EpiSweep<4>, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_planes, tm_planes, sw, ep);
+            launch_gemm<EpiSweep, 0, 0>(c, cg_fwd, 0, tmHc_k, tmW_fwd, tm_planes, tm_planes, sw, ep);
           }
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;

@@ -27,6 +27,9 @@ def _rel(a, b):
     (0, 70001, 64, 0.0, 12.0),       # default limits: one slab
     (128, 1500, 64, 0.01, 0.0),      # slabs of half a row tile
     (384, 700, 128, 0.0, 0.0),       # slabs of one row tile and a half
+    # the same for heads wide enough that the logits are kept, above they are formed twice
+    (256, 300, 896, 0.0, 0.0), (256, 1024, 960, 0.01, 0.0), (512, 1025, 896, 0.01, 20.0), (0, 20001, 896, 0.0, 12.0),
+    (128, 1500, 960, 0.01, 0.0), (384, 700, 896, 0.0, 0.0),
 ])
 def test_one_sweep_matches_oracle(cta_group, rows, V, d, ent, off):
     from paper_2512_21450_b200 import Context
@@ -70,7 +73,7 @@ def test_one_sweep_matches_oracle(cta_group, rows, V, d, ent, off):
 # the logits again from the same operands.  Entropy term alone, so that no entry is larger than its row's others together.
 # The log-sum-exp of a row may differ by its last bits (2e-6 of about 10: another split into column ranges), which turns
 # over the bf16 rounding (spacing 2^-8 to 2^-7) of 2e-6 / 0.0055 = 4e-4 of the entries: sqrt(4e-4) * 0.0055 = 1.1e-4 of G.
-@pytest.mark.parametrize("d,V", [(256, 9000), (1344, 5001)])
+@pytest.mark.parametrize("d,V", [(896, 9000), (1344, 5001)])
 def test_one_sweep_keeps_fp32_logits(d, V):
     from paper_2512_21450_b200 import Context
     from paper_2512_21450_b200.workloads import make_workload
