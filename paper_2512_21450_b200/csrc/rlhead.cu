@@ -178,13 +178,16 @@ inline size_t carve_stage(char* base, int64_t T, int64_t d, HostStage* hs) {
 }
 
 // host_slots > 0 adds room for that many sets of host-call inputs behind the scratch proper.
-WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_slots, int64_t d_ref = 0) {
+// by_columns: slabs of many rows and some columns even where whole rows would fit, for calls that form the logits twice
+// whatever the slab's shape is: fewer, longer row slabs for dW (sequence-level ratio against the library that knew column slabs
+// only: 67 thousand rows at d = 3584 1.4 % slower with slabs of whole rows, 2 % faster by columns; 34 thousand at d = 2048 level).
+WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_slots, int64_t d_ref = 0, bool by_columns = false) {
   WsLayout L;
   L.Tpad = (int)align_up((size_t)(T > 0 ? T : 1), 128);
   const int Vpad = (int)align_up((size_t)V, 256);
   long long rows = c->slab_rows, one = 0;
   L.Vs = Vpad < c->slab_cols ? Vpad : c->slab_cols;
-  if (c->slab_auto) {
+  if (c->slab_auto && !by_columns) {
     // as many rows as kSlabBytes allows, and no more than keep the compact rows, which the dW pass reads once per row
     // panel of dW, in L2 beside the streamed slab
     long long whole = kSlabBytes / slab_entry_bytes(d, d_ref) / Vpad / 256 * 256;
@@ -251,6 +254,13 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   o += (size_t)host_slots * carve_stage(nullptr, T, d, nullptr);
   L.total = o;
   return L;
+}
+
+// Workspace of any call without a reference model: a loss per response may need either shape.
+size_t ws_bytes(const rl_ctx* c, int64_t T, int64_t d, int64_t V) {
+  const WsLayout L = ws_layout(c, T, d, V, 0);
+  const size_t twice = L.n_row_slabs > 1 ? ws_layout(c, T, d, V, 0, 0, true).total : 0;
+  return twice > L.total ? twice : L.total;
 }
 
 // K-major operand: global tensor [rows, k] with k contiguous, row stride ld elements.
@@ -719,7 +729,7 @@ rl_status rl_set_stream(rl_ctx* c, void* s) {
 
 rl_status rl_workspace_bytes(rl_ctx* c, int64_t T, int64_t d, int64_t V, size_t* bytes) {
   if (!c || !bytes || T < 0 || d <= 0 || V <= 0) return RL_ERR_INVALID_ARG;
-  *bytes = ws_layout(c, T, d, V, false).total;
+  *bytes = ws_bytes(c, T, d, V);
   return RL_OK;
 }
 
@@ -1134,7 +1144,9 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     klref.W_ref = o.W_ref; klref.ldW_ref = o.ldW_ref;
     klref.d_ref = o.d_ref;
   }
-  const WsLayout L = ws_layout(c, T, d, V, false, o.kl_full ? o.d_ref : 0);
+  WsLayout L = ws_layout(c, T, d, V, 0, o.kl_full ? o.d_ref : 0);
+  // the coefficients of a response's rows need rows of other slabs: the logits are formed twice
+  if (seq_path && L.n_row_slabs > 1) L = ws_layout(c, T, d, V, 0, 0, true);
   if ((s = check_ws(c, L.total)) != RL_OK) return s;
   char* ws = static_cast<char*>(c->ws);
   cudaStream_t st = c->stream;
@@ -1855,7 +1867,7 @@ rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int
   c.grid_full[1] = n_sm;
   c.grid_full[2] = n_sm / 2 * 2;
   const WsLayout L = ws_layout(&c, T, d, V, 0, d_ref);
-  bytes[0] = (int64_t)L.total;
+  bytes[0] = (int64_t)(d_ref > 0 || static_scratch ? L.total : ws_bytes(&c, T, d, V));
   bytes[1] = (int64_t)L.G;
   bytes[2] = (int64_t)(L.row_pos + (T > kPrepRows ? (size_t)T * 4 : 0));
   return RL_OK;
