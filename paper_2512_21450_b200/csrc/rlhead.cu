@@ -180,7 +180,7 @@ inline size_t carve_stage(char* base, int64_t T, int64_t d, HostStage* hs) {
 // host_slots > 0 adds room for that many sets of host-call inputs behind the scratch proper.
 // by_columns: slabs of many rows and some columns even where whole rows would fit, for calls that form the logits twice
 // whatever the slab's shape is: fewer, longer row slabs for dW (sequence-level ratio against the library that knew column slabs
-// only: 67 thousand rows at d = 3584 1.4 % slower with slabs of whole rows, 2 % faster by columns; 34 thousand at d = 2048 level).
+// only: 74 thousand rows at d = 3584 1.4 % slower with slabs of whole rows, up to 2 % faster by columns; 37 thousand at d = 2048 level).
 WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_slots, int64_t d_ref = 0, bool by_columns = false) {
   WsLayout L;
   L.Tpad = (int)align_up((size_t)(T > 0 ? T : 1), 128);

@@ -116,6 +116,32 @@ def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
     assert _rel(_np64(a["dH"]), _np64(b["dH"])) <= 4e-3 and _rel(_np64(a["dW"]), _np64(b["dW"])) <= 4e-3
 
 
+def test_sequence_level_ratio_over_several_slabs_takes_column_slabs():
+    # more rows than a slab of whole rows holds by default (2048 of a million words): the slabs are those of the documented
+    # limits for column slabs, to the bit
+    from paper_2512_21450_b200 import Context
+    T, d, V = 2304, 64, 1000001
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    H = torch.randn(T, d, generator=gen, device="cuda").to(torch.bfloat16)
+    W = (0.1 * torch.randn(V, d, generator=gen, device="cuda")).to(torch.bfloat16)
+    tok = torch.randint(0, V, (T,), generator=gen, device="cuda", dtype=torch.int32)
+    old, adv = torch.full((T,), -14.0, device="cuda"), torch.randn(T, generator=gen, device="cuda")
+    off = torch.arange(0, T + 1, 96, dtype=torch.int32, device="cuda")
+    outs = []
+    for limits in ((0, 0), (32768, 37888)):
+        c = Context(0)
+        try:
+            c.set_slab_limits(*limits)
+            outs.append(c.rl_policy_loss_fwd_bwd(H, W, tok, old, None, adv, None, 0.2, 0.2, 0.0, sequence_level=True,
+                                                 seq_offsets=off))
+            assert c.last_device_status()[0] == 0
+        finally:
+            c.close()
+    assert torch.isfinite(outs[0]["loss"]).all()
+    for key in ("loss", "dH", "dW", "logp", "metrics"):
+        assert torch.equal(outs[0][key], outs[1][key]), key
+
+
 # full-distribution KL with the logits of both models formed once: hidden sizes on both sides of the rule that chooses it,
 # slabs of one and several row tiles, a single-CTA case (at most 128 rows), ragged vocabulary, an entropy term, and rows
 # whose behaviour log-probability is far off; regulariser alone (adv = 0) so that its own term is what is compared
