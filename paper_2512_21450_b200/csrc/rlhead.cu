@@ -78,6 +78,9 @@ constexpr size_t kCountOffset = 256;
 constexpr size_t kSumsOffset = kCountOffset + kCountBlocks * sizeof(unsigned);
 constexpr size_t kStatusBytes = kSumsOffset + (size_t)kTokenLossBlocks * kLossSums * sizeof(double);
 constexpr int kAdvRowsMinGroups = 2048;     // from this many groups on, GRPO advantages run one thread per group
+// Rows up to which the broadcast works the advantages out itself, once per thread and response it meets: one launch of 8.6-11.2 us
+// in place of two of 10.7-15.6 up to 2^19 rows; at 2^20 / 2^21 rows 8.7-36 / 8.7-99 against 10.6-20 / 10.6-21 (16 to 2000 groups of 8 to 32).
+constexpr int64_t kFusedAdvRows = 1 << 19;
 constexpr int kWideGain = 96;              // time of a 256 x 512 tile, in % of two 256 x 256 tiles of the same K
 constexpr int kMergeBlocks = 512;          // blocks per merge launch when a call makes several (kLossThreads threads each)
 constexpr size_t kTicketOffset = 192;      // in the device block: blocks that are done, of the loss kernels of a step (cleared by
@@ -894,8 +897,8 @@ rl_status rl_grpo_advantages_ex(rl_ctx* c, const float* rewards, int64_t n_seq, 
   // many groups of 4, 8, ... 32 responses in 16-byte aligned arrays: one thread per group; else shuffle segments
   const bool rows_path = n_groups >= kAdvRowsMinGroups && group_size % 4 == 0 && group_size <= 32 &&
                          ((reinterpret_cast<uintptr_t>(rewards) | reinterpret_cast<uintptr_t>(adv_seq)) & 15) == 0;
-  // few groups of few responses: the broadcast works the advantages out itself
-  const bool fused = adv_tok && T > 0 && n_groups < kAdvRowsMinGroups && group_size <= 32 && rewards != adv_seq;
+  // few groups of few responses and rows: the broadcast works the advantages out itself
+  const bool fused = adv_tok && T > 0 && T <= kFusedAdvRows && n_groups < kAdvRowsMinGroups && group_size <= 32 && rewards != adv_seq;
   if (fused) {
   } else if (rows_path) {
     const int blocks = (n_groups + 255) / 256;

@@ -55,13 +55,18 @@ def test_loss_per_response(L_max, agg_mode, sequence_level):
         c.close()
 
 
-@pytest.mark.parametrize("n_groups,G", [(1, 2), (2047, 3), (2048, 3), (40, 32), (40, 33)])
+@pytest.mark.parametrize("n_groups,G", [(1, 2), (2047, 3), (2048, 3), (40, 32), (40, 33), (5, 17), (5, 18)])
 def test_advantages_in_the_broadcast(n_groups, G):
     from paper_2512_21450_b200 import Context
     rng = np.random.default_rng(G)
     r = (10 + rng.uniform(size=n_groups * G)).astype(np.float32)
     r[:G] = r[0]
-    off = np.concatenate([[3], 3 + np.cumsum(rng.integers(0, 9, size=r.size))]).astype(np.int32)
+    lens = rng.integers(0, 9, size=r.size)
+    if n_groups == 5:      # the most rows for which the broadcast works them out (17), and one more (18)
+        lens[:40] = (2 ** 19 - 8) // 40
+        lens[40:] = 0
+        lens[-1] = 2 ** 19 - 8 - lens.sum() + (G == 18)
+    off = np.concatenate([[3], 3 + np.cumsum(lens)]).astype(np.int32)
     c = Context(0)
     try:
         seq, tok = c.rl_grpo_advantages(torch.from_numpy(r).cuda(), G, seq_offsets=torch.from_numpy(off).cuda(), T=int(off[-1]) + 5)
