@@ -93,9 +93,15 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // fp32 accumulator buffers of the dH pass: one per K slice, or two when stream-K balancing is on
 inline bool dh_uses_stream_k(const rl_ctx* c) { return c->dh_stream_k && c->dh_k_slices == 1; }
 inline int dh_buffers(const rl_ctx* c) { return dh_uses_stream_k(c) ? 2 : c->dh_k_slices; }
-// Blocks of the merge of `rows` rows, 32 at a time; all launches of a call together have at most kMergeBlocks * (1 + slabs).
-inline int merge_blocks(int64_t rows, int slabs) {
-  const int64_t n = (rows + 31) / 32, most = slabs > 1 ? kMergeBlocks : 2 * kMergeBlocks;
+// The merge of `rows` rows with at most `ranges` column ranges each (0: nothing to merge): a thread per row, else eight warps per
+// 32 rows.  Merge and loss, thread against eight warps: 2 ranges 10.6 / 10.6 / 10.6 / 27 us against 12.1 / 15.0 / 20.9 / 101 at 8 / 16 /
+// 32 / 524 thousand rows, 16 ranges 12.7 / 12.7 / 13.1 / 20.9 against 12.7 / 16.8 / 22.9 / 39.4 at 8 / 16 / 32 / 131 thousand, 75 ranges
+// 14.1 / 22.9 / 25.0 / 24.8 / 39.5 against 11.9 / 12.7 / 18.8 / 26.6 / 42.7 at 4 / 8 / 16 / 32 / 65 thousand.
+inline bool merge_by_thread(int64_t rows, int ranges) { return rows >= (ranges <= kMaxSplit ? 8192 : 32768) || ranges == 0; }
+// Its blocks; all launches of a call together have at most kMergeBlocks * (1 + slabs).
+inline int merge_blocks(int64_t rows, int slabs, int ranges) {
+  const int64_t per = merge_by_thread(rows, ranges) ? kLossThreads : 32;
+  const int64_t n = (rows + per - 1) / per, most = slabs > 1 ? kMergeBlocks : 2 * kMergeBlocks;
   return (int)(n < most ? n : most);
 }
 // Neither option set: the tiles of the dH pass's ragged last wave are cut into parts that lie in slots.
@@ -475,6 +481,13 @@ inline int row_group_tiles(const rl_ctx* c, int64_t k) {
   const long long panel = (long long)BM * c->cta_group * k * 2;
   const long long n = c->row_group_bytes / panel;
   return n < 1 ? 1 : (n > (1 << 20) ? (1 << 20) : (int)n);
+}
+
+void launch_merge(rl_ctx* c, const LossParams& p, int64_t rows, int ranges, int slabs = 1) {
+  const int blocks = merge_blocks(rows, slabs, ranges);
+  if (merge_by_thread(rows, ranges)) launch(c, combine_loss_kernel<1>, blocks, kLossThreads, p, c->dstatus);
+  else                               launch(c, combine_loss_kernel<kLossThreads / 32>, blocks, kLossThreads, p, c->dstatus);
+  c->launches++;
 }
 
 // Compute capability and SM count (cudaGetDeviceProperties takes 2.5 ms, these two queries a microsecond).
@@ -1095,9 +1108,7 @@ rl_status rl_token_logprobs(rl_ctx* c, const void* H, int64_t ldH, const void* W
   p.logp_out = logp;
   p.ent_out = entropy;
   p.lse_out = lse;
-  const int blocks = merge_blocks(T, 1);
-  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
-  c->launches++;
+  launch_merge(c, p, T, L.part_ranges);
   return cuda_ok();
 }
 
@@ -1226,20 +1237,21 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   fin.metrics = o.metrics_out;
   auto merge_and_loss = [&](int r) {
     const int slabs = sweep ? L.n_row_slabs : 1;
-    const int nb = merge_blocks(sweep ? L.Ts : T, slabs);
+    const int64_t rows = sweep ? L.Ts : T;
+    const int ranges = shard ? 0 : L.part_ranges;
+    const int nb = merge_blocks(rows, slabs, ranges);
     const int pr_loss = prof_begin(c, 6);
     if (!seq_path) {
       p.fin = fin;
       p.fin.base = r * nb;
       p.fin.total = slabs * nb;
-      launch(c, combine_loss_kernel, nb, kLossThreads, p, c->dstatus);
-      c->launches++;
+      launch_merge(c, p, rows, ranges, slabs);
     } else {
       // merge the statistics first, then one team per response forms weights, ratios and the loss; valid rows that lie
       // outside every response range take no part: their coefficients stay 0
       p.with_loss = 0;
       p.zero_coef = 1;
-      launch(c, combine_loss_kernel, nb, kLossThreads, p, c->dstatus);
+      launch_merge(c, p, rows, ranges, slabs);
       SeqParams q;
       memset(&q, 0, sizeof(q));
       q.seq_offsets = o.seq_offsets;
@@ -1269,7 +1281,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       q.fin.total = (int)(teams < 1024 ? teams : 1024);
       if (by_block) launch(c, seq_loss_kernel<kLossThreads>, q.fin.total, kLossThreads, q, c->dstatus);
       else          launch(c, seq_loss_kernel<32>, q.fin.total, kLossThreads, q, c->dstatus);
-      c->launches += 2;
+      c->launches++;
     }
     prof_end(c, pr_loss, 6);
   };
@@ -1544,11 +1556,9 @@ rl_status rl_shard_logit_stats(rl_ctx* c, const void* H, int64_t ldH, const void
   p.part_stride = L.Tpad;
   p.row_map = reinterpret_cast<const int*>(ws + L.row_map);
   p.stats_out = reinterpret_cast<float4*>(stats);
-  const int blocks = merge_blocks(T, 1);
   const int pr = prof_begin(c, 6);
-  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
+  launch_merge(c, p, T, L.part_ranges);
   prof_end(c, pr, 6);
-  c->launches++;
   return cuda_ok();
 }
 
@@ -1601,9 +1611,7 @@ rl_status rl_token_logprobs_multi(rl_ctx* c, int n_models, const void* const* H,
     p.ent_c = reinterpret_cast<float*>(ws + L.ent_c);
     p.logp_out = logp[i];
     p.ent_out = entropy ? entropy[i] : nullptr;
-    const int blocks = merge_blocks(T, 1);
-    launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
-    c->launches++;
+    launch_merge(c, p, T, L.part_ranges);
   }
   return cuda_ok();
 }
@@ -2058,8 +2066,7 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
   p.logp_out = logp;
   p.ent_out = entropy;
   p.lse_out = lse;
-  const int blocks = merge_blocks(T, 1);
-  launch(c, combine_loss_kernel, blocks, kLossThreads, p, c->dstatus);
+  launch_merge(c, p, T, L.part_ranges);
   if (dev_status &&
       cudaMemcpyAsync(dev_status, c->dstatus, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
     return RL_ERR_CUDA;

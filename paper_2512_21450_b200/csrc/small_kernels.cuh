@@ -804,16 +804,18 @@ __device__ __forceinline__ void finish_loss(const double (&acc)[kLossSums], cons
   }
 }
 
-// A block takes 32 rows at a time, lane = row; its eight warps share the column ranges (with one thread per row a call of
-// a few hundred rows and 75 to 148 ranges was a chain of that many loads: 17 us) and warp 0 goes on with the sums.  What
-// the loss needs besides is loaded before the merge, one round trip instead of three.
+// A team of kW warps takes 32 rows at a time, lane = row, and shares their column ranges; its first warp goes on with the sums.
+// What the loss needs besides is loaded before the merge, one round trip instead of three.  kW = 8 (a block) where rows are
+// few: with one thread per row a call of a few hundred rows and 75 to 148 ranges was a chain of that many loads, 17 us.
+// kW = 1 where there are rows enough to fill the machine, and where there is nothing to merge (merge_by_thread).
+template <int kW>
 __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossParams p, DevStatus* st) {
   chain_begin();
-  constexpr int kW = kLossThreads / 32;
-  __shared__ float part_s[2][7][kW][32];
+  constexpr int kTeams = kLossThreads / 32 / kW;
+  __shared__ float part_s[2][7][kW][kW > 1 ? 32 : 1];
   const int n = st->n_valid;
   const int n_ranges = p.ext_lse ? 0 : st->n_ranges;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % kW, team = (threadIdx.x >> 5) / kW;
   double acc[kLossSums];
 #pragma unroll
   for (int k = 0; k < kLossSums; ++k) acc[k] = 0.0;
@@ -825,7 +827,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     i_end += i_begin;
   }
   int turn = 0;
-  for (int i0 = i_begin + blockIdx.x * 32; i0 < i_end; i0 += gridDim.x * 32, turn ^= 1) {
+  for (int i0 = i_begin + (blockIdx.x * kTeams + team) * 32; i0 < i_end; i0 += gridDim.x * kTeams * 32, turn ^= 1) {
     const int i = i0 + lane;
     const bool in = i < i_end;
     float lse, logp, ent, kl = 0.f;
@@ -865,39 +867,41 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
         }
         M = m;
       }
-      float (*ps)[kW][32] = part_s[turn];   // the other buffer may still be read by warp 0
-      ps[0][warp][lane] = M;
-      ps[1][warp][lane] = S;
-      ps[2][warp][lane] = A;
-      ps[3][warp][lane] = zy;
-      if (p.kl_full) {
-        ps[4][warp][lane] = D;
-        ps[5][warp][lane] = Mr;
-        ps[6][warp][lane] = Sr;
-      }
-      __syncthreads();
-      if (warp != 0) continue;
-      float Mt = M, Mrt = Mr;
-#pragma unroll
-      for (int w = 1; w < kW; ++w) {
-        Mt = fmaxf(Mt, ps[0][w][lane]);
-        if (p.kl_full) Mrt = fmaxf(Mrt, ps[5][w][lane]);
-      }
-      S = A = zy = D = Sr = 0.f;
-#pragma unroll
-      for (int w = 0; w < kW; ++w) {
-        const float m = ps[0][w][lane], b = m == -CUDART_INF_F ? 0.f : exp2f((m - Mt) * kLog2e);   // -inf: no range
-        S = fmaf(ps[1][w][lane], b, S);
-        A = fmaf(ps[2][w][lane], b, A);
-        zy += ps[3][w][lane];
+      if constexpr (kW > 1) {
+        auto ps = part_s[turn];   // the other buffer may still be read by warp 0
+        ps[0][warp][lane] = M;
+        ps[1][warp][lane] = S;
+        ps[2][warp][lane] = A;
+        ps[3][warp][lane] = zy;
         if (p.kl_full) {
-          const float mr = ps[5][w][lane];
-          D = fmaf(ps[4][w][lane], b, D);
-          Sr = fmaf(ps[6][w][lane], mr == -CUDART_INF_F ? 0.f : exp2f((mr - Mrt) * kLog2e), Sr);
+          ps[4][warp][lane] = D;
+          ps[5][warp][lane] = Mr;
+          ps[6][warp][lane] = Sr;
         }
+        __syncthreads();
+        if (warp != 0) continue;
+        float Mt = M, Mrt = Mr;
+#pragma unroll
+        for (int w = 1; w < kW; ++w) {
+          Mt = fmaxf(Mt, ps[0][w][lane]);
+          if (p.kl_full) Mrt = fmaxf(Mrt, ps[5][w][lane]);
+        }
+        S = A = zy = D = Sr = 0.f;
+#pragma unroll
+        for (int w = 0; w < kW; ++w) {
+          const float m = ps[0][w][lane], b = m == -CUDART_INF_F ? 0.f : exp2f((m - Mt) * kLog2e);   // -inf: no range
+          S = fmaf(ps[1][w][lane], b, S);
+          A = fmaf(ps[2][w][lane], b, A);
+          zy += ps[3][w][lane];
+          if (p.kl_full) {
+            const float mr = ps[5][w][lane];
+            D = fmaf(ps[4][w][lane], b, D);
+            Sr = fmaf(ps[6][w][lane], mr == -CUDART_INF_F ? 0.f : exp2f((mr - Mrt) * kLog2e), Sr);
+          }
+        }
+        M = Mt;
+        Mr = Mrt;
       }
-      M = Mt;
-      Mr = Mrt;
       if (!in) continue;
       if (p.stats_out) {
         p.stats_out[row] = make_float4(M, S, A, zy);

@@ -135,3 +135,19 @@ def test_loss_after_a_call_that_failed_half_way(kw):
         assert torch.isfinite(outs[1]["loss"]).all()
     finally:
         c.close()
+
+
+# the most rows whose statistics are merged by eight warps per 32 rows, and the fewest by a thread per row (8192, few ranges)
+@pytest.mark.parametrize("L_max,kw", [(63, {}), (64, {}), (65, {}), (64, dict(agg_mode=1)), (64, dict(token_weight=True))])
+def test_merge_by_warps_and_by_threads(L_max, kw):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    from tests.test_gpu_parity import _check_against_oracle
+    w = make_workload(1, prompts=16, L_max=L_max, d=64, V=4500, seed=7000 + L_max)
+    if "token_weight" in kw:
+        kw = dict(token_weight=torch.rand(w.T, device="cuda") / w.T)
+    c = Context(0)
+    try:
+        _check_against_oracle(c, w, **kw)
+    finally:
+        c.close()
