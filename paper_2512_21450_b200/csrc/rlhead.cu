@@ -1275,8 +1275,10 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         launch(c, seq_lmax_kernel, 1, 1024, o.seq_offsets, (int)o.n_seq, q.l_max);
         c->launches++;
       }
-      // a block per response unless that would be mostly idle threads
-      const bool by_block = T >= 64 * o.n_seq;
+      // A block per response, else a warp.  Merge and loss, block against warp: 64 responses 16.9 / 18.5 / 22.8 / 34 us against 17.1 /
+      // 21.0 / 43 / 134 at 128 / 256 / 1024 / 4096 rows, 512 responses 22.8 / 25.2 / 34 / 72 against 21.0 / 27.1 / 56 / 204; 1024
+      // responses 31.7 / 38.7 / 45.7 / 53 against 21.0 / 28.6 / 40.0 / 62 at 64 / 256 / 512 / 1024 rows, 8192 responses of 256 rows 190 against 79.
+      const bool by_block = T >= 128 * o.n_seq && (o.n_seq <= (int64_t)c->n_sm * 4 || T >= 1024 * o.n_seq);
       const int64_t teams = by_block ? o.n_seq : (o.n_seq + kLossThreads / 32 - 1) / (kLossThreads / 32);
       q.fin.total = (int)(teams < 1024 ? teams : 1024);
       if (by_block) launch(c, seq_loss_kernel<kLossThreads>, q.fin.total, kLossThreads, q, c->dstatus);

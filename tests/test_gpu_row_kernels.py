@@ -41,15 +41,16 @@ def test_rows_are_scored_in_place_and_masked_rows_are_zero(T, shift):
         c.close()
 
 
-@pytest.mark.parametrize("L_max", [7, 63, 64, 150])    # a warp per response below 64 rows each, a block from there on
+# a warp per response below 128 rows each, a block from there on unless there are more than four responses per SM
+@pytest.mark.parametrize("prompts,L_max", [(3, 7), (3, 63), (3, 64), (3, 127), (3, 128), (3, 150), (75, 128)])
 @pytest.mark.parametrize("agg_mode,sequence_level", [(0, True), (1, False), (2, True)])
-def test_loss_per_response(L_max, agg_mode, sequence_level):
+def test_loss_per_response(prompts, L_max, agg_mode, sequence_level):
     from paper_2512_21450_b200 import Context
     from paper_2512_21450_b200.workloads import make_workload
     from tests.test_gpu_parity import _check_against_oracle
     c = Context(0)
     try:
-        _check_against_oracle(c, make_workload(1, prompts=3, L_max=L_max, d=64, V=500, seed=6000 + L_max, sigma_old=0.3),
+        _check_against_oracle(c, make_workload(1, prompts=prompts, L_max=L_max, d=64, V=500, seed=6000 + L_max, sigma_old=0.3),
                               agg_mode=agg_mode, sequence_level=sequence_level)
     finally:
         c.close()
