@@ -1402,13 +1402,11 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           lg.zr = zr;
           lg.lse_ref = p.lse_ref_c; lg.kl = p.kl_c; lg.cb = p.cb_c;
           const long long padded = (long long)align_up(rows_cap, 128);
-          const bool few = padded * ((L.Vs + 256 * kGradVecs - 1) / (256 * kGradVecs)) < kGradFewUnits;
-          const int unit = 256 * (o.kl_full ? kGradVecsKL : few ? kGradVecsFew : kGradVecs);
+          const int unit = 256 * (o.kl_full ? kGradVecsKL : kGradVecs);
           long long grad_blocks = (padded * ((L.Vs + unit - 1) / unit) + 7) / 8;   // a warp each
           if (grad_blocks > c->n_sm * 64) grad_blocks = c->n_sm * 64;
           if (o.kl_full) launch(c, logit_grad_kl_kernel, (int)grad_blocks, 256, lg, c->dstatus);
-          else if (few)  launch(c, logit_grad_kernel<kGradVecsFew>, (int)grad_blocks, 256, lg, c->dstatus);
-          else           launch(c, logit_grad_kernel<kGradVecs>, (int)grad_blocks, 256, lg, c->dstatus);
+          else           launch(c, logit_grad_kernel, (int)grad_blocks, 256, lg, c->dstatus);
           prof_end(c, pr_lg, 1);
           c->launches++;
         } else {

@@ -961,12 +961,12 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
 // One-sweep path: the fp32 logits of a slab become the bf16 gradient with respect to the logits, in the arithmetic of EpiGrad:
 //   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),
 // written in place of their upper halves; rows past the slab's valid rows (up to a multiple of 128) and columns past V
-// become zero.  Bound by memory: 4 bytes in and 2 out per entry and nothing read twice.  A warp takes VECS * 256
-// consecutive columns of one row, all its 16-byte loads in flight before the first is used.
-constexpr int kGradVecs = 4;         // pairs of 16-byte words per lane and unit of VECS * 256 columns
-constexpr int kGradVecsFew = 2;      // the same with few rows (twice the warps)
-constexpr int kGradVecsKL = 2;       // the KL kernel loads four words per output
-constexpr long long kGradFewUnits = 65536;   // units of kGradVecs below which it is few
+// become zero.  Bound by memory: 4 bytes in and 2 out per entry and nothing read twice.  A warp takes kGradVecs * 256
+// consecutive columns of one row, all its 16-byte loads in flight before the first is used.  151936 columns: 17 / 45 / 146 / 556 /
+// 986 us at 64 / 276 / 1000 / 4000 / 6912 rows, 5.5 TB/s at 276 and 6.3-6.6 from 600 on (two pairs in flight 17 / 49 / 150 / 590 /
+// 1089, eight 17 / 49 / 148 / 565 / 1012).
+constexpr int kGradVecs = 4;         // pairs of 16-byte words per lane and unit of kGradVecs * 256 columns
+constexpr int kGradVecsKL = 2;       // the KL kernel loads four words per output: 68 / 232 / 462 us at 276 / 1000 / 2000 rows (one: 72 / 247 / 481)
 struct LogitGradParams {
   uint16_t* slab;          // [slab rows][ld] upper halves of the logits, then the gradient
   const uint16_t* lo;      // lower halves
@@ -1051,30 +1051,29 @@ __global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParam
   }
 }
 
-template <int VECS>
 __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
   chain_begin();
   int off, rows;
   slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
   const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + (VECS * 256) - 1) / (VECS * 256);
+  const int units_per_row = (p.ld + (kGradVecs * 256) - 1) / (kGradVecs * 256);
   const long long n_units = (long long)rows_pad * units_per_row;
   const int lane = threadIdx.x & 31;
   const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
     const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * (VECS * 256);
+    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecs * 256);
     uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
     if (r >= rows) {
 #pragma unroll
-      for (int k = 0; k < VECS; ++k)
+      for (int k = 0; k < kGradVecs; ++k)
         if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
       continue;
     }
     const uint4* low = reinterpret_cast<const uint4*>(p.lo + (size_t)r * p.ld + c0) + lane;
-    uint4 h[VECS], l[VECS];
+    uint4 h[kGradVecs], l[kGradVecs];
 #pragma unroll
-    for (int k = 0; k < VECS; ++k)
+    for (int k = 0; k < kGradVecs; ++k)
       if (c0 + k * 256 < p.ld) {
         h[k] = base[k * 32];
         l[k] = __ldcs(low + k * 32);
@@ -1083,7 +1082,7 @@ __global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p
     const float lse = p.lse[i], cp = p.cp[i], ce = p.ce[i], kc = fmaf(ce, p.ent[i], cp);
     const int y = p.tokens_c[i];
 #pragma unroll
-    for (int k = 0; k < VECS; ++k) {
+    for (int k = 0; k < kGradVecs; ++k) {
       const int c = c0 + k * 256 + lane * 8;
       if (c0 + k * 256 >= p.ld) break;
       const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, lw[4] = {l[k].x, l[k].y, l[k].z, l[k].w};
