@@ -62,7 +62,9 @@ constexpr int kBoxBytes = 4096;                        // one 32 x 32 fp32 or 32
 constexpr int kEpiStaging = 8 * kBoxBytes;             // of an epilogue that stores boxes: two per warp, or one of eight
 constexpr int kTmemCols = 512;
 constexpr int kMaxSplit = 16;   // most column ranges per row tile unless GemmShape::n_split_max says otherwise
-constexpr int kFewRowTiles = 16;   // row tiles up to which the column split is chosen by waves (choose_split)
+// Row tiles up to which the column split is chosen by waves (choose_split).  Score pass, d = 2048 against 152 K words: 202 / 393 / 595 /
+// 1711 us at 300 / 900 / 1500 / 4096 rows, 202 / 400 / 597 / 1724 by the rule for plenty of work, and level from there on.
+constexpr int kFewRowTiles = 16;
 constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
 constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)

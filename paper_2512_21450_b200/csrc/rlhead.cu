@@ -120,6 +120,11 @@ constexpr int64_t kSweepMinK = 896;
 inline int slab_entry_bytes(int64_t d, int64_t d_ref) {
   return d_ref > 0 ? (kl_one_sweep(d, d_ref) ? 8 : 2) : (d >= kSweepMinK ? 4 : 2);
 }
+// A narrow head keeps them too while they stay in L2, and up to 128 rows, where the logit pass is a stream of W: a whole call,
+// kept against formed twice, 53.8 / 77.3 / 113 us against 58.6 / 79.4 / 106 at d = 256, 4 / 34 / 67 MB of logits (4096 words), 63.5 / 77.5 /
+// 100.5 against 68.3 / 77.3 / 96.9 (16384 words, 17 / 34 / 67 MB), 188 / 192 / 253 against 215 / 200 / 232 at 64 / 128 / 256 rows of 151936 words.
+constexpr size_t kKeepBytes = 40u << 20;
+constexpr int kKeepRows = 128;
 // 256 x 512 tiles: fewer operand bytes per flop, but a tile's epilogue does not overlap the next main loop, and a last
 // tile that is half empty costs as much as a full one.  For dH, whose K is the vocabulary: 7 % of the pass (8.59 / 53.1 /
 // 58.9 ms against 9.35 / 57.3 / 63.1 at d = 2048 / 2560 / 3584).  Not for dW, whose K is a slab of rows: 256 x 256 tiles
@@ -245,9 +250,15 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   }
   L.block_sums = take((size_t)kMergeBlocks * (1 + L.n_row_slabs) * kLossSums * sizeof(double));
   L.Hc = take((size_t)L.Tpad * d * 2);
-  L.keeps_logits = L.Vs == Vpad && slab_entry_bytes(d, d_ref) >= 4;
+  const size_t entries = (size_t)L.Ts * L.Vs;
+  const bool narrow = d_ref == 0 && d < kSweepMinK;
+  const bool small = narrow && L.n_row_slabs == 1 && (L.Tpad <= kKeepRows || entries * 4 <= kKeepBytes);
+  L.keeps_logits = L.Vs == Vpad && (slab_entry_bytes(d, d_ref) >= 4 || small);
+  size_t slab = entries * (L.keeps_logits ? 4 : 2);
+  // (so that the size does not fall where a batch gets too large for its logits to be kept)
+  if (narrow && L.Vs == Vpad && slab < kKeepBytes) slab = entries * 4 < kKeepBytes ? entries * 4 : kKeepBytes;
   // what run_forward() touches lies before this point (without a reference model)
-  L.G = take((size_t)L.Ts * L.Vs * (L.keeps_logits ? 4 : 2));
+  L.G = take(slab);
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
   L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = 0;

@@ -27,7 +27,7 @@ def _rel(a, b):
     (0, 70001, 64, 0.0, 12.0),       # default limits: one slab
     (128, 1500, 64, 0.01, 0.0),      # slabs of half a row tile
     (384, 700, 128, 0.0, 0.0),       # slabs of one row tile and a half
-    # the same for heads wide enough that the logits are kept, above they are formed twice
+    # the same for heads wide enough that the logits are kept with several slabs as well
     (256, 300, 896, 0.0, 0.0), (256, 1024, 960, 0.01, 0.0), (512, 1025, 896, 0.01, 20.0), (0, 20001, 896, 0.0, 12.0),
     (128, 1500, 960, 0.01, 0.0), (384, 700, 896, 0.0, 0.0),
 ])
@@ -114,6 +114,21 @@ def test_sequence_level_ratio_over_several_slabs_forms_logits_twice():
     assert torch.allclose(a["loss"], b["loss"], rtol=1e-5)
     # two roundings to bf16 (2^-9 each) of the same gradient
     assert _rel(_np64(a["dH"]), _np64(b["dH"])) <= 4e-3 and _rel(_np64(a["dW"]), _np64(b["dW"])) <= 4e-3
+
+
+# a narrow head keeps its logits up to 40 MB of them, and up to 128 rows: both sides of the two lines
+@pytest.mark.parametrize("L_max,V", [(16, 90000), (17, 90000), (80, 16384), (80, 16640)])
+def test_narrow_head_on_both_sides_of_the_rule(L_max, V):
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    from tests.test_gpu_parity import _check_against_oracle
+    w = make_workload(1, prompts=1, L_max=L_max, d=64, V=V, seed=8000 + L_max)
+    assert w.T in (128, 136, 640)          # 640 rows x 16384 words x 4 bytes are 40 MB
+    c = Context(0)
+    try:
+        _check_against_oracle(c, w, dH_fp32=True)
+    finally:
+        c.close()
 
 
 def test_sequence_level_ratio_over_several_slabs_takes_column_slabs():
