@@ -22,7 +22,7 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 METRIC = "fused LM-head logprob+GRPO loss fwd+bwd tokens/s; % of bf16 tensor peak"
-KIND_NAMES = ["gemm_kernel<EpiSweep,square> (logits: statistics and codes)", "logit_grad_kernel (codes -> dlogits, HBM bound)",
+KIND_NAMES = ["gemm_kernel<EpiSweep,square> (logits: statistics, kept in fp32)", "logit_grad_kernel (logits -> dlogits, HBM bound)",
               "gemm_kernel<EpiAcc,K,MN,wide> (dH)", "gemm_kernel<EpiAcc,MN,MN,square> (dW)"]
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the tensor-core kernels from one ncu capture
@@ -30,8 +30,8 @@ KIND_NAMES = ["gemm_kernel<EpiSweep,square> (logits: statistics and codes)", "lo
 # for the sources of those kernels (main loop, epilogues, PTX wrappers, small kernels) whose hash is recorded with it.  Bytes
 # per AVERAGE launch of a step.
 KERNEL_SOURCES = ("epilogues.cuh", "gemm_engine.cuh", "ptx.cuh", "small_kernels.cuh")
-NCU_TRAFFIC = {"sources_sha256": "90e82871bb4e166aad8732371092da458a6bfc1d1b3abea8f69c4bf9a0538974", "config": 1,
-               "bytes_per_avg_launch": {0: 2608919000, 1: 3383986000, 2: 6038128000, 3: 4450700000}}
+NCU_TRAFFIC = {"sources_sha256": "974afb17ccff8b4e180740900905df1a9baf4332a7b0028b505c8bea258641f5", "config": 1,
+               "bytes_per_avg_launch": {0: 2600224000, 1: 3048739000, 2: 2320441000, 3: 2605237000}}
 
 
 def sources_hash():
@@ -337,8 +337,7 @@ SEED_STRESS = 251221450 + 99
 def run_reduced_case(args):
     """A reduced copy of the bench workload for profiler captures: same d and distributions, 37888 vocabulary
     rows (W = 155 MB, larger than L2), two prompts (about 4.6 K valid rows), a few steps, nothing timed.
-    Four tensor-core launches per step: the logit pass, the pass that redoes row tiles whose codes could not hold their
-    logits (none here: it returns at once), dH and dW."""
+    Three tensor-core launches per step: the logit pass, dH and dW."""
     import torch
     from paper_2512_21450_b200 import Context
     from paper_2512_21450_b200.workloads import make_workload
@@ -446,14 +445,14 @@ def measure_config(ctx, w, steps, warmup, dev, world=1, reducer=None, token_coun
 
 def kernel_table(w, r, peaks):
     """Per kernel kind: TFLOP/s from the profiling pass (2 d V flop per valid token and tensor-core pass), GB/s for the
-    elementwise pass over the slab (2 bytes read and 2 written per token and vocabulary column)."""
+    elementwise pass over the slab (4 bytes read and 2 written per token and vocabulary column)."""
     flops_step = 2.0 * w.d * w.V * w.n_valid
     out = []
     for k in range(4):
         if r["kind_n"][k]:
             t_ms = r["kind_ms"][k] / r["profile_steps"]
             if k == 1:
-                gbs = 4.0 * w.n_valid * (-(-w.V // 256) * 256) / (t_ms / 1e3) / 1e9
+                gbs = 6.0 * w.n_valid * (-(-w.V // 256) * 256) / (t_ms / 1e3) / 1e9
                 out.append(dict(kernel=KIND_NAMES[k], launches_per_step=r["kind_n"][k] // r["profile_steps"],
                                 ms_per_step=t_ms, gbs=gbs, frac_of_hbm_peak=gbs / peaks["hbm"]))
                 continue

@@ -78,8 +78,8 @@ rl_status rl_workspace_bytes_kl(rl_ctx* ctx, int64_t T, int64_t d, int64_t V, in
  * them is 32768 rows or 37888 columns.  (0, 0) restores the default: rows over the whole vocabulary, at most
  * 4.3 GB and 58 MB of hidden states (6912 rows at 152 K words), or 32768 x 37888 for vocabularies of which fewer
  * than 2048 rows would fit.  With whole rows in the slab (max_cols covers the vocabulary) and d >= 896 the loss calls keep
- * the fp32 logits there, 4 bytes per entry, and form them once instead of twice: 13-18 % of a step.  Below that the slab
- * takes 2 bytes per entry and 4.3 GB hold 14080 rows.  Changes what
+ * the fp32 logits there, 4 bytes per entry, and form them once instead of twice: 8-18 % of a step.  Below that they do so
+ * for 128 rows or 40 MB of logits at most, otherwise the slab takes 2 bytes per entry and 4.3 GB hold 14080 rows.  Changes what
  * rl_workspace_bytes() returns: call it first. */
 rl_status rl_set_slab_limits(rl_ctx* ctx, int max_rows, int max_cols);
 /* Tile shape of the tensor-core passes: 1 = one CTA per 128x256 output tile, 2 = CTA pairs
@@ -111,9 +111,10 @@ rl_status rl_set_wide_tiles(rl_ctx* ctx, int on);
  * Measured: 2 % (16896 rows, d = 2048) to 11 % (32768-row slabs, d = 2560 / 3584) of a step. */
 rl_status rl_set_row_group_bytes(rl_ctx* ctx, int64_t bytes);
 /* Load balancing of the dH pass (default off).  The pass has (row tiles x d/256) output tiles; when
- * that count is not a multiple of the number of SM pairs the last wave of tiles leaves most SMs
- * idle (7.14 waves at d = 2048 with 16896 rows).  With stream-K on, the last full wave and the
- * ragged wave are instead cut, by tile x k-block iterations, into equal contiguous shares, one per
+ * that count is not a multiple of the number of SM pairs the last wave of tiles would leave most SMs
+ * idle (7.14 waves at d = 2048 with 16896 rows).  By default the tiles of that wave alone are cut along K, into parts
+ * that lie in slots and are added when dH is written.  With this option on, the last full wave and the
+ * ragged wave are cut instead, by tile x k-block iterations, into equal contiguous shares, one per
  * SM pair; a tile that straddles two shares is completed in a second fp32 accumulator buffer,
  * summed when dH is written.  Every element still has one writer per buffer and launch, so
  * results stay reproducible run to run.  Costs one extra [slab rows x d] fp32 buffer of
@@ -125,8 +126,9 @@ rl_status rl_set_dh_stream_k(rl_ctx* ctx, int on);
 /* Upper bound on the CTAs of the persistent tensor-core grids (default: one per SM).  A caller that
  * overlaps a collective with the backward pass (sections 4.3 / 4.4: sharded training engines) can
  * leave a few SMs to the collective's kernels this way; an odd bound is rounded down to whole CTA
- * pairs.  0 restores the default.  Results do not depend on it except where the forward pass
- * chooses its vocabulary split from the number of workers (summation order of the merge).
+ * pairs.  0 restores the default.  Results depend on it only in the order of fp32 sums, in two places: the passes that
+ * form logits choose their vocabulary split from the number of workers, and so does dH how it cuts its last tiles into
+ * parts.
  * Errors: max_ctas < 0 or, after rounding, fewer than 2 -> RL_ERR_INVALID_ARG. */
 rl_status rl_set_max_ctas(rl_ctx* ctx, int max_ctas);
 /* Gradient hand-over for data-parallel training (the paper has no kernel-level counterpart; its
