@@ -364,7 +364,9 @@ struct EpiAcc {
   static constexpr int kStagingBytes = kEpiStaging;
   struct Params {
     int n_cols;
-    int accumulate;
+    int accumulate;  // 0 store, 1 add, 2 (slabs walked from the last to the first): add unless this is the last slab that has rows
+    const int* n_valid;                      // 2 only
+    int slab_cap, slab_one, slab_index;
     int row_base;
     int slice_add;   // stream-K launches: output slices past the first are always added to
     int tile_cols;   // > 0: k_slice > 0 names slot k_slice - 1, a box of tile_cols columns x tile_rows rows of its own
@@ -372,6 +374,7 @@ struct EpiAcc {
   };
   struct State {
     int k_slice;
+    int add;
     uint32_t n_issued;   // chunks handed to the TMA unit so far (selects the staging buffer)
   };
   __device__ static __forceinline__ void init(State& st) { st.n_issued = 0; }
@@ -379,8 +382,9 @@ struct EpiAcc {
     if ((threadIdx.x & 31) == 0 && st.n_issued) bulk_wait_group_all();
     __syncwarp();
   }
-  __device__ static __forceinline__ void begin_unit(const Params&, State& st, int, int, int, int, int, int k_slice) {
+  __device__ static __forceinline__ void begin_unit(const Params& p, State& st, int, int, int, int, int, int k_slice) {
     st.k_slice = k_slice;
+    st.add = p.accumulate == 2 ? p.slab_index + 1 < slab_count(*p.n_valid, p.slab_cap, p.slab_one) : p.accumulate;
   }
   __device__ static __forceinline__ void chunk(const Params& p, State& st, int m_tile, int n_tile, int c,
                                                int row_in_tile, int m_rows, const float (&v)[32],
@@ -407,7 +411,7 @@ struct EpiAcc {
     __syncwarp();
     if (lane == 0) {
       if (part) tma_store_3d(tmC, buf, col0 % p.tile_cols, row0 % p.tile_rows, st.k_slice - 1);
-      else if (p.accumulate || (p.slice_add && st.k_slice > 0)) tma_reduce_add_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
+      else if (st.add || (p.slice_add && st.k_slice > 0)) tma_reduce_add_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
       else              tma_store_3d(tmC, buf, col0, p.row_base + row0, st.k_slice);
       bulk_commit_group();
     }

@@ -225,8 +225,9 @@ __host__ __device__ inline int choose_k_split(long tiles, int n_workers, int sma
 
 // Offset and row count of slab `index` when n_valid rows are cut into equal slabs of at most cap rows.
 // Up to `one` rows (at least cap) stay in one slab: two half slabs would be worse than one that is a little long.
+__host__ __device__ inline int slab_count(int n_valid, int cap, int one) { return n_valid <= one ? 1 : (n_valid + cap - 1) / cap; }
 __host__ __device__ inline void slab_extent(int n_valid, int cap, int one, int index, int& off, int& rows) {
-  int n_slabs = n_valid <= one ? 1 : (n_valid + cap - 1) / cap;
+  const int n_slabs = slab_count(n_valid, cap, one);
   int per = ((n_valid + n_slabs - 1) / n_slabs + 255) / 256 * 256;
   if (per > one) per = one;
   off = index * per;

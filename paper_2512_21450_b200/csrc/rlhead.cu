@@ -1344,7 +1344,12 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int n_col_slabs = (int)((V + L.Vs - 1) / L.Vs);
   const int d_tiles = (int)((d + BN - 1) / BN);
   int hook_slab = 0;
-  for (int r = 0; r < n_row_slabs; ++r) {
+  // Slabs are sized for T rows, and how many of them have any is known to the device alone.  Whoever wants to be told as rows of dW
+  // are completed has them walked from the last to the first, so that the one that completes them has rows: its dW launches, in
+  // pieces and before its dH, are what is told about while they and dH still run.
+  const bool reverse = c->dw_hook && n_row_slabs > 1;
+  for (int q = 0; q < n_row_slabs; ++q) {
+    const int r = reverse ? n_row_slabs - 1 - q : q;
     GemmShape dh_shape;
     memset(&dh_shape, 0, sizeof(dh_shape));
     const int rows_cap = L.Ts;   // the valid rows are cut into equal slabs of at most Ts rows on the device
@@ -1451,7 +1456,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         }
       }
       // (2) dH_slab (+)= G * W_slab        [rows x d], K = vocabulary columns of the slab
-      {
+      auto launch_dH = [&]() {
         GemmShape sh;
         memset(&sh, 0, sizeof(sh));
         sh.n_valid = n_valid;
@@ -1464,16 +1469,16 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.k_split_max = c->dh_k_slices;
         sh.stream_k = dh_uses_stream_k(c) ? 1 : (L.dH_slots ? 2 : 0);
         dh_shape = sh;      // how tiles are cut depends only on rows, d tiles and grid: same for every slab
-        EpiAcc::Params ep;
+        EpiAcc::Params ep = {};
         ep.n_cols = (int)d; ep.accumulate = cs > 0; ep.row_base = 0; ep.slice_add = sh.stream_k == 1;
         ep.tile_cols = sh.stream_k == 2 ? dh_cols : 0;
         ep.tile_rows = dh_tile_rows;
         if (use_wide(c, d)) launch_wide<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
         else launch_gemm<EpiAcc, 0, 1>(c, c->cta_group, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
-      }
-      // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab.  A caller that wants to
-      // be told as rows of dW are completed gets them in pieces.
-      const bool report = c->dw_hook && r == n_row_slabs - 1;
+      };
+      // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab
+      const bool report = c->dw_hook && q == n_row_slabs - 1;
+      if (!report) launch_dH();
       const int step = report && cols > kSlabColsMax ? kSlabColsMax : cols;
       for (int c0 = 0; c0 < cols; c0 += step) {
         GemmShape sh;
@@ -1487,16 +1492,18 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.a_mn_off = c0;
         sh.b_k_slab = 1;
         sh.n_fastest = 1;
-        EpiAcc::Params ep;
-        ep.n_cols = (int)d; ep.accumulate = (r > 0 || o.accumulate_dW) ? 1 : 0;
+        EpiAcc::Params ep = {};
+        ep.n_cols = (int)d; ep.accumulate = o.accumulate_dW ? 1 : reverse ? 2 : (r > 0 ? 1 : 0);
+        ep.n_valid = n_valid; ep.slab_cap = L.Tc; ep.slab_one = L.Ts; ep.slab_index = r;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
         launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
-        // these rows of dW are complete once the last row slab has added to them
+        // these rows of dW are complete once the row slab that is walked last has added to them
         if (report) {
           const int64_t row0 = (int64_t)vocab_base + c0;
           c->dw_hook(c->dw_hook_user, hook_slab++, row0, row0 + sh.m_rows_cap);
         }
       }
+      if (report) launch_dH();
     }
     const int pr_sc = prof_begin(c, 7);
     DhSource src;
@@ -1976,7 +1983,7 @@ rl_status rl_selftest_gemm(rl_ctx* c, const void* A, const void* B, float* C, in
   sh.n_fastest = 1;   // walk the column tiles of one row panel first, as the gradient passes do
   CUtensorMap tc;
   if (!map_out_f32(c, &tc, C, (uint64_t)M, (uint64_t)N, (uint64_t)N, 1, (uint64_t)M)) return RL_ERR_CUDA;
-  EpiAcc::Params ep;
+  EpiAcc::Params ep = {};
   ep.n_cols = (int)N; ep.accumulate = accumulate; ep.row_base = 0; ep.slice_add = 0; ep.tile_cols = 0;
   if (c->wide_tiles && c->cta_group == 2 && !a_mn && b_mn) {   // the operand layout of dH, the one pass that has wide tiles
     sh.n_tiles = (int)((N + 2 * BN - 1) / (2 * BN));

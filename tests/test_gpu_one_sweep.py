@@ -251,3 +251,52 @@ def test_one_sweep_full_kl_outlier_rows():
     # an entry of G is rounded to bf16 once (2^-9 at most, 1.7e-3 rms over a row of many entries), and a row of dH is the sum
     # of its entries times random rows of W, which keeps the ratio up to 1/sqrt(d)
     assert err.max() <= 4e-3, np.sort(err)[-5:]
+
+
+# Rows of dW are reported while there is still work to run beside what the hook starts: slabs are sized for all rows, of which half
+# are masked here, and the slab that is walked last is one that has rows.  At the moment of a report those rows are complete.
+@pytest.mark.parametrize("valid,accumulate", [(0.5, False), (0.5, True), (0.0, False), (1.0, False)])
+def test_rows_of_dW_are_reported_before_the_end(valid, accumulate):
+    from paper_2512_21450_b200 import Context
+    T, d, V = 2048, 896, 80000
+    gen = torch.Generator(device="cuda").manual_seed(31)
+    H = torch.randn(T, d, generator=gen, device="cuda").to(torch.bfloat16)
+    W = (0.02 * torch.randn(V, d, generator=gen, device="cuda")).to(torch.bfloat16)
+    tok = torch.randint(0, V, (T,), generator=gen, device="cuda", dtype=torch.int32)
+    mask = torch.zeros(T, dtype=torch.uint8, device="cuda")
+    mask[:int(valid * T)] = 1
+    old, adv = torch.full((T,), -11.4, device="cuda"), torch.randn(T, generator=gen, device="cuda")
+    dW0 = 1e-3 * torch.randn(V, d, generator=gen, device="cuda")
+    c = Context(0)
+    try:
+        c.set_slab_limits(512, 80128)                 # four slabs of whole rows
+        outs, seen, copies, events = [], [], [], []
+        for hook in (False, True, True):              # the second call with the hook is the timed one
+            seen.clear(), copies.clear(), events.clear()
+
+            def fn(slab, r0, r1):
+                event = torch.cuda.Event(enable_timing=True)
+                event.record()
+                events.append(event)
+                seen.append((slab, r0, r1))
+                copies.append(dW[r0:r1].clone())
+
+            c.set_dw_slab_hook(fn if hook else None)
+            dW = dW0.clone()
+            begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            begin.record()
+            outs.append(c.rl_policy_loss_fwd_bwd(H, W, tok, old, None, adv, mask, 0.2, 0.2, 0.0, dW=dW,
+                                                 accumulate_dW=accumulate, dH_fp32=True))
+            end.record()
+            assert c.last_device_status()[0] == 0
+        assert seen == [(i, 37888 * i, min(V, 37888 * (i + 1))) for i in range(3)]
+        assert torch.equal(torch.cat(copies), outs[2]["dW"])
+        assert torch.equal(outs[1]["dW"], outs[2]["dW"])
+        for key in ("loss", "dH", "logp"):
+            assert torch.equal(outs[0][key], outs[2][key]), key
+        # another order of the slabs: fp32 sums of at most four terms, each within an ulp of the largest
+        assert (outs[0]["dW"] - outs[2]["dW"]).norm() <= 1e-6 * outs[0]["dW"].norm() + 1e-30
+        if valid > 0:      # what is left after the first piece is most of dW and all of dH of that slab, half of its work
+            assert events[0].elapsed_time(end) >= 0.25 * begin.elapsed_time(end) / (4 * valid)
+    finally:
+        c.close()
