@@ -498,6 +498,11 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
  * max_slots = 0, *n_slots = number of pairs. */
 rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers,
                               int32_t* slots, int64_t max_slots, int64_t* n_slots);
+/* The order in which the dH pass forms its operand while it reads it, for K = ld columns of which k_len are in the
+ * vocabulary: the pairs {128-row tile, chunk of 512 columns} of int32, each once; pairs may be NULL when max_pairs = 0.
+ * *pays (may be NULL): 1 if it does so at all with so many rows, 0 if a launch before it forms the operand. */
+rl_status rl_debug_feed_order(int64_t n_valid, int64_t k_len, int64_t ld, int64_t n_tiles, int cta_group, int n_workers,
+                              int32_t* pairs, int64_t max_pairs, int64_t* n_pairs, int* pays);
 /* Host-only view of the workspace layout (works without a GPU; the paper has no counterpart) with default
  * options on a GPU of n_sm SMs: bytes[0] = what rl_workspace_bytes[_kl] returns (d_ref = 0: no reference model),
  * bytes[1] = what rl_workspace_bytes_logprobs returns, where the arrays that forming log-probabilities uses end, bytes[2] = where the row positions, which only

@@ -125,6 +125,8 @@ def load_library():
     lib.rl_debug_schedule.restype = c_int
     lib.rl_debug_tile_slots.argtypes = [c_int64, c_int64, c_int64, c_int, c_int, P, c_int64, POINTER(c_int64)]
     lib.rl_debug_tile_slots.restype = c_int
+    lib.rl_debug_feed_order.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, P, c_int64, POINTER(c_int64), POINTER(c_int)]
+    lib.rl_debug_feed_order.restype = c_int
     lib.rl_debug_workspace.argtypes = [c_int64, c_int64, c_int64, c_int64, c_int, c_int, POINTER(c_int64)]
     lib.rl_debug_workspace.restype = c_int
     lib.rl_selftest_cluster_exchange.argtypes = [P, c_int, c_int, c_int, c_int, c_int, POINTER(c_float), POINTER(c_int)]
@@ -606,6 +608,17 @@ def debug_tile_slots(n_valid, k_len, n_tiles, cta_group=2, n_workers=74):
     out = np.empty((n.value, 2), dtype=np.int32)
     _check(lib.rl_debug_tile_slots(*args, out.ctypes.data_as(c_void_p), n.value, byref(n)), "rl_debug_tile_slots")
     return out
+
+
+def debug_feed_order(n_valid, k_len, ld, n_tiles, cta_group=2, n_workers=74):
+    """Host-only: pairs (128-row tile, column chunk) in the order in which the dH pass forms its operand, and whether it does."""
+    import numpy as np
+    lib, n, pays = load_library(), c_int64(), c_int()
+    args = (n_valid, k_len, ld, n_tiles, cta_group, n_workers)
+    _check(lib.rl_debug_feed_order(*args, None, 0, byref(n), None), "rl_debug_feed_order")
+    out = np.empty((n.value, 2), dtype=np.int32)
+    _check(lib.rl_debug_feed_order(*args, out.ctypes.data_as(c_void_p), n.value, byref(n), byref(pays)), "rl_debug_feed_order")
+    return out, bool(pays.value)
 
 
 def debug_workspace(T, d, V, d_ref=0, n_sm=148, static_scratch=False):

@@ -24,6 +24,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
 struct RowStats {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;   // [rows] compact sampled-token ids
@@ -168,6 +169,7 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // the statistics alone 1.36 / 1.65 / 2.85 / 5.16).
 struct EpiSweep {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 4;
   static constexpr int kStagingBytes = kEpiStaging;
   using Params = RowStats::Params;
@@ -260,6 +262,7 @@ struct GradParams {
 template <int W>
 struct EpiGrad {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = W;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;
@@ -357,21 +360,23 @@ struct EpiGrad {
 // accumulating.  The output is seen through a 3-D fp32 tensor map {columns, rows, K slices}, which
 // also clips rows past the tensor.  Every element is written by exactly one tile per launch, so
 // the result does not depend on timing.
+struct AccParams {
+  int n_cols;
+  int accumulate;  // 0 store, 1 add, 2 (slabs walked from the last to the first): add unless this is the last slab that has rows
+  const int* n_valid;                      // 2 only
+  int slab_cap, slab_one, slab_index;
+  int row_base;
+  int slice_add;   // stream-K launches: output slices past the first are always added to
+  int tile_cols;   // > 0: k_slice > 0 names slot k_slice - 1, a box of tile_cols columns x tile_rows rows of its own
+  int tile_rows;
+};
 struct EpiAcc {
   static constexpr bool kParts = true;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 4;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;
-  struct Params {
-    int n_cols;
-    int accumulate;  // 0 store, 1 add, 2 (slabs walked from the last to the first): add unless this is the last slab that has rows
-    const int* n_valid;                      // 2 only
-    int slab_cap, slab_one, slab_index;
-    int row_base;
-    int slice_add;   // stream-K launches: output slices past the first are always added to
-    int tile_cols;   // > 0: k_slice > 0 names slot k_slice - 1, a box of tile_cols columns x tile_rows rows of its own
-    int tile_rows;
-  };
+  using Params = AccParams;
   struct State {
     int k_slice;
     int add;
@@ -419,5 +424,4 @@ struct EpiAcc {
   }
   __device__ static __forceinline__ void end_unit(const Params&, State&, int, int, int, int) {}
 };
-
 }  // namespace rlh

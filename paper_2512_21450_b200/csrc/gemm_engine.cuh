@@ -10,6 +10,9 @@
 //                 that its rank modulo 4 may read, pulls its columns of the accumulator (all, or one half of
 //                 them) out in 32-column chunks and hands them to the epilogue functor.  With eight, the functor's
 //                 per-row state of the second half is merged into the first's at the end of a unit.
+//   feed warps  : behind them, where the A operand is still being formed (Epi::kFeedWarps > 0): they write it in the order in which
+//                 the producers read it, which wait for the part they are about to load.  Parts are handed out by a counter to
+//                 warps that run, so none is waited for that nobody works on, however many blocks are resident.
 //
 // Tile modes (per CTA 128 accumulator rows):
 //   kTileSquare : a tile is 256 columns wide and lives in ONE accumulator; tile t uses accumulator
@@ -55,7 +58,8 @@ constexpr int BM = 128;   // accumulator rows per CTA
 constexpr int BN = 256;   // accumulator columns
 constexpr int BK = 64;
 constexpr int kAStageBytes = BM * BK * 2;
-constexpr int gemm_threads(int epi_warps) { return 64 + 32 * epi_warps; }
+// feed_warps > 0: those, and one that watches what they have done
+constexpr int gemm_threads(int epi_warps, int feed_warps) { return 64 + 32 * (epi_warps + feed_warps + (feed_warps > 0)); }
 constexpr int kTileSmemBytes = 224 * 1024;             // operand ring + epilogue staging
 constexpr int kMaxSmemBytes = 227 * 1024;              // static + dynamic shared memory of a block
 constexpr int kBoxBytes = 4096;                        // one 32 x 32 fp32 or 32 x 64 bf16 box
@@ -69,6 +73,12 @@ constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
 constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
+// An A operand that is formed while it is read (Epi::kFeedWarps > 0): a job is kFeedRows rows x kFeedCols columns (of K).
+constexpr int kFeedRows = 16;
+constexpr int kFeedCols = 512;
+constexpr int kFeedJobs = BM / kFeedRows;   // jobs per 128-row tile and column chunk
+// Column chunks that k-blocks [kb0, kb1) touch.
+__host__ __device__ inline int feed_chunks(int kb0, int kb1) { return (kb1 * BK + kFeedCols - 1) / kFeedCols - kb0 * BK / kFeedCols; }
 
 enum TileMode { kTileSquare = 0, kTileWide = 1, kTileDual = 2 };
 
@@ -425,15 +435,18 @@ struct UnitWalk {
       ks = 1 + r * S + s;
       it = it_end;
     } else {
+      // from the last piece to the first, so that only the one done last may start inside an end: where A is still being
+      // formed, from the start of every part and every end on, a helper that started there waited (1700 rows, 28 tiles: for a
+      // quarter of the pass)
       const int ends = cut_tile_ends(ex);
-      r = (int)div_floor(it, ends);
-      const int pos = (int)(it - (long long)r * ends);
-      for (s = 0; s + 1 < S && cut_end_pos(ex, s + 1) <= pos; ++s) {}
-      kb0 = cut_begin(ex, s) + ex.cut_len + pos - cut_end_pos(ex, s);
-      kb1 = cut_begin(ex, s + 1);
-      if (kb1 - kb0 > it_end - it) kb1 = kb0 + (int)(it_end - it);
+      r = (int)div_floor(it_end - 1, ends);
+      const int pos = (int)(it_end - (long long)r * ends);   // behind the piece, in the ends of its tile
+      for (s = 0; s + 1 < S && cut_end_pos(ex, s + 1) < pos; ++s) {}
+      kb0 = cut_begin(ex, s) + ex.cut_len;
+      kb1 = kb0 + pos - cut_end_pos(ex, s);
+      if (kb1 - kb0 > it_end - it) kb0 = kb1 - (int)(it_end - it);
       ks = 1 + mains + r * S + s + (me - mains);
-      it += kb1 - kb0;
+      it_end -= kb1 - kb0;
     }
     const int tile = plain_units + r;
     if (sh.n_fastest) { nr = tile % ex.n_ranges; mu = tile / ex.n_ranges; }
@@ -453,12 +466,15 @@ struct UnitWalk {
 //     static constexpr int kMerge;                             // floats of state that pack() hands to the other half's
 //     static void pack(const State&, float (&)[kMerge]); static void merge(State&, const float (&)[kMerge]);   // if > 0
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
-//     static constexpr bool kParts; };                         // knows what to do with parts of tiles (stream_k == 2)
+//     static constexpr bool kParts;                            // knows what to do with parts of tiles (stream_k == 2)
+//     static constexpr int kFeedWarps; };                      // warps that form A; if > 0:
+//     static bool feeds(const Params&, const GemmExtents&, int n_workers);   // or A is complete when the launch starts
+//     static void feed(const Params&, const GemmExtents&, int cg, int n_workers); static const unsigned* feed_flag(const Params&, int m_tile, int chunk);
 //   kTileDual: chunk receives the chunk of the second product as well (..., v, v2, out_map, staging).
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
 // sh.n_tiles then counts 512-wide tiles).  tmA2 / tmB2 / k2_len are read by kTileDual only.
 template <class Epi, int A_MN, int B_MN, int CG, int MODE>
-__global__ void __launch_bounds__(gemm_threads(Epi::kWarps), 1)
+__global__ void __launch_bounds__(gemm_threads(Epi::kWarps, Epi::kFeedWarps), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
@@ -481,6 +497,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   __shared__ float merge_s[kMerges ? Epi::kMerge : 1][kMerges ? BM : 1];
   __shared__ __align__(8) uint64_t bar_merge[2][4];   // full, empty
   __shared__ int abort_flag;
+  __shared__ int fed_s;   // feed warps: chunks of A, in the order of this worker's units, that are there
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -501,6 +518,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int w = 0; w < 4; ++w) { mbar_init(smem_u32(&bar_merge[0][w]), 1); mbar_init(smem_u32(&bar_merge[1][w]), 1); }
     mbar_init(smem_u32(&bar_drain), 1);
     abort_flag = 0;
+    fed_s = 0;
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
@@ -517,6 +535,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   chain_wait();
   const uint32_t tmem_base = tmem_base_smem;
   volatile int* abort_p = &abort_flag;
+  volatile int* fed_p = &fed_s;
 
   // parts of cut tiles go to slots, seen through the second map of operand A (one-product passes only)
   const CUtensorMap* part_map = MODE == kTileDual ? &tmC : &tmA2;
@@ -532,6 +551,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      int fed = 0, fed0 = 0;   // chunks of A, in the order of the walk, that were there when last looked; behind the last unit
       UnitWalk walk(sh, ex, worker, n_workers);
       int mu, nr, ks, kb0, kb1;
       while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
@@ -548,6 +568,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 latch_status(status, kStatusTimeout, (1 << 28) | (blockIdx.x << 8) | stage);
                 ok = false;
                 break;
+              }
+              if constexpr (Epi::kFeedWarps > 0) {
+                // the chunks of A that this stage needs are there
+                const int need = fed0 + feed_chunks(kb0, min(kb + Cfg::kKSub, hi));
+                if (fed < need) {
+                  while (ok && (fed = *fed_p) < need) ok = !*abort_p;
+                  if (!ok) break;
+                  __threadfence_block();
+                }
               }
               const uint32_t full_local = smem_u32(&bar_full[stage]);
               // the even CTA's barrier counts the bytes of both CTAs' copies
@@ -585,6 +614,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
           }
         }
+        if constexpr (Epi::kFeedWarps > 0) fed0 += feed_chunks(kb0, kb1);
       }
       if (!ok && (CG == 1 || rank == 0)) {
         // let copies that were already issued land before the block's shared memory goes away
@@ -685,6 +715,36 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       bool drained = false;
       for (int it = 0; it < (1 << 22) && !drained; ++it) drained = mbar_try_wait(smem_u32(&bar_drain), 0) != 0;
       if (!drained) latch_status(status, kStatusTimeout, (4 << 28) | (blockIdx.x << 8));
+    }
+  } else if (Epi::kFeedWarps > 0 && warp >= 2 + Epi::kWarps) {
+    // ------------------------------------------------------------- feed warps (both CTAs)
+    if constexpr (Epi::kFeedWarps > 0) {
+      if (warp == 2 + Epi::kWarps + Epi::kFeedWarps) {
+        // The counters of the producer's chunks, one after the other, on its behalf: looking at one takes a microsecond.
+        // (By the producer itself, at every eighth k-block, dH of 6912 rows at d = 1024 took 2.0 ms in place of 1.5.)
+        if (lane == 0 && !Epi::feeds(ep, ex, n_workers)) {
+          *fed_p = 1 << 30;   // A is complete
+        } else if (lane == 0) {
+          UnitWalk walk(sh, ex, worker, n_workers);
+          int mu, nr, ks, kb0, kb1, n = 0;
+          bool ok = true;
+          while (ok && walk.next(mu, nr, ks, kb0, kb1)) {
+            const int m = mu * CG + (int)rank, c0 = kb0 * BK / kFeedCols, c1 = c0 + feed_chunks(kb0, kb1);
+            for (int c = c0; c < c1 && ok; ++c) {
+              // (a pair's second tile may lie past the rows: nobody forms it and what is loaded is not used)
+              if (m * BM < ex.m_rows) {
+                ok = count_wait_bounded(Epi::feed_flag(ep, m, c), kFeedJobs, abort_p);
+                fence_proxy_async_global();
+              }
+              __threadfence_block();
+              if (ok) *fed_p = ++n;
+            }
+          }
+          if (!ok) latch_status(status, kStatusTimeout, (6 << 28) | (blockIdx.x << 8) | 0xff);
+        }
+      } else if (Epi::feeds(ep, ex, n_workers)) {
+        Epi::feed(ep, ex, CG, n_workers);
+      }
     }
   } else {
     // ------------------------------------------------------------- epilogue warps (both CTAs)

@@ -14,6 +14,7 @@ namespace rlh {
 // statistics 1200 / 1474 / 1858 / 4775 us with four, 985 / 1246 / 1607 / 4395 with eight).
 struct EpiStatsKL {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -141,6 +142,7 @@ __device__ __forceinline__ void st_planes(const float (&v)[32], uint16_t* hi, ui
 // A thread holds 32 consecutive columns of its row: four 32-byte stores, every sector written whole.
 struct EpiRefSweep {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -189,6 +191,7 @@ struct EpiRefSweep {
 // logits of the next 32 columns are loaded while these are worked on.
 struct EpiSweepKL {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -283,6 +286,7 @@ struct EpiSweepKL {
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
   static constexpr bool kParts = false;
+  static constexpr int kFeedWarps = 0;
   static constexpr int kWarps = 8;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;

@@ -120,6 +120,9 @@ constexpr int64_t kSweepMinK = 896;
 inline int slab_entry_bytes(int64_t d, int64_t d_ref) {
   return d_ref > 0 ? (kl_one_sweep(d, d_ref) ? 8 : 2) : (d >= kSweepMinK ? 4 : 2);
 }
+// Entries of a slab from which on dH may form its operand itself (feed_pays): below, the start of the feed shows, and a larger launch
+// that does not feed 1 % of a call.  100 and 300 rows x 151936 words, d = 2048, 1 % slower and level; 256 rows of 40000 words 169 / 188 us.
+constexpr long long kFeedEntries = 128 << 20;
 // A narrow head keeps them too while they stay in L2, and up to 128 rows, where the logit pass is a stream of W: a whole call,
 // kept against formed twice, 53.8 / 77.3 / 113 us against 58.6 / 79.4 / 106 at d = 256, 4 / 34 / 67 MB of logits (4096 words), 63.5 / 77.5 /
 // 100.5 against 68.3 / 77.3 / 96.9 (16384 words, 17 / 34 / 67 MB), 188 / 192 / 253 against 215 / 200 / 232 at 64 / 128 / 256 rows of 151936 words.
@@ -149,6 +152,7 @@ struct WsLayout {
                                                      // the plane behind it their lower halves
   int part_ranges;                                   // column ranges per row that the partials have room for
   size_t dH_slots;                                   // parts of cut dH tiles (0: none)
+  size_t feed, feed_bytes;                           // ticket and counters of the gradient jobs (logits are kept)
   int n_row_slabs;
   size_t Hc_ref, partials2, lse_ref_c, kl_c, cb_c;   // only with a reference model (full KL)
   size_t zr;                                         // the reference's logits of the slab (one-sweep form)
@@ -261,6 +265,8 @@ WsLayout ws_layout(const rl_ctx* c, int64_t T, int64_t d, int64_t V, int host_sl
   L.G = take(slab);
   L.dH_acc = take((size_t)dh_buffers(c) * L.Ts * d * 4);
   L.dH_slots = dh_cuts_tiles(c) && L.Vs == Vpad ? take(dh_slot_bytes(c, d)) : 0;
+  L.feed_bytes = L.keeps_logits ? feed_words(L.Ts, L.Vs) * 4 : 0;
+  L.feed = take(L.feed_bytes);
   L.Hc_ref = L.partials2 = L.lse_ref_c = L.kl_c = L.cb_c = L.zr = 0;
   if (d_ref > 0) {
     L.Hc_ref = take((size_t)L.Tpad * d_ref * 2);
@@ -418,7 +424,7 @@ void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUten
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(c->grid[cg]);
-  cfg.blockDim = dim3(gemm_threads(Epi::kWarps));
+  cfg.blockDim = dim3(gemm_threads(Epi::kWarps, Epi::kFeedWarps));
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -691,7 +697,9 @@ rl_status rl_create(rl_ctx** out, int device) {
             set_smem_attr<EpiAcc, 0, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 0, 1>() == cudaSuccess &&
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
-            set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess;
+            set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess &&
+            set_smem_attr<EpiAccFed, 0, 1>() == cudaSuccess &&
+            set_smem_attr_one<EpiAccFed, 0, 1, 2, kTileWide>() == cudaSuccess;
   if (!ok) { cudaFree(c->dstatus); delete c; return RL_ERR_CUDA; }
   {
     // how many CTA pairs can be resident at once (pairs must share a TPC): the persistent grid
@@ -699,7 +707,7 @@ rl_status rl_create(rl_ctx** out, int device) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(c->grid[2]);
-    cfg.blockDim = dim3(gemm_threads(EpiAcc::kWarps));
+    cfg.blockDim = dim3(gemm_threads(EpiAcc::kWarps, EpiAcc::kFeedWarps));
     cfg.dynamicSmemBytes = g_smem_bytes<EpiAcc, 0, 0, 2, kTileSquare>;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1358,6 +1366,22 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     for (int cs = 0; cs < n_col_slabs; ++cs) {
       const int vocab_base = cs * L.Vs;
       const int cols = (int)((V - vocab_base) < L.Vs ? (V - vocab_base) : L.Vs);
+      // dH may form its operand itself where it comes next and takes its tiles whole or cut; whether it does is decided on the
+      // device (feed_pays), and logit_grad_kernel has nothing to do then
+      const bool report = c->dw_hook && q == n_row_slabs - 1;
+      const bool fed = sweep && !report && !o.kl_full && dh_cuts_tiles(c) && (long long)L.Ts * L.Vs >= kFeedEntries;
+      // how tiles of dH are cut depends only on rows, d tiles and grid: same for every column slab
+      dh_shape.n_valid = n_valid;
+      dh_shape.m_rows_cap = rows_cap; dh_shape.m_dyn = 1; dh_shape.slab_cap = L.Tc; dh_shape.slab_one = L.Ts; dh_shape.slab_index = r;
+      dh_shape.k_cap = cols;
+      dh_shape.n_tiles = (int)((d + dh_cols - 1) / dh_cols);
+      dh_shape.n_range = 1;
+      dh_shape.b_k_off = vocab_base;
+      dh_shape.n_fastest = 1;   // the CTAs that share a panel of G rows run together
+      dh_shape.k_split_max = c->dh_k_slices;
+      dh_shape.stream_k = dh_uses_stream_k(c) ? 1 : (L.dH_slots ? 2 : 0);
+      FeedParams lg;
+      memset(&lg, 0, sizeof(lg));
       // (1) the slab's G = dloss/dlogits as bf16: from the logits of a first pass, or by forming them again
       {
         if (sweep) {
@@ -1405,26 +1429,38 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
           }
           p.slab_cap = L.Tc; p.slab_one = L.Ts;
           p.slab_index = r;
+          p.clear = reinterpret_cast<uint4*>(ws + L.feed);
+          p.n_clear = fed ? (int)(L.feed_bytes / 16) : 0;
           merge_and_loss(r);
-          LogitGradParams lg;
           lg.slab = z_hi;
+          lg.lo = z_lo;
           lg.ld = L.Vs;
           lg.V = (int)V;
           lg.slab_cap = L.Tc; lg.slab_one = L.Ts; lg.slab_index = r;
           lg.tokens_c = ep.tokens_c;
           lg.lse = p.lse_c; lg.ent = p.ent_c; lg.cp = p.cp_c; lg.ce = p.ce_c;
-          const int pr_lg = prof_begin(c, 1);
-          lg.lo = z_lo;
           lg.zr = zr;
           lg.lse_ref = p.lse_ref_c; lg.kl = p.kl_c; lg.cb = p.cb_c;
-          const long long padded = (long long)align_up(rows_cap, 128);
-          const int unit = 256 * (o.kl_full ? kGradVecsKL : kGradVecs);
-          long long grad_blocks = (padded * ((L.Vs + unit - 1) / unit) + 7) / 8;   // a warp each
-          if (grad_blocks > c->n_sm * 64) grad_blocks = c->n_sm * 64;
-          if (o.kl_full) launch(c, logit_grad_kl_kernel, (int)grad_blocks, 256, lg, c->dstatus);
-          else           launch(c, logit_grad_kernel, (int)grad_blocks, 256, lg, c->dstatus);
-          prof_end(c, pr_lg, 1);
-          c->launches++;
+          if (fed) {
+            lg.dh = dh_shape;
+            lg.cg = c->cta_group;
+            lg.workers = dh_workers;
+            lg.ticket = reinterpret_cast<unsigned*>(ws + L.feed);
+            lg.ready = lg.ticket + 4;
+          }
+          {
+            const int pr_lg = prof_begin(c, 1);
+            const long long padded = (long long)align_up(rows_cap, 128);
+            const int unit = 256 * (o.kl_full ? kGradVecs<true> : kGradVecs<false>);
+            long long grad_blocks = (padded * ((L.Vs + unit - 1) / unit) + 7) / 8;   // a warp each
+            if (grad_blocks > c->n_sm * 64) grad_blocks = c->n_sm * 64;
+            const LogitGradParams& alone = lg;
+            if (fed)            launch(c, logit_grad_kernel<false, FeedParams>, (int)grad_blocks, 256, lg, c->dstatus);
+            else if (o.kl_full) launch(c, logit_grad_kernel<true, LogitGradParams>, (int)grad_blocks, 256, alone, c->dstatus);
+            else                launch(c, logit_grad_kernel<false, LogitGradParams>, (int)grad_blocks, 256, alone, c->dstatus);
+            prof_end(c, pr_lg, 1);
+            c->launches++;
+          }
         } else {
           GemmShape sh;
           memset(&sh, 0, sizeof(sh));
@@ -1457,27 +1493,26 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       }
       // (2) dH_slab (+)= G * W_slab        [rows x d], K = vocabulary columns of the slab
       auto launch_dH = [&]() {
-        GemmShape sh;
-        memset(&sh, 0, sizeof(sh));
-        sh.n_valid = n_valid;
-        sh.m_rows_cap = rows_cap; sh.m_dyn = 1; sh.slab_cap = L.Tc; sh.slab_one = L.Ts; sh.slab_index = r;
-        sh.k_cap = cols;
-        sh.n_tiles = (int)((d + dh_cols - 1) / dh_cols);
-        sh.n_range = 1;
-        sh.b_k_off = vocab_base;
-        sh.n_fastest = 1;   // the CTAs that share a panel of G rows run together
-        sh.k_split_max = c->dh_k_slices;
-        sh.stream_k = dh_uses_stream_k(c) ? 1 : (L.dH_slots ? 2 : 0);
-        dh_shape = sh;      // how tiles are cut depends only on rows, d tiles and grid: same for every slab
-        EpiAcc::Params ep = {};
+        const GemmShape& sh = dh_shape;
+        AccParams ep = {};
         ep.n_cols = (int)d; ep.accumulate = cs > 0; ep.row_base = 0; ep.slice_add = sh.stream_k == 1;
         ep.tile_cols = sh.stream_k == 2 ? dh_cols : 0;
         ep.tile_rows = dh_tile_rows;
-        if (use_wide(c, d)) launch_wide<EpiAcc, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
-        else launch_gemm<EpiAcc, 0, 1>(c, c->cta_group, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, ep);
+        auto tiles = [&](auto epi, const auto& params) {
+          using Epi = decltype(epi);
+          if (use_wide(c, d)) launch_wide<Epi, 0, 1>(c, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, params);
+          else launch_gemm<Epi, 0, 1>(c, c->cta_group, 2, tmG_k, tmW_mn, tm_dH, tm_slots, sh, params);
+        };
+        if (fed) {
+          EpiAccFed::Params params = {};
+          static_cast<AccParams&>(params) = ep;
+          params.grad = lg;
+          tiles(EpiAccFed(), params);
+        } else {
+          tiles(EpiAcc(), ep);
+        }
       };
       // (3) dW_slab (+)= G^T * H_slab      [vocabulary rows x d], K = valid rows of the slab
-      const bool report = c->dw_hook && q == n_row_slabs - 1;
       if (!report) launch_dH();
       const int step = report && cols > kSlabColsMax ? kSlabColsMax : cols;
       for (int c0 = 0; c0 < cols; c0 += step) {
@@ -1492,7 +1527,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         sh.a_mn_off = c0;
         sh.b_k_slab = 1;
         sh.n_fastest = 1;
-        EpiAcc::Params ep = {};
+        AccParams ep = {};
         ep.n_cols = (int)d; ep.accumulate = o.accumulate_dW ? 1 : reverse ? 2 : (r > 0 ? 1 : 0);
         ep.n_valid = n_valid; ep.slab_cap = L.Tc; ep.slab_one = L.Ts; ep.slab_index = r;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
@@ -1849,16 +1884,11 @@ rl_status rl_debug_schedule(int64_t n_valid, int64_t rows_cap, int64_t k_len, in
   return RL_OK;
 }
 
-rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers, int32_t* slots,
-                              int64_t max_slots, int64_t* n_slots) {
-  if (!n_slots || n_valid <= 0 || k_len <= 0 || n_tiles <= 0 || n_workers <= 0 || max_slots < 0 ||
-      (cta_group != 1 && cta_group != 2) || (max_slots > 0 && !slots))
-    return RL_ERR_INVALID_ARG;
-  const int nv = (int)n_valid;
+// Extents of a dH pass over n_valid rows.
+static GemmExtents dh_extents(int n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers) {
   GemmShape sh;
   memset(&sh, 0, sizeof(sh));
-  sh.n_valid = &nv;
-  sh.m_rows_cap = nv;
+  sh.m_rows_cap = n_valid;
   sh.m_dyn = 1;
   sh.k_cap = (int)k_len;
   sh.n_tiles = (int)n_tiles;
@@ -1866,7 +1896,15 @@ rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, i
   sh.n_fastest = 1;
   sh.k_split_max = 1;
   sh.stream_k = 2;
-  const GemmExtents ex = gemm_extents(sh, nv, cta_group, n_workers);
+  return gemm_extents(sh, n_valid, cta_group, n_workers);
+}
+
+rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, int cta_group, int n_workers, int32_t* slots,
+                              int64_t max_slots, int64_t* n_slots) {
+  if (!n_slots || n_valid <= 0 || k_len <= 0 || n_tiles <= 0 || n_workers <= 0 || max_slots < 0 ||
+      (cta_group != 1 && cta_group != 2) || (max_slots > 0 && !slots))
+    return RL_ERR_INVALID_ARG;
+  const GemmExtents ex = dh_extents((int)n_valid, k_len, n_tiles, cta_group, n_workers);
   int64_t n = 0;
   auto put = [&](int tile, int slot) {
     if (n < max_slots) { slots[2 * n] = tile; slots[2 * n + 1] = slot; }
@@ -1879,6 +1917,25 @@ rl_status rl_debug_tile_slots(int64_t n_valid, int64_t k_len, int64_t n_tiles, i
       for (int h = c.first; h <= c.last; ++h) put(ex.n_units - ex.cut + r, h);
     }
   *n_slots = n;
+  return RL_OK;
+}
+
+rl_status rl_debug_feed_order(int64_t n_valid, int64_t k_len, int64_t ld, int64_t n_tiles, int cta_group, int n_workers,
+                              int32_t* pairs, int64_t max_pairs, int64_t* n_pairs, int* pays) {
+  if (!n_pairs || n_valid <= 0 || k_len <= 0 || ld < k_len || n_tiles <= 0 || n_workers <= 0 || max_pairs < 0 ||
+      (cta_group != 1 && cta_group != 2) || (max_pairs > 0 && !pairs))
+    return RL_ERR_INVALID_ARG;
+  const GemmExtents ex = dh_extents((int)n_valid, k_len, n_tiles, cta_group, n_workers);
+  const FeedOrder o = feed_order(ex, (int)n_valid, (int)ld, cta_group, n_workers);
+  const int64_t n = (int64_t)o.m_tiles * o.chunks;
+  for (int64_t q = 0; q < n && q < max_pairs; ++q) {
+    int tile, chunk;
+    feed_pair(ex, o, (int)q, tile, chunk);
+    pairs[2 * q] = tile;
+    pairs[2 * q + 1] = chunk;
+  }
+  *n_pairs = n;
+  if (pays) *pays = feed_pays(ex, n_workers) ? 1 : 0;
   return RL_OK;
 }
 
@@ -1983,7 +2040,7 @@ rl_status rl_selftest_gemm(rl_ctx* c, const void* A, const void* B, float* C, in
   sh.n_fastest = 1;   // walk the column tiles of one row panel first, as the gradient passes do
   CUtensorMap tc;
   if (!map_out_f32(c, &tc, C, (uint64_t)M, (uint64_t)N, (uint64_t)N, 1, (uint64_t)M)) return RL_ERR_CUDA;
-  EpiAcc::Params ep = {};
+  AccParams ep = {};
   ep.n_cols = (int)N; ep.accumulate = accumulate; ep.row_base = 0; ep.slice_add = 0; ep.tile_cols = 0;
   if (c->wide_tiles && c->cta_group == 2 && !a_mn && b_mn) {   // the operand layout of dH, the one pass that has wide tiles
     sh.n_tiles = (int)((N + 2 * BN - 1) / (2 * BN));

@@ -4,7 +4,7 @@
 // conversion of dH.  All of them are bandwidth- or latency-bound; loads are coalesced and
 // vectorised where a row is wide enough to matter.
 #pragma once
-#include "kl_epilogues.cuh"
+#include "logit_grad.cuh"
 
 namespace rlh {
 
@@ -745,6 +745,8 @@ struct LossParams {
   const float* ext_lse;
   // one row slab of the one-sweep path (slab_cap > 0): only its rows are merged
   int slab_cap, slab_one, slab_index;
+  uint4* clear;            // ticket and counters of the gradient jobs that follow
+  int n_clear;
 };
 // Fixed-order sum of column k of the block partials by one warp: lane l adds blocks l, l + 32, ... in order, then a
 // butterfly over the lanes; the order depends on n_blocks alone, so the result is reproducible.
@@ -813,6 +815,7 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
   chain_begin();
   constexpr int kTeams = kLossThreads / 32 / kW;
   __shared__ float part_s[2][7][kW][kW > 1 ? 32 : 1];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n_clear; i += gridDim.x * blockDim.x) p.clear[i] = make_uint4(0, 0, 0, 0);
   const int n = st->n_valid;
   const int n_ranges = p.ext_lse ? 0 : st->n_ranges;
   const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % kW, team = (threadIdx.x >> 5) / kW;
@@ -955,162 +958,6 @@ __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossPa
     }
   }
   if (p.with_loss) finish_loss(acc, p.fin, (float)n);
-}
-
-// ------------------------------------------------------------------------------------------
-// One-sweep path: the fp32 logits of a slab become the bf16 gradient with respect to the logits, in the arithmetic of EpiGrad:
-//   g_tj = cp_t (p_tj - 1[j = y_t]) + ce_t p_tj (log p_tj + Ent_t),
-// written in place of their upper halves; rows past the slab's valid rows (up to a multiple of 128) and columns past V
-// become zero.  Bound by memory: 4 bytes in and 2 out per entry and nothing read twice.  A warp takes kGradVecs * 256
-// consecutive columns of one row, all its 16-byte loads in flight before the first is used.  151936 columns: 17 / 45 / 146 / 556 /
-// 986 us at 64 / 276 / 1000 / 4000 / 6912 rows, 5.5 TB/s at 276 and 6.3-6.6 from 600 on (two pairs in flight 17 / 49 / 150 / 590 /
-// 1089, eight 17 / 49 / 148 / 565 / 1012).
-constexpr int kGradVecs = 4;         // pairs of 16-byte words per lane and unit of kGradVecs * 256 columns
-constexpr int kGradVecsKL = 2;       // the KL kernel loads four words per output: 68 / 232 / 462 us at 276 / 1000 / 2000 rows (one: 72 / 247 / 481)
-struct LogitGradParams {
-  uint16_t* slab;          // [slab rows][ld] upper halves of the logits, then the gradient
-  const uint16_t* lo;      // lower halves
-  int ld;                  // multiple of 256
-  int V;
-  int slab_cap, slab_one, slab_index;
-  const int* tokens_c;     // per compact row, as the arrays below
-  const float* lse;
-  const float* ent;
-  const float* cp;
-  const float* ce;
-  // full-distribution KL: the reference's logits
-  const float* zr;
-  const float* lse_ref;
-  const float* kl;
-  const float* cb;
-};
-
-// The same with the regulariser's term, from the fp32 logits of both models, in the arithmetic of EpiGradKL:
-//   g_tj = cp_t (p_tj - 1[j = y_t]) + cb_t p_tj (log p_tj - log q_tj - KL_t) + ce_t p_tj (log p_tj + Ent_t).
-// 8 bytes in and 2 out per entry.
-__global__ void __launch_bounds__(256) logit_grad_kl_kernel(const LogitGradParams p, const DevStatus* st) {
-  chain_begin();
-  int off, rows;
-  slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
-  const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + (kGradVecsKL * 256) - 1) / (kGradVecsKL * 256);
-  const long long n_units = (long long)rows_pad * units_per_row;
-  const int lane = threadIdx.x & 31;
-  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
-    const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecsKL * 256);
-    const size_t at = (size_t)r * p.ld + c0;
-    uint4* base = reinterpret_cast<uint4*>(p.slab + at) + lane;
-    if (r >= rows) {
-#pragma unroll
-      for (int k = 0; k < kGradVecsKL; ++k)
-        if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
-      continue;
-    }
-    const uint4* low = reinterpret_cast<const uint4*>(p.lo + at) + lane;
-    const float4* ref = reinterpret_cast<const float4*>(p.zr + at) + 2 * lane;
-    uint4 h[kGradVecsKL], l[kGradVecsKL];
-    float4 z0[kGradVecsKL], z1[kGradVecsKL];
-#pragma unroll
-    for (int k = 0; k < kGradVecsKL; ++k)
-      if (c0 + k * 256 < p.ld) {
-        h[k] = base[k * 32];
-        l[k] = __ldcs(low + k * 32);
-        z0[k] = __ldcs(ref + k * 64);
-        z1[k] = __ldcs(ref + k * 64 + 1);
-      }
-    const int i = off + r;
-    const float lse = p.lse[i], lse_ref = p.lse_ref[i], cp = p.cp[i], ce = p.ce[i], cb = p.cb[i];
-    const float rest = cp + ce * p.ent[i] - cb * p.kl[i];   // terms that do not depend on j
-    const float k_lp = cb + ce;                             // coefficient of log p_j
-    const int y = p.tokens_c[i];
-#pragma unroll
-    for (int k = 0; k < kGradVecsKL; ++k) {
-      const int c = c0 + k * 256 + lane * 8;
-      if (c0 + k * 256 >= p.ld) break;
-      const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, lw[4] = {l[k].x, l[k].y, l[k].z, l[k].w};
-      const float zr[8] = {z0[k].x, z0[k].y, z0[k].z, z0[k].w, z1[k].x, z1[k].y, z1[k].z, z1[k].w};
-      float g[8];
-      const unsigned rel = (unsigned)(y - c);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float lp = __uint_as_float(__byte_perm(lw[j / 2], hw[j / 2], j & 1 ? 0x7632 : 0x5410)) - lse;
-        g[j] = ex2_approx(lp * kLog2e) * (fmaf(k_lp, lp, rest) - cb * (zr[j] - lse_ref));
-        if (rel == (unsigned)j) g[j] -= cp;
-        if (c + j >= p.V) g[j] = 0.f;
-      }
-      uint32_t o[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
-        o[j] = *reinterpret_cast<const uint32_t*>(&b);
-      }
-      base[k * 32] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256) logit_grad_kernel(const LogitGradParams p, const DevStatus* st) {
-  chain_begin();
-  int off, rows;
-  slab_extent(st->n_valid, p.slab_cap, p.slab_one, p.slab_index, off, rows);
-  const int rows_pad = (rows + 127) / 128 * 128;
-  const int units_per_row = (p.ld + (kGradVecs * 256) - 1) / (kGradVecs * 256);
-  const long long n_units = (long long)rows_pad * units_per_row;
-  const int lane = threadIdx.x & 31;
-  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n_units; u += n_warps) {
-    const int r = (int)(u / units_per_row);
-    const int c0 = (int)(u - (long long)r * units_per_row) * (kGradVecs * 256);
-    uint4* base = reinterpret_cast<uint4*>(p.slab + (size_t)r * p.ld + c0) + lane;
-    if (r >= rows) {
-#pragma unroll
-      for (int k = 0; k < kGradVecs; ++k)
-        if (c0 + k * 256 < p.ld) base[k * 32] = make_uint4(0, 0, 0, 0);
-      continue;
-    }
-    const uint4* low = reinterpret_cast<const uint4*>(p.lo + (size_t)r * p.ld + c0) + lane;
-    uint4 h[kGradVecs], l[kGradVecs];
-#pragma unroll
-    for (int k = 0; k < kGradVecs; ++k)
-      if (c0 + k * 256 < p.ld) {
-        h[k] = base[k * 32];
-        l[k] = __ldcs(low + k * 32);
-      }
-    const int i = off + r;
-    const float lse = p.lse[i], cp = p.cp[i], ce = p.ce[i], kc = fmaf(ce, p.ent[i], cp);
-    const int y = p.tokens_c[i];
-#pragma unroll
-    for (int k = 0; k < kGradVecs; ++k) {
-      const int c = c0 + k * 256 + lane * 8;
-      if (c0 + k * 256 >= p.ld) break;
-      const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, lw[4] = {l[k].x, l[k].y, l[k].z, l[k].w};
-      float g[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float z = __uint_as_float(__byte_perm(lw[j / 2], hw[j / 2], j & 1 ? 0x7632 : 0x5410));
-        const float e = ex2_approx(fmaf(z, kLog2e, -lse * kLog2e));
-        g[j] = ce == 0.f ? e * cp : e * fmaf(ce, z - lse, kc);
-      }
-      const unsigned rel = (unsigned)(y - c);
-      if (rel < 8u) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) g[j] = rel == (unsigned)j ? g[j] - cp : g[j];
-      }
-      if (c + 8 > p.V) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) g[j] = c + j < p.V ? g[j] : 0.f;
-      }
-      uint32_t o[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
-        o[j] = *reinterpret_cast<const uint32_t*>(&b);
-      }
-      base[k * 32] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-  }
 }
 
 // ------------------------------------------------------------------------------------------
