@@ -24,7 +24,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // the logit of the sampled token.  Logits never leave the chip; one float4 per (range, row) does.
 struct RowStats {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;   // [rows] compact sampled-token ids
@@ -169,7 +170,8 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 // the statistics alone 1.36 / 1.65 / 2.85 / 5.16).
 struct EpiSweep {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 4;
   static constexpr int kStagingBytes = kEpiStaging;
   using Params = RowStats::Params;
@@ -262,7 +264,8 @@ struct GradParams {
 template <int W>
 struct EpiGrad {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = W;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;
@@ -372,7 +375,8 @@ struct AccParams {
 };
 struct EpiAcc {
   static constexpr bool kParts = true;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 4;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;

@@ -10,9 +10,10 @@
 //                 that its rank modulo 4 may read, pulls its columns of the accumulator (all, or one half of
 //                 them) out in 32-column chunks and hands them to the epilogue functor.  With eight, the functor's
 //                 per-row state of the second half is merged into the first's at the end of a unit.
-//   feed warps  : behind them, where the A operand is still being formed (Epi::kFeedWarps > 0): they write it in the order in which
-//                 the producers read it, which wait for the part they are about to load.  Parts are handed out by a counter to
-//                 warps that run, so none is waited for that nobody works on, however many blocks are resident.
+//   side warps  : behind them (Epi::kSideWarps), work that runs beside the products.  Where they form the A operand itself
+//                 (Epi::kFeeds) they write it in the order in which the producers read it, which wait for the part they are about to
+//                 load.  Parts are handed out by a counter to warps that run, so none is waited for that nobody works on, however
+//                 many blocks are resident.
 //
 // Tile modes (per CTA 128 accumulator rows):
 //   kTileSquare : a tile is 256 columns wide and lives in ONE accumulator; tile t uses accumulator
@@ -58,8 +59,8 @@ constexpr int BM = 128;   // accumulator rows per CTA
 constexpr int BN = 256;   // accumulator columns
 constexpr int BK = 64;
 constexpr int kAStageBytes = BM * BK * 2;
-// feed_warps > 0: those, and one that watches what they have done
-constexpr int gemm_threads(int epi_warps, int feed_warps) { return 64 + 32 * (epi_warps + feed_warps + (feed_warps > 0)); }
+// feeds: one warp more, which watches what the side warps have done
+constexpr int gemm_threads(int epi_warps, int side_warps, bool feeds) { return 64 + 32 * (epi_warps + side_warps + (feeds ? 1 : 0)); }
 constexpr int kTileSmemBytes = 224 * 1024;             // operand ring + epilogue staging
 constexpr int kMaxSmemBytes = 227 * 1024;              // static + dynamic shared memory of a block
 constexpr int kBoxBytes = 4096;                        // one 32 x 32 fp32 or 32 x 64 bf16 box
@@ -73,7 +74,7 @@ constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
 constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
-// An A operand that is formed while it is read (Epi::kFeedWarps > 0): a job is kFeedRows rows x kFeedCols columns (of K).
+// An A operand that is formed while it is read (Epi::kFeeds): a job is kFeedRows rows x kFeedCols columns (of K).
 constexpr int kFeedRows = 16;
 constexpr int kFeedCols = 512;
 constexpr int kFeedJobs = BM / kFeedRows;   // jobs per 128-row tile and column chunk
@@ -467,14 +468,16 @@ struct UnitWalk {
 //     static void pack(const State&, float (&)[kMerge]); static void merge(State&, const float (&)[kMerge]);   // if > 0
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
 //     static constexpr bool kParts;                            // knows what to do with parts of tiles (stream_k == 2)
-//     static constexpr int kFeedWarps; };                      // warps that form A; if > 0:
+//     static constexpr int kSideWarps; static constexpr bool kFeeds; };   // if kSideWarps > 0:
+//     static void side(const Params&, const GemmExtents&, int cg, int n_workers, int warp);
+//   if kFeeds:
 //     static bool feeds(const Params&, const GemmExtents&, int n_workers);   // or A is complete when the launch starts
-//     static void feed(const Params&, const GemmExtents&, int cg, int n_workers); static const unsigned* feed_flag(const Params&, int m_tile, int chunk);
+//     static const unsigned* feed_flag(const Params&, int m_tile, int chunk);
 //   kTileDual: chunk receives the chunk of the second product as well (..., v, v2, out_map, staging).
 // m_tile counts 128-row tiles, n_tile 256-column tiles (a wide tile n covers column tiles 2n and 2n + 1;
 // sh.n_tiles then counts 512-wide tiles).  tmA2 / tmB2 / k2_len are read by kTileDual only.
 template <class Epi, int A_MN, int B_MN, int CG, int MODE>
-__global__ void __launch_bounds__(gemm_threads(Epi::kWarps, Epi::kFeedWarps), 1)
+__global__ void __launch_bounds__(gemm_threads(Epi::kWarps, Epi::kSideWarps, Epi::kFeeds), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ CUtensorMap tmC, const GemmShape sh, const int k2_len,
@@ -497,7 +500,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   __shared__ float merge_s[kMerges ? Epi::kMerge : 1][kMerges ? BM : 1];
   __shared__ __align__(8) uint64_t bar_merge[2][4];   // full, empty
   __shared__ int abort_flag;
-  __shared__ int fed_s;   // feed warps: chunks of A, in the order of this worker's units, that are there
+  __shared__ int fed_s;   // kFeeds: chunks of A, in the order of this worker's units, that are there
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -569,7 +572,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 ok = false;
                 break;
               }
-              if constexpr (Epi::kFeedWarps > 0) {
+              if constexpr (Epi::kFeeds) {
                 // the chunks of A that this stage needs are there
                 const int need = fed0 + feed_chunks(kb0, min(kb + Cfg::kKSub, hi));
                 if (fed < need) {
@@ -614,7 +617,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
           }
         }
-        if constexpr (Epi::kFeedWarps > 0) fed0 += feed_chunks(kb0, kb1);
+        if constexpr (Epi::kFeeds) fed0 += feed_chunks(kb0, kb1);
       }
       if (!ok && (CG == 1 || rank == 0)) {
         // let copies that were already issued land before the block's shared memory goes away
@@ -716,10 +719,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       for (int it = 0; it < (1 << 22) && !drained; ++it) drained = mbar_try_wait(smem_u32(&bar_drain), 0) != 0;
       if (!drained) latch_status(status, kStatusTimeout, (4 << 28) | (blockIdx.x << 8));
     }
-  } else if (Epi::kFeedWarps > 0 && warp >= 2 + Epi::kWarps) {
-    // ------------------------------------------------------------- feed warps (both CTAs)
-    if constexpr (Epi::kFeedWarps > 0) {
-      if (warp == 2 + Epi::kWarps + Epi::kFeedWarps) {
+  } else if (Epi::kSideWarps > 0 && warp >= 2 + Epi::kWarps) {
+    // ------------------------------------------------------------- side warps (both CTAs)
+    if constexpr (Epi::kFeeds) {
+      if (warp == 2 + Epi::kWarps + Epi::kSideWarps) {
         // The counters of the producer's chunks, one after the other, on its behalf: looking at one takes a microsecond.
         // (By the producer itself, at every eighth k-block, dH of 6912 rows at d = 1024 took 2.0 ms in place of 1.5.)
         if (lane == 0 && !Epi::feeds(ep, ex, n_workers)) {
@@ -743,8 +746,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           if (!ok) latch_status(status, kStatusTimeout, (6 << 28) | (blockIdx.x << 8) | 0xff);
         }
       } else if (Epi::feeds(ep, ex, n_workers)) {
-        Epi::feed(ep, ex, CG, n_workers);
+        Epi::side(ep, ex, CG, n_workers, warp - 2 - Epi::kWarps);
       }
+    } else if constexpr (Epi::kSideWarps > 0) {
+      Epi::side(ep, ex, CG, n_workers, warp - 2 - Epi::kWarps);
     }
   } else {
     // ------------------------------------------------------------- epilogue warps (both CTAs)

@@ -14,7 +14,8 @@ namespace rlh {
 // statistics 1200 / 1474 / 1858 / 4775 us with four, 985 / 1246 / 1607 / 4395 with eight).
 struct EpiStatsKL {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -142,7 +143,8 @@ __device__ __forceinline__ void st_planes(const float (&v)[32], uint16_t* hi, ui
 // A thread holds 32 consecutive columns of its row: four 32-byte stores, every sector written whole.
 struct EpiRefSweep {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -191,7 +193,8 @@ struct EpiRefSweep {
 // logits of the next 32 columns are loaded while these are worked on.
 struct EpiSweepKL {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -286,7 +289,8 @@ struct EpiSweepKL {
 // written to the bf16 slab exactly as EpiGrad does (swizzled staging + TMA bulk stores).
 struct EpiGradKL {
   static constexpr bool kParts = false;
-  static constexpr int kFeedWarps = 0;
+  static constexpr int kSideWarps = 0;
+  static constexpr bool kFeeds = false;
   static constexpr int kWarps = 8;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;

@@ -319,11 +319,12 @@ struct LogitGradWarp {
 // dH of one slab while its operand G is still being formed: kFeedWarps warps of every CTA do the jobs of LogitGradWarp, the
 // producer waits for the chunks it is about to load.
 struct EpiAccFed : EpiAcc {
-  static constexpr int kFeedWarps = 9;   // with the one that watches, sixteen warps in all: 128 registers a thread
+  static constexpr int kSideWarps = 9;   // with the one that watches, sixteen warps in all: 128 registers a thread
+  static constexpr bool kFeeds = true;
   struct Params : AccParams {
     FeedParams grad;
   };
-  __device__ static __forceinline__ void feed(const Params& p, const GemmExtents& ex, int cg, int n_workers) {
+  __device__ static __forceinline__ void side(const Params& p, const GemmExtents& ex, int cg, int n_workers, int) {
     LogitGradWarp::run(p.grad, ex, feed_order(ex, ex.m_rows, p.grad.ld, cg, n_workers), ex.slab_off, ex.m_rows);
   }
   __device__ static __forceinline__ bool feeds(const Params& p, const GemmExtents& ex, int n_workers) { return feed_pays(ex, n_workers); }

@@ -424,7 +424,7 @@ void launch_tiles(rl_ctx* c, int cg, int kind, const CUtensorMap& a, const CUten
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(c->grid[cg]);
-  cfg.blockDim = dim3(gemm_threads(Epi::kWarps, Epi::kFeedWarps));
+  cfg.blockDim = dim3(gemm_threads(Epi::kWarps, Epi::kSideWarps, Epi::kFeeds));
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -698,7 +698,7 @@ rl_status rl_create(rl_ctx** out, int device) {
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
             set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess &&
-            set_smem_attr<EpiAccFed, 0, 1>() == cudaSuccess &&
+            set_smem_attr<EpiAccScatter, 1, 1>() == cudaSuccess && set_smem_attr<EpiAccFed, 0, 1>() == cudaSuccess &&
             set_smem_attr_one<EpiAccFed, 0, 1, 2, kTileWide>() == cudaSuccess;
   if (!ok) { cudaFree(c->dstatus); delete c; return RL_ERR_CUDA; }
   {
@@ -707,7 +707,7 @@ rl_status rl_create(rl_ctx** out, int device) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(c->grid[2]);
-    cfg.blockDim = dim3(gemm_threads(EpiAcc::kWarps, EpiAcc::kFeedWarps));
+    cfg.blockDim = dim3(gemm_threads(EpiAcc::kWarps, EpiAcc::kSideWarps, EpiAcc::kFeeds));
     cfg.dynamicSmemBytes = g_smem_bytes<EpiAcc, 0, 0, 2, kTileSquare>;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1360,6 +1360,18 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
     const int r = reverse ? n_row_slabs - 1 - q : q;
     GemmShape dh_shape;
     memset(&dh_shape, 0, sizeof(dh_shape));
+    DhSource src;
+    src.acc = dH_acc;
+    src.d = (int)d;
+    src.cg = c->cta_group;
+    src.workers = dh_workers;
+    src.split_stride = (long long)L.Ts * d;
+    src.slots = dH_slots;
+    src.tile_rows = dh_tile_rows;
+    src.tile_cols = dh_cols;
+    src.row_map = row_map;
+    src.dH = dH;
+    src.f32 = o.dH_dtype;
     const int rows_cap = L.Ts;   // the valid rows are cut into equal slabs of at most Ts rows on the device
     // stream-K parts that finish a tile are added to the second accumulator buffer: it starts at zero
     if (dh_uses_stream_k(c)) cudaMemsetAsync(dH_acc + (size_t)L.Ts * d, 0, (size_t)L.Ts * d * 4, st);
@@ -1531,7 +1543,15 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         ep.n_cols = (int)d; ep.accumulate = o.accumulate_dW ? 1 : reverse ? 2 : (r > 0 ? 1 : 0);
         ep.n_valid = n_valid; ep.slab_cap = L.Tc; ep.slab_one = L.Ts; ep.slab_index = r;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
-        launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
+        if (!report && cs == n_col_slabs - 1) {
+          EpiAccScatter::Params es = {};
+          static_cast<AccParams&>(es) = ep;
+          src.shape = dh_shape;
+          es.dh = src;
+          launch_gemm<EpiAccScatter, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, es);
+        } else {
+          launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
+        }
         // these rows of dW are complete once the row slab that is walked last has added to them
         if (report) {
           const int64_t row0 = (int64_t)vocab_base + c0;
@@ -1540,21 +1560,14 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       }
       if (report) launch_dH();
     }
-    const int pr_sc = prof_begin(c, 7);
-    DhSource src;
-    src.acc = dH_acc;
-    src.d = (int)d;
-    src.shape = dh_shape;
-    src.cg = c->cta_group;
-    src.workers = dh_workers;
-    src.split_stride = (long long)L.Ts * d;
-    src.slots = dH_slots;
-    src.tile_rows = dh_tile_rows;
-    src.tile_cols = dh_cols;
-    if (o.dH_dtype) launch(c, scatter_dH_kernel<true>, c->n_sm * 8, 256, src, row_map, dH, c->dstatus);
-    else            launch(c, scatter_dH_kernel<false>, c->n_sm * 8, 256, src, row_map, dH, c->dstatus);
-    prof_end(c, pr_sc, 7);
-    c->launches++;
+    // dW of the last column slab has written dH in passing, unless it came before dH
+    if (c->dw_hook && q == n_row_slabs - 1) {
+      src.shape = dh_shape;
+      const int pr_sc = prof_begin(c, 7);
+      launch(c, scatter_dH_kernel, c->n_sm * 8, 256, src, c->dstatus);
+      prof_end(c, pr_sc, 7);
+      c->launches++;
+    }
   }
   return cuda_ok();
 }

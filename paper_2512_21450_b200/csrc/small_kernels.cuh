@@ -1284,7 +1284,8 @@ __global__ void __launch_bounds__(256) merge_shard_stats_kernel(const float4* __
 }
 
 // ------------------------------------------------------------------------------------------
-// dH of one row slab: fp32 accumulator rows -> rows of the caller's dH at their original positions, fp32 or bf16.
+// dH of one row slab: fp32 accumulator rows -> rows of the caller's dH at their original positions, fp32 or bf16.  Done by four
+// extra warps of the dW launch that follows (EpiAccScatter), or by a launch of its own where dW comes first.
 // The dH pass may have cut K into slices that accumulate in separate buffers, split_stride elements apart, or cut the
 // tiles of its last wave into parts that lie in slots: summed here in a fixed order.
 struct DhSource {
@@ -1295,6 +1296,9 @@ struct DhSource {
   long long split_stride;
   const float* slots;      // [slots][tile_rows][tile_cols], tiles cut by stream_k == 2
   int tile_rows, tile_cols;
+  const int* row_map;
+  void* dH;
+  int f32;                 // dH is fp32
 };
 
 __device__ __forceinline__ void add_piece(float4 (&x)[4], const float* q, int cols, int lane) {
@@ -1310,20 +1314,16 @@ __device__ __forceinline__ void add_piece(float4 (&x)[4], const float* q, int co
   }
 }
 
-// One warp per row and column tile (at most 512 columns: two groups of eight per lane).
-template <bool F32>
-__global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const int* __restrict__ row_map,
-                                                         void* __restrict__ dH, const DevStatus* st) {
-  chain_begin();
+// One warp per row and column tile (at most 512 columns: two groups of eight per lane); this is warp `warp` of n_warps.
+__device__ __forceinline__ void scatter_rows(const DhSource& s, int n_valid, unsigned warp, unsigned n_warps) {
   int slab_base, rows;
-  slab_extent(st->n_valid, s.shape.slab_cap, s.shape.slab_one, s.shape.slab_index, slab_base, rows);
-  const GemmExtents ex = gemm_extents(s.shape, st->n_valid, s.cg, s.workers);
+  slab_extent(n_valid, s.shape.slab_cap, s.shape.slab_one, s.shape.slab_index, slab_base, rows);
+  const GemmExtents ex = gemm_extents(s.shape, n_valid, s.cg, s.workers);
   const int slices = s.shape.stream_k == 1 ? 2 : ex.k_split;   // stream-K launches always keep two buffers
   const int lane = threadIdx.x & 31;
-  const int warps_per_block = blockDim.x >> 5;
   const unsigned col_tiles = (s.d + s.tile_cols - 1) / s.tile_cols;
   const unsigned units = (unsigned)rows * col_tiles;
-  for (unsigned u = blockIdx.x * warps_per_block + (threadIdx.x >> 5); u < units; u += gridDim.x * warps_per_block) {
+  for (unsigned u = warp; u < units; u += n_warps) {
     const int i = (int)(u / col_tiles), nt = (int)(u - i * col_tiles);
     const int cols = min(s.tile_cols, s.d - nt * s.tile_cols);
     const size_t col0 = (size_t)nt * s.tile_cols;
@@ -1348,14 +1348,14 @@ __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const
       const float* q = s.acc + (size_t)i * s.d + col0;
       for (int k = 0; k < slices; ++k, q += s.split_stride) add_piece(x, q, cols, lane);
     }
-    const size_t out = (size_t)row_map[slab_base + i] * s.d + col0;
+    const size_t out = (size_t)s.row_map[slab_base + i] * s.d + col0;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int v = lane + 32 * k;
       if (v * 8 >= cols) break;
       const float4 a = x[2 * k], b = x[2 * k + 1];
-      if (F32) {
-        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(dH) + out) + 2 * v;
+      if (s.f32) {
+        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(s.dH) + out) + 2 * v;
         __stcs(dst, a);
         __stcs(dst + 1, b);
       } else {
@@ -1366,11 +1366,28 @@ __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const
         o.y = *reinterpret_cast<uint32_t*>(&b1);
         o.z = *reinterpret_cast<uint32_t*>(&b2);
         o.w = *reinterpret_cast<uint32_t*>(&b3);
-        __stcs(reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(dH) + out) + v, o);
+        __stcs(reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(s.dH) + out) + v, o);
       }
     }
   }
 }
+
+__global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const DevStatus* st) {
+  chain_begin();
+  const unsigned per_block = blockDim.x >> 5;
+  scatter_rows(s, st->n_valid, blockIdx.x * per_block + (threadIdx.x >> 5), gridDim.x * per_block);
+}
+
+// dW of one slab; extra warps write dH of the same slab, which the launch before has left, meanwhile: a launch less.
+struct EpiAccScatter : EpiAcc {
+  static constexpr int kSideWarps = 4;
+  struct Params : AccParams {
+    DhSource dh;
+  };
+  __device__ static __forceinline__ void side(const Params& p, const GemmExtents&, int, int, int warp) {
+    scatter_rows(p.dh, *p.n_valid, blockIdx.x * kSideWarps + warp, gridDim.x * kSideWarps);
+  }
+};
 
 // ------------------------------------------------------------------------------------------
 // Exercises the bounded wait: one warp waits on an mbarrier that nothing ever arrives on, with a
