@@ -25,7 +25,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 struct RowStats {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kStagingBytes = 0;
   struct Params {
     const int* tokens_c;   // [rows] compact sampled-token ids
@@ -171,7 +171,7 @@ __device__ __forceinline__ void stage_half_box(const uint32_t (&w)[16], int c, u
 struct EpiSweep {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = 4;
   static constexpr int kStagingBytes = kEpiStaging;
   using Params = RowStats::Params;
@@ -265,7 +265,7 @@ template <int W>
 struct EpiGrad {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = W;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;
@@ -373,11 +373,17 @@ struct AccParams {
   int tile_cols;   // > 0: k_slice > 0 names slot k_slice - 1, a box of tile_cols columns x tile_rows rows of its own
   int tile_rows;
 };
-struct EpiAcc {
+// W: four warps, or eight for dW of few rows, where the time is the output's (K of a tile is short, and its 128 KB per CTA leave
+// through the epilogue).  Adding, the boxes of this worker's next tile are brought to L2 meanwhile: the adds otherwise wait for
+// DRAM one box at a time.  dW of 151936 words, d = 2048, four warps / eight: stores 282 / 264 us at 100 rows, 380 / 340 at 300, 468 / 430 at
+// 512, and slower from 1000 rows on; adds 542 / 425, 587 / 446, 602 / 524 (the four without prefetches; with them 413 / 494 / 544; a
+// plain kernel that adds in this order takes 400).
+template <int W>
+struct EpiAccW {
   static constexpr bool kParts = true;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
-  static constexpr int kWarps = 4;
+  static constexpr bool kFeeds = false, kAhead = W == 8;
+  static constexpr int kWarps = W;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;
   using Params = AccParams;
@@ -385,6 +391,7 @@ struct EpiAcc {
     int k_slice;
     int add;
     uint32_t n_issued;   // chunks handed to the TMA unit so far (selects the staging buffer)
+    int next_row, next_col;   // this warp's part of the next tile (row -1: none)
   };
   __device__ static __forceinline__ void init(State& st) { st.n_issued = 0; }
   __device__ static __forceinline__ void finish(State& st) {
@@ -408,6 +415,8 @@ struct EpiAcc {
     // the last store issued from this buffer must have finished reading it
     if (lane == 0) bulk_wait_group_read<kBufs - 1>();
     __syncwarp();
+    if (kAhead && lane == 0 && st.add && st.next_row >= 0 && st.next_row < m_rows && st.next_col + c * 32 < p.n_cols)
+      tma_prefetch_3d(tmC, st.next_col + c * 32, p.row_base + st.next_row, 0);
     // row `lane` of the box: 8 chunks of 16 bytes, chunk j stored at position j ^ (row & 7)
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -427,5 +436,6 @@ struct EpiAcc {
     st.n_issued++;
   }
   __device__ static __forceinline__ void end_unit(const Params&, State&, int, int, int, int) {}
-};
+};using EpiAcc = EpiAccW<4>;
+
 }  // namespace rlh

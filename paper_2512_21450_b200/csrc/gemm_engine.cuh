@@ -74,6 +74,9 @@ constexpr int kMinShare = 8;    // least k-blocks of a part of a cut tile
 constexpr int kPartCost = 20;   // k-blocks in whose time the output of one part leaves the chip (cut_tiles)
 constexpr int kHelpSplit = 16;  // most parts per cut tile for which the workers left over are given work (cut_tiles)
 constexpr int kFwdRange = 8;    // column tiles per work unit when there is plenty of work
+// K-blocks up to which an epilogue is told where this worker's next tile lies (Epi::kAhead): with more, the products take longer
+// than the output, and prefetches only get in the way.
+constexpr int kAheadBlocks = 10;
 // An A operand that is formed while it is read (Epi::kFeeds): a job is kFeedRows rows x kFeedCols columns (of K).
 constexpr int kFeedRows = 16;
 constexpr int kFeedCols = 512;
@@ -468,6 +471,7 @@ struct UnitWalk {
 //     static void pack(const State&, float (&)[kMerge]); static void merge(State&, const float (&)[kMerge]);   // if > 0
 //     static constexpr int kStagingBytes;                      // shared memory behind the ring (0 or 32 KB)
 //     static constexpr bool kParts;                            // knows what to do with parts of tiles (stream_k == 2)
+//     static constexpr bool kAhead;                            // State has next_row and next_col: this warp's first row and column of the next tile
 //     static constexpr int kSideWarps; static constexpr bool kFeeds; };   // if kSideWarps > 0:
 //     static void side(const Params&, const GemmExtents&, int cg, int n_workers, int warp);
 //   if kFeeds:
@@ -770,6 +774,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const int m = mu * CG + (int)rank;
       const int n0 = nr * ex.n_range, n1 = min(n0 + ex.n_range, sh.n_tiles);
       Epi::begin_unit(ep, st, m, nr, row_in_tile, ex.m_rows, ex.slab_off, ks);
+      if constexpr (Epi::kAhead) {
+        UnitWalk peek = walk;
+        int mu2, nr2, ks2, lo2, hi2;
+        const bool more = ex.k_blocks <= kAheadBlocks && peek.next(mu2, nr2, ks2, lo2, hi2);
+        st.next_row = more ? (mu2 * CG + (int)rank) * BM + q * 32 : -1;
+        st.next_col = more ? nr2 * BN : 0;
+      }
       for (int n = n0; n < n1 && ok; ++n, t += has_k ? 1u : 0u) {
         const uint32_t a = MODE == kTileSquare ? (t & 1u) : 0u;
         if (has_k) {

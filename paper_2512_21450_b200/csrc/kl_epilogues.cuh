@@ -15,7 +15,7 @@ namespace rlh {
 struct EpiStatsKL {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -144,7 +144,7 @@ __device__ __forceinline__ void st_planes(const float (&v)[32], uint16_t* hi, ui
 struct EpiRefSweep {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -194,7 +194,7 @@ struct EpiRefSweep {
 struct EpiSweepKL {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = 8;
   static constexpr int kStagingBytes = 0;
   struct Params {
@@ -290,7 +290,7 @@ struct EpiSweepKL {
 struct EpiGradKL {
   static constexpr bool kParts = false;
   static constexpr int kSideWarps = 0;
-  static constexpr bool kFeeds = false;
+  static constexpr bool kFeeds = false, kAhead = false;
   static constexpr int kWarps = 8;
   static constexpr int kMerge = 0;
   static constexpr int kStagingBytes = kEpiStaging;

@@ -153,6 +153,12 @@ __device__ __forceinline__ void tma_reduce_add_3d(const void* tmap, uint32_t src
                "r"(src), "r"(c0), "r"(c1), "r"(c2)
                : "memory");
 }
+// The box to L2.
+__device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0),
+               "r"(c1), "r"(c2)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Wait until at most N of this thread's bulk groups still have to read their shared-memory source.
 template <int N>

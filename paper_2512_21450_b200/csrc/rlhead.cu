@@ -136,6 +136,8 @@ inline bool use_wide(const rl_ctx* c, int64_t d) {
   const int64_t wide = (d + 2 * BN - 1) / (2 * BN) * 2, square = (d + BN - 1) / BN;
   return c->wide_tiles && c->cta_group == 2 && wide * kWideGain <= square * 100;
 }
+// Rows of a call up to which dW runs with eight epilogue warps (EpiAccW; how many of them are valid only the device knows).
+constexpr int64_t kFewRows = 640;
 // Width of a dH tile, and bytes of the slots its parts may need (two per worker).
 inline int dh_tile_cols(const rl_ctx* c, int64_t d) { return use_wide(c, d) ? 2 * BN : BN; }
 inline size_t dh_slot_bytes(const rl_ctx* c, int64_t d) {
@@ -698,7 +700,7 @@ rl_status rl_create(rl_ctx** out, int device) {
             set_smem_attr<EpiAcc, 1, 0>() == cudaSuccess && set_smem_attr<EpiAcc, 1, 1>() == cudaSuccess &&
             set_smem_attr_dual<EpiStatsKL>() == cudaSuccess && set_smem_attr_dual<EpiGradKL>() == cudaSuccess &&
             set_smem_attr_one<EpiAcc, 0, 1, 2, kTileWide>() == cudaSuccess &&
-            set_smem_attr<EpiAccScatter, 1, 1>() == cudaSuccess && set_smem_attr<EpiAccFed, 0, 1>() == cudaSuccess &&
+            set_smem_attr<EpiAccScatter<4>, 1, 1>() == cudaSuccess && set_smem_attr<EpiAccScatter<8>, 1, 1>() == cudaSuccess && set_smem_attr<EpiAccFed, 0, 1>() == cudaSuccess &&
             set_smem_attr_one<EpiAccFed, 0, 1, 2, kTileWide>() == cudaSuccess;
   if (!ok) { cudaFree(c->dstatus); delete c; return RL_ERR_CUDA; }
   {
@@ -1544,11 +1546,17 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         ep.n_valid = n_valid; ep.slab_cap = L.Tc; ep.slab_one = L.Ts; ep.slab_index = r;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
         if (!report && cs == n_col_slabs - 1) {
-          EpiAccScatter::Params es = {};
-          static_cast<AccParams&>(es) = ep;
           src.shape = dh_shape;
-          es.dh = src;
-          launch_gemm<EpiAccScatter, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, es);
+          auto dW_and_dH = [&](auto epi) {
+            typename decltype(epi)::Params es = {};
+            static_cast<AccParams&>(es) = ep;
+            es.dh = src;
+            launch_gemm<decltype(epi), 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, es);
+          };
+          // (a worker with one or two tiles has nothing for more epilogue warps to overlap: the smallest step 52.2 -> 52.9 us)
+          const long long tiles = (long long)d_tiles * ((cols + BN - 1) / BN);
+          if (T <= kFewRows && tiles >= 4 * dh_workers) dW_and_dH(EpiAccScatter<8>());
+          else                                          dW_and_dH(EpiAccScatter<4>());
         } else {
           launch_gemm<EpiAcc, 1, 1>(c, c->cta_group, 3, tmG_mn, tmHc_mn, tm_dW, tm_dW, sh, ep);
         }

@@ -1379,7 +1379,8 @@ __global__ void __launch_bounds__(256) scatter_dH_kernel(const DhSource s, const
 }
 
 // dW of one slab; extra warps write dH of the same slab, which the launch before has left, meanwhile: a launch less.
-struct EpiAccScatter : EpiAcc {
+template <int W>
+struct EpiAccScatter : EpiAccW<W> {
   static constexpr int kSideWarps = 4;
   struct Params : AccParams {
     DhSource dh;

@@ -130,3 +130,30 @@ def test_helped_parts_match_oracle(L_max, d, V, max_ctas, tiles, parts):
         _check_against_oracle(c, w, dH_fp32=True)
     finally:
         c.close()
+
+
+# dW of few rows on eight epilogue warps, stored and added to what was there (whose next tile is then on its way to L2): one and
+# several tiles per worker, a ragged last row tile and last column tile, K of one to ten blocks, a grid of few workers
+@pytest.mark.gpu
+@pytest.mark.parametrize("L_max,d,V,kw", [(2, 256, 80000, {}), (20, 320, 50001, {}), (75, 704, 33000, {}), (80, 1024, 20300, {}),
+                                         (40, 512, 9000, dict(max_ctas=6))])
+def test_dw_of_few_rows_adds_to_what_was_there(L_max, d, V, kw):
+    import torch
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.workloads import make_workload
+    from tests.test_gpu_parity import _check_against_oracle
+    w = make_workload(1, prompts=1, L_max=L_max, d=d, V=V, seed=6000 + V + L_max)
+    c = Context(0)
+    try:
+        c.set_max_ctas(kw.get("max_ctas", 0))
+        assert w.T <= 640 and -(-V // 256) * -(-d // 256) >= 2 * (kw.get("max_ctas", 148))
+        _check_against_oracle(c, w)
+        _, adv = c.rl_grpo_advantages(w.rewards, w.G, seq_offsets=w.seq_offsets, T=w.T)
+        args = (w.H, w.W, w.tokens, w.old_logp, w.ref_logp, adv, w.mask, w.eps_low, w.eps_high, w.beta)
+        plain = c.rl_policy_loss_fwd_bwd(*args)["dW"]
+        before = torch.randn(V, d, device="cuda") * float(plain.abs().max())
+        added = c.rl_policy_loss_fwd_bwd(*args, dW=before.clone(), accumulate_dW=True)["dW"]
+        torch.cuda.synchronize()
+        assert torch.equal(added, before + plain)   # one fp32 addition per entry
+    finally:
+        c.close()
