@@ -1,4 +1,5 @@
-"""ctypes binding of librlhead.so (C ABI declared in include/rlhead.h).
+"""ctypes binding of librlhead.so (C ABI declared in include/rlhead.h); the short calls go through _host_calls.so, which does
+the same marshalling natively, and fall back to ctypes for whatever that does not handle.
 
 Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  torch is used for device memory and streams.  There is no CPU
@@ -8,6 +9,7 @@ calls raise.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from ctypes import POINTER, byref, c_char_p, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 
@@ -157,7 +159,35 @@ def load_library():
                  "rl_profile_read"):
         getattr(lib, name).restype = c_int
     _lib = lib
+    _load_host_calls(lib)
     return lib
+
+
+_host = None
+HOST_PATH = os.path.join(_HERE, "_host_calls.so")
+
+
+def _load_host_calls(lib):
+    """The native host side of the short calls, handed the addresses of the functions that it calls."""
+    global _host
+    if not os.path.exists(HOST_PATH):
+        raise RuntimeError(f"{HOST_PATH} not built: run `python -m paper_2512_21450_b200.build`")
+    spec = importlib.util.spec_from_file_location("paper_2512_21450_b200._host_calls", HOST_PATH)
+    host = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(host)
+    host.bind(*(ctypes.cast(getattr(lib, name), c_void_p).value for name in (
+        "rl_workspace_bytes", "rl_workspace_bytes_logprobs", "rl_set_workspace", "rl_grpo_advantages_ex", "rl_kl_shaped_returns",
+        "rl_token_loss", "rl_token_logprobs", "rl_policy_loss_fwd_bwd_ex")))
+    _host = host
+
+
+def _handled(out, where):
+    """Whether _host_calls did the call; a status instead of results is raised."""
+    if out is NotImplemented:
+        return False
+    if type(out) is int:
+        raise RLHeadError(out, where)
+    return True
 
 
 def _ptr(t):
@@ -180,6 +210,7 @@ class Context:
         self.device = torch.device("cuda", device)
         self.handle = c_void_p()
         _check(self.lib.rl_create(byref(self.handle), device), "rl_create")
+        self._address = self.handle.value
         self._ws = None
         self._ws_key = None
         self._slot_busy = [False, False]
@@ -189,6 +220,7 @@ class Context:
         if self.handle:
             self.lib.rl_destroy(self.handle)
             self.handle = c_void_p()
+            self._address = 0
 
     def __del__(self):
         try:
@@ -258,6 +290,10 @@ class Context:
     # ------------------------------------------------------------------ calls
     def rl_grpo_advantages(self, rewards, group_size, ddof=1, eps_std=1e-6, seq_offsets=None, T=None):
         self._bind_stream()
+        if seq_offsets is not None:
+            out = _host.grpo_advantages(self._address, rewards, group_size, ddof, eps_std, seq_offsets, T)
+            if _handled(out, "rl_grpo_advantages_ex"):
+                return out
         assert rewards.dtype == torch.float32 and rewards.is_cuda and rewards.is_contiguous()
         adv_seq = torch.empty_like(rewards)
         if seq_offsets is None:
@@ -289,6 +325,10 @@ class Context:
 
     def rl_token_logprobs(self, H, W, tokens, mask=None):
         self._bind_stream()
+        if self._ws is not None:
+            out = _host.token_logprobs(self._address, self._ws, H, W, tokens, mask)
+            if _handled(out, "rl_token_logprobs"):
+                return out
         T, d = H.shape
         V = W.shape[0]
         assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and tokens.dtype == torch.int32
@@ -309,6 +349,13 @@ class Context:
         """H_ref [T, d_ref] and W_ref [V, d_ref] (bf16) switch the regulariser to the full-distribution
         KL(pi_theta || pi_ref) against softmax(W_ref h_ref); ref_logp is then unused."""
         self._bind_stream()
+        if (want_aux and H_ref is None and W_ref is None and dW is not None and dH is not None and loss is not None
+                and self._ws is not None):
+            out = _host.policy_loss(self._address, self._ws, H, W, tokens, old_logp, ref_logp, adv, mask, eps_low, eps_high, beta,
+                                    ent_coef, token_weight, accumulate_dW, dW, dH, loss, agg_mode, sequence_level, seq_offsets,
+                                    dH_fp32, token_count)
+            if _handled(out, "rl_policy_loss_fwd_bwd_ex"):
+                return dict(loss=loss, dH=dH, dW=dW, logp=out[0], entropy=out[1], metrics=out[2])
         T, d = H.shape
         V = W.shape[0]
         assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and tokens.dtype == torch.int32
@@ -375,6 +422,11 @@ class Context:
                              kl_tok=None, want_shaped=True, returns=None):
         """Token-level KL reward shaping: returns (shaped_reward [T] or None, returns [T])."""
         self._bind_stream()
+        if want_shaped and returns is None:
+            out = _host.kl_shaped_returns(self._address, seq_value, logp, ref_logp, mask, seq_offsets, T, beta, gamma,
+                                          self.KL_ESTIMATES[kind], kl_tok)
+            if _handled(out, "rl_kl_shaped_returns"):
+                return out
         assert seq_value.dtype == torch.float32 and seq_offsets.dtype == torch.int32
         for x in (logp, ref_logp, kl_tok):
             assert x is None or (x.dtype == torch.float32 and x.is_contiguous() and x.numel() == T)
@@ -393,6 +445,11 @@ class Context:
         """The per-token loss arithmetic on its own, from log-probabilities (and entropies) the caller holds:
         returns dict(loss [1], dlogp [T], dentropy [T], metrics [8]); `out` may carry preallocated tensors."""
         self._bind_stream()
+        if out is None and want_grads and want_metrics:
+            got = _host.token_loss(self._address, logp, entropy, old_logp, ref_logp, adv, mask, eps_low, eps_high, beta, ent_coef,
+                                   token_weight, token_count)
+            if _handled(got, "rl_token_loss"):
+                return dict(loss=got[0], dlogp=got[1], dentropy=got[2], metrics=got[3])
         T = logp.numel()
         for x in (logp, entropy, old_logp, ref_logp, adv, token_weight):
             assert x is None or (x.dtype == torch.float32 and x.is_contiguous() and x.numel() == T)

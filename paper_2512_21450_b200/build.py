@@ -1,15 +1,20 @@
-"""Build librlhead.so for sm_100a in-tree:  python -m paper_2512_21450_b200.build"""
+"""Build librlhead.so (the library, for sm_100a) and _host_calls.so (host side of the short calls) in-tree:
+python -m paper_2512_21450_b200.build"""
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-SRC = os.path.join(HERE, "csrc", "rlhead.cu")
+CSRC = os.path.join(HERE, "csrc")
+HEADER = os.path.join(ROOT, "include", "rlhead.h")
+SRC = os.path.join(CSRC, "rlhead.cu")
 OUT = os.path.join(HERE, "librlhead.so")
-DEPS = [os.path.join(HERE, "csrc", f) for f in os.listdir(os.path.join(HERE, "csrc"))] + \
-       [os.path.join(ROOT, "include", "rlhead.h")]
+DEPS = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [HEADER]
+HOST_SRC = os.path.join(CSRC, "host_calls.cpp")
+HOST_OUT = os.path.join(HERE, "_host_calls.so")
 
 
 def nvcc_path():
@@ -19,8 +24,28 @@ def nvcc_path():
     raise RuntimeError("nvcc not found")
 
 
+def current(out, deps):
+    return os.path.exists(out) and all(os.path.getmtime(out) >= os.path.getmtime(p) for p in deps)
+
+
+def build_host_calls(force=False):
+    if not force and current(HOST_OUT, [HOST_SRC, HEADER]):
+        return HOST_OUT
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], "-o", HOST_OUT, HOST_SRC,
+           "-L", lib, "-lc10", "-ltorch_cpu", "-ltorch_python"]
+    subprocess.run(cmd, check=True)
+    return HOST_OUT
+
+
 def build(force=False, verbose=False):
-    if not force and os.path.exists(OUT) and all(os.path.getmtime(OUT) >= os.path.getmtime(p) for p in DEPS):
+    build_host_calls(force)
+    if not force and current(OUT, DEPS):
         return OUT
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
            "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(HERE, "csrc"),

@@ -1,0 +1,92 @@
+"""The native host side of the short calls: what it does not handle it leaves to the general path, what it handles gives the same."""
+import pytest
+import torch
+
+
+def _host():
+    from paper_2512_21450_b200 import binding
+    binding.load_library()
+    return binding._host
+
+
+def test_unusual_arguments_are_left_to_the_general_path():
+    import numpy as np
+    h, x, i32 = _host(), torch.zeros(8), torch.zeros(3, dtype=torch.int32)
+
+    class Sub(torch.Tensor):
+        pass
+    for out in (h.token_loss(), h.token_loss(0, x),                                          # too few arguments
+                h.token_loss(0, x, x, x, x, x, None, 0.2, 0.2, 0.0, 0.0, None, None),        # memory of the host
+                h.token_loss(0, "x", x, x, x, x, None, 0.2, 0.2, 0.0, 0.0, None, None),
+                h.token_loss(2 ** 70, x, x, x, x, x, None, 0.2, 0.2, 0.0, 0.0, None, None),
+                h.token_loss(0, x.as_subclass(Sub), x, x, x, x, None, 0.2, 0.2, 0.0, 0.0, None, None),
+                h.grpo_advantages(0, x, np.int64(4), 1, 1e-6, i32, 8), h.grpo_advantages(0, x, 4, 1, 1e-6, i32, None),
+                h.kl_shaped_returns(0, x, x, x, None, i32, 8, 0.1, 1.0, 1, None),
+                h.token_logprobs(0, None, x, x, i32, None), h.policy_loss(*range(23))):
+        assert out is NotImplemented
+
+
+class _General:
+    """Leaves every call to the general path."""
+
+    def __getattr__(self, name):
+        return lambda *args: NotImplemented
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opt", [{}, dict(ent_coef=1e-2, agg_mode=1), dict(sequence_level=True), dict(accumulate_dW=True, agg_mode=2),
+                                 dict(weight=True), dict(count=True, dH_fp32=True), dict(beta=0.0), dict(strided=True)])
+def test_native_and_general_paths_agree(monkeypatch, opt):
+    from paper_2512_21450_b200 import Context, binding
+    g = torch.Generator(device="cuda").manual_seed(5)
+    n_seq, L, d, V = 6, 20, 192, 900
+    T = n_seq * L
+    wide = torch.randn(T, d + 64, generator=g, device="cuda", dtype=torch.bfloat16)
+    H = wide[:, :d] if opt.get("strided") else wide[:, :d].contiguous()
+    W = torch.randn(V, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    tok = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    mask = (torch.rand(T, generator=g, device="cuda") < 0.8).to(torch.uint8)
+    logp = -torch.rand(T, generator=g, device="cuda") * 9
+    old, ref, ent = logp + 0.05, logp - 0.1, -logp
+    rewards = torch.rand(n_seq, generator=g, device="cuda")
+    off = torch.arange(0, T + 1, L, dtype=torch.int32, device="cuda")
+    weight = torch.rand(T, generator=g, device="cuda") if opt.get("weight") else None
+    count = torch.tensor([100], device="cuda") if opt.get("count") else None
+    beta = opt.get("beta", 0.04)
+    out = []
+    for native in (True, False):
+        if not native:
+            monkeypatch.setattr(binding, "_host", _General())
+        c = Context(0)
+        try:
+            got = {}
+            for _ in range(2):   # the first call makes the workspace
+                got["adv_seq"], adv = c.rl_grpo_advantages(rewards, 3, seq_offsets=off, T=T)
+                got["adv"] = adv
+                got["shaped"], got["returns"] = c.rl_kl_shaped_returns(got["adv_seq"], logp, ref, mask, off, T, 0.02)
+                tl = c.rl_token_loss(logp, ent, old, ref if beta else None, adv, mask, 0.2, 0.3, beta, ent_coef=1e-2,
+                                     token_weight=weight, token_count=count)
+                got.update({"t_" + k: v for k, v in tl.items()})
+                got["score"], got["score_ent"], got["score_lse"] = c.rl_token_logprobs(H, W, tok, mask)
+                dH = torch.zeros(T, d, device="cuda", dtype=torch.float32 if opt.get("dH_fp32") else torch.bfloat16)
+                dW = torch.ones(V, d, device="cuda")
+                kw = {k: v for k, v in opt.items() if k in ("ent_coef", "agg_mode", "sequence_level", "accumulate_dW", "dH_fp32")}
+                got.update(c.rl_policy_loss_fwd_bwd(H, W, tok, old, ref if beta else None, adv, mask, 0.2, 0.3, beta, dW=dW, dH=dH,
+                                                    loss=torch.zeros(1, device="cuda"), seq_offsets=off, token_weight=weight,
+                                                    token_count=count, **kw))
+            # what the library refuses is refused alike
+            with pytest.raises(binding.RLHeadError, match="rl_token_loss"):
+                c.rl_token_loss(logp, ent, old, None, adv, mask, 0.2, 0.3, 0.04)
+            with pytest.raises(binding.RLHeadError, match="rl_grpo_advantages_ex"):
+                c.rl_grpo_advantages(rewards, 4, seq_offsets=off, T=T)
+            with pytest.raises(AssertionError):
+                c.rl_token_loss(logp, ent[:-1], old, ref, adv, mask, 0.2, 0.3, 0.04)
+            with pytest.raises(AssertionError):
+                c.rl_token_logprobs(H, W, tok.long(), mask)
+            torch.cuda.synchronize()
+            out.append(got)
+        finally:
+            c.close()
+    assert out[0].keys() == out[1].keys()
+    for k in out[0]:
+        assert out[0][k].dtype == out[1][k].dtype and out[0][k].shape == out[1][k].shape and torch.equal(out[0][k], out[1][k]), k
