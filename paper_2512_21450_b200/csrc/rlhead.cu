@@ -504,8 +504,9 @@ inline int row_group_tiles(const rl_ctx* c, int64_t k) {
 
 void launch_merge(rl_ctx* c, const LossParams& p, int64_t rows, int ranges, int slabs = 1) {
   const int blocks = merge_blocks(rows, slabs, ranges);
-  if (merge_by_thread(rows, ranges)) launch(c, combine_loss_kernel<1>, blocks, kLossThreads, p, c->dstatus);
-  else                               launch(c, combine_loss_kernel<kLossThreads / 32>, blocks, kLossThreads, p, c->dstatus);
+  auto merge = [&](auto plain, auto clearing) { launch(c, p.n_clear > 0 ? clearing : plain, blocks, kLossThreads, p, c->dstatus); };
+  if (merge_by_thread(rows, ranges)) merge(combine_loss_kernel<1, false>, combine_loss_kernel<1, true>);
+  else merge(combine_loss_kernel<kLossThreads / 32, false>, combine_loss_kernel<kLossThreads / 32, true>);
   c->launches++;
 }
 

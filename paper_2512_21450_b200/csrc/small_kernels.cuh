@@ -810,12 +810,14 @@ __device__ __forceinline__ void finish_loss(const double (&acc)[kLossSums], cons
 // What the loss needs besides is loaded before the merge, one round trip instead of three.  kW = 8 (a block) where rows are
 // few: with one thread per row a call of a few hundred rows and 75 to 148 ranges was a chain of that many loads, 17 us.
 // kW = 1 where there are rows enough to fill the machine, and where there is nothing to merge (merge_by_thread).
-template <int kW>
+// CLEAR: the counters of gradient jobs that follow are cleared in passing.
+template <int kW, bool CLEAR>
 __global__ void __launch_bounds__(kLossThreads) combine_loss_kernel(const LossParams p, DevStatus* st) {
   chain_begin();
   constexpr int kTeams = kLossThreads / 32 / kW;
   __shared__ float part_s[2][7][kW][kW > 1 ? 32 : 1];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n_clear; i += gridDim.x * blockDim.x) p.clear[i] = make_uint4(0, 0, 0, 0);
+  if (CLEAR)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n_clear; i += gridDim.x * blockDim.x) p.clear[i] = make_uint4(0, 0, 0, 0);
   const int n = st->n_valid;
   const int n_ranges = p.ext_lse ? 0 : st->n_ranges;
   const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % kW, team = (threadIdx.x >> 5) / kW;
