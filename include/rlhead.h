@@ -447,7 +447,8 @@ rl_status rl_token_logprobs_static(void* cuda_stream, const void* H, int64_t ldH
  * on the context's stream (at most 65536 launch groups are kept between two reads; later ones go untimed).
  * rl_profile_read: synchronises the stream and returns, per kernel kind (0 logits (statistics, and
  * the logits themselves where they are formed once), 1 gradient-of-logits slab, 2 dH, 3 dW, 4 mask scan, 5 row preparation, 6 merge + loss,
- * 7 dH scatter, 8 advantages), the summed device time in milliseconds ms[9] (host) and the number
+ * 7 dH to the caller's rows in a launch of its own, 8 advantages; the gradient of kept logits may be formed, and dH written, by extra warps of the
+ * launches of kinds 2 and 3), the summed device time in milliseconds ms[9] (host) and the number
  * of timed launch groups launches[9] (host) since the previous read.  The paper has no
  * counterpart; these exist so that a benchmark can report per-kernel roofline figures. */
 rl_status rl_launch_count(rl_ctx* ctx, int64_t* n);
