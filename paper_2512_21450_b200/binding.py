@@ -158,8 +158,8 @@ def load_library():
                  "rl_policy_loss_fwd_bwd_host", "rl_selftest_gemm", "rl_launch_count", "rl_set_profiling",
                  "rl_profile_read"):
         getattr(lib, name).restype = c_int
-    _lib = lib
     _load_host_calls(lib)
+    _lib = lib   # last: whoever finds it finds the host half too
     return lib
 
 

@@ -9,6 +9,18 @@ def _host():
     return binding._host
 
 
+def test_library_is_published_with_its_host_half(monkeypatch):
+    from paper_2512_21450_b200 import binding
+
+    def fails(lib):
+        raise RuntimeError("no host half")
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_load_host_calls", fails)
+    for _ in range(2):   # the second call must not return a library whose short calls have no host half
+        with pytest.raises(RuntimeError, match="no host half"):
+            binding.load_library()
+
+
 def test_unusual_arguments_are_left_to_the_general_path():
     import numpy as np
     h, x, i32 = _host(), torch.zeros(8), torch.zeros(3, dtype=torch.int32)
