@@ -1,4 +1,4 @@
-"""ctypes binding of librlhead.so (C ABI declared in include/rlhead.h); the short calls go through _host_calls.so, which does
+"""ctypes binding of librlhead.so (C ABI declared in include/rlhead.h); the short calls go through _host_calls.*.so, which does
 the same marshalling natively, and fall back to ctypes for whatever that does not handle.
 
 Argument marshalling only: every step of the path runs in the library's CUDA
@@ -11,6 +11,8 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sys
+import warnings
 from ctypes import POINTER, byref, c_char_p, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 
 import torch
@@ -164,17 +166,30 @@ def load_library():
 
 
 _host = None
-HOST_PATH = os.path.join(_HERE, "_host_calls.so")
+# It is compiled against one Python and one torch: another of either needs another file.
+HOST_PATH = os.path.join(_HERE, f"_host_calls.{sys.implementation.cache_tag}-torch-{torch.__version__}.so")
+
+
+class _NoHostCalls:
+    """Leaves every call to the general path."""
+
+    def __getattr__(self, name):
+        return lambda *args: NotImplemented
 
 
 def _load_host_calls(lib):
-    """The native host side of the short calls, handed the addresses of the functions that it calls."""
+    """The native host side of the short calls, handed the addresses of the functions that it calls.  Without it every call takes
+    the general path, which handles them all: the GPU's work is the same, the host's takes longer."""
     global _host
-    if not os.path.exists(HOST_PATH):
-        raise RuntimeError(f"{HOST_PATH} not built: run `python -m paper_2512_21450_b200.build`")
     spec = importlib.util.spec_from_file_location("paper_2512_21450_b200._host_calls", HOST_PATH)
-    host = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(host)
+    try:
+        host = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(host)
+    except ImportError as e:
+        warnings.warn(f"calls are marshalled in Python, {HOST_PATH} cannot be loaded ({e}): run `python -m paper_2512_21450_b200.build`",
+                      RuntimeWarning, stacklevel=3)
+        _host = _NoHostCalls()
+        return
     host.bind(*(ctypes.cast(getattr(lib, name), c_void_p).value for name in (
         "rl_workspace_bytes", "rl_workspace_bytes_logprobs", "rl_set_workspace", "rl_grpo_advantages_ex", "rl_kl_shaped_returns",
         "rl_token_loss", "rl_token_logprobs", "rl_policy_loss_fwd_bwd_ex")))

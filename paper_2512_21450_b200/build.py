@@ -1,10 +1,12 @@
-"""Build librlhead.so (the library, for sm_100a) and _host_calls.so (host side of the short calls) in-tree:
+"""Build librlhead.so (the library, for sm_100a) and _host_calls.*.so (host side of the short calls) in-tree:
 python -m paper_2512_21450_b200.build"""
 import os
 import shutil
 import subprocess
 import sys
 import sysconfig
+
+from .binding import HOST_PATH as HOST_OUT
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -14,7 +16,6 @@ SRC = os.path.join(CSRC, "rlhead.cu")
 OUT = os.path.join(HERE, "librlhead.so")
 DEPS = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [HEADER]
 HOST_SRC = os.path.join(CSRC, "host_calls.cpp")
-HOST_OUT = os.path.join(HERE, "_host_calls.so")
 
 
 def nvcc_path():
@@ -44,8 +45,8 @@ def build_host_calls(force=False):
 
 
 def build(force=False, verbose=False):
-    build_host_calls(force)
     if not force and current(OUT, DEPS):
+        build_host_calls(force)
         return OUT
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
            "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(HERE, "csrc"),
@@ -54,6 +55,7 @@ def build(force=False, verbose=False):
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
     subprocess.run(cmd, check=True)
+    build_host_calls(force)   # last: the library does not need it
     return OUT
 
 

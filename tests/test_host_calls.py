@@ -21,6 +21,28 @@ def test_library_is_published_with_its_host_half(monkeypatch):
             binding.load_library()
 
 
+@pytest.mark.parametrize("content", [None, b"", b"\x7fELF of another Python"])
+def test_calls_are_general_without_a_loadable_host_half(monkeypatch, tmp_path, content):
+    from paper_2512_21450_b200 import binding
+    path = tmp_path / "_host_calls.so"
+    if content is not None:
+        path.write_bytes(content)
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_host", None)
+    monkeypatch.setattr(binding, "HOST_PATH", str(path))
+    with pytest.warns(RuntimeWarning, match="marshalled in Python"):
+        lib = binding.load_library()
+    assert binding.load_library() is lib and binding.debug_workspace(256, 256, 4096)[0] > 0
+    assert not binding._handled(binding._host.token_loss(0, None), "rl_token_loss")
+
+
+def test_host_half_is_named_after_what_it_was_built_for():
+    import sys
+    from paper_2512_21450_b200 import binding, build
+    assert build.HOST_OUT == binding.HOST_PATH
+    assert sys.implementation.cache_tag in build.HOST_OUT and torch.__version__ in build.HOST_OUT
+
+
 def test_unusual_arguments_are_left_to_the_general_path():
     import numpy as np
     h, x, i32 = _host(), torch.zeros(8), torch.zeros(3, dtype=torch.int32)
