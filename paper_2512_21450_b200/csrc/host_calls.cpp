@@ -250,7 +250,7 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
       o.seq_offsets = data<int32_t>(offsets);
       o.n_seq = offsets->numel() - 1;
     }
-    o.dH_dtype = a.integer() != 0;
+    o.dH_dtype = a.small();   // (the library says which values it knows)
     const at::Tensor* count = a.of(at::kLong, true);
     if (count && count->numel() != 1) throw General();
     o.token_count = data<int64_t>(count);

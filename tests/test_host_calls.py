@@ -113,6 +113,10 @@ def test_native_and_general_paths_agree(monkeypatch, opt):
                 c.rl_token_loss(logp, ent, old, None, adv, mask, 0.2, 0.3, 0.04)
             with pytest.raises(binding.RLHeadError, match="rl_grpo_advantages_ex"):
                 c.rl_grpo_advantages(rewards, 4, seq_offsets=off, T=T)
+            for bad in (2, -1):
+                with pytest.raises(binding.RLHeadError, match="rl_policy_loss_fwd_bwd_ex"):
+                    c.rl_policy_loss_fwd_bwd(H, W, tok, old, ref, adv, mask, 0.2, 0.3, 0.04, dW=dW, dH=torch.zeros(T, d, device="cuda"),
+                                             loss=torch.zeros(1, device="cuda"), dH_fp32=bad)
             with pytest.raises(AssertionError):
                 c.rl_token_loss(logp, ent[:-1], old, ref, adv, mask, 0.2, 0.3, 0.04)
             with pytest.raises(AssertionError):
