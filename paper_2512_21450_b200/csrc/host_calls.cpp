@@ -89,44 +89,58 @@ struct Args {
 
 template <class T>
 T* data(const at::Tensor* t) { return t ? static_cast<T*>(t->data_ptr()) : nullptr; }
-at::Tensor fresh(int64_t n, const at::Tensor& like) { return at::empty({n}, like.options().dtype(at::kFloat).requires_grad(false)); }
 
-PyObject* general() { return Py_NewRef(Py_NotImplemented); }
+// The interpreter's lock is given up for as long as this lives, as ctypes and torch give it up: an allocation may wait for the GPU,
+// the call may lead back into Python (a hook), and other threads launch what the GPU waits for.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
 
-// The ABI call without the interpreter's lock, as ctypes makes it (a hook may call back into Python).
-template <class F>
-rl_status unlocked(F f) {
-  rl_status s;
-  Py_BEGIN_ALLOW_THREADS
-  s = f();
-  Py_END_ALLOW_THREADS
-  return s;
-}
+// What a call returns.
+struct Outputs {
+  at::Tensor t[4];
+  int n = 0;
+  void* add(at::Tensor x) {
+    t[n] = std::move(x);
+    return t[n++].data_ptr();
+  }
+  // [n] fp32 on the device of `like`
+  float* values(int64_t n_values, const at::Tensor& like) {
+    return static_cast<float*>(add(at::empty({n_values}, like.options().dtype(at::kFloat).requires_grad(false))));
+  }
+};
 
-// Runs f, which returns a new reference, or a status other than RL_OK as an int for the caller to raise.
+// f reads the arguments, allocates the outputs and makes the call, last; a status other than RL_OK is returned as an int for the
+// caller to raise.  Only what is thrown before the call sends its caller to the general path, which makes the call again.
 template <class F>
 PyObject* guarded(F f) {
+  Outputs out;
+  rl_status s;
   try {
-    return f();
-  } catch (const General&) {
-    return general();
-  } catch (...) {   // e.g. a tensor whose memory cannot be taken: the general path says why
+    s = f(out);
+  } catch (...) {   // General, or e.g. a tensor whose memory cannot be taken: the general path says why
     PyErr_Clear();
-    return general();
+    return Py_NewRef(Py_NotImplemented);
   }
-}
-PyObject* failed(rl_status s) { return PyLong_FromLong((long)s); }
-
-PyObject* tuple_of(std::initializer_list<at::Tensor> ts) {
-  PyObject* out = PyTuple_New((Py_ssize_t)ts.size());
-  Py_ssize_t i = 0;
-  for (const at::Tensor& t : ts) PyTuple_SET_ITEM(out, i++, THPVariable_Wrap(t));
-  return out;
+  if (s != RL_OK) return PyLong_FromLong((long)s);
+  PyObject* result = PyTuple_New(out.n);
+  for (int i = 0; result && i < out.n; ++i) {
+    PyObject* o = nullptr;
+    try {
+      o = THPVariable_Wrap(std::move(out.t[i]));
+    } catch (...) {
+      if (!PyErr_Occurred()) PyErr_NoMemory();
+    }
+    if (o) PyTuple_SET_ITEM(result, i, o);
+    else   Py_CLEAR(result);
+  }
+  return result;
 }
 
 // (context, rewards, group_size, ddof, eps_std, seq_offsets, T) -> (adv_seq, adv_tok)
 PyObject* grpo_advantages(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  return guarded([&]() -> PyObject* {
+  return guarded([&](Outputs& out) {
     Args a(args, nargs, 7);
     rl_ctx* c = a.context();
     const at::Tensor* rewards = a.of(at::kFloat, false);
@@ -136,19 +150,19 @@ PyObject* grpo_advantages(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     const at::Tensor* offsets = a.of(at::kInt, false);
     const int64_t T = a.integer();
     if (T < 0) throw General();
-    at::Tensor seq = at::empty(rewards->sizes(), rewards->options().requires_grad(false)), tok = fresh(T, *rewards);
     const float* r = data<float>(rewards);
     const int32_t* o = data<int32_t>(offsets);
-    float *ps = data<float>(&seq), *pt = data<float>(&tok);
     const int64_t n = rewards->numel();
-    const rl_status s = unlocked([&] { return abi.grpo_advantages_ex(c, r, n, group, ddof, eps, o, T, ps, pt); });
-    return s == RL_OK ? tuple_of({seq, tok}) : failed(s);
+    Unlocked u;
+    float* seq = static_cast<float*>(out.add(at::empty(rewards->sizes(), rewards->options().requires_grad(false))));
+    float* tok = out.values(T, *rewards);
+    return abi.grpo_advantages_ex(c, r, n, group, ddof, eps, o, T, seq, tok);
   });
 }
 
 // (context, seq_value, logp, ref_logp, mask, seq_offsets, T, beta, gamma, kind, kl_tok) -> (shaped, returns)
 PyObject* kl_shaped_returns(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  return guarded([&]() -> PyObject* {
+  return guarded([&](Outputs& out) {
     Args a(args, nargs, 11);
     rl_ctx* c = a.context();
     const at::Tensor* value = a.of(at::kFloat, false);
@@ -161,21 +175,20 @@ PyObject* kl_shaped_returns(PyObject*, PyObject* const* args, Py_ssize_t nargs) 
     const float beta = a.real(), gamma = a.real();
     const int kind = a.small();
     const at::Tensor* kl = a.values(T, true);
-    at::Tensor shaped = fresh(T, *value), returns = fresh(T, *value);
     const float *pv = data<float>(value), *pl = data<float>(logp), *pr = data<float>(ref), *pk = data<float>(kl);
     const uint8_t* pm = static_cast<const uint8_t*>(data<void>(mask));
     const int32_t* po = data<int32_t>(offsets);
-    float *ps = data<float>(&shaped), *pt = data<float>(&returns);
     const int64_t n = offsets->numel() - 1;
-    const rl_status s = unlocked([&] { return abi.kl_shaped_returns(c, pv, pl, pr, pk, pm, po, n, T, beta, gamma, kind, ps, pt); });
-    return s == RL_OK ? tuple_of({shaped, returns}) : failed(s);
+    Unlocked u;
+    float *shaped = out.values(T, *value), *returns = out.values(T, *value);
+    return abi.kl_shaped_returns(c, pv, pl, pr, pk, pm, po, n, T, beta, gamma, kind, shaped, returns);
   });
 }
 
 // (context, logp, entropy, old_logp, ref_logp, adv, mask, eps_low, eps_high, beta, ent_coef, token_weight, token_count)
 // -> (loss, dlogp, dentropy, metrics)
 PyObject* token_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  return guarded([&]() -> PyObject* {
+  return guarded([&](Outputs& out) {
     Args a(args, nargs, 13);
     rl_ctx* c = a.context();
     const at::Tensor* logp = a.of(at::kFloat, false);
@@ -186,15 +199,13 @@ PyObject* token_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     if (mask && mask->numel() != T) throw General();
     const float lo = a.real(), hi = a.real(), beta = a.real(), ec = a.real();
     const at::Tensor *weight = a.values(T, true), *count = a.of(at::kLong, true);
-    at::Tensor loss = fresh(1, *logp), dlogp = fresh(T, *logp), dent = fresh(T, *logp), metrics = fresh(8, *logp);
     const float *pl = data<float>(logp), *pe = data<float>(ent), *po = data<float>(old), *pr = data<float>(ref), *pa = data<float>(adv),
                 *pw = data<float>(weight);
     const uint8_t* pm = data<uint8_t>(mask);
     const void* pc = data<void>(count);
-    float *q0 = data<float>(&loss), *q1 = data<float>(&dlogp), *q2 = data<float>(&dent), *q3 = data<float>(&metrics);
-    const rl_status s =
-        unlocked([&] { return abi.token_loss(c, pl, pe, po, pr, pa, pm, T, lo, hi, beta, ec, pw, pc, q0, q1, q2, q3); });
-    return s == RL_OK ? tuple_of({loss, dlogp, dent, metrics}) : failed(s);
+    Unlocked u;
+    float *loss = out.values(1, *logp), *dlogp = out.values(T, *logp), *dent = out.values(T, *logp), *metrics = out.values(8, *logp);
+    return abi.token_loss(c, pl, pe, po, pr, pa, pm, T, lo, hi, beta, ec, pw, pc, loss, dlogp, dent, metrics);
   });
 }
 
@@ -206,29 +217,28 @@ void bind_workspace(rl_ctx* c, const at::Tensor* ws, decltype(&rl_workspace_byte
 
 // (context, workspace, H, W, tokens, mask) -> (logp, entropy, lse)
 PyObject* token_logprobs(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  return guarded([&]() -> PyObject* {
+  return guarded([&](Outputs& out) {
     Args a(args, nargs, 6);
     rl_ctx* c = a.context();
     const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows(), *tokens = a.of(at::kInt, false), *mask = a.tensor(true);
     const int64_t T = H->size(0), d = H->size(1), V = W->size(0);
     if (T == 0) throw General();
     bind_workspace(c, ws, abi.workspace_bytes_logprobs, T, d, V);
-    at::Tensor logp = fresh(T, *H), ent = fresh(T, *H), lse = fresh(T, *H);
     const void *ph = H->data_ptr(), *pw = W->data_ptr();
     const int64_t ldH = H->stride(0), ldW = W->stride(0);
     const int32_t* pt = data<int32_t>(tokens);
     const uint8_t* pm = static_cast<const uint8_t*>(data<void>(mask));
-    float *q0 = data<float>(&logp), *q1 = data<float>(&ent), *q2 = data<float>(&lse);
-    const rl_status s = unlocked([&] { return abi.token_logprobs(c, ph, ldH, pw, ldW, pt, pm, T, d, V, q0, q1, q2); });
-    return s == RL_OK ? tuple_of({logp, ent, lse}) : failed(s);
+    Unlocked u;
+    float *logp = out.values(T, *H), *ent = out.values(T, *H), *lse = out.values(T, *H);
+    return abi.token_logprobs(c, ph, ldH, pw, ldW, pt, pm, T, d, V, logp, ent, lse);
   });
 }
 
 // (context, workspace, H, W, tokens, old_logp, ref_logp, adv, mask, eps_low, eps_high, beta, ent_coef, token_weight, accumulate_dW,
-//  dW, dH, loss, agg_mode, sequence_level, seq_offsets, dH_fp32, token_count) -> (loss, logp, entropy, metrics); loss, dH and dW are
-// the caller's
+//  dW, dH, loss, agg_mode, sequence_level, seq_offsets, dH_fp32, token_count) -> (logp, entropy, metrics); loss, dH and dW are the
+// caller's
 PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  return guarded([&]() -> PyObject* {
+  return guarded([&](Outputs& out) {
     Args a(args, nargs, 23);
     rl_ctx* c = a.context();
     const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows(), *tokens = a.of(at::kInt, false);
@@ -255,10 +265,6 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     if (count && count->numel() != 1) throw General();
     o.token_count = data<int64_t>(count);
     bind_workspace(c, ws, abi.workspace_bytes, T, d, V);
-    at::Tensor logp = fresh(T, *W), ent = fresh(T, *W), metrics = fresh(8, *W);
-    o.logp_out = data<float>(&logp);
-    o.entropy_out = data<float>(&ent);
-    o.metrics_out = data<float>(&metrics);
     const void *ph = H->data_ptr(), *pw = W->data_ptr();
     const int64_t ldH = H->stride(0), ldW = W->stride(0);
     const int32_t* pt = data<int32_t>(tokens);
@@ -266,10 +272,11 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     const uint8_t* pm = static_cast<const uint8_t*>(data<void>(mask));
     float *pl = static_cast<float*>(data<void>(loss)), *pd = static_cast<float*>(data<void>(dW));
     void* ph_out = data<void>(dH);
-    const rl_status s = unlocked([&] {
-      return abi.policy_loss_fwd_bwd_ex(c, ph, ldH, pw, ldW, pt, po, pr, pa, pm, T, d, V, lo, hi, beta, pl, ph_out, pd, &o);
-    });
-    return s == RL_OK ? tuple_of({logp, ent, metrics}) : failed(s);
+    Unlocked u;
+    o.logp_out = out.values(T, *W);
+    o.entropy_out = out.values(T, *W);
+    o.metrics_out = out.values(8, *W);
+    return abi.policy_loss_fwd_bwd_ex(c, ph, ldH, pw, ldW, pt, po, pr, pa, pm, T, d, V, lo, hi, beta, pl, ph_out, pd, &o);
   });
 }
 

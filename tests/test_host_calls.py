@@ -128,3 +128,68 @@ def test_native_and_general_paths_agree(monkeypatch, opt):
     assert out[0].keys() == out[1].keys()
     for k in out[0]:
         assert out[0][k].dtype == out[1][k].dtype and out[0][k].shape == out[1][k].shape and torch.equal(out[0][k], out[1][k]), k
+
+
+# A device allocator that counts its calls, and those made by a thread that holds the interpreter's lock
+_PROBE = """
+#include <Python.h>
+#include <cuda_runtime_api.h>
+extern "C" {
+int calls = 0, held = 0;
+void* probe_alloc(ssize_t n, int, cudaStream_t) {
+  void* p = nullptr;
+  ++calls;
+  held += PyGILState_Check();
+  cudaMalloc(&p, n);
+  return p;
+}
+void probe_free(void* p, ssize_t, int, cudaStream_t) { cudaFree(p); }
+}
+"""
+
+
+@pytest.mark.gpu
+def test_other_threads_run_while_outputs_are_allocated(tmp_path):
+    """An allocation may wait for the GPU, and the GPU for what another thread is about to launch."""
+    import ctypes
+    import os
+    import subprocess
+    import sysconfig
+    from paper_2512_21450_b200 import Context
+    from paper_2512_21450_b200.build import nvcc_path
+    src, so = tmp_path / "probe.cpp", str(tmp_path / "probe.so")
+    src.write_text(_PROBE)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
+    subprocess.run(["g++", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", cuda, "-o", so, str(src)], check=True)
+    T, d, V = 5000, 64, 300
+    x = -torch.rand(T, device="cuda") - 1
+    H = torch.randn(T, d, device="cuda").bfloat16()
+    W = torch.randn(V, d, device="cuda").bfloat16()
+    tok, mask = torch.zeros(T, dtype=torch.int32, device="cuda"), torch.ones(T, dtype=torch.uint8, device="cuda")
+    off = torch.arange(0, T + 1, 1000, dtype=torch.int32, device="cuda")
+    rewards = torch.rand(5, device="cuda")
+    dH, dW, loss = torch.zeros(T, d, device="cuda", dtype=torch.bfloat16), torch.zeros(V, d, device="cuda"), torch.zeros(1, device="cuda")
+    c = Context(0)
+    try:
+        c.ensure_workspace(T, d, V)
+        c._bind_stream()
+        h, probe = _host(), ctypes.CDLL(so)
+        allocator = torch.cuda.memory.CUDAPluggableAllocator(so, "probe_alloc", "probe_free").allocator()
+        calls, held = (ctypes.c_int.in_dll(probe, name) for name in ("calls", "held"))
+        for call in (lambda: h.grpo_advantages(c._address, rewards, 5, 1, 1e-6, off, T),
+                     lambda: h.kl_shaped_returns(c._address, rewards, x, x, mask, off, T, 0.1, 1.0, 1, None),
+                     lambda: h.token_loss(c._address, x, x, x, x, x, mask, 0.2, 0.2, 0.04, 0.0, None, None),
+                     lambda: h.token_logprobs(c._address, c._ws, H, W, tok, mask),
+                     lambda: h.policy_loss(c._address, c._ws, H, W, tok, x, x, x, mask, 0.2, 0.2, 0.04, 0.0, None, False, dW, dH, loss,
+                                           0, False, None, False, None)):
+            before = calls.value
+            pool = torch.cuda.MemPool(allocator)
+            with torch.cuda.use_mem_pool(pool):
+                out = call()
+            assert type(out) is tuple and calls.value > before
+            torch.cuda.synchronize()
+            del out, pool
+            torch.cuda.empty_cache()   # what the pool held goes back while the allocator is there
+        assert held.value == 0
+    finally:
+        c.close()
