@@ -210,6 +210,16 @@ def _ptr(t):
     return 0 if t is None else t.data_ptr()
 
 
+def _check_array(x, n, dtype=torch.float32):
+    """x (None: not given) is read or written by address: n entries of dtype, one behind the other."""
+    assert x is None or (x.dtype == dtype and x.is_contiguous() and x.numel() >= n)
+
+
+def _check_rows(T, tokens, mask):
+    _check_array(tokens, T, torch.int32)
+    assert mask is None or (mask.element_size() == 1 and mask.is_contiguous() and mask.numel() >= T)
+
+
 def _check(status, where):
     if status != 0:
         raise RLHeadError(status, where)
@@ -346,8 +356,9 @@ class Context:
                 return out
         T, d = H.shape
         V = W.shape[0]
-        assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and tokens.dtype == torch.int32
+        assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16
         assert H.stride(1) == 1 and W.stride(1) == 1
+        _check_rows(T, tokens, mask)
         self.ensure_workspace(T, d, V, scoring=True)
         logp = torch.empty(T, dtype=torch.float32, device=H.device)
         ent = torch.empty_like(logp)
@@ -373,8 +384,14 @@ class Context:
                 return dict(loss=loss, dH=dH, dW=dW, logp=out[0], entropy=out[1], metrics=out[2])
         T, d = H.shape
         V = W.shape[0]
-        assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and tokens.dtype == torch.int32
+        assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16
         assert H.stride(1) == 1 and W.stride(1) == 1
+        _check_rows(T, tokens, mask)
+        for x in (old_logp, ref_logp, adv, token_weight):
+            _check_array(x, T)
+        _check_array(loss, 1)
+        _check_array(dH, T * d, torch.float32 if dH_fp32 else torch.bfloat16)
+        _check_array(dW, V * d)
         kl_full = W_ref is not None
         if kl_full:
             assert H_ref is not None and H_ref.dtype == torch.bfloat16 and W_ref.dtype == torch.bfloat16
@@ -443,6 +460,8 @@ class Context:
             if _handled(out, "rl_kl_shaped_returns"):
                 return out
         assert seq_value.dtype == torch.float32 and seq_offsets.dtype == torch.int32
+        _check_array(seq_value, seq_offsets.numel() - 1)
+        _check_rows(T, None, mask)
         for x in (logp, ref_logp, kl_tok):
             assert x is None or (x.dtype == torch.float32 and x.is_contiguous() and x.numel() == T)
         dev = seq_value.device
@@ -506,7 +525,7 @@ class Context:
         for H, W in zip(Hs, Ws):
             assert H.dtype == torch.bfloat16 and W.dtype == torch.bfloat16 and H.shape[0] == T and W.shape[0] == V
             assert H.stride(1) == 1 and W.stride(1) == 1 and H.shape[1] == W.shape[1]
-        assert tokens.dtype == torch.int32
+        _check_rows(T, tokens, mask)
         self.ensure_workspace(T, max(W.shape[1] for W in Ws), V, scoring=True)
         dev = Ws[0].device
         logp = [torch.empty(T, dtype=torch.float32, device=dev) for _ in range(n)]
@@ -525,8 +544,9 @@ class Context:
         self._bind_stream()
         T, d = H.shape
         Vs = W_shard.shape[0]
-        assert H.dtype == torch.bfloat16 and W_shard.dtype == torch.bfloat16 and tokens.dtype == torch.int32
+        assert H.dtype == torch.bfloat16 and W_shard.dtype == torch.bfloat16
         assert H.stride(1) == 1 and W_shard.stride(1) == 1
+        _check_rows(T, tokens, mask)
         self.ensure_workspace(T, d, Vs, scoring=True)
         if stats is None:
             stats = torch.empty(T, 4, dtype=torch.float32, device=H.device)
@@ -557,8 +577,14 @@ class Context:
         self._bind_stream()
         T, d = H.shape
         Vs = W_shard.shape[0]
-        assert H.dtype == torch.bfloat16 and W_shard.dtype == torch.bfloat16 and tokens.dtype == torch.int32
+        assert H.dtype == torch.bfloat16 and W_shard.dtype == torch.bfloat16
         assert H.stride(1) == 1 and W_shard.stride(1) == 1
+        _check_rows(T, tokens, mask)
+        for x in (old_logp, ref_logp, adv, token_weight):
+            _check_array(x, T)
+        # dH of either type, whatever dH_fp32 says
+        _check_array(dH, T * d, dH.dtype if dH is not None and dH.dtype == torch.float32 else torch.bfloat16)
+        _check_array(dW, Vs * d)
         for x in (logp, entropy, lse):
             assert x.dtype == torch.float32 and x.is_contiguous() and x.numel() == T
         self.ensure_workspace(T, d, Vs)

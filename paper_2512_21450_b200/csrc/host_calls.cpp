@@ -73,10 +73,17 @@ struct Args {
     if (t && t->scalar_type() != type) throw General();
     return t;
   }
-  // [n] contiguous fp32
-  const at::Tensor* values(int64_t n, bool none_ok) {
-    const at::Tensor* t = of(at::kFloat, none_ok);
+  // [n] contiguous entries of a type
+  const at::Tensor* array(at::ScalarType type, int64_t n, bool none_ok) {
+    const at::Tensor* t = of(type, none_ok);
     if (t && (t->numel() != n || !t->is_contiguous())) throw General();
+    return t;
+  }
+  const at::Tensor* values(int64_t n, bool none_ok) { return array(at::kFloat, n, none_ok); }
+  // [n] one-byte entries or None
+  const at::Tensor* mask(int64_t n) {
+    const at::Tensor* t = tensor(true);
+    if (t && (t->element_size() != 1 || t->numel() != n || !t->is_contiguous())) throw General();
     return t;
   }
   // rows of bf16, contiguous within a row
@@ -166,11 +173,12 @@ PyObject* kl_shaped_returns(PyObject*, PyObject* const* args, Py_ssize_t nargs) 
     Args a(args, nargs, 11);
     rl_ctx* c = a.context();
     const at::Tensor* value = a.of(at::kFloat, false);
+    if (!value->is_contiguous()) throw General();
     Args peek = a;
     peek.i += 4;
     const int64_t T = peek.integer();
     if (T < 0) throw General();
-    const at::Tensor *logp = a.values(T, true), *ref = a.values(T, true), *mask = a.tensor(true), *offsets = a.of(at::kInt, false);
+    const at::Tensor *logp = a.values(T, true), *ref = a.values(T, true), *mask = a.mask(T), *offsets = a.of(at::kInt, false);
     ++a.i;
     const float beta = a.real(), gamma = a.real();
     const int kind = a.small();
@@ -179,6 +187,7 @@ PyObject* kl_shaped_returns(PyObject*, PyObject* const* args, Py_ssize_t nargs) 
     const uint8_t* pm = static_cast<const uint8_t*>(data<void>(mask));
     const int32_t* po = data<int32_t>(offsets);
     const int64_t n = offsets->numel() - 1;
+    if (value->numel() != n) throw General();
     Unlocked u;
     float *shaped = out.values(T, *value), *returns = out.values(T, *value);
     return abi.kl_shaped_returns(c, pv, pl, pr, pk, pm, po, n, T, beta, gamma, kind, shaped, returns);
@@ -195,8 +204,7 @@ PyObject* token_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     const int64_t T = logp->numel();
     if (!logp->is_contiguous()) throw General();
     const at::Tensor *ent = a.values(T, true), *old = a.values(T, true), *ref = a.values(T, true), *adv = a.values(T, true);
-    const at::Tensor* mask = a.of(at::kByte, true);
-    if (mask && mask->numel() != T) throw General();
+    const at::Tensor* mask = a.array(at::kByte, T, true);
     const float lo = a.real(), hi = a.real(), beta = a.real(), ec = a.real();
     const at::Tensor *weight = a.values(T, true), *count = a.of(at::kLong, true);
     const float *pl = data<float>(logp), *pe = data<float>(ent), *po = data<float>(old), *pr = data<float>(ref), *pa = data<float>(adv),
@@ -220,9 +228,10 @@ PyObject* token_logprobs(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   return guarded([&](Outputs& out) {
     Args a(args, nargs, 6);
     rl_ctx* c = a.context();
-    const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows(), *tokens = a.of(at::kInt, false), *mask = a.tensor(true);
+    const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows();
     const int64_t T = H->size(0), d = H->size(1), V = W->size(0);
     if (T == 0) throw General();
+    const at::Tensor *tokens = a.array(at::kInt, T, false), *mask = a.mask(T);
     bind_workspace(c, ws, abi.workspace_bytes_logprobs, T, d, V);
     const void *ph = H->data_ptr(), *pw = W->data_ptr();
     const int64_t ldH = H->stride(0), ldW = W->stride(0);
@@ -241,18 +250,19 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   return guarded([&](Outputs& out) {
     Args a(args, nargs, 23);
     rl_ctx* c = a.context();
-    const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows(), *tokens = a.of(at::kInt, false);
+    const at::Tensor *ws = a.tensor(true), *H = a.rows(), *W = a.rows();
     const int64_t T = H->size(0), d = H->size(1), V = W->size(0);
     if (T == 0) throw General();
-    const at::Tensor *old = a.tensor(false), *ref = a.tensor(true), *adv = a.tensor(false), *mask = a.tensor(true);
+    const at::Tensor *tokens = a.array(at::kInt, T, false), *old = a.values(T, false), *ref = a.values(T, true), *adv = a.values(T, false),
+                     *mask = a.mask(T);
     const float lo = a.real(), hi = a.real(), beta = a.real();
     rl_loss_opts o;
     memset(&o, 0, sizeof(o));
     o.struct_size = sizeof(o);
     o.ent_coef = a.real();
-    o.token_weight = data<float>(a.tensor(true));
+    o.token_weight = data<float>(a.values(T, true));
     o.accumulate_dW = a.integer() != 0;
-    const at::Tensor *dW = a.tensor(false), *dH = a.tensor(false), *loss = a.tensor(false);
+    const at::Tensor *dW = a.values(V * d, false), *dH = a.tensor(false), *loss = a.values(1, false);
     o.agg_mode = a.small();
     o.sequence_level = a.integer() != 0;
     const at::Tensor* offsets = a.of(at::kInt, true);
@@ -261,6 +271,7 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
       o.n_seq = offsets->numel() - 1;
     }
     o.dH_dtype = a.small();   // (the library says which values it knows)
+    if (dH->scalar_type() != (o.dH_dtype ? at::kFloat : at::kBFloat16) || dH->numel() != T * d || !dH->is_contiguous()) throw General();
     const at::Tensor* count = a.of(at::kLong, true);
     if (count && count->numel() != 1) throw General();
     o.token_count = data<int64_t>(count);
@@ -268,9 +279,9 @@ PyObject* policy_loss(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     const void *ph = H->data_ptr(), *pw = W->data_ptr();
     const int64_t ldH = H->stride(0), ldW = W->stride(0);
     const int32_t* pt = data<int32_t>(tokens);
-    const float *po = static_cast<float*>(data<void>(old)), *pr = static_cast<float*>(data<void>(ref)), *pa = static_cast<float*>(data<void>(adv));
+    const float *po = data<float>(old), *pr = data<float>(ref), *pa = data<float>(adv);
     const uint8_t* pm = static_cast<const uint8_t*>(data<void>(mask));
-    float *pl = static_cast<float*>(data<void>(loss)), *pd = static_cast<float*>(data<void>(dW));
+    float *pl = data<float>(loss), *pd = data<float>(dW);
     void* ph_out = data<void>(dH);
     Unlocked u;
     o.logp_out = out.values(T, *W);

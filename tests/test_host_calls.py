@@ -60,6 +60,51 @@ def test_unusual_arguments_are_left_to_the_general_path():
         assert out is NotImplemented
 
 
+def test_arrays_that_do_not_fit_their_call_are_refused(monkeypatch):
+    """Arrays are read and written by address: a short one, one of another type or with gaps would be read or written past."""
+    from paper_2512_21450_b200 import Context, binding
+
+    class Library:
+        def __getattr__(self, name):
+            return lambda *args: 0
+    monkeypatch.setattr(binding, "_host", _General())
+    c = Context.__new__(Context)
+    c.lib, c.handle, c._address, c._ws = Library(), None, 0, None
+    c._bind_stream, c.ensure_workspace = lambda: None, lambda *args, **kw: None
+    T, d, V = 12, 64, 300
+    H, W = torch.zeros(T, d, dtype=torch.bfloat16), torch.zeros(V, d, dtype=torch.bfloat16)
+    tok, x, mask, off = torch.zeros(T, dtype=torch.int32), torch.zeros(T), torch.ones(T, dtype=torch.uint8), torch.tensor([0, 5, T]).int()
+    gaps = torch.zeros(T, 2)[:, 0]
+    good = dict(tokens=tok, old_logp=x, ref_logp=x, adv=x, mask=mask, token_weight=x, loss=torch.zeros(1), dW=torch.zeros(V, d),
+                dH=torch.zeros(T, d, dtype=torch.bfloat16))
+
+    def loss(**kw):
+        a = dict(good, **kw)
+        fixed = [a.pop(k) for k in ("tokens", "old_logp", "ref_logp", "adv", "mask")]
+        return c.rl_policy_loss_fwd_bwd(H, W, *fixed, 0.2, 0.2, 0.04, **a)
+    # what was taken is taken: more than is needed, other shapes of as many entries, masks of any one-byte type, nothing at all
+    for kw in (dict(), dict(mask=mask.bool()), dict(mask=None, token_weight=None), dict(adv=torch.zeros(T + 3)), dict(old_logp=x.view(3, 4)),
+               dict(dW=torch.zeros(V * d), dH=torch.zeros(T + 4, d, dtype=torch.bfloat16)), dict(loss=None, dW=None, dH=None),
+               dict(dH=torch.zeros(T, d), dH_fp32=True)):
+        loss(**kw)
+    for kw in (dict(dH=torch.zeros(T, d, dtype=torch.bfloat16), dH_fp32=True), dict(dH=torch.zeros(T, d)), dict(dH=torch.zeros(T - 1, d).bfloat16()),
+               dict(dH=torch.zeros(d, T).bfloat16().t()), dict(dW=torch.zeros(V, d).bfloat16()), dict(dW=torch.zeros(V - 1, d)),
+               dict(dW=torch.zeros(d, V).t()), dict(loss=torch.zeros(1).double()), dict(adv=x.double()), dict(adv=x[:-1]), dict(adv=gaps),
+               dict(old_logp=gaps), dict(ref_logp=x[:-1]), dict(token_weight=x.double()), dict(token_weight=x[:1].expand(T)),
+               dict(mask=mask.int()), dict(mask=mask[:-1]), dict(tokens=tok[:-1]), dict(tokens=tok.long())):
+        with pytest.raises(AssertionError):
+            loss(**kw)
+    c.rl_token_logprobs(H, W, tok, mask.bool())
+    c.rl_kl_shaped_returns(x[:2], x, x, mask.bool(), off, T, 0.1)
+    for bad in (mask.float(), mask[:-1], torch.ones(T, 2, dtype=torch.uint8)[:, 0]):
+        with pytest.raises(AssertionError):
+            c.rl_token_logprobs(H, W, tok, bad)
+        with pytest.raises(AssertionError):
+            c.rl_kl_shaped_returns(x[:2], x, x, bad, off, T, 0.1)
+    with pytest.raises(AssertionError):
+        c.rl_kl_shaped_returns(x[:1], x, x, mask, off, T, 0.1)
+
+
 class _General:
     """Leaves every call to the general path."""
 
