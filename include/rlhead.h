@@ -512,8 +512,9 @@ rl_status rl_debug_workspace(int64_t T, int64_t d, int64_t V, int64_t d_ref, int
                              int64_t* bytes);
 
 /* Self-test of the bounded waits every kernel of this library uses: launches one warp that waits,
- * for at most limit_ms (1..1000) milliseconds, on a barrier nothing ever signals.  The kernel
- * returns by itself with RL_ERR_TIMEOUT latched (detail 0x70000000); rl_last_device_status()
+ * for at most limit_ms (1..1000) milliseconds each, on a barrier nothing ever signals, on a counter nothing adds to and on a
+ * word nothing raises.  The kernel returns by itself with RL_ERR_TIMEOUT latched (detail 0x70000000; a low bit is set for
+ * each wait that did not run out); rl_last_device_status()
  * reports and clears it and the context stays usable.  The paper has no counterpart. */
 rl_status rl_selftest_wait_timeout(rl_ctx* ctx, int limit_ms);
 

@@ -580,8 +580,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 // the chunks of A that this stage needs are there
                 const int need = fed0 + feed_chunks(kb0, min(kb + Cfg::kKSub, hi));
                 if (fed < need) {
-                  while (ok && (fed = *fed_p) < need) ok = !*abort_p;
-                  if (!ok) break;
+                  ok = word_wait_bounded(fed_p, need, fed, abort_p);
+                  if (!ok) {
+                    latch_status(status, kStatusTimeout, (1 << 28) | (blockIdx.x << 8) | 0xff);
+                    break;
+                  }
                   __threadfence_block();
                 }
               }

@@ -95,7 +95,7 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   return v;
 }
 // Until *p has reached n; bounded as the mbarrier waits are.
-__device__ __forceinline__ bool count_wait_bounded(const unsigned* p, unsigned n, volatile int* abort_flag) {
+__device__ __forceinline__ bool count_wait_bounded(const unsigned* p, unsigned n, volatile int* abort_flag, uint64_t limit_ns = kWaitLimitNs) {
   if (ld_acquire(p) >= n) return true;
   const uint64_t t0 = global_timer_ns();
   for (uint32_t it = 1;; ++it) {
@@ -103,7 +103,22 @@ __device__ __forceinline__ bool count_wait_bounded(const unsigned* p, unsigned n
     __nanosleep(64);
     if ((it & 63u) == 0u) {
       if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
+      if (global_timer_ns() - t0 > limit_ns) { *abort_flag = 1; return false; }
+    }
+  }
+}
+// Until *p, a word of shared memory that another warp raises, has reached n; `seen` is what it was.  That warp itself waits twice at
+// most (count_wait_bounded) before it raises the word by two.
+__device__ __forceinline__ bool word_wait_bounded(volatile int* p, int n, int& seen, volatile int* abort_flag,
+                                                  uint64_t limit_ns = 2 * kWaitLimitNs) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 1;; ++it) {
+    if ((seen = *p) >= n) return true;
+    if (*abort_flag) return false;
+    if ((it & 255u) == 0u) {
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit_ns) { *abort_flag = 1; return false; }
     }
   }
 }

@@ -1393,20 +1393,29 @@ struct EpiAccScatter : EpiAccW<W> {
 };
 
 // ------------------------------------------------------------------------------------------
-// Exercises the bounded wait: one warp waits on an mbarrier that nothing ever arrives on, with a
-// short limit, and must come back with the timeout latched instead of spinning forever.
+// Exercises the bounded waits, each with a short limit: on an mbarrier that nothing ever arrives on, on a counter in global memory and
+// on a word in shared memory that nobody raises.  Each must come back with the abort flag raised; the detail's low bits name those that did not.
+__device__ unsigned g_never_counted;
 __global__ void __launch_bounds__(32) wait_timeout_probe_kernel(unsigned long long limit_ns, DevStatus* st) {
   __shared__ __align__(8) uint64_t bar;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, word;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
-    abort_flag = 0;
+    word = 0;
     fence_mbar_init();
   }
   __syncwarp();
-  volatile int* abort_p = &abort_flag;
   if (threadIdx.x == 0) {
-    if (!mbar_wait_bounded(smem_u32(&bar), 0, abort_p, limit_ns)) latch_status(st, kStatusTimeout, 0x70000000);
+    volatile int *abort_p = &abort_flag, *word_p = &word;
+    int kept = 0, seen;
+    auto runs_out = [&](int bit, auto wait) {
+      *abort_p = 0;
+      if (wait() || *abort_p != 1) kept |= bit;
+    };
+    runs_out(1, [&] { return mbar_wait_bounded(smem_u32(&bar), 0, abort_p, limit_ns); });
+    runs_out(2, [&] { return count_wait_bounded(&g_never_counted, 1, abort_p, limit_ns); });
+    runs_out(4, [&] { return word_wait_bounded(word_p, 1, seen, abort_p, limit_ns); });
+    latch_status(st, kStatusTimeout, 0x70000000 | kept);
   }
   __syncwarp();
 }

@@ -865,7 +865,8 @@ def test_calls_can_be_captured_in_a_cuda_graph():
 
 
 def test_bounded_wait_times_out_cleanly(ctx):
-    # a wait that nothing satisfies ends by itself, reports RL_ERR_TIMEOUT and leaves the context usable
+    # a wait that nothing satisfies (mbarrier, counter, word: low bits for those that did not run out) ends by itself, reports
+    # RL_ERR_TIMEOUT and leaves the context usable
     import time
     from paper_2512_21450_b200.workloads import make_workload
     t0 = time.time()
@@ -873,6 +874,7 @@ def test_bounded_wait_times_out_cleanly(ctx):
     s, detail = ctx.last_device_status()
     assert s == 8 and (detail & 0xffffffff) == 0x70000000
     assert time.time() - t0 < 5.0
+    assert time.time() - t0 > 0.06                    # three waits of 20 ms
     assert ctx.last_device_status()[0] == 0           # cleared
     w = make_workload(0, seed=71)
     lp, _, _ = ctx.rl_token_logprobs(w.H, w.W, w.tokens, w.mask)
