@@ -105,11 +105,28 @@ def test_arrays_that_do_not_fit_their_call_are_refused(monkeypatch):
         c.rl_kl_shaped_returns(x[:1], x, x, mask, off, T, 0.1)
 
 
+_CALLS = ("grpo_advantages", "kl_shaped_returns", "token_loss", "token_logprobs", "policy_loss")
+
+
 class _General:
     """Leaves every call to the general path."""
 
     def __getattr__(self, name):
         return lambda *args: NotImplemented
+
+
+class _Recorder:
+    """Passes calls on and notes which of them were handled."""
+
+    def __init__(self, host):
+        self.host, self.seen = host, []
+
+    def __getattr__(self, name):
+        def call(*args):
+            out = getattr(self.host, name)(*args)
+            self.seen.append((name, out is not NotImplemented))
+            return out
+        return call
 
 
 @pytest.mark.gpu
@@ -134,8 +151,8 @@ def test_native_and_general_paths_agree(monkeypatch, opt):
     beta = opt.get("beta", 0.04)
     out = []
     for native in (True, False):
-        if not native:
-            monkeypatch.setattr(binding, "_host", _General())
+        recorder = _Recorder(_host()) if native else _General()
+        monkeypatch.setattr(binding, "_host", recorder)
         c = Context(0)
         try:
             got = {}
@@ -153,6 +170,10 @@ def test_native_and_general_paths_agree(monkeypatch, opt):
                 got.update(c.rl_policy_loss_fwd_bwd(H, W, tok, old, ref if beta else None, adv, mask, 0.2, 0.3, beta, dW=dW, dH=dH,
                                                     loss=torch.zeros(1, device="cuda"), seq_offsets=off, token_weight=weight,
                                                     token_count=count, **kw))
+                if native:
+                    handled, recorder.seen = recorder.seen, []
+            if native:   # each of the five once, and none was left to the general path
+                assert sorted(handled) == [(name, True) for name in sorted(_CALLS)]
             # what the library refuses is refused alike
             with pytest.raises(binding.RLHeadError, match="rl_token_loss"):
                 c.rl_token_loss(logp, ent, old, None, adv, mask, 0.2, 0.3, 0.04)
@@ -173,6 +194,57 @@ def test_native_and_general_paths_agree(monkeypatch, opt):
     assert out[0].keys() == out[1].keys()
     for k in out[0]:
         assert out[0][k].dtype == out[1][k].dtype and out[0][k].shape == out[1][k].shape and torch.equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.gpu
+def test_one_unusual_argument_leaves_the_call_to_the_general_path():
+    """Each from a call that is handled, by changing one argument."""
+    import numpy as np
+    from paper_2512_21450_b200 import Context
+
+    class Sub(torch.Tensor):
+        pass
+    T, d, V, n = 60, 64, 300, 6
+    x = -torch.rand(T, device="cuda") - 1
+    gaps = torch.zeros(T, 2, device="cuda")[:, 0]
+    H, W = torch.randn(T, d, device="cuda").bfloat16(), torch.randn(V, d, device="cuda").bfloat16()
+    tok, mask = torch.zeros(T, dtype=torch.int32, device="cuda"), torch.ones(T, dtype=torch.uint8, device="cuda")
+    off, rewards = torch.arange(0, T + 1, 10, dtype=torch.int32, device="cuda"), torch.rand(n, device="cuda")
+    count = torch.tensor([T], device="cuda")
+    dH, dW, loss = torch.zeros(T, d, device="cuda", dtype=torch.bfloat16), torch.zeros(V, d, device="cuda"), torch.zeros(1, device="cuda")
+    c = Context(0)
+    try:
+        c.ensure_workspace(T, d, V)
+        c._bind_stream()
+        a, ws = c._address, c._ws
+        good = dict(grpo_advantages=[a, rewards, 3, 1, 1e-6, off, T],
+                    kl_shaped_returns=[a, rewards, x, x, mask, off, T, 0.1, 1.0, 1, None],
+                    token_loss=[a, x, x, x, x, x, mask, 0.2, 0.2, 0.04, 0.01, x, count],
+                    token_logprobs=[a, ws, H, W, tok, mask],
+                    policy_loss=[a, ws, H, W, tok, x, x, x, mask, 0.2, 0.2, 0.04, 0.01, x, False, dW, dH, loss, 1, False, off, False, count])
+        bad = dict(
+            grpo_advantages=[(0, 2 ** 70), (1, rewards.double()), (1, rewards.cpu()), (1, rewards[::2]), (1, None), (2, np.int64(3)),
+                             (2, 2 ** 40), (3, 1.0), (4, np.float64(1e-6)), (5, off.long()), (6, None), (6, -1)],
+            kl_shaped_returns=[(1, rewards.double()), (1, rewards[:5]), (2, x[:-1]), (3, gaps), (4, mask.int()), (4, mask[:-1]), (5, off.long()),
+                               (6, None), (6, -1), (7, "0.1"), (9, None), (10, x.double())],
+            token_loss=[(1, "x"), (1, x.as_subclass(Sub)), (1, x.double()), (1, gaps), (2, x[:-1]), (3, x.cpu()), (6, mask.bool()),
+                        (6, mask[:-1]), (7, np.float32(0.2)), (7, None), (8, 10 ** 400), (11, x.double()), (12, count.int())],
+            token_logprobs=[(1, None), (1, ws[:16]), (2, H.float()), (2, H.t().contiguous().t()), (2, H[:0]), (2, H[0]), (3, W.cpu()),
+                            (4, tok.long()), (4, tok[:-1]), (5, mask[:-1]), (5, mask.int())],
+            policy_loss=[(1, ws[:16]), (2, H[:0]), (4, tok[:-1]), (5, None), (5, x.double()), (6, gaps), (7, x[:-1]), (8, mask[:-1]), (9, "0.2"),
+                         (13, x.double()), (14, "no"), (15, dW[:-1]), (15, dW.bfloat16()), (15, None), (16, dH.float()), (16, dH[:-1]),
+                         (16, dH.t().contiguous().t()), (17, loss.double()), (18, 1.5), (19, None), (20, off.long()), (21, True),
+                         (22, count.int()), (22, count.repeat(2))])
+        for name in _CALLS:
+            call = getattr(_host(), name)
+            assert type(call(*good[name])) is tuple, name
+            assert call(*good[name][:-1]) is NotImplemented, name
+            for i, value in bad[name]:
+                assert call(*[value if k == i else v for k, v in enumerate(good[name])]) is NotImplemented, (name, i, value)
+        torch.cuda.synchronize()
+        assert c.last_device_status()[0] == 0
+    finally:
+        c.close()
 
 
 # A device allocator that counts its calls, and those made by a thread that holds the interpreter's lock
