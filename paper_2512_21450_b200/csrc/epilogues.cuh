@@ -366,7 +366,7 @@ struct EpiGrad {
 struct AccParams {
   int n_cols;
   int accumulate;  // 0 store, 1 add, 2 (slabs walked from the last to the first): add unless this is the last slab that has rows
-  const int* n_valid;                      // 2 only
+  const int* n_valid;                      // 2, and where side warps write dH (EpiAccScatter)
   int slab_cap, slab_one, slab_index;
   int row_base;
   int slice_add;   // stream-K launches: output slices past the first are always added to
@@ -436,6 +436,7 @@ struct EpiAccW {
     st.n_issued++;
   }
   __device__ static __forceinline__ void end_unit(const Params&, State&, int, int, int, int) {}
-};using EpiAcc = EpiAccW<4>;
+};
+using EpiAcc = EpiAccW<4>;
 
 }  // namespace rlh

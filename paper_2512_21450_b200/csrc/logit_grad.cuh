@@ -5,7 +5,8 @@
 // written in place of the policy logits' upper halves; rows past the slab's valid rows (up to a multiple of 128) and
 // columns past V become zero.  4 bytes in (8 with the KL) and 2 out per entry, nothing read twice: bound by memory.
 // The work is done by extra warps of the dH kernel (EpiAccFed), which read and write DRAM while the tensor cores
-// multiply what they have finished, or by a kernel of its own (logit_grad_kernel) where dH does not come next.
+// multiply what they have finished, or by a kernel of its own (logit_grad_kernel) where dH does not come next, where that does
+// not pay (feed_pays) and with the full KL.
 #pragma once
 #include <type_traits>
 
@@ -45,8 +46,8 @@ inline size_t feed_words(long long rows, long long ld) {
 // Whether dH pays for forming its operand itself, known once the rows are counted.  While its tiles run in whole waves, and
 // where helpers are many or none; a few helpers ask for the ends of nearly all tiles at once, beside the parts, and where
 // parts are many and short the start shows.  A whole step,
-// apart against fed, sustained at the board's power limit, d = 2048: 4.71 / 5.93 / 7.78 / 9.09 / 11.06 ms against 4.51 / 5.90 / 7.60 /
-// 8.82 / 10.75 at 2600 / 3500 / 4864 / 5632 / 6912 rows (30, 18 helpers, waves), but 3.40 / 6.66 against 3.51 / 6.78 at 2000 /
+// apart against fed, sustained at the board's power limit, d = 2048: 4.71 / 7.78 / 9.09 / 11.06 ms against 4.51 / 7.60 / 8.82 / 10.75 at
+// 2600 / 4864 / 5632 / 6912 rows (30 helpers, waves), level at 3500 (18 helpers: 5.93 / 5.90), but 3.40 / 6.66 against 3.51 / 6.78 at 2000 /
 // 4096 (10 helpers); 45.3 against 44.4 at 16896 rows, d = 3584; 16.41 against 16.12 at 16896 rows, d = 1024; in 6 parts 1.49 against 1.47 at
 // 1000 rows, d = 1536, in 9 and 12 1.24 against 1.26 at 447, d = 2048, and 0.89 against 0.90 at 700, d = 1024.
 __host__ __device__ inline bool feed_pays(const GemmExtents& ex, int n_workers) {
@@ -316,7 +317,7 @@ struct LogitGradWarp {
   }
 };
 
-// dH of one slab while its operand G is still being formed: kFeedWarps warps of every CTA do the jobs of LogitGradWarp, the
+// dH of one slab while its operand G is still being formed: kSideWarps warps of every CTA do the jobs of LogitGradWarp, the
 // producer waits for the chunks it is about to load.
 struct EpiAccFed : EpiAcc {
   static constexpr int kSideWarps = 9;   // with the one that watches, sixteen warps in all: 128 registers a thread
