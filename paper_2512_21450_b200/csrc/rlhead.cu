@@ -138,6 +138,17 @@ inline bool use_wide(const rl_ctx* c, int64_t d) {
 }
 // Rows of a call up to which dW runs with eight epilogue warps (EpiAccW; how many of them are valid only the device knows).
 constexpr int64_t kFewRows = 640;
+// Whether dW's launch writes dH to the caller's rows as well (EpiAccScatter), or a launch of its own behind it does.  Four warps a CTA
+// copy at 1.5 TB/s, a launch of its own at 4.7; beside, the copy is hidden as far as dW lasts, which is as long as the waves of its
+// tiles: with few words and many columns it ends first.  Per row dW takes 7 ns a wave, a copy beside it 4.1 ps a column, one behind it
+// 1.3: level near 2500 columns a wave.  A call, beside against behind: d = 3584, 16384 rows, 256 / 600 / 1000 / 1500 / 2000 words (1, 1, 1, 2,
+// 2 waves) 487 / 560 / 592 / 708 / 826 us against 441 / 512 / 541 / 723 / 845, d = 4096, 1000 / 2000 / 3000 (1, 2, 3) 746 / 1008 / 1263 against
+// 675 / 999 / 1318, d = 2048, 8192 rows, 256 / 1000 142 / 182 against 158 / 190.  Up to a thousand rows the launch saved is worth as much.
+inline bool dH_beside_dW(const rl_ctx* c, int64_t T, int64_t d, int64_t cols) {
+  const int64_t tiles = (d + BN - 1) / BN * ((cols + BN - 1) / BN) * 2;   // of 128 rows
+  const int64_t waves = (tiles + c->grid[c->cta_group] - 1) / c->grid[c->cta_group];
+  return T <= 1024 || d < 2000 * waves + 64;
+}
 // Width of a dH tile, and bytes of the slots its parts may need (two per worker).
 inline int dh_tile_cols(const rl_ctx* c, int64_t d) { return use_wide(c, d) ? 2 * BN : BN; }
 inline size_t dh_slot_bytes(const rl_ctx* c, int64_t d) {
@@ -1355,6 +1366,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
   const int n_col_slabs = (int)((V + L.Vs - 1) / L.Vs);
   const int d_tiles = (int)((d + BN - 1) / BN);
   int hook_slab = 0;
+  const bool dH_beside = dH_beside_dW(c, T, d, V - (int64_t)(n_col_slabs - 1) * L.Vs);
   // Slabs are sized for T rows, and how many of them have any is known to the device alone.  Whoever wants to be told as rows of dW
   // are completed has them walked from the last to the first, so that the one that completes them has rows: its dW launches, in
   // pieces and before its dH, are what is told about while they and dH still run.
@@ -1549,7 +1561,7 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
         ep.n_cols = (int)d; ep.accumulate = o.accumulate_dW ? 1 : reverse ? 2 : (r > 0 ? 1 : 0);
         ep.n_valid = n_valid; ep.slab_cap = L.Tc; ep.slab_one = L.Ts; ep.slab_index = r;
         ep.row_base = vocab_base + c0; ep.slice_add = 0; ep.tile_cols = 0;
-        if (!report && cs == n_col_slabs - 1) {
+        if (dH_beside && !report && cs == n_col_slabs - 1) {
           src.shape = dh_shape;
           auto dW_and_dH = [&](auto epi) {
             typename decltype(epi)::Params es = {};
@@ -1572,8 +1584,8 @@ static rl_status loss_fwd_bwd_impl(rl_ctx* c, const void* H, int64_t ldH, const 
       }
       if (report) launch_dH();
     }
-    // dW of the last column slab has written dH in passing, unless it came before dH
-    if (c->dw_hook && q == n_row_slabs - 1) {
+    // dW of the last column slab has written dH in passing, unless it came before dH or is too short for that
+    if (!dH_beside || (c->dw_hook && q == n_row_slabs - 1)) {
       src.shape = dh_shape;
       const int pr_sc = prof_begin(c, 7);
       launch(c, scatter_dH_kernel, c->n_sm * 8, 256, src, c->dstatus);

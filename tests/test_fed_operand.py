@@ -95,3 +95,50 @@ def test_fed_matches_a_launch_of_its_own(T, d, V, kw, fed):
         a, b = out[False]["dW"], out[True]["dW"]
         assert float((a - b).norm() / b.norm()) < 1e-6   # fp32 sums of three addends in another order
     assert torch.isfinite(out[False]["dH"].float()).all() and torch.isfinite(out[False]["dW"]).all()
+
+
+# dH to the caller's rows beside dW, or by a launch of its own where dW's tiles are few and rows long: the last size on either side of
+# the rule in words, in columns and in rows, and several column slabs of which the last is narrow
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,d,V,kw,beside", [
+    (1025, 2048, 300, {}, True), (1025, 2112, 300, {}, False), (1024, 2112, 300, {}, True), (1100, 2112, 2048, {}, False), (1100, 2112, 2100, {}, True),
+    (1300, 2112, 700, dict(cta_group=1), False), (1300, 2304, 700, dict(fp32=True), False), (3000, 2304, 1300, dict(limits=(1024, 1024)), False),
+])
+def test_dH_beside_dW_or_behind(T, d, V, kw, beside):
+    import torch
+    from paper_2512_21450_b200 import Context
+    g = torch.Generator(device="cuda").manual_seed(T + d + V)
+    H = torch.randn(T, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    W = torch.randn(V, d, generator=g, device="cuda", dtype=torch.bfloat16) * 0.02
+    tok = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    old = -torch.rand(T, generator=g, device="cuda") - 5
+    adv = torch.randn(T, generator=g, device="cuda")
+    mask = (torch.rand(T, generator=g, device="cuda") >= 0.2).to(torch.uint8)
+    fp32 = kw.get("fp32", False)
+    out, behind = {}, {}
+    for hook in (False, True):
+        c = Context(0)
+        try:
+            c.set_cta_group(kw.get("cta_group", 2))
+            if "limits" in kw:
+                c.set_slab_limits(*kw["limits"])
+            if hook:   # dW of the slab that is walked last comes before its dH, which then has a launch of its own
+                c.set_dw_slab_hook(lambda slab_index, lo, hi: None)
+            c.set_profiling(True)
+            o = c.rl_policy_loss_fwd_bwd(H, W, tok, old, old, adv, mask, 0.2, 0.2, 0.04, dH_fp32=fp32,
+                                         dH=torch.full((T, d), float("nan"), device="cuda", dtype=torch.float32 if fp32 else torch.bfloat16))
+            behind[hook] = c.profile_read()[1][7]
+            assert c.last_device_status()[0] == 0
+            out[hook] = o
+        finally:
+            c.close()
+    slabs = -(-T // kw["limits"][0]) if "limits" in kw else 1
+    assert behind[False] == (0 if beside else slabs) and behind[True] == (1 if beside else slabs)
+    assert torch.equal(out[False]["dH"], out[True]["dH"]) and bool(torch.isfinite(out[False]["dH"].float()).all())
+    p = torch.softmax(H.float() @ W.float().t(), 1)
+    # dH = G W with G's rows proportional to p - onehot(token) (no entropy term): the direction of every row
+    ref = (p - torch.nn.functional.one_hot(tok.long(), V)) @ W.float()
+    cos = torch.nn.functional.cosine_similarity(out[False]["dH"].float(), ref, dim=1).abs()
+    rows = (mask == 1) & (out[False]["dH"].float().norm(dim=1) > 0)
+    assert int(rows.sum()) > 0.5 * T and float(cos[rows].min()) > 0.999
+    assert float(out[False]["dH"][mask == 0].float().abs().max()) == 0.0
