@@ -136,7 +136,10 @@ inline bool use_wide(const rl_ctx* c, int64_t d) {
   const int64_t wide = (d + 2 * BN - 1) / (2 * BN) * 2, square = (d + BN - 1) / BN;
   return c->wide_tiles && c->cta_group == 2 && wide * kWideGain <= square * 100;
 }
-// Rows of a call up to which dW runs with eight epilogue warps (EpiAccW; how many of them are valid only the device knows).
+// Rows of a call up to which dW runs with eight epilogue warps (EpiAccW).  dW of 151936 words, d = 2048, four warps against eight, adding
+// 577 / 449, 602 / 517, 604 / 572, 634 / 641 us at 300 / 512 / 640 / 768 rows, storing 368 / 336, 414 / 419, 515 / 504, 519 / 535; d = 3584, adding
+// 1021 / 845, 1059 / 925, 1047 / 1018, 1112 / 1099: level at 700.  By the rows of the call, since how many are valid only the device knows: 300 valid
+// rows among 1024 keep four (600 against 474 us adding).
 constexpr int64_t kFewRows = 640;
 // Whether dW's launch writes dH to the caller's rows as well (EpiAccScatter), or a launch of its own behind it does.  Four warps a CTA
 // copy at 1.5 TB/s, a launch of its own at 4.7; beside, the copy is hidden as far as dW lasts, which is as long as the waves of its
